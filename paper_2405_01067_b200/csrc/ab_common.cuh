@@ -179,16 +179,35 @@ struct SvdItem {
 size_t svd_batch_ws(const SvdItem* items, int L);
 int svd_batch(const SvdItem* items, int L, float sigma_cutoff, void* ws, size_t ws_bytes, cudaStream_t st);
 
+// ---- direct symmetric eigensolver (ab_eig.cu) ---------------------------------------------------
+// Leading eigenvectors of `count` symmetric matrices of order s <= kEigSmallMax, fp64 inside.  Everything an EigJob
+// points to is device memory; eig_bind carves the scratch of one matrix (eig_ws_doubles(s) doubles).
+constexpr int kEigSmallMax = 256;
+struct EigJob {
+  const float* X;     // s x s, row stride s
+  int gram;           // 0: the matrix is X (symmetric); 1: it is X^T X, formed in fp64 from X
+  int s, need;        // order; how many eigenvectors are wanted
+  float* rows;        // need x s: unit rows, descending eigenvalue
+  float* vals;        // need: the eigenvalue (gram 0) or its square root, 0 below 1e-6 of the largest (gram 1); may be null
+  int* flag;          // set to 1 when close vectors came out less than orthogonal (the caller clears it)
+  double *refl, *zp, *zm, *d, *e, *gam, *lam, *inv, *cross, *norm;
+};
+size_t eig_ws_doubles(int s);
+void eig_bind(EigJob& j, double* ws);
+// status: device int that receives AB_ERR_TIMEOUT if a bounded wait ran out
+int eig_direct(const EigJob* d_jobs, int count, int smax, int* status, cudaStream_t st);
+
 // ---- factored group sync (ab_sync_fast.cu) ------------------------------------------------------
 // One-sided Jacobi on the rows of `count` s x s matrices (s <= 256) kept in shared memory, one CTA or
 // one cluster of CTAs per matrix (ab_sync_fast.cu).  X: count matrices, s * s apart.  rows: the
 // orthogonalised rows scaled to unit length, sorted by descending norm; norms: those norms.  status:
 // one int per matrix, status_stride_bytes apart (AB_OK / AB_ERR_NOT_CONVERGED).  scratch: device memory
-// of rows_jacobi_scratch_bytes(count).
+// of rows_jacobi_scratch_bytes(count).  flags: one int per matrix in device memory; a matrix whose flag is zero is
+// left alone.
 bool rows_jacobi_fits(int count, int s);
 size_t rows_jacobi_scratch_bytes(int count);
-int rows_jacobi(const float* X, float* rows, float* norms, int* status, size_t status_stride_bytes, int count, int s,
-                void* scratch, cudaStream_t st);
+int rows_jacobi(const float* X, float* rows, float* norms, int* status, size_t status_stride_bytes, const int* flags,
+                int count, int s, void* scratch, cudaStream_t st);
 bool sync_factored_supported(const ab_sync_desc* d, int L);
 size_t sync_factored_ws(const ab_sync_desc* d, int L);
 int sync_factored(const ab_sync_desc* d, int L, int K, float sigma_cutoff, int dt, int* dev_status,

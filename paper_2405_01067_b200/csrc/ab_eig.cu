@@ -1,0 +1,845 @@
+// Direct eigensolver for symmetric matrices, batched: the r x r core of the factored group synchronisation and
+// the Gram matrices of the dense split (short side up to kEigSmallMax).
+//
+//   1. tridiag_small_kernel : Householder reduction C = H T H^T (a cluster of CTAs per matrix, C in registers)
+//   2. tri_values_kernel    : eigenvalues of T, multisection on Sturm counts
+//   3. tri_vectors_kernel   : eigenvectors of T, twisted factorisation at each eigenvalue
+//   4. back_transform_kernel: u = H z, rows sorted by descending eigenvalue, rounded to fp32
+//
+// Everything up to the last rounding is fp64.  C = M^T M is formed in fp64 from the fp32 matrix M, so an
+// eigenvalue carries an absolute error of 1e-16 of the largest and squaring costs no accuracy: a singular value
+// of 1 % of the largest is good to 1e-12 before it is rounded to fp32.
+//
+// Why not the one-sided Jacobi that this replaces (it stays as the fallback, see below): its sweeps are chains of
+// dependent steps -- s - 1 rounds a sweep, eight to thirteen sweeps, every step a dot product, a reduction across a warp, a
+// rotation and a write-back -- while the reduction to tridiagonal form has s - 2 steps in all.
+//
+// Vectors of eigenvalues that are closer than about 1e-10 of the norm and not separated by a zero off-diagonal
+// come out of step 3 less than orthogonal.  Step 4 checks every pair that is close and raises the matrix's flag
+// when a pair fails; the caller then runs the Jacobi route for that matrix (a kernel that returns at once when
+// the flag is clear).
+#include <cooperative_groups.h>
+
+#include <algorithm>
+
+#include "ab_common.cuh"
+#include "ab_tc_ptx.cuh"
+
+namespace ab {
+namespace {
+
+namespace cg = cooperative_groups;
+
+constexpr double kSplitRel = 2.3e-16;   // an off-diagonal below this fraction of the norm splits T
+constexpr double kCloseRel = 1e-7;      // eigenvalues closer than this fraction of the norm are checked for orthogonality
+constexpr double kOrthTol = 1e-6;
+constexpr int kGroup = 4;               // reflectors applied together in the back transform
+
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+__device__ __forceinline__ uint32_t map_rank(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+// 16 bytes to a CTA of the cluster; its barrier counts them.
+__device__ __forceinline__ void st_async(uint32_t addr, double x, double y, uint32_t bar) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f64 [%0], {%1, %2}, [%3];" ::"r"(addr), "d"(x), "d"(y),
+               "r"(bar)
+               : "memory");
+}
+
+// ---- 1. Householder reduction ---------------------------------------------------------------------------
+// The matrix lives in registers: element (i, k) in warp i mod (warps of the cluster), lane k mod 32, so a warp
+// holds R whole rows, E elements of each per lane.  Step j:
+//   - warp 0 of each CTA has received p = A v of the reflector before (v, gamma) and column j of
+//     the matrix as it was before that reflector's update;  w = gamma p - (gamma^2 p.v / 2) v;  it works out column j of the
+//     updated matrix and the next reflector v', and hands w and v' to the other warps;
+//   - all warps pass over their rows in registers: A -= v w^T + w v^T, p' = A v';  every row's p'_i and A[i][j+1] go
+//     to warp 0 of every CTA of the cluster.
+// So the rank-two update and the product with the next vector touch an element once, and a step is a chain of two
+// warp reductions, a square root, the pass and one exchange.  The vectors are worked out by one warp because fp64 issues
+// at half rate: with every warp doing it for itself (no hand-over) the copies took more issue slots than the pass (8100 cycles a step
+// at order 192).  Finished 32-column groups are dropped at compile time (segment<E0>).
+// The exchange is st.async onto an mbarrier of each receiver (two, used in turn): the data carry their own
+// completion.  With a cluster barrier in its place, whose release also waits for the step's global stores, a step
+// of order 256 (8 CTAs) took 2.6 us against 1.9 us.  A CTA may overwrite a peer's buffer of step j once it has everything of step
+// j + 1 from that peer: warp 0 of each CTA sends a 16-byte token once it has read its buffer.
+// Where the matrix fits one CTA (kSingle) plain shared memory and named barriers take the place of the exchange.
+constexpr int kMaxCl = 8;
+
+__device__ __forceinline__ void bar_arrive(int id, int threads) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+
+template <int E, int R, int W, bool kSingle>
+struct Tridiag {
+  static_assert(R % 4 == 0, "rows go through the warp reduction in fours");
+  static constexpr int S = 32 * E;
+  static constexpr int kChunk = 16;
+  static constexpr int kThreads = 32 * W;
+  struct Shared {
+    double2 pa[2][S + kMaxCl];   // p and the next column; behind them the peers' tokens
+    double2 stage_or_col[kChunk * S / 2];   // start: rows of X as fp64; afterwards each row warp's piece of column j + 1
+    double v[2][S], w[S];
+    uint64_t bar[2];
+    int dead;
+  };
+
+  Shared& sh;
+  const EigJob& job;
+  int s, CL, rank, warp, lane;
+  int* status;
+
+  struct Rows { double A[R][E]; double v[E]; double gam, v1; bool ok; uint32_t dst, dbar; };
+
+  // Warp 0, step j: from p and the column to w and the next reflector (left in shared memory).  Returns through vn,
+  // dj, beta what is to be stored, through nrm, alpha what gamma follows from.
+  template <int E0>
+  __device__ __forceinline__ void vec_step(Rows& x, int j, double (&vn)[E], double& dj, double& beta, double& den) {
+    const int par = j & 1;
+    if constexpr (kSingle) tc::named_bar_sync(2, kThreads);
+    else x.ok = x.ok && tc::mbar_wait(&sh.bar[par], (j >> 1) & 1);
+    const double2* pb = sh.pa[par];
+    double w[E], pv = 0.0;
+#pragma unroll
+    for (int e = E0; e < E; ++e) {
+      const double2 q = pb[lane + 32 * e];
+      w[e] = q.x; vn[e] = q.y;
+    }
+    const int j1 = j + 1 < s ? j + 1 : j;
+    const double2 qj = pb[j], qj1 = pb[j1];
+    const double vj1 = sh.v[par][j1];
+#pragma unroll
+    for (int e = E0; e < E; ++e) pv = fma(w[e], x.v[e], pv);
+    pv = warp_sum(pv);
+    const double c = 0.5 * x.gam * x.gam * pv;
+    const double wj = x.gam * qj.x - c * x.v1;
+    double sq = 0.0;
+#pragma unroll
+    for (int e = E0; e < E; ++e) {
+      w[e] = x.gam * w[e] - c * x.v[e];
+      vn[e] = vn[e] - x.v1 * w[e] - wj * x.v[e];
+      if (e <= E0 + 1 && lane + 32 * e <= j + 1) vn[e] = 0.0;
+      sq = fma(vn[e], vn[e], sq);
+      sh.w[lane + 32 * e] = w[e];
+    }
+    sq = warp_sum(sq);
+    dj = qj.y - 2.0 * x.v1 * wj;
+    const double alpha = (j + 1 < s) ? qj1.y - x.v1 * (x.gam * qj1.x - c * vj1) - wj * vj1 : 0.0;
+    const bool live = sq > 0.0;
+    const double nrm = sqrt(fma(alpha, alpha, sq));
+    beta = live ? (alpha > 0.0 ? -nrm : nrm) : alpha;
+    x.v1 = live ? alpha - beta : 0.0;
+    den = live ? nrm * (nrm + fabs(alpha)) : 0.0;
+#pragma unroll
+    for (int e = E0; e < E; ++e) {
+      if (e <= E0 + 1 && lane + 32 * e == j + 1) vn[e] = x.v1;
+      sh.v[par ^ 1][lane + 32 * e] = vn[e];
+    }
+    if constexpr (!kSingle) {
+      if (lane == 0 && !x.ok) sh.dead = 1;                 // a peer never answered: all warps leave
+      if (x.ok && j + 1 < s) open_step(par ^ 1, s - 1 - j);
+    }
+  }
+  // opens the barrier of buffer buf for the bytes of a step with n live rows; the token says that this CTA has
+  // read the buffer of the step before
+  __device__ __forceinline__ void open_step(int buf, int n) {
+    if (lane == 0) tc::mbar_arrive_expect_tx(&sh.bar[buf], (uint32_t)(16 * (n + CL)));
+    if (lane < CL) st_async(map_rank(tc::smem_u32(&sh.pa[buf][S + rank]), lane), 0.0, 0.0, map_rank(tc::smem_u32(&sh.bar[buf]), lane));
+  }
+
+  __device__ __forceinline__ void send(const Rows& x, int buf, int row, double p, double a) {
+    if constexpr (kSingle) {
+      if ((lane & 7) == 0) sh.pa[buf][row] = make_double2(p, a);
+    } else {
+      if ((lane & 7) < CL) st_async(x.dst + (uint32_t)((buf * (S + kMaxCl) + row) * 16), p, a, x.dbar + (uint32_t)(buf * 8));
+    }
+  }
+  // steps whose first live column lies in the 32-column group E0; groups before it are finished
+  template <int E0>
+  __device__ __forceinline__ void segment(Rows& x) {
+    const int gw = rank * W + warp, gs = CL * W;
+    double* col = reinterpret_cast<double*>(sh.stage_or_col) + warp * R;
+    const int jend = min(32 * E0 + 32, s);
+    for (int j = 32 * E0; j < jend; ++j) {
+      const int par = j & 1;
+      double w[E], vn[E], dj = 0.0, beta = 0.0, den = 0.0;
+      if (warp == 0) vec_step<E0>(x, j, vn, dj, beta, den);
+      tc::named_bar_sync(1, kThreads);               // w and v' are there
+      if constexpr (!kSingle) {
+        if (*reinterpret_cast<volatile int*>(&sh.dead)) return;
+      }
+      if (gw + gs * (R - 1) > j) {                   // this warp still has a live row
+#pragma unroll
+        for (int e = E0; e < E; ++e) {
+          w[e] = sh.w[lane + 32 * e];
+          vn[e] = sh.v[par ^ 1][lane + 32 * e];
+        }
+#pragma unroll
+        for (int g = 0; g < R / 4; ++g) {
+          if (gw + gs * (4 * g + 3) <= j) continue;  // rows of a live group that are finished are updated for nothing
+          double ps[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const int r = 4 * g + q;
+            const int i = min(gw + gs * r, S - 1);
+            const double vi = sh.v[par][i], wi = sh.w[i];
+            double acc = 0.0;
+#pragma unroll
+            for (int e = E0; e < E; ++e) {
+              x.A[r][e] = fma(-vi, w[e], fma(-wi, x.v[e], x.A[r][e]));
+              acc = fma(x.A[r][e], vn[e], acc);
+            }
+            ps[q] = acc;
+          }
+          if (lane == ((j + 1) & 31)) {              // column j + 1 of the rows
+            const bool next = ((j + 1) >> 5) > E0;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) col[4 * g + q] = (next && E0 + 1 < E) ? x.A[4 * g + q][E0 + 1 < E ? E0 + 1 : E0] : x.A[4 * g + q][E0];
+          }
+          // four row sums across the warp, each exchange halving what a lane still carries: lanes 8 q .. hold sum q
+          const bool h2 = (lane & 16) != 0, h1 = (lane & 8) != 0;
+          double t0 = (h2 ? ps[2] : ps[0]) + __shfl_xor_sync(0xffffffffu, h2 ? ps[0] : ps[2], 16);
+          double t1 = (h2 ? ps[3] : ps[1]) + __shfl_xor_sync(0xffffffffu, h2 ? ps[1] : ps[3], 16);
+          double t = (h1 ? t1 : t0) + __shfl_xor_sync(0xffffffffu, h1 ? t0 : t1, 8);
+          t += __shfl_xor_sync(0xffffffffu, t, 4);
+          t += __shfl_xor_sync(0xffffffffu, t, 2);
+          t += __shfl_xor_sync(0xffffffffu, t, 1);
+          const int row = gw + gs * (4 * g + (lane >> 3));
+          if (row > j && row < s) send(x, par ^ 1, row, t, col[4 * g + (lane >> 3)]);
+        }
+      }
+      if constexpr (kSingle) { if (warp != 0) bar_arrive(2, kThreads); }
+      if (warp == 0) {                               // off the chain: gamma, and what later kernels need
+        x.gam = den > 0.0 ? 1.0 / den : 0.0;
+        if (rank == j % CL) {
+          double* dst = job.refl + (size_t)j * s;
+#pragma unroll
+          for (int e = 0; e < E; ++e)
+            if (lane + 32 * e < s) dst[lane + 32 * e] = e < E0 ? 0.0 : vn[e];
+          if (lane == 0) { job.d[j] = dj; job.e[j] = (j + 1 < s) ? beta : 0.0; job.gam[j] = x.gam; }
+        }
+      }
+#pragma unroll
+      for (int e = E0; e < E; ++e) x.v[e] = vn[e];
+    }
+    if constexpr (E0 + 1 < E) {
+      if (32 * (E0 + 1) < s) segment<E0 + 1>(x);
+    }
+  }
+
+  __device__ __forceinline__ void load_rows(Rows& x) {
+    const int gw = rank * W + warp, gs = CL * W;
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+      for (int e = 0; e < E; ++e) x.A[r][e] = 0.0;
+    if (job.gram) {           // C = X^T X, rows of X staged a chunk at a time as fp64
+      double (*stage)[S] = reinterpret_cast<double (*)[S]>(sh.stage_or_col);
+      for (int t0 = 0; t0 < s; t0 += kChunk) {
+        const int tn = min(kChunk, s - t0);
+        tc::named_bar_sync(3, 32 * W);
+        for (int idx = 32 * warp + lane; idx < tn * S; idx += 32 * W) {
+          const int t = idx / S, k = idx - t * S;
+          stage[t][k] = (k < s) ? (double)job.X[(size_t)(t0 + t) * s + k] : 0.0;
+        }
+        tc::named_bar_sync(3, 32 * W);
+        for (int t = 0; t < tn; ++t) {
+          double xk[E];
+#pragma unroll
+          for (int e = 0; e < E; ++e) xk[e] = stage[t][lane + 32 * e];
+#pragma unroll
+          for (int r = 0; r < R; ++r) {
+            const double xi = stage[t][min(gw + gs * r, S - 1)];
+#pragma unroll
+            for (int e = 0; e < E; ++e) x.A[r][e] = fma(xi, xk[e], x.A[r][e]);
+          }
+        }
+      }
+      tc::named_bar_sync(3, 32 * W);
+    } else {
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int i = gw + gs * r;
+        if (i < s) {
+#pragma unroll
+          for (int e = 0; e < E; ++e) {
+            const int k = lane + 32 * e;
+            if (k < s) x.A[r][e] = (double)job.X[(size_t)i * s + k];
+          }
+        }
+      }
+    }
+  }
+
+  __device__ __forceinline__ void run() {
+    for (int i = threadIdx.x; i < S + kMaxCl; i += kThreads) sh.pa[0][i] = sh.pa[1][i] = make_double2(0.0, 0.0);
+    for (int i = threadIdx.x; i < S; i += kThreads) sh.v[0][i] = sh.v[1][i] = sh.w[i] = 0.0;
+    if (threadIdx.x == 0) {
+      sh.dead = 0;
+      if (!kSingle) { tc::mbar_init(&sh.bar[0], 1); tc::mbar_init(&sh.bar[1], 1); tc::fence_barrier_init(); }
+    }
+    if constexpr (kSingle) __syncthreads(); else cg::this_cluster().sync();   // buffers and barriers are ready before a peer writes
+    Rows x;
+    load_rows(x);
+#pragma unroll
+    for (int e = 0; e < E; ++e) x.v[e] = 0.0;
+    x.gam = 0.0; x.v1 = 0.0; x.ok = true;
+    x.dst = x.dbar = 0;
+    if constexpr (!kSingle) {
+      const int c = (lane & 7) < CL ? (lane & 7) : 0;
+      x.dst = map_rank(tc::smem_u32(&sh.pa[0][0]), c);
+      x.dbar = map_rank(tc::smem_u32(&sh.bar[0]), c);
+      if (warp == 0) open_step(0, s);
+    }
+    const int gw = rank * W + warp, gs = CL * W;
+    double* col = reinterpret_cast<double*>(sh.stage_or_col) + warp * R;
+    if (lane == 0) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) col[r] = x.A[r][0];
+    }
+    __syncwarp();
+#pragma unroll
+    for (int g = 0; g < R / 4; ++g) {
+      const int row = gw + gs * (4 * g + (lane >> 3));
+      if (row < s) send(x, 0, row, 0.0, col[4 * g + (lane >> 3)]);
+    }
+    __syncwarp();
+    if constexpr (kSingle) { if (warp != 0) bar_arrive(2, kThreads); }
+    segment<0>(x);
+    if (!x.ok && lane == 0) atomicExch(status, (int)AB_ERR_TIMEOUT);
+    if constexpr (!kSingle) cg::this_cluster().sync();         // nobody leaves while a peer may still send to it
+  }
+};
+
+template <int E, int R, int W, bool kSingle>
+__global__ void __launch_bounds__(32 * W, 1)
+tridiag_small_kernel(const EigJob* __restrict__ jobs, int* status) {
+  using T = Tridiag<E, R, W, kSingle>;
+  extern __shared__ __align__(16) unsigned char tri_sm[];
+  const int CL = kSingle ? 1 : (int)cg::this_cluster().num_blocks();
+  const EigJob job = jobs[blockIdx.x / CL];
+  T t{*reinterpret_cast<typename T::Shared*>(tri_sm), job, job.s, CL, kSingle ? 0 : (int)cg::this_cluster().block_rank(),
+      (int)threadIdx.x >> 5, (int)threadIdx.x & 31, status};
+  t.run();
+}
+
+// ---- 2. and 3. the tridiagonal problem ------------------------------------------------------------------
+// Shared by both kernels: d and e of T scaled by 1 / norm, the positions where T splits.
+struct TriShared {
+  double2* de;               // (d[k], e[k]); e[k] couples k and k + 1 and is zero where T splits
+  unsigned* mask;            // bit k set: T splits between k and k + 1
+  double norm;
+};
+__device__ __forceinline__ void tri_load(const EigJob& job, TriShared& t, double2* sm, unsigned* mask, double* red) {
+  const int s = job.s;
+  t.de = sm; t.mask = mask;
+  double big = 0.0;
+  for (int k = threadIdx.x; k < s; k += blockDim.x) {
+    const double l = k > 0 ? fabs(job.e[k - 1]) : 0.0, r = k + 1 < s ? fabs(job.e[k]) : 0.0;
+    big = fmax(big, fabs(job.d[k]) + l + r);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) big = fmax(big, __shfl_xor_sync(0xffffffffu, big, o));
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = big;
+  for (int k = threadIdx.x; k < (s + 31) / 32; k += blockDim.x) mask[k] = 0u;
+  __syncthreads();
+  big = 0.0;
+  for (int k = 0; k < (int)(blockDim.x >> 5); ++k) big = fmax(big, red[k]);
+  t.norm = big;
+  const double inv = big > 0.0 ? 1.0 / big : 0.0;
+  for (int k = threadIdx.x; k < s; k += blockDim.x) {
+    const double e = k + 1 < s ? job.e[k] * inv : 0.0;
+    const bool cut = fabs(e) <= kSplitRel;
+    t.de[k] = make_double2(job.d[k] * inv, cut ? 0.0 : e);
+    if (cut) atomicOr(&mask[k >> 5], 1u << (k & 31));
+  }
+  __syncthreads();
+}
+// the unreduced block [b0, b1) that position i lies in
+__device__ __forceinline__ void tri_block(const TriShared& t, int s, int i, int& b0, int& b1) {
+  b0 = 0;
+  for (int w = (i - 1) >> 5; w >= 0 && i > 0; --w) {
+    unsigned m = t.mask[w];
+    if (w == ((i - 1) >> 5)) m &= 0xffffffffu >> (31 - ((i - 1) & 31));
+    if (m) { b0 = 32 * w + 32 - __clz(m); break; }
+  }
+  b1 = s;
+  for (int w = i >> 5; w < (s + 31) / 32; ++w) {
+    unsigned m = t.mask[w];
+    if (w == (i >> 5)) m &= 0xffffffffu << (i & 31);
+    if (m) { b1 = 32 * w + __ffs(m); break; }
+  }
+}
+
+// Eigenvalues below x of the block [b0, b1): sign changes of the leading principal minors of T - x I.  The
+// three-term recurrence has one dependent multiply-add a step (8.6 cycles; a division form has a division, 63);
+// eight steps' coefficients are fetched ahead of their use, and every eight steps the pair is brought back to unit size.
+__device__ __forceinline__ int sturm_count(const double2* de, int b0, int b1, double x) {
+  double p0 = 0.0, p1 = 1.0, e2 = 0.0;
+  int cnt = 0;
+  for (int k = b0; k < b1; k += 8) {
+    double2 q[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) q[u] = de[k + u];        // (d, e^2); eight entries of padding behind the last
+    if (k + 8 > b1) {                                    // what is not in the block: a diagonal of 2, no sign change
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (k + u >= b1) q[u] = make_double2(2.0, 0.0);
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const double p2 = fma(q[u].x - x, p1, -(e2 * p0));
+      cnt += (unsigned)(__double2hiint(p2) ^ __double2hiint(p1)) >> 31;
+      p0 = p1; p1 = p2;
+      e2 = q[u].y;
+    }
+    const int h = max(__double2hiint(p0) & 0x7ff00000, __double2hiint(p1) & 0x7ff00000);
+    if (h > 0 && h < 0x7fe00000) {
+      const double sc = __hiloint2double(0x7fe00000 - h, 0);
+      p0 *= sc; p1 *= sc;
+    }
+  }
+  return cnt;
+}
+
+// Position i of T carries the (i - b0)-th smallest eigenvalue of its block.  kLanes lanes share the position: each
+// pass cuts the interval into kLanes + 1 parts, so a lone matrix takes 32 lanes (11 passes) and a batch that fills the
+// device by itself 4 (23 passes, least work in all).
+template <int kLanes>
+__global__ void __launch_bounds__(128)
+tri_values_kernel(const EigJob* __restrict__ jobs) {
+  extern __shared__ __align__(16) double2 eig_sm[];
+  __shared__ unsigned mask[32];
+  __shared__ double red[4];
+  const EigJob job = jobs[blockIdx.y];
+  const int s = job.s;
+  const int per = 128 / kLanes;
+  if ((int)blockIdx.x * per >= s) return;
+  TriShared t;
+  tri_load(job, t, eig_sm, mask, red);
+  for (int k = threadIdx.x; k < s + 8; k += 128) {
+    const double e = k < s ? eig_sm[k].y : 0.0;
+    eig_sm[k] = make_double2(k < s ? eig_sm[k].x : 2.0, e * e);
+  }
+  __syncthreads();
+  const int i = blockIdx.x * per + threadIdx.x / kLanes, sub = threadIdx.x % kLanes;
+  const bool in = i < s;
+  int b0 = 0, b1 = 1;
+  if (in) tri_block(t, s, i, b0, b1);
+  const int want = i - b0;
+  double lo = -1.0000001, hi = 1.0000001;
+  const unsigned gmask = (0xffffffffu >> (32 - kLanes)) << ((threadIdx.x & 31) / kLanes * kLanes);
+  if (in && b1 - b0 == 1) { lo = hi = t.de[b0].x; }
+  constexpr int kPasses = kLanes == 4 ? 24 : kLanes == 8 ? 18 : 11;
+  for (int pass = 0; pass < kPasses; ++pass) {
+    const double wdt = (hi - lo) * (1.0 / (kLanes + 1));
+    const double x = lo + wdt * (sub + 1);
+    int below = 0;                                    // x is at or below the wanted eigenvalue
+    if (in && hi - lo > 2e-16 * fmax(fabs(lo), fabs(hi)) + 1e-18) below = sturm_count(t.de, b0, b1, x) <= want ? 1 : 0;
+    else below = 2;
+    const unsigned bal = __ballot_sync(0xffffffffu, below == 1) & gmask;
+    if (below != 2) {
+      const int nb = __popc(bal);                     // counts rise with x: the first nb points are below
+      const double l0 = lo;
+      if (nb > 0) lo = l0 + wdt * nb;
+      if (nb < kLanes) hi = l0 + wdt * (nb + 1);
+    }
+  }
+  if (in && sub == 0) { job.lam[i] = 0.5 * (lo + hi); if (i == 0) job.norm[0] = t.norm; }
+}
+
+// Eigenvector of T at lam: L from the factorisation from the top, U from the one from the bottom, joined where the
+// joint pivot is smallest (twisted factorisation; Fernando, and Dhillon and Parlett).  Warp 0 of a block works
+// from the top, warp 1 from the bottom, a lane per eigenvalue.  z[k][i]: component k of vector i, not normalised;
+// outside its block a vector is zero.
+// The blocks behind the vector blocks form the dot products inside each group of kGroup reflectors that the back
+// transform needs.
+__global__ void __launch_bounds__(64)
+tri_vectors_kernel(const EigJob* __restrict__ jobs, int vec_blocks) {
+  extern __shared__ __align__(16) double2 eig_sm[];
+  __shared__ unsigned mask[32];
+  __shared__ double red[2];
+  __shared__ double best_g[2][32];
+  __shared__ int best_k[2][32];
+  const EigJob job = jobs[blockIdx.y];
+  const int s = job.s;
+  const int half = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if ((int)blockIdx.x >= vec_blocks) {
+    const int g = ((int)blockIdx.x - vec_blocks) * 2 + half, j0 = g * kGroup;
+    if (j0 >= s) return;
+    int idx = 0;
+    for (int a = 0; a < kGroup; ++a)
+      for (int b = a + 1; b < kGroup; ++b, ++idx) {
+        double acc = 0.0;
+        if (j0 + b < s)
+          for (int k = j0 + b + lane; k < s; k += 32) acc = fma(job.refl[(size_t)(j0 + a) * s + k], job.refl[(size_t)(j0 + b) * s + k], acc);
+        acc = warp_sum(acc);
+        if (lane == 0) job.cross[g * 6 + idx] = acc;
+      }
+    return;
+  }
+  if ((int)blockIdx.x * 32 >= s) return;
+  TriShared t;
+  tri_load(job, t, eig_sm, mask, red);
+  const int i = blockIdx.x * 32 + lane;
+  const bool in = i < s;
+  double* Lp = job.zp + i;
+  double* Up = job.zm + i;
+  int b0 = 0, b1 = 0;
+  double lam = 0.0;
+  constexpr double tiny = 1e-290;
+  const double2* de = t.de;
+  if (in) {
+    tri_block(t, s, i, b0, b1);
+    lam = job.lam[i];
+    if (half == 0) {          // L[k] = e[k] / D+[k], k = b0 .. b1 - 2
+      double2 c = de[b0];
+      double D = c.x - lam;
+      for (int k = b0; k + 1 < b1; ++k) {
+        const double2 cn = de[k + 1];
+        if (fabs(D) < tiny) D = D < 0.0 ? -tiny : tiny;
+        const double L = c.y / D;
+        Lp[(size_t)k * s] = L;
+        D = fma(-L, c.y, cn.x - lam);
+        c = cn;
+      }
+    } else {                  // U[k] = e[k - 1] / D-[k], k = b1 - 1 .. b0 + 1
+      double D = de[b1 - 1].x - lam;
+      for (int k = b1 - 1; k > b0; --k) {
+        const double2 cn = de[k - 1];
+        if (fabs(D) < tiny) D = D < 0.0 ? -tiny : tiny;
+        const double U = cn.y / D;
+        Up[(size_t)k * s] = U;
+        D = fma(-U, cn.y, cn.x - lam);
+      }
+    }
+  }
+  __syncthreads();
+  {                           // joint pivot at k: d - lam - e[k-1] L[k-1] - e[k] U[k+1]
+    double bg = 1e300;
+    int bk = b0;
+    if (in) {
+      const int mid = (b0 + b1) >> 1;
+      const int k0 = half ? mid : b0, k1 = half ? b1 : mid;
+#pragma unroll 8
+      for (int k = k0; k < k1; ++k) {
+        const double2 c = de[k];
+        double g = c.x - lam;
+        if (k > b0) g = fma(-de[k - 1].y, __ldcg(Lp + (size_t)(k - 1) * s), g);
+        if (k + 1 < b1) g = fma(-c.y, __ldcg(Up + (size_t)(k + 1) * s), g);
+        if (fabs(g) < bg) { bg = fabs(g); bk = k; }
+      }
+    }
+    best_g[half][lane] = bg;
+    best_k[half][lane] = bk;
+  }
+  __syncthreads();
+  double n2 = 0.0;
+  const int tw = best_g[1][lane] < best_g[0][lane] ? best_k[1][lane] : best_k[0][lane];
+  if (in) {                   // eight factors fetched ahead of the chain that uses them
+    double z = 1.0;
+    if (half == 0) {
+      n2 = 1.0;
+      for (int k = tw - 1; k >= b0; k -= 8) {
+        double f[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) f[u] = k - u >= b0 ? Lp[(size_t)(k - u) * s] : 0.0;
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          if (k - u >= b0) { z *= -f[u]; n2 = fma(z, z, n2); Lp[(size_t)(k - u) * s] = z; }
+      }
+      for (int k = 0; k < b0; ++k) Lp[(size_t)k * s] = 0.0;
+    } else {
+      for (int k = tw + 1; k < b1; k += 8) {
+        double f[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) f[u] = k + u < b1 ? Up[(size_t)(k + u) * s] : 0.0;
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          if (k + u < b1) { z *= -f[u]; n2 = fma(z, z, n2); Lp[(size_t)(k + u) * s] = z; }
+      }
+      for (int k = b1; k < s; ++k) Lp[(size_t)k * s] = 0.0;
+      Lp[(size_t)tw * s] = 1.0;
+    }
+  }
+  best_g[half][lane] = n2;
+  __syncthreads();
+  if (in && half == 0) job.inv[i] = 1.0 / sqrt(best_g[0][lane] + best_g[1][lane]);
+}
+
+// ---- 4. back transform ----------------------------------------------------------------------------------
+// A warp carries NV vectors of E elements a lane through all reflectors, last one first.  kGroup reflectors are
+// applied together: their dot products with the vectors go through the warp reduction side by side, and the
+// products among themselves (cross) turn them into the coefficients one after the other would have had.  The eight
+// warps of a block share the reflectors through shared memory, the next group on its way while one is applied
+// (each warp fetching its own was bound by L2: 259 us for 72 matrices of order 192).
+constexpr int kBackWarps = 8;
+template <int E, int NV>
+struct BackGroups {
+  double (&z)[NV][E];
+  double (*fs)[kGroup][32 * E];
+  const double *gs, *xs;
+  double* red;               // this warp's NV x kGroup sums
+  int lane;
+  bool wanted;
+  // the reflectors whose first element lies in the 32-column group E0
+  template <int E0, typename F>
+  __device__ __forceinline__ void segment(int ngroups, F& fetch) {
+    constexpr int kPer = 32 / kGroup;
+    for (int g = min(ngroups, (E0 + 1) * kPer) - 1; g >= E0 * kPer; --g) {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+      __syncthreads();                     // group g is here, and nobody reads the buffer of group g + 1 any more
+      if (g > 0) fetch(g - 1);
+      if (!wanted) continue;
+      double f[kGroup][E];
+#pragma unroll
+      for (int a = 0; a < kGroup; ++a)
+#pragma unroll
+        for (int e = E0; e < E; ++e) f[a][e] = fs[g & 1][a][lane + 32 * e];
+      double dt[NV * kGroup];
+#pragma unroll
+      for (int v = 0; v < NV; ++v)
+#pragma unroll
+        for (int a = 0; a < kGroup; ++a) {
+          double acc = 0.0;
+#pragma unroll
+          for (int e = E0; e < E; ++e) acc = fma(f[a][e], z[v][e], acc);
+          dt[v * kGroup + a] = acc;
+        }
+      // NV * kGroup sums across the warp, each exchange halving what a lane still carries; the sums then go round
+      // through shared memory
+      int width = 16;
+      double t;
+      if constexpr (NV == 4) {
+        const bool h = (lane & 16) != 0;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) dt[q] = (h ? dt[q + 8] : dt[q]) + __shfl_xor_sync(0xffffffffu, h ? dt[q] : dt[q + 8], 16);
+        width = 8;
+      }
+      {
+        const bool h = (lane & width) != 0;
+        if constexpr (NV >= 2) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q) dt[q] = (h ? dt[q + 4] : dt[q]) + __shfl_xor_sync(0xffffffffu, h ? dt[q] : dt[q + 4], width);
+          width >>= 1;
+        }
+      }
+      {
+        const bool h = (lane & width) != 0;
+#pragma unroll
+        for (int q = 0; q < 2; ++q) dt[q] = (h ? dt[q + 2] : dt[q]) + __shfl_xor_sync(0xffffffffu, h ? dt[q] : dt[q + 2], width);
+        width >>= 1;
+        const bool h1 = (lane & width) != 0;
+        t = (h1 ? dt[1] : dt[0]) + __shfl_xor_sync(0xffffffffu, h1 ? dt[0] : dt[1], width);
+      }
+      constexpr int kRest = 32 / (NV * kGroup);        // lanes that still hold parts of the same sum
+#pragma unroll
+      for (int o = kRest / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      __syncwarp();
+      if (lane % kRest == 0) red[lane / kRest] = t;
+      __syncwarp();
+      const double2 g01 = *reinterpret_cast<const double2*>(gs + g * kGroup), g23 = *reinterpret_cast<const double2*>(gs + g * kGroup + 2);
+      const double2 x01 = *reinterpret_cast<const double2*>(xs + g * 6), x23 = *reinterpret_cast<const double2*>(xs + g * 6 + 2),
+                    x45 = *reinterpret_cast<const double2*>(xs + g * 6 + 4);
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        const double2 d01 = *reinterpret_cast<const double2*>(red + v * kGroup), d23 = *reinterpret_cast<const double2*>(red + v * kGroup + 2);
+        // cross: (0,1) (0,2) (0,3) (1,2) (1,3) (2,3); the last reflector acts first
+        const double c3 = g23.y * d23.y;
+        const double c2 = g23.x * fma(-c3, x45.y, d23.x);
+        const double c1 = g01.y * fma(-c3, x45.x, fma(-c2, x23.y, d01.y));
+        const double c0 = g01.x * fma(-c3, x23.x, fma(-c2, x01.y, fma(-c1, x01.x, d01.x)));
+#pragma unroll
+        for (int e = E0; e < E; ++e)
+          z[v][e] = fma(-c0, f[0][e], fma(-c1, f[1][e], fma(-c2, f[2][e], fma(-c3, f[3][e], z[v][e]))));
+      }
+    }
+    if constexpr (E0 > 0) segment<E0 - 1>(ngroups, fetch);
+  }
+};
+
+template <int E, int NV>
+__global__ void __launch_bounds__(32 * kBackWarps)
+back_transform_kernel(const EigJob* __restrict__ jobs) {
+  constexpr int S = 32 * E;
+  extern __shared__ __align__(16) double back_sm[];
+  double (*fs)[kGroup][S] = reinterpret_cast<double (*)[kGroup][S]>(back_sm);   // two groups of reflectors
+  double* gs = back_sm + 2 * kGroup * S;                                           // gamma, padded to a whole group
+  __shared__ __align__(16) double red[kBackWarps][NV * kGroup];
+  double* xs = gs + S + kGroup;                                                    // six products a group
+  const EigJob job = jobs[blockIdx.y];
+  const int s = job.s;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if ((int)blockIdx.x * kBackWarps * NV >= s) return;
+  const int i0 = (blockIdx.x * kBackWarps + warp) * NV;
+  const int ngroups = (s + kGroup - 1) / kGroup;
+  for (int k = tid; k < ngroups * kGroup; k += 32 * kBackWarps) gs[k] = k < s ? job.gam[k] : 0.0;
+  for (int k = tid; k < ngroups * 6; k += 32 * kBackWarps) xs[k] = job.cross[k];
+  auto fetch = [&](int g) {              // reflector a of group g has its first element at j0 + a + 1
+    const int j0 = g * kGroup, k0 = j0 & ~31, w = S - k0;
+    for (int idx = tid; idx < kGroup * w; idx += 32 * kBackWarps) {
+      const int a = idx / w, k = k0 + idx - a * w;
+      double* d = &fs[g & 1][a][k];
+      if (k < s && j0 + a < s)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(tc::smem_u32(d)), "l"(job.refl + (size_t)(j0 + a) * s + k) : "memory");
+      else
+        *d = 0.0;
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  fetch(ngroups - 1);
+  // rank of each vector's eigenvalue among all (descending, ties by position)
+  int rank[NV];
+  double lam[NV];
+  bool wanted = false;
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    const int i = i0 + v;
+    lam[v] = i < s ? job.lam[i] : 0.0;
+    int c = 0;
+    for (int k = lane; k < s; k += 32) {
+      const double lk = job.lam[k];
+      c += (lk > lam[v] || (lk == lam[v] && k < i)) ? 1 : 0;
+    }
+    rank[v] = __reduce_add_sync(0xffffffffu, c);
+    if (i >= s) rank[v] = s;
+    wanted = wanted || rank[v] < job.need;
+  }
+  double z[NV][E];
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    const int i = i0 + v;
+    const double inv = i < s ? job.inv[i] : 0.0;
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      const int k = lane + 32 * e;
+      z[v][e] = (wanted && i < s && k < s) ? job.zp[(size_t)k * s + i] * inv : 0.0;
+    }
+    // neighbours too close for the factorisation to keep apart: is this vector orthogonal to them?
+    if (i < s && rank[v] < job.need) {
+      for (int k0 = 0; k0 < s; k0 += 32) {
+        const int k = k0 + lane;
+        bool close = false;
+        if (k < s && k != i) {
+          const double lk = job.lam[k];
+          close = fabs(lk - lam[v]) < kCloseRel && (lk > lam[v] || (lk == lam[v] && k < i));
+        }
+        unsigned bal = __ballot_sync(0xffffffffu, close);
+        while (bal) {
+          const int kk = k0 + __ffs(bal) - 1;
+          bal &= bal - 1;
+          double acc = 0.0;
+#pragma unroll
+          for (int e = 0; e < E; ++e) {
+            const int q = lane + 32 * e;
+            if (q < s) acc = fma(z[v][e], job.zp[(size_t)q * s + kk], acc);
+          }
+          acc = warp_sum(acc) * job.inv[kk];
+          if (!(fabs(acc) <= kOrthTol) && lane == 0) *job.flag = 1;
+        }
+      }
+    }
+  }
+  BackGroups<E, NV> bg{z, fs, gs, xs, red[warp], lane, wanted};
+  bg.template segment<E - 1>(ngroups, fetch);
+  const double norm = job.norm[0];
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    if (rank[v] >= job.need) continue;
+    float* dst = job.rows + (size_t)rank[v] * s;
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      const int k = lane + 32 * e;
+      if (k < s) dst[k] = (float)z[v][e];
+    }
+    if (lane == 0 && job.vals) {
+      const double l = lam[v] * norm;
+      job.vals[rank[v]] = (float)(job.gram ? (l > 1e-12 * norm ? sqrt(l) : 0.0) : l);
+    }
+  }
+}
+
+template <int E, int R, int W, bool kSingle>
+int launch_tridiag(const EigJob* jobs, int count, int CL, int* status, cudaStream_t st) {
+  const size_t sm = sizeof(typename Tridiag<E, R, W, kSingle>::Shared);
+  AB_CUDA_OK(cudaFuncSetAttribute(tridiag_small_kernel<E, R, W, kSingle>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(count * CL));
+  cfg.blockDim = dim3(32 * W);
+  cfg.dynamicSmemBytes = sm;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = CL; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr; cfg.numAttrs = 1;
+  AB_CUDA_OK(cudaLaunchKernelEx(&cfg, tridiag_small_kernel<E, R, W, kSingle>, jobs, status));
+  AB_LAUNCH_OK();
+  return AB_OK;
+}
+
+template <int L>
+int launch_values(const EigJob* jobs, int count, int smax, cudaStream_t st) {
+  const int per = 128 / L;
+  tri_values_kernel<L><<<dim3((unsigned)((smax + per - 1) / per), (unsigned)count), 128, (smax + 8) * sizeof(double2), st>>>(jobs);
+  AB_LAUNCH_OK();
+  return AB_OK;
+}
+
+template <int E, int NV>
+int launch_back(const EigJob* jobs, int count, int smax, cudaStream_t st) {
+  const int per = kBackWarps * NV;
+  const size_t sm = sizeof(double) * (2 * kGroup * 32 * E + 32 * E + kGroup + (32 * E / kGroup + 1) * 6);
+  back_transform_kernel<E, NV><<<dim3((unsigned)((smax + per - 1) / per), (unsigned)count), 32 * kBackWarps, sm, st>>>(jobs);
+  AB_LAUNCH_OK();
+  return AB_OK;
+}
+// Four vectors a warp where the batch fills the device; one where it does not (the chain of a warp is then what counts).
+template <int E>
+int launch_back_e(const EigJob* jobs, int count, int smax, int sms, cudaStream_t st) {
+  return (long long)count * smax >= 32LL * sms ? launch_back<E, 4>(jobs, count, smax, st) : launch_back<E, 1>(jobs, count, smax, st);
+}
+
+}  // namespace
+
+size_t eig_ws_doubles(int s) { return (size_t)3 * s * s + 5 * (size_t)s + 2 * (size_t)s + 64; }
+
+void eig_bind(EigJob& j, double* ws) {
+  const size_t s = (size_t)j.s;
+  j.refl = ws; j.zp = j.refl + s * s; j.zm = j.zp + s * s;
+  j.d = j.zm + s * s; j.e = j.d + s; j.gam = j.e + s; j.lam = j.gam + s; j.inv = j.lam + s; j.cross = j.inv + s;
+  j.norm = j.cross + (s + 3) / 4 * 6;
+}
+
+int eig_direct(const EigJob* d_jobs, int count, int smax, int* status, cudaStream_t st) {
+  if (smax > kEigSmallMax) return AB_ERR_UNSUPPORTED;
+  const int sms = sm_count();
+  if (sms <= 0) return AB_ERR_CUDA;
+  int rc;
+  if (smax <= 64) rc = launch_tridiag<2, 8, 8, true>(d_jobs, count, 1, status, st);
+  else if (smax <= 128) rc = launch_tridiag<4, 16, 8, true>(d_jobs, count, 1, status, st);
+  else if (smax <= 192)
+    rc = 6 * count <= sms ? launch_tridiag<6, 4, 8, false>(d_jobs, count, 6, status, st) : launch_tridiag<6, 12, 8, false>(d_jobs, count, 2, status, st);
+  else
+    rc = 8 * count <= sms ? launch_tridiag<8, 4, 8, false>(d_jobs, count, 8, status, st) : launch_tridiag<8, 8, 8, false>(d_jobs, count, 4, status, st);
+  AB_TRY(rc);
+  const long long values = (long long)count * smax;
+  if (values <= 16LL * sms) rc = launch_values<32>(d_jobs, count, smax, st);
+  else if (values <= 64LL * sms) rc = launch_values<8>(d_jobs, count, smax, st);
+  else rc = launch_values<4>(d_jobs, count, smax, st);
+  AB_TRY(rc);
+  const int vb = (smax + 31) / 32, gb = ((smax + kGroup - 1) / kGroup + 1) / 2;
+  tri_vectors_kernel<<<dim3((unsigned)(vb + gb), (unsigned)count), 64, smax * sizeof(double2), st>>>(d_jobs, vb);
+  AB_LAUNCH_OK();
+  if (smax <= 64) return launch_back_e<2>(d_jobs, count, smax, sms, st);
+  if (smax <= 128) return launch_back_e<4>(d_jobs, count, smax, sms, st);
+  if (smax <= 192) return launch_back_e<6>(d_jobs, count, smax, sms, st);
+  return launch_back_e<8>(d_jobs, count, smax, sms, st);
+}
+
+}  // namespace ab

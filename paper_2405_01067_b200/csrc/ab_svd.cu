@@ -14,6 +14,9 @@
 // and |x_i| = sigma_i^2.  The long-side factor is W V_r (or V_r^T W) by a GEMM; sigma_i is
 // re-measured as the norm of that product, which makes A^T A = B B^T = diag(sigma) hold by
 // construction.  No wait in these kernels can spin: every loop has a fixed trip count.
+//
+// Short sides up to kEigSmallMax take the direct solver of ab_eig.cu in place of the block Jacobi (256 x 2304:
+// 2.87 ms in the shared-memory Jacobi that they took before -> 0.47 ms); the shared-memory Jacobi is its fallback.
 #include <vector>
 #include <algorithm>
 #include <map>
@@ -377,7 +380,9 @@ norms_sort_kernel(const float* __restrict__ Xall, int s, float* __restrict__ lam
 // projection becomes zero (it then contributes nothing to either factor).  Only the first r_need rows
 // are ever used.  One CTA per matrix.
 __global__ void __launch_bounds__(256)
-complete_basis_kernel(float* __restrict__ rows_all, const float* __restrict__ lam_all, int s, int r_need) {
+complete_basis_kernel(float* __restrict__ rows_all, const float* __restrict__ lam_all, const int* __restrict__ flags, int s,
+                      int r_need) {
+  if (flags[blockIdx.x] == 0) return;
   extern __shared__ float cb_sm[];
   float* v = cb_sm;            // s
   float* coef = cb_sm + s;     // s
@@ -426,11 +431,6 @@ complete_basis_kernel(float* __restrict__ rows_all, const float* __restrict__ la
     for (int u = tid; u < s; u += 256) rows[(size_t)k * s + u] = v[u] * inv;
     __syncthreads();                                         // the next row reads this one from global memory
   }
-}
-
-__global__ void identity_perm_kernel(int* __restrict__ perm, int s, int total) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < total) perm[i] = i % s;
 }
 
 // Vr[k][:] = Vt[perm[k]][:] scaled to unit length, k < r_cap (thousands of fp32 rotations leave
@@ -564,7 +564,10 @@ struct Layout {
   std::map<int, std::vector<int>> groups;     // s -> item indices
   std::map<int, float*> X, Vt;
   std::map<int, JState*> st;
-  std::map<int, void*> jobs;                  // scratch of the in-shared-memory solver
+  std::map<int, void*> jobs;                  // short side up to kEigSmallMax: EigJobs, scratch of the eigensolver,
+  std::map<int, double*> eig;                 //   fallback flags and the in-shared-memory Jacobi's scratch
+  std::map<int, int*> flags;
+  std::map<int, EigJob*> ejobs;
   std::vector<ItemWs> item;
   size_t bytes;
 };
@@ -578,7 +581,12 @@ Layout make_layout(const SvdItem* items, int L, void* ws) {
     lo.X[g.first] = ar.take_n<float>(cnt * s * s);
     lo.Vt[g.first] = ar.take_n<float>(cnt * s * s);
     lo.st[g.first] = ar.take_n<JState>(cnt);
-    lo.jobs[g.first] = ar.take_n<char>(rows_jacobi_scratch_bytes((int)cnt));
+    if (g.first <= kEigSmallMax) {
+      lo.jobs[g.first] = ar.take_n<char>(rows_jacobi_scratch_bytes((int)cnt));
+      lo.ejobs[g.first] = ar.take_n<EigJob>(cnt);
+      lo.flags[g.first] = ar.take_n<int>(cnt);
+      lo.eig[g.first] = ar.take_n<double>(cnt * eig_ws_doubles(g.first));
+    }
   }
   lo.item.resize(L);
   for (int i = 0; i < L; ++i) {
@@ -667,18 +675,27 @@ int svd_batch(const SvdItem* items, int L, float sigma_cutoff, void* ws, size_t 
   for (auto& g : lo.groups) {
     const int s = g.first, count = (int)g.second.size();
     Plan p = make_plan(items[g.second[0]]);
-    if (rows_jacobi_fits(count, s)) {
-      // small enough to stay in shared memory for the whole iteration: the rows of G rotated until
-      // orthogonal are lambda_i v_i^T, so the unit rows are the eigenvectors, already sorted
+    if (s <= kEigSmallMax && rows_jacobi_fits(count, s)) {
+      // The direct solver leaves the leading eigenvectors as unit rows in descending order in Vt.  A flagged matrix
+      // goes through the Jacobi kernel that keeps it in shared memory (the rows of G rotated until orthogonal are
+      // lambda_i v_i^T), which returns at once for the others.
+      std::vector<EigJob> ej((size_t)count);
+      for (int j = 0; j < count; ++j) {
+        EigJob& q = ej[j];
+        q.X = lo.X[s] + (size_t)j * s * s; q.gram = 0; q.s = s; q.need = make_plan(items[g.second[j]]).r_cap;
+        q.rows = lo.Vt[s] + (size_t)j * s * s; q.vals = nullptr; q.flag = lo.flags[s] + j;
+        eig_bind(q, lo.eig[s] + (size_t)j * eig_ws_doubles(s));
+      }
       AB_CUDA_OK(cudaMemsetAsync(lo.st[s], 0, sizeof(JState) * count, stream));
-      AB_TRY(rows_jacobi(lo.X[s], lo.Vt[s], lo.item[g.second[0]].lam, &lo.st[s]->status, sizeof(JState), count, s,
-                         lo.jobs[s], stream));
+      AB_CUDA_OK(cudaMemsetAsync(lo.flags[s], 0, sizeof(int) * count, stream));
+      AB_CUDA_OK(cudaMemcpyAsync(lo.ejobs[s], ej.data(), ej.size() * sizeof(EigJob), cudaMemcpyHostToDevice, stream));
+      AB_TRY(eig_direct(lo.ejobs[s], count, s, &lo.st[s]->status, stream));
+      AB_TRY(rows_jacobi(lo.X[s], lo.Vt[s], lo.item[g.second[0]].lam, &lo.st[s]->status, sizeof(JState), lo.flags[s], count,
+                         s, lo.jobs[s], stream));
       int r_need = 0;
       for (int idx : g.second) r_need = std::max(r_need, make_plan(items[idx]).r_cap);
-      complete_basis_kernel<<<count, 256, 2 * (size_t)s * sizeof(float), stream>>>(lo.Vt[s], lo.item[g.second[0]].lam, s,
-                                                                                  r_need);
-      AB_LAUNCH_OK();
-      identity_perm_kernel<<<(count * s + 255) / 256, 256, 0, stream>>>(lo.item[g.second[0]].perm, s, count * s);
+      complete_basis_kernel<<<count, 256, 2 * (size_t)s * sizeof(float), stream>>>(lo.Vt[s], lo.item[g.second[0]].lam,
+                                                                                  lo.flags[s], s, r_need);
       AB_LAUNCH_OK();
       continue;
     }
@@ -700,10 +717,14 @@ int svd_batch(const SvdItem* items, int L, float sigma_cutoff, void* ws, size_t 
       const int i = g.second[j];
       const SvdItem& it = items[i];
       Plan p = make_plan(it);
-      const ItemWs& w = lo.item[i];
-      const float* Vt = lo.Vt[s] + j * (size_t)s * s;
-      gather_rows_kernel<<<p.r_cap, 256, 0, stream>>>(Vt, w.perm, s, p.r_cap, w.Vr);
-      AB_LAUNCH_OK();
+      ItemWs w = lo.item[i];
+      float* Vt = lo.Vt[s] + j * (size_t)s * s;
+      if (s <= kEigSmallMax && rows_jacobi_fits((int)g.second.size(), s)) {
+        w.Vr = Vt;                  // unit rows in order already
+      } else {
+        gather_rows_kernel<<<p.r_cap, 256, 0, stream>>>(Vt, w.perm, s, p.r_cap, w.Vr);
+        AB_LAUNCH_OK();
+      }
       int64_t yt, yk;   // Ylong(k,t) = Y[t*yt + k*yk]
       if (p.tall) {     // Y (m x r_cap) = W Vr^T
         AB_TRY(gemm_simt(it.W, it.w_dt, it.n, 1, w.Vr, AB_F32, 1, s, w.Y, AB_F32, p.r_cap, it.m, p.r_cap, it.n, stream));

@@ -5,9 +5,12 @@
 //   Abar = Q_A R_A,  Bbar^T = Q_B R_B   with Q_A = Abar R_A^-1, Q_B = Bbar^T R_B^-1 orthonormal
 //   W = Q_A M Q_B^T,  M = R_A R_B^T  (r x r),   M = U_M S V_M^T         (SVD, r x r)
 //   A' = Abar Z_A,  Z_A = R_A^-1 (M V_M) S^(-1/2);   B' = Z_B Bbar,  Z_B = S^(1/2) V_M^T R_B^-T
-// One CTA per Gram matrix factors it in shared memory and inverts the triangle in place; one CTA
-// per M keeps it in shared memory and orthogonalises its ROWS with one-sided Jacobi rotations
-// (the rows of the result are sigma_i v_i^T), so no kernel boundary and no global traffic sits
+// One CTA per Gram matrix factors it in shared memory and inverts the triangle in place.  The SVD of M is the
+// direct eigensolver of ab_eig.cu on M^T M in fp64 (whole ViT-B/16, 72 cores of order 192: 2183 -> 770 us for its four
+// kernels against the one-sided Jacobi alone; a lone core of order 64: 234 -> 106 us).  A core whose vectors that solver could not
+// keep orthogonal goes through the Jacobi kernel below, which returns at once for all others: one CTA or cluster
+// per M keeps it in shared memory and orthogonalises its ROWS with one-sided rotations (the rows of the result are
+// sigma_i v_i^T), so no kernel boundary and no global traffic sits
 // between rotations.  Cholesky pivots below 1e-6 of the largest diagonal entry of G are treated
 // as zero: the row of R and the row and column of its inverse are dropped, which is exactly right
 // for factors truncated by the rank rule (zero columns of A, zero rows of B).  Otherwise the
@@ -46,6 +49,7 @@ struct JacobiJob {
   float* rows;      // k x r output: unit rows, sorted by descending norm (zero rows stay zero)
   float* norms;     // k
   int* status;      // AB_OK / AB_ERR_NOT_CONVERGED (may be null)
+  const int* flag;  // run only if *flag is set
   int k, r;
 };
 
@@ -76,6 +80,7 @@ jacobi_rows_cluster_kernel(const JacobiJob* __restrict__ jobs, float tol) {
   extern __shared__ __align__(16) float sm[];
   const int crank = (kC == 1) ? 0 : (int)cluster.block_rank();
   const JacobiJob job = jobs[blockIdx.x / kC];
+  if (*job.flag == 0) return;                  // the same for every CTA of the cluster
   const int k = job.k, r = job.r, ld = r + 1;
   const int nb = (k + 3) / 4;                  // blocks of 4 rows
   const int nbl = (nb + kC - 1) / kC;          // blocks held by each CTA (same layout in all)
@@ -548,9 +553,10 @@ __global__ void fast_rank_rule_kernel(const float* const* __restrict__ sigma, co
   }
 }
 
-// A bounded wait that ran out inside one of the tensor-core launches of the call reaches every matrix's status.
+// A bounded wait that ran out inside one of the tensor-core launches or the eigensolver of the call reaches every matrix's status.
 __global__ void fold_tc_status_kernel(const int* __restrict__ tc_status, int* __restrict__ dev_status, int L) {
-  const int bad = (tc_status[0] != AB_OK) ? tc_status[0] : (tc_status[1] != AB_OK) ? tc_status[1] : tc_status[2];
+  int bad = AB_OK;
+  for (int k = 0; k < 4; ++k) if (tc_status[k] != AB_OK) bad = tc_status[k];
   if (bad == AB_OK) return;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < L; i += gridDim.x * blockDim.x) dev_status[i] = bad;
 }
@@ -571,6 +577,7 @@ struct FastWs {
   CholJob* cjobs;       // 2 L
   AvgJob* ajobs;        // 2 L
   JacobiJob* jobs;      // L
+  EigJob* ejobs;        // L
   int* jstatus;         // 3 L
   const float** sig_ptrs;
   int** rout_ptrs;
@@ -579,7 +586,8 @@ struct FastWs {
   SplitJob* sjobs;      // 4 L
   std::vector<bf16*> Asp, Bsp, ZAsp, ZBsp;    // each: three pieces one after the other
   void* tc_table[3];    // problem tables of the three tensor-core launches
-  int* tc_status;
+  int* tc_status;       // 64, and behind them one fallback flag per matrix (see EigJob)
+  std::vector<double*> eig;   // scratch of the eigensolver
   size_t bytes;
 };
 
@@ -604,6 +612,7 @@ FastWs fast_layout(const ab_sync_desc* d, int L, void* ws) {
   w.cjobs = ar.take_n<CholJob>((size_t)2 * L);
   w.ajobs = ar.take_n<AvgJob>((size_t)2 * L);
   w.jobs = ar.take_n<JacobiJob>((size_t)L);
+  w.ejobs = ar.take_n<EigJob>((size_t)L);
   w.jstatus = ar.take_n<int>((size_t)3 * L);
   w.sig_ptrs = ar.take_n<const float*>(L);
   w.rout_ptrs = ar.take_n<int*>(L);
@@ -620,7 +629,9 @@ FastWs fast_layout(const ab_sync_desc* d, int L, void* ws) {
   w.tc_table[0] = ar.take(gemm_tc_table_bytes(2 * L));
   w.tc_table[1] = ar.take(gemm_tc_table_bytes(2 * L));
   w.tc_table[2] = ar.take(gemm_tc_table_bytes(L));
-  w.tc_status = ar.take_n<int>(64);
+  w.tc_status = ar.take_n<int>(64 + (size_t)L);
+  w.eig.resize(L);
+  for (int i = 0; i < L; ++i) w.eig[i] = ar.take_n<double>(eig_ws_doubles(d[i].r));
   w.bytes = align_up(ar.used, 256);
   return w;
 }
@@ -681,12 +692,12 @@ bool rows_jacobi_fits(int count, int s) {
 
 size_t rows_jacobi_scratch_bytes(int count) { return align_up((size_t)count * sizeof(JacobiJob), 256); }
 
-int rows_jacobi(const float* X, float* rows, float* norms, int* status, size_t status_stride_bytes, int count, int s,
-                void* scratch, cudaStream_t st) {
+int rows_jacobi(const float* X, float* rows, float* norms, int* status, size_t status_stride_bytes, const int* flags,
+                int count, int s, void* scratch, cudaStream_t st) {
   std::vector<JacobiJob> jb((size_t)count);
   for (int j = 0; j < count; ++j) {
     int* stj = reinterpret_cast<int*>(reinterpret_cast<char*>(status) + (size_t)j * status_stride_bytes);
-    jb[j] = JacobiJob{X + (size_t)j * s * s, rows + (size_t)j * s * s, norms + (size_t)j * s, stj, s, s};
+    jb[j] = JacobiJob{X + (size_t)j * s * s, rows + (size_t)j * s * s, norms + (size_t)j * s, stj, flags + j, s, s};
   }
   AB_CUDA_OK(cudaMemcpyAsync(scratch, jb.data(), jb.size() * sizeof(JacobiJob), cudaMemcpyHostToDevice, st));
   return launch_jacobi(static_cast<const JacobiJob*>(scratch), count, s, rows_jacobi_tol(s), st);
@@ -728,6 +739,7 @@ int sync_factored(const ab_sync_desc* d, int L, int K, float sigma_cutoff, int d
   std::vector<GemmDesc> gg;
   gg.reserve((size_t)2 * kGramMaxParts * L);
   std::vector<JacobiJob> jb((size_t)L);
+  std::vector<EigJob> ej((size_t)L);
   std::vector<const float*> sigp(L);
   std::vector<int*> routp(L);
   std::vector<int> rs(L);
@@ -812,7 +824,11 @@ int sync_factored(const ab_sync_desc* d, int L, int K, float sigma_cutoff, int d
       x.upper_only = 1;
       gg.push_back(x);
     }
-    jb[i] = JacobiJob{w.M[i], w.Vs[i], d[i].sigma, w.jstatus + 3 * i + 2, r, r};
+    int* flag = w.tc_status + 64 + i;
+    jb[i] = JacobiJob{w.M[i], w.Vs[i], d[i].sigma, w.jstatus + 3 * i + 2, flag, r, r};
+    EigJob& q = ej[i];
+    q.X = w.M[i]; q.gram = 1; q.s = r; q.need = r; q.rows = w.Vs[i]; q.vals = d[i].sigma; q.flag = flag;
+    eig_bind(q, w.eig[i]);
     sigp[i] = d[i].sigma; routp[i] = d[i].r_out; rs[i] = r;
   }
   // All tables sit back to back in the workspace (descs ... rs): one host image, one copy.
@@ -838,6 +854,7 @@ int sync_factored(const ab_sync_desc* d, int L, int K, float sigma_cutoff, int d
     put(w.cjobs, cj.data(), cj.size() * sizeof(CholJob));
     put(w.ajobs, aj.data(), aj.size() * sizeof(AvgJob));
     put(w.jobs, jb.data(), jb.size() * sizeof(JacobiJob));
+    put(w.ejobs, ej.data(), ej.size() * sizeof(EigJob));
     put(w.sig_ptrs, sigp.data(), L * sizeof(float*));
     put(w.rout_ptrs, routp.data(), L * sizeof(int*));
     put(w.rs, rs.data(), L * sizeof(int));
@@ -875,10 +892,8 @@ int sync_factored(const ab_sync_desc* d, int L, int K, float sigma_cutoff, int d
     if (use_tc) return gemm_tc_batched(tp_w.data(), (int)tp_w.size(), w.tc_table[2], w.tc_status + 2, s2);
     return gemm_simt_batched(w.descs + 8 * L, L, mmax, nmax, s2);
   };
-  if (use_tc) {
-    AB_CUDA_OK(cudaMemsetAsync(w.tc_status, 0, 4 * sizeof(int), st));
-    AB_TRY(split3_batched(w.sjobs, 2 * L, split_blocks[0], st));                            // pieces of Abar, Bbar
-  }
+  AB_CUDA_OK(cudaMemsetAsync(w.tc_status, 0, (64 + (size_t)L) * sizeof(int), st));          // launch status and flags
+  if (use_tc) AB_TRY(split3_batched(w.sjobs, 2 * L, split_blocks[0], st));                  // pieces of Abar, Bbar
   if (any_w && !side) AB_TRY(product_w(st));
   if (use_tc) AB_TRY(gemm_tc_batched(tp_gram.data(), (int)tp_gram.size(), w.tc_table[0], w.tc_status, st));
   else AB_TRY(gemm_simt_batched(w.gram_descs, (int)gg.size(), rmax, rmax, st));             // Gram slices
@@ -889,7 +904,8 @@ int sync_factored(const ab_sync_desc* d, int L, int K, float sigma_cutoff, int d
   AB_TRY(gemm_simt_batched(w.descs + 2 * L, L, rmax, rmax, st));                            // M
   int side_rc = AB_OK;
   if (side && cudaEventRecord(fork, st) != cudaSuccess) side_rc = AB_ERR_CUDA;
-  AB_TRY(launch_jacobi(w.jobs, L, rmax, tol, st));                                    // SVD of M
+  AB_TRY(eig_direct(w.ejobs, L, rmax, w.tc_status + 3, st));                                                 // SVD of M: right vectors, sigma
+  AB_TRY(launch_jacobi(w.jobs, L, rmax, tol, st));                                          // of flagged matrices, from M
   if (side) {
     if (side_rc == AB_OK && cudaStreamWaitEvent(side, fork, 0) != cudaSuccess) side_rc = AB_ERR_CUDA;
     if (side_rc == AB_OK) side_rc = product_w(side);
@@ -911,7 +927,7 @@ int sync_factored(const ab_sync_desc* d, int L, int K, float sigma_cutoff, int d
     if (side_rc == AB_OK && cudaStreamWaitEvent(st, join, 0) != cudaSuccess) side_rc = AB_ERR_CUDA;
     if (side_rc != AB_OK) { (void)cudaGetLastError(); return side_rc; }
   }
-  if (use_tc && dev_status) {
+  if (dev_status) {
     fold_tc_status_kernel<<<1, 128, 0, st>>>(w.tc_status, dev_status, L);
     AB_LAUNCH_OK();
   }
