@@ -180,22 +180,25 @@ size_t svd_batch_ws(const SvdItem* items, int L);
 int svd_batch(const SvdItem* items, int L, float sigma_cutoff, void* ws, size_t ws_bytes, cudaStream_t st);
 
 // ---- direct symmetric eigensolver (ab_eig.cu) ---------------------------------------------------
-// Leading eigenvectors of `count` symmetric matrices of order s <= kEigSmallMax, fp64 inside.  Everything an EigJob
-// points to is device memory; eig_bind carves the scratch of one matrix (eig_ws_doubles(s) doubles).
+// Leading eigenvectors of `count` symmetric matrices, fp64 inside: any orders up to kEigSmallMax in one call, or
+// matrices of one order up to eig_max().  Everything an EigJob points to is device memory; eig_bind carves the
+// scratch of one matrix (eig_ws_doubles(s) doubles, 16-byte aligned).
 constexpr int kEigSmallMax = 256;
+int eig_max();
 struct EigJob {
   const float* X;     // s x s, row stride s
-  int gram;           // 0: the matrix is X (symmetric); 1: it is X^T X, formed in fp64 from X
+  int gram;           // 0: the matrix is X (symmetric); 1: it is X^T X, formed in fp64 from X (s <= kEigSmallMax)
   int s, need;        // order; how many eigenvectors are wanted
   float* rows;        // need x s: unit rows, descending eigenvalue
   float* vals;        // need: the eigenvalue (gram 0) or its square root, 0 below 1e-6 of the largest (gram 1); may be null
   int* flag;          // set to 1 when close vectors came out less than orthogonal (the caller clears it)
-  double *refl, *zp, *zm, *d, *e, *gam, *lam, *inv, *cross, *norm;
+  double *xbuf, *refl, *zp, *zm, *d, *e, *gam, *lam, *inv, *cross, *norm;
 };
 size_t eig_ws_doubles(int s);
 void eig_bind(EigJob& j, double* ws);
 // status: device int that receives AB_ERR_TIMEOUT if a bounded wait ran out
-int eig_direct(const EigJob* d_jobs, int count, int smax, int* status, cudaStream_t st);
+// h_jobs: the same table in host memory
+int eig_direct(const EigJob* h_jobs, const EigJob* d_jobs, int count, int smax, int* status, cudaStream_t st);
 
 // ---- factored group sync (ab_sync_fast.cu) ------------------------------------------------------
 // One-sided Jacobi on the rows of `count` s x s matrices (s <= 256) kept in shared memory, one CTA or

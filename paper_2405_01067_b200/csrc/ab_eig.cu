@@ -1,7 +1,8 @@
 // Direct eigensolver for symmetric matrices, batched: the r x r core of the factored group synchronisation and
-// the Gram matrices of the dense split (short side up to kEigSmallMax).
+// the Gram matrices of the dense split (short side up to eig_max()).
 //
-//   1. tridiag_small_kernel : Householder reduction C = H T H^T (a cluster of CTAs per matrix, C in registers)
+//   1. tridiag_small_kernel : Householder reduction C = H T H^T, order up to kEigSmallMax (a cluster of CTAs per
+//      matrix, C in registers); tridiag_grid_kernel above that (eight rows of C in the registers of each CTA)
 //   2. tri_values_kernel    : eigenvalues of T, multisection on Sturm counts
 //   3. tri_vectors_kernel   : eigenvectors of T, twisted factorisation at each eigenvalue
 //   4. back_transform_kernel: u = H z, rows sorted by descending eigenvalue, rounded to fp32
@@ -15,8 +16,8 @@
 // rotation and a write-back -- while the reduction to tridiagonal form has s - 2 steps in all.
 //
 // Vectors of eigenvalues that are closer than about 1e-10 of the norm and not separated by a zero off-diagonal
-// come out of step 3 less than orthogonal.  Step 4 checks every pair that is close and raises the matrix's flag
-// when a pair fails; the caller then runs the Jacobi route for that matrix (a kernel that returns at once when
+// come out of step 3 less than orthogonal.  Step 4 checks every pair that is close and not null (one that is zero to
+// the caller contributes nothing to either factor) and raises the matrix's flag when a pair fails; the caller then runs the Jacobi route for that matrix (a kernel that returns at once when
 // the flag is clear).
 #include <cooperative_groups.h>
 
@@ -32,8 +33,14 @@ namespace cg = cooperative_groups;
 
 constexpr double kSplitRel = 2.3e-16;   // an off-diagonal below this fraction of the norm splits T
 constexpr double kCloseRel = 1e-7;      // eigenvalues closer than this fraction of the norm are checked for orthogonality
-constexpr double kOrthTol = 1e-6;
+constexpr double kOrthTol = 4e-6;       // what the Jacobi route leaves at small orders
+constexpr int kMaxOrder = 1280;         // masks are sized for this order
+constexpr double kLive2 = 1e-290;       // a column whose squared norm is below this needs no reflector
 constexpr int kGroup = 4;               // reflectors applied together in the back transform
+
+// Eigenvalues (fractions of the norm) that carry nothing: a core's sigma below 1e-6 of the largest is zero to its
+// caller; a Gram matrix that was rounded to fp32 has noise of 2^-24 of its entries for eigenvalues down there.
+__device__ __forceinline__ double null_rel(const EigJob& job) { return job.gram ? 1e-12 : 1e-7; }
 
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
@@ -117,7 +124,7 @@ struct Tridiag {
 #pragma unroll
     for (int e = E0; e < E; ++e) pv = fma(w[e], x.v[e], pv);
     pv = warp_sum(pv);
-    const double c = 0.5 * x.gam * x.gam * pv;
+    const double c = 0.5 * x.gam * (x.gam * pv);    // gamma alone may be as large as 1e290
     const double wj = x.gam * qj.x - c * x.v1;
     double sq = 0.0;
 #pragma unroll
@@ -131,7 +138,7 @@ struct Tridiag {
     sq = warp_sum(sq);
     dj = qj.y - 2.0 * x.v1 * wj;
     const double alpha = (j + 1 < s) ? qj1.y - x.v1 * (x.gam * qj1.x - c * vj1) - wj * vj1 : 0.0;
-    const bool live = sq > 0.0;
+    const bool live = sq > kLive2;
     const double nrm = sqrt(fma(alpha, alpha, sq));
     beta = live ? (alpha > 0.0 ? -nrm : nrm) : alpha;
     x.v1 = live ? alpha - beta : 0.0;
@@ -329,6 +336,200 @@ tridiag_small_kernel(const EigJob* __restrict__ jobs, int* status) {
   t.run();
 }
 
+// ---- 1b. Householder reduction over the whole device ------------------------------------------------------
+// The same steps for orders a cluster cannot hold.  CTA c of the matrix's C = ceil(s / kGridRows) keeps rows c, c + C, ... in
+// registers; thread t owns columns t, t + 256, ... of all of them, so the vectors are spread over the CTA (every CTA works
+// out w and the next reflector for itself) and what crosses the device in a step is one (p_i, A[i][j+1]) pair per row.
+// A pair is two 8-byte words, each carrying the step in its eight lowest mantissa bits (2^-44 of the value): a reader
+// polls the words of its own columns until the step matches, so data and signal are one trip through L2.
+// A CTA leaves when its last row is finished; every CTA that still reads the pairs of step j therefore sends a row
+// of step j + 1, and whoever has all of step j + 1 may overwrite the buffer of step j (two buffers, cleared before the launch).
+// All CTAs of a matrix have to be resident together: cooperative launch.  The polls are bounded.
+// Order 768: 2.21 ms, 2.9 us a step, nearly all of it latency (the poll, three barriers, three warp reductions, a
+// square root); the pass over 8 x 768 elements is 24 multiply-adds a thread.
+constexpr int kGridRows = 8, kGridThreads = 256;
+
+__device__ __forceinline__ double tag_word(double x, unsigned tag) {
+  return __longlong_as_double((__double_as_longlong(x) & ~0xffll) | (long long)tag);
+}
+__device__ __forceinline__ unsigned word_tag(double x) { return (unsigned)__double2loint(x) & 0xffu; }
+__device__ __forceinline__ double2 ld_relaxed(const double2* p) {
+  double2 v;
+  asm volatile("ld.relaxed.gpu.global.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_relaxed(double2* p, double x, double y) {
+  asm volatile("st.relaxed.gpu.global.v2.f64 [%0], {%1, %2};" ::"l"(p), "d"(x), "d"(y) : "memory");
+}
+__device__ __forceinline__ unsigned step_tag(int j) { return 1u + (unsigned)(j % 255); }
+// waits for the pair of a step; false after about a second
+__device__ __forceinline__ bool poll_pair(const double2* p, unsigned tag, double2& v) {
+  v = ld_relaxed(p);
+  if (word_tag(v.x) == tag && word_tag(v.y) == tag) return true;
+  const uint64_t t0 = tc::globaltimer_ns();
+  for (unsigned it = 0;; ++it) {
+    v = ld_relaxed(p);
+    if (word_tag(v.x) == tag && word_tag(v.y) == tag) return true;
+    if ((it & 1023u) == 1023u && tc::globaltimer_ns() - t0 > tc::kWaitLimitNs) return false;
+  }
+}
+// sum over the CTA's eight warps of a value each warp has reduced into red[warp]
+__device__ __forceinline__ double sum8(const double* red) {
+  const double2* r = reinterpret_cast<const double2*>(red);
+  const double2 a = r[0], b = r[1], c = r[2], d = r[3];
+  return ((a.x + a.y) + (b.x + b.y)) + ((c.x + c.y) + (d.x + d.y));
+}
+
+template <int E>
+__global__ void __launch_bounds__(kGridThreads, E <= 3 ? 2 : 1)
+tridiag_grid_kernel(const EigJob* __restrict__ jobs, int count, int C, int* status) {
+  constexpr int R = kGridRows;
+  __shared__ __align__(16) double red_pv[8], red_sq[8], red_row[R][8];
+  __shared__ double2 vw[R];              // (v_i, w_i) of this CTA's rows
+  __shared__ double colbuf[R];
+  __shared__ double sc[5];               // p_j, a_j, p_j+1, a_j+1, v_j+1
+  __shared__ int dead;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int ngroups = gridDim.x / C, group = blockIdx.x / C, cta = blockIdx.x - group * C;
+  if (tid == 0) dead = 0;
+  for (int mat = group; mat < count; mat += ngroups) {
+    const EigJob job = jobs[mat];
+    const int s = job.s;
+    double2* xb = reinterpret_cast<double2*>(job.xbuf);        // 2 x s pairs
+    double A[R][E];
+    int slot[E];                         // which of this CTA's rows column k is, or -1
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      const int k = tid + kGridThreads * e;
+      slot[e] = (k < s && k % C == cta) ? k / C : -1;
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int i = cta + C * r;
+        A[r][e] = (i < s && k < s) ? (double)job.X[(size_t)i * s + k] : 0.0;
+      }
+    }
+    int last = -1;                       // this CTA's last row
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+      if (cta + C * r < s) last = cta + C * r;
+    if (tid < R && cta + C * tid < s) {
+      const int i = cta + C * tid;
+      st_relaxed(xb + i, tag_word(0.0, step_tag(0)), tag_word((double)job.X[(size_t)i * s], step_tag(0)));
+    }
+    double v[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) v[e] = 0.0;
+    double gam = 0.0, v1 = 0.0;
+    for (int j = 0; j < last; ++j) {
+      const unsigned tag = step_tag(j);
+      const double2* rb = xb + (size_t)(j & 1) * s;
+      double w[E], vn[E], pv = 0.0;
+      bool ok = true;
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        const int k = tid + kGridThreads * e;
+        w[e] = 0.0; vn[e] = 0.0;
+        if (k >= j && k < s) {
+          double2 q;
+          ok = poll_pair(rb + k, tag, q) && ok;
+          w[e] = q.x; vn[e] = q.y;
+          pv = fma(q.x, v[e], pv);
+          if (k == j) { sc[0] = q.x; sc[1] = q.y; }
+          if (k == j + 1) { sc[2] = q.x; sc[3] = q.y; sc[4] = v[e]; }
+        }
+      }
+      if (!ok) *reinterpret_cast<volatile int*>(&dead) = 1;
+      pv = warp_sum(pv);
+      if (lane == 0) red_pv[warp] = pv;
+      __syncthreads();
+      if (*reinterpret_cast<volatile int*>(&dead)) break;      // the same for all threads: a peer never answered
+      const double c = 0.5 * gam * (gam * sum8(red_pv));
+      const double wj = gam * sc[0] - c * v1;
+      double sq = 0.0;
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        const int k = tid + kGridThreads * e;
+        w[e] = gam * w[e] - c * v[e];
+        vn[e] = (k > j + 1) ? vn[e] - v1 * w[e] - wj * v[e] : 0.0;
+        sq = fma(vn[e], vn[e], sq);
+        if (slot[e] >= 0) vw[slot[e]] = make_double2(v[e], w[e]);
+      }
+      sq = warp_sum(sq);
+      if (lane == 0) red_sq[warp] = sq;
+      const double dj = sc[1] - 2.0 * v1 * wj;
+      const double alpha = sc[3] - v1 * (gam * sc[2] - c * sc[4]) - wj * sc[4];
+      __syncthreads();
+      sq = sum8(red_sq);
+      const bool live = sq > kLive2;
+      const double nrm = sqrt(fma(alpha, alpha, sq));
+      const double beta = live ? (alpha > 0.0 ? -nrm : nrm) : alpha;
+      v1 = live ? alpha - beta : 0.0;
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        if (!live) vn[e] = 0.0;
+        if (tid + kGridThreads * e == j + 1) vn[e] = v1;
+      }
+      double ps[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        ps[r] = 0.0;
+        if (cta + C * r > j) {
+          const double2 q = vw[r];
+#pragma unroll
+          for (int e = 0; e < E; ++e) {
+            A[r][e] = fma(-q.x, w[e], fma(-q.y, v[e], A[r][e]));
+            ps[r] = fma(A[r][e], vn[e], ps[r]);
+          }
+        }
+      }
+#pragma unroll
+      for (int e = 0; e < E; ++e)
+        if (tid + kGridThreads * e == j + 1) {
+#pragma unroll
+          for (int r = 0; r < R; ++r) colbuf[r] = A[r][e];
+        }
+      // eight row sums across the warp, each exchange halving what a lane still carries: lanes 4 r .. hold sum r
+      {
+        const bool h3 = (lane & 16) != 0, h2 = (lane & 8) != 0, h1 = (lane & 4) != 0;
+        double t4[4], t2[2];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) t4[q] = (h3 ? ps[q + 4] : ps[q]) + __shfl_xor_sync(0xffffffffu, h3 ? ps[q] : ps[q + 4], 16);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) t2[q] = (h2 ? t4[q + 2] : t4[q]) + __shfl_xor_sync(0xffffffffu, h2 ? t4[q] : t4[q + 2], 8);
+        double t = (h1 ? t2[1] : t2[0]) + __shfl_xor_sync(0xffffffffu, h1 ? t2[0] : t2[1], 4);
+        t += __shfl_xor_sync(0xffffffffu, t, 2);
+        t += __shfl_xor_sync(0xffffffffu, t, 1);
+        if ((lane & 3) == 0) red_row[lane >> 2][warp] = t;
+      }
+      __syncthreads();
+      if (tid < R) {
+        const int i = cta + C * tid;
+        if (i > j && i < s)
+          st_relaxed(xb + (size_t)((j + 1) & 1) * s + i, tag_word(sum8(red_row[tid]), step_tag(j + 1)), tag_word(colbuf[tid], step_tag(j + 1)));
+      }
+      gam = live ? 1.0 / (nrm * (nrm + fabs(alpha))) : 0.0;
+      // what later kernels need, from the owner of row j + 1 (it is still here)
+      if ((j + 1) % C == cta) {
+        double* dst = job.refl + (size_t)j * s;
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+          if (tid + kGridThreads * e < s) dst[tid + kGridThreads * e] = vn[e];
+        if (tid == 0) { job.d[j] = dj; job.e[j] = beta; job.gam[j] = gam; }
+      }
+#pragma unroll
+      for (int e = 0; e < E; ++e) v[e] = vn[e];
+    }
+    if (*reinterpret_cast<volatile int*>(&dead)) break;
+    if (last == s - 1) {                 // the last diagonal element is what its row would have sent
+      double* dst = job.refl + (size_t)(s - 1) * s;
+      for (int k = tid; k < s; k += kGridThreads) dst[k] = 0.0;
+      if (tid == 0) { job.d[s - 1] = colbuf[(s - 1) / C]; job.e[s - 1] = 0.0; job.gam[s - 1] = 0.0; }
+    }
+    __syncthreads();                     // colbuf is read before the next matrix writes it
+  }
+  if (tid == 0 && dead) atomicExch(status, (int)AB_ERR_TIMEOUT);
+}
+
 // ---- 2. and 3. the tridiagonal problem ------------------------------------------------------------------
 // Shared by both kernels: d and e of T scaled by 1 / norm, the positions where T splits.
 struct TriShared {
@@ -415,7 +616,7 @@ template <int kLanes>
 __global__ void __launch_bounds__(128)
 tri_values_kernel(const EigJob* __restrict__ jobs) {
   extern __shared__ __align__(16) double2 eig_sm[];
-  __shared__ unsigned mask[32];
+  __shared__ unsigned mask[kMaxOrder / 32];
   __shared__ double red[4];
   const EigJob job = jobs[blockIdx.y];
   const int s = job.s;
@@ -463,7 +664,7 @@ tri_values_kernel(const EigJob* __restrict__ jobs) {
 __global__ void __launch_bounds__(64)
 tri_vectors_kernel(const EigJob* __restrict__ jobs, int vec_blocks) {
   extern __shared__ __align__(16) double2 eig_sm[];
-  __shared__ unsigned mask[32];
+  __shared__ unsigned mask[kMaxOrder / 32];
   __shared__ double red[2];
   __shared__ double best_g[2][32];
   __shared__ int best_k[2][32];
@@ -693,7 +894,6 @@ back_transform_kernel(const EigJob* __restrict__ jobs) {
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
-  fetch(ngroups - 1);
   // rank of each vector's eigenvalue among all (descending, ties by position)
   int rank[NV];
   double lam[NV];
@@ -711,6 +911,7 @@ back_transform_kernel(const EigJob* __restrict__ jobs) {
     if (i >= s) rank[v] = s;
     wanted = wanted || rank[v] < job.need;
   }
+  if (!__syncthreads_or(wanted)) return;
   double z[NV][E];
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
@@ -722,7 +923,7 @@ back_transform_kernel(const EigJob* __restrict__ jobs) {
       z[v][e] = (wanted && i < s && k < s) ? job.zp[(size_t)k * s + i] * inv : 0.0;
     }
     // neighbours too close for the factorisation to keep apart: is this vector orthogonal to them?
-    if (i < s && rank[v] < job.need) {
+    if (i < s && rank[v] < job.need && lam[v] > null_rel(job)) {
       for (int k0 = 0; k0 < s; k0 += 32) {
         const int k = k0 + lane;
         bool close = false;
@@ -746,6 +947,7 @@ back_transform_kernel(const EigJob* __restrict__ jobs) {
       }
     }
   }
+  fetch(ngroups - 1);
   BackGroups<E, NV> bg{z, fs, gs, xs, red[warp], lane, wanted};
   bg.template segment<E - 1>(ngroups, fetch);
   const double norm = job.norm[0];
@@ -763,6 +965,141 @@ back_transform_kernel(const EigJob* __restrict__ jobs) {
       job.vals[rank[v]] = (float)(job.gram ? (l > 1e-12 * norm ? sqrt(l) : 0.0) : l);
     }
   }
+}
+
+// The same for orders above kEigSmallMax: one vector a warp, reflectors read from shared memory where they are
+// used, finished columns dropped 128 at a time.
+constexpr int kBigWarps = 4;
+template <int EB>
+struct BackBig {
+  static constexpr int E = 4 * EB, S = 32 * E;
+  double (&z)[E];
+  double (*fs)[kGroup][S];
+  const double *gs, *xs;
+  double* red;
+  int lane;
+  bool wanted;
+  template <int B0, typename F>
+  __device__ __forceinline__ void segment(int ngroups, F& fetch) {
+    constexpr int kPer = 128 / kGroup, E0 = 4 * B0;
+    for (int g = min(ngroups, (B0 + 1) * kPer) - 1; g >= B0 * kPer; --g) {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+      __syncthreads();                     // group g is here, and nobody reads the buffer of group g + 1 any more
+      if (g > 0) fetch(g - 1);
+      if (!wanted) continue;
+      const double (*f)[S] = fs[g & 1];
+      double d0 = 0.0, d1 = 0.0, d2 = 0.0, d3 = 0.0;
+#pragma unroll
+      for (int e = E0; e < E; ++e) {
+        const int k = lane + 32 * e;
+        d0 = fma(f[0][k], z[e], d0); d1 = fma(f[1][k], z[e], d1); d2 = fma(f[2][k], z[e], d2); d3 = fma(f[3][k], z[e], d3);
+      }
+      const bool h2 = (lane & 16) != 0, h1 = (lane & 8) != 0;
+      const double t0 = (h2 ? d2 : d0) + __shfl_xor_sync(0xffffffffu, h2 ? d0 : d2, 16);
+      const double t1 = (h2 ? d3 : d1) + __shfl_xor_sync(0xffffffffu, h2 ? d1 : d3, 16);
+      double t = (h1 ? t1 : t0) + __shfl_xor_sync(0xffffffffu, h1 ? t0 : t1, 8);
+      t += __shfl_xor_sync(0xffffffffu, t, 4);
+      t += __shfl_xor_sync(0xffffffffu, t, 2);
+      t += __shfl_xor_sync(0xffffffffu, t, 1);
+      __syncwarp();
+      if ((lane & 7) == 0) red[lane >> 3] = t;
+      __syncwarp();
+      const double* x = xs + g * 6;
+      const double* gm = gs + g * kGroup;
+      const double c3 = gm[3] * red[3];
+      const double c2 = gm[2] * fma(-c3, x[5], red[2]);
+      const double c1 = gm[1] * fma(-c3, x[4], fma(-c2, x[3], red[1]));
+      const double c0 = gm[0] * fma(-c3, x[2], fma(-c2, x[1], fma(-c1, x[0], red[0])));
+#pragma unroll
+      for (int e = E0; e < E; ++e) {
+        const int k = lane + 32 * e;
+        z[e] = fma(-c0, f[0][k], fma(-c1, f[1][k], fma(-c2, f[2][k], fma(-c3, f[3][k], z[e]))));
+      }
+    }
+    if constexpr (B0 > 0) segment<B0 - 1>(ngroups, fetch);
+  }
+};
+template <int EB>
+__global__ void __launch_bounds__(32 * kBigWarps)
+back_transform_big_kernel(const EigJob* __restrict__ jobs) {
+  constexpr int E = 4 * EB, S = 32 * E;
+  extern __shared__ __align__(16) double back_sm[];
+  double (*fs)[kGroup][S] = reinterpret_cast<double (*)[kGroup][S]>(back_sm);
+  double* gs = back_sm + 2 * kGroup * S;
+  double* xs = gs + S + kGroup;
+  __shared__ __align__(16) double red[kBigWarps][kGroup];
+  const EigJob job = jobs[blockIdx.y];
+  const int s = job.s;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int i = blockIdx.x * kBigWarps + warp;
+  const int ngroups = (s + kGroup - 1) / kGroup;
+  const double lam = i < s ? job.lam[i] : 0.0;
+  int rank = s;
+  if (i < s) {
+    int c = 0;
+    for (int k = lane; k < s; k += 32) {
+      const double lk = job.lam[k];
+      c += (lk > lam || (lk == lam && k < i)) ? 1 : 0;
+    }
+    rank = __reduce_add_sync(0xffffffffu, c);
+  }
+  const bool wanted = rank < job.need;
+  if (!__syncthreads_or(wanted)) return;
+  for (int k = tid; k < ngroups * kGroup; k += 32 * kBigWarps) gs[k] = k < s ? job.gam[k] : 0.0;
+  for (int k = tid; k < ngroups * 6; k += 32 * kBigWarps) xs[k] = job.cross[k];
+  auto fetch = [&](int g) {
+    const int j0 = g * kGroup, k0 = j0 & ~127, w = S - k0;
+    for (int idx = tid; idx < kGroup * w; idx += 32 * kBigWarps) {
+      const int a = idx / w, k = k0 + idx - a * w;
+      double* d = &fs[g & 1][a][k];
+      if (k < s && j0 + a < s)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(tc::smem_u32(d)), "l"(job.refl + (size_t)(j0 + a) * s + k) : "memory");
+      else
+        *d = 0.0;
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  fetch(ngroups - 1);
+  double z[E];
+  const double inv = i < s ? job.inv[i] : 0.0;
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const int k = lane + 32 * e;
+    z[e] = (wanted && k < s) ? job.zp[(size_t)k * s + i] * inv : 0.0;
+  }
+  if (wanted && lam > null_rel(job)) {
+    for (int k0 = 0; k0 < s; k0 += 32) {
+      const int k = k0 + lane;
+      bool close = false;
+      if (k < s && k != i) {
+        const double lk = job.lam[k];
+        close = fabs(lk - lam) < kCloseRel && (lk > lam || (lk == lam && k < i));
+      }
+      unsigned bal = __ballot_sync(0xffffffffu, close);
+      while (bal) {
+        const int kk = k0 + __ffs(bal) - 1;
+        bal &= bal - 1;
+        double acc = 0.0;
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+          const int q = lane + 32 * e;
+          if (q < s) acc = fma(z[e], job.zp[(size_t)q * s + kk], acc);
+        }
+        acc = warp_sum(acc) * job.inv[kk];
+        if (!(fabs(acc) <= kOrthTol) && lane == 0) *job.flag = 1;
+      }
+    }
+  }
+  BackBig<EB> bb{z, fs, gs, xs, red[warp], lane, wanted};
+  bb.template segment<EB - 1>(ngroups, fetch);
+  if (!wanted) return;
+  float* dst = job.rows + (size_t)rank * s;
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const int k = lane + 32 * e;
+    if (k < s) dst[k] = (float)z[e];
+  }
+  if (lane == 0 && job.vals) job.vals[rank] = (float)(lam * job.norm[0]);
 }
 
 template <int E, int R, int W, bool kSingle>
@@ -805,23 +1142,56 @@ int launch_back_e(const EigJob* jobs, int count, int smax, int sms, cudaStream_t
   return (long long)count * smax >= 32LL * sms ? launch_back<E, 4>(jobs, count, smax, st) : launch_back<E, 1>(jobs, count, smax, st);
 }
 
+template <int E>
+int launch_grid(const EigJob* jobs, int count, int smax, int sms, int* status, cudaStream_t st) {
+  int per_sm = 0;
+  AB_CUDA_OK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tridiag_grid_kernel<E>, kGridThreads, 0));
+  int C = (smax + kGridRows - 1) / kGridRows;
+  if (per_sm * sms < C) return AB_ERR_UNSUPPORTED;
+  const int groups = std::min(count, per_sm * sms / C);
+  void* args[] = {(void*)&jobs, (void*)&count, (void*)&C, (void*)&status};
+  AB_CUDA_OK(cudaLaunchCooperativeKernel(tridiag_grid_kernel<E>, dim3((unsigned)(groups * C)), dim3(kGridThreads), args, 0, st));
+  AB_LAUNCH_OK();
+  return AB_OK;
+}
+
+template <int EB>
+int launch_back_big(const EigJob* jobs, int count, int smax, cudaStream_t st) {
+  constexpr int S = 128 * EB;
+  const size_t sm = sizeof(double) * (2 * kGroup * S + S + kGroup + (S / kGroup + 1) * 6);
+  AB_CUDA_OK(cudaFuncSetAttribute(back_transform_big_kernel<EB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+  back_transform_big_kernel<EB><<<dim3((unsigned)((smax + kBigWarps - 1) / kBigWarps), (unsigned)count), 32 * kBigWarps, sm, st>>>(jobs);
+  AB_LAUNCH_OK();
+  return AB_OK;
+}
+
 }  // namespace
 
-size_t eig_ws_doubles(int s) { return (size_t)3 * s * s + 5 * (size_t)s + 2 * (size_t)s + 64; }
+size_t eig_ws_doubles(int s) { return align_up((size_t)3 * s * s + (4 + 5 + 2) * (size_t)s + 64, 2); }
+
+// The largest order: the grid kernel needs all CTAs of a matrix resident together.
+int eig_max() { return std::min(1184, kGridRows * std::max(sm_count(), 1)); }
 
 void eig_bind(EigJob& j, double* ws) {
   const size_t s = (size_t)j.s;
-  j.refl = ws; j.zp = j.refl + s * s; j.zm = j.zp + s * s;
+  j.xbuf = ws; j.refl = j.xbuf + 4 * s; j.zp = j.refl + s * s; j.zm = j.zp + s * s;     // xbuf first: 16-byte aligned
   j.d = j.zm + s * s; j.e = j.d + s; j.gam = j.e + s; j.lam = j.gam + s; j.inv = j.lam + s; j.cross = j.inv + s;
   j.norm = j.cross + (s + 3) / 4 * 6;
 }
 
-int eig_direct(const EigJob* d_jobs, int count, int smax, int* status, cudaStream_t st) {
-  if (smax > kEigSmallMax) return AB_ERR_UNSUPPORTED;
+int eig_direct(const EigJob* h_jobs, const EigJob* d_jobs, int count, int smax, int* status, cudaStream_t st) {
+  if (smax > eig_max()) return AB_ERR_UNSUPPORTED;
   const int sms = sm_count();
   if (sms <= 0) return AB_ERR_CUDA;
   int rc;
-  if (smax <= 64) rc = launch_tridiag<2, 8, 8, true>(d_jobs, count, 1, status, st);
+  if (smax > kEigSmallMax) {
+    for (int i = 0; i < count; ++i)       // no word of a step is there yet
+      AB_CUDA_OK(cudaMemsetAsync(h_jobs[i].xbuf, 0, (size_t)4 * h_jobs[i].s * sizeof(double), st));
+    if (smax <= 512) rc = launch_grid<2>(d_jobs, count, smax, sms, status, st);
+    else if (smax <= 768) rc = launch_grid<3>(d_jobs, count, smax, sms, status, st);
+    else if (smax <= 1024) rc = launch_grid<4>(d_jobs, count, smax, sms, status, st);
+    else rc = launch_grid<5>(d_jobs, count, smax, sms, status, st);
+  } else if (smax <= 64) rc = launch_tridiag<2, 8, 8, true>(d_jobs, count, 1, status, st);
   else if (smax <= 128) rc = launch_tridiag<4, 16, 8, true>(d_jobs, count, 1, status, st);
   else if (smax <= 192)
     rc = 6 * count <= sms ? launch_tridiag<6, 4, 8, false>(d_jobs, count, 6, status, st) : launch_tridiag<6, 12, 8, false>(d_jobs, count, 2, status, st);
@@ -836,6 +1206,10 @@ int eig_direct(const EigJob* d_jobs, int count, int smax, int* status, cudaStrea
   const int vb = (smax + 31) / 32, gb = ((smax + kGroup - 1) / kGroup + 1) / 2;
   tri_vectors_kernel<<<dim3((unsigned)(vb + gb), (unsigned)count), 64, smax * sizeof(double2), st>>>(d_jobs, vb);
   AB_LAUNCH_OK();
+  if (smax > 1024) return launch_back_big<10>(d_jobs, count, smax, st);
+  if (smax > 768) return launch_back_big<8>(d_jobs, count, smax, st);
+  if (smax > 512) return launch_back_big<6>(d_jobs, count, smax, st);
+  if (smax > kEigSmallMax) return launch_back_big<4>(d_jobs, count, smax, st);
   if (smax <= 64) return launch_back_e<2>(d_jobs, count, smax, sms, st);
   if (smax <= 128) return launch_back_e<4>(d_jobs, count, smax, sms, st);
   if (smax <= 192) return launch_back_e<6>(d_jobs, count, smax, sms, st);

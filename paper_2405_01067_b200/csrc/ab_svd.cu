@@ -15,8 +15,10 @@
 // re-measured as the norm of that product, which makes A^T A = B B^T = diag(sigma) hold by
 // construction.  No wait in these kernels can spin: every loop has a fixed trip count.
 //
-// Short sides up to kEigSmallMax take the direct solver of ab_eig.cu in place of the block Jacobi (256 x 2304:
-// 2.87 ms in the shared-memory Jacobi that they took before -> 0.47 ms); the shared-memory Jacobi is its fallback.
+// Short sides up to eig_max() (1184) take the direct solver of ab_eig.cu; the Jacobi in shared memory (up to
+// kEigSmallMax) or the block Jacobi in one cooperative launch is its fallback.  Larger ones take the block Jacobi.
+// Eigensolve of 256 x 2304: 2.87 ms in the shared-memory Jacobi -> 0.47 ms; of 3072 x 768: 21.9 ms in 1410 launches of the
+// block Jacobi -> 2.94 ms.
 #include <vector>
 #include <algorithm>
 #include <map>
@@ -24,6 +26,7 @@
 #include <cooperative_groups.h>
 
 #include "ab_common.cuh"
+#include "ab_tc_ptx.cuh"
 
 namespace ab {
 namespace {
@@ -55,8 +58,10 @@ __host__ __device__ inline float jacobi_tol(int s) {
   return t < 4e-6f ? 4e-6f : t;
 }
 
-__global__ void init_state_kernel(float* __restrict__ Vt, JState* __restrict__ st, int s, int count) {
+// flags: null, or one int per matrix; a matrix whose flag is zero is left alone (also in the kernels below)
+__global__ void init_state_kernel(float* __restrict__ Vt, JState* __restrict__ st, int s, const int* __restrict__ flags) {
   const int mat = blockIdx.y;
+  if (flags && flags[mat] == 0) return;
   float* V = Vt + (size_t)mat * s * s;
   const size_t total = (size_t)s * s;
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x)
@@ -69,9 +74,7 @@ __global__ void init_state_kernel(float* __restrict__ Vt, JState* __restrict__ s
   }
 }
 
-__global__ void sweep_end_kernel(JState* __restrict__ st, int count, float tol) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= count) return;
+__device__ __forceinline__ void sweep_end(JState* st, int i, float tol) {
   JState z = st[i];
   if (z.done) return;
   if (z.sweeps < 26) z.off_hist[z.sweeps] = __uint_as_float(z.off_bits);
@@ -82,6 +85,10 @@ __global__ void sweep_end_kernel(JState* __restrict__ st, int count, float tol) 
   if (z.next_maxn2_bits) z.maxn2_bits = z.next_maxn2_bits;
   z.next_maxn2_bits = 0;
   st[i] = z;
+}
+__global__ void sweep_end_kernel(JState* __restrict__ st, int count, float tol) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < count) sweep_end(st, i, tol);
 }
 
 // Index pair k of round t in a round-robin over an even number `ne` of players.
@@ -177,19 +184,16 @@ __device__ __forceinline__ void cta_eig32(float* Ms, float* Qs, int ldm, float t
 // the X panel and of the V^T panel.  No wait spins: the only waits are cluster barriers that every CTA of the
 // cluster reaches (all early exits depend on values the whole cluster agrees on).
 template <int PB, int kCl>
-__global__ void __launch_bounds__(256, 2)
-jacobi_pair_kernel(float* __restrict__ Xall, float* __restrict__ Vall, int s, int nb, int round,
-                   float tol, JState* __restrict__ states) {
+__device__ __forceinline__ void jacobi_pair(float* Xall, float* Vall, int s, int nb, int round, int mat, int pair, int crank,
+                                            float tol, JState* states) {
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
   constexpr int HB = PB / 2;          // rows per block
   constexpr int LDM = 33;
   constexpr int LDQ = PB + 4;
   extern __shared__ __align__(16) float smem[];
-  const int mat = blockIdx.y;
-  const int pair = blockIdx.x / kCl, crank = blockIdx.x % kCl;
   JState* st = states + mat;
-  if (st->done) return;               // the same for the whole cluster
+  if (*reinterpret_cast<volatile int*>(&st->done)) return;               // the same for the whole cluster
   const int nbe = nb + (nb & 1);
   int bi, bj;
   rr_pair(nbe, round, pair, bi, bj);
@@ -340,6 +344,68 @@ jacobi_pair_kernel(float* __restrict__ Xall, float* __restrict__ Vall, int s, in
 }
 
 template <int PB, int kCl>
+__global__ void __launch_bounds__(256, 2)
+jacobi_pair_kernel(float* __restrict__ Xall, float* __restrict__ Vall, int s, int nb, int round,
+                   float tol, JState* __restrict__ states) {
+  jacobi_pair<PB, kCl>(Xall, Vall, s, nb, round, blockIdx.y, blockIdx.x / kCl, blockIdx.x % kCl, tol, states);
+}
+
+// All sweeps of the flagged matrices in one launch, for when the block Jacobi is the fallback of the direct solver:
+// nearly always no flag is set and one empty launch is all it costs.  The blocks meet between rounds (cooperative
+// launch, so all of them are resident); bar[0] counts arrivals, bar[1] is set when a wait gave up.
+__device__ __forceinline__ bool grid_meet(unsigned* bar, unsigned& round_no) {
+  __shared__ int ok;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    ++round_no;
+    __threadfence();
+    atomicAdd(bar, 1u);
+    const unsigned want = round_no * gridDim.x;
+    const uint64_t t0 = tc::globaltimer_ns();
+    ok = 1;
+    for (unsigned it = 0; *reinterpret_cast<volatile unsigned*>(bar) < want; ++it) {
+      if (*reinterpret_cast<volatile unsigned*>(bar + 1) || ((it & 1023u) == 1023u && tc::globaltimer_ns() - t0 > tc::kWaitLimitNs)) {
+        atomicExch(bar + 1, 1u);
+        ok = 0;
+        break;
+      }
+    }
+    __threadfence();
+  }
+  __syncthreads();
+  return ok != 0;
+}
+template <int PB>
+__global__ void __launch_bounds__(256)
+jacobi_sweeps_kernel(float* Xall, float* Vall, int s, int nb, int count, float tol, JState* states, const int* flags, unsigned* bar) {
+  bool any = false;
+  for (int m = 0; m < count; ++m) any = any || flags[m] != 0;
+  if (!any) return;
+  const int nbe = nb + (nb & 1), pairs = nbe / 2, rounds = nbe > 2 ? nbe - 1 : 1;
+  unsigned round_no = 0;
+  bool met = true;
+  for (int sweep = 0; sweep < kMaxSweeps && met; ++sweep) {
+    for (int r = 0; r < rounds && met; ++r) {
+      for (int t = blockIdx.x; t < pairs * count; t += gridDim.x) {
+        const int mat = t / pairs;
+        __syncthreads();                               // the panel of the task before is no longer read
+        if (flags[mat]) jacobi_pair<PB, 1>(Xall, Vall, s, nb, r, mat, t - mat * pairs, 0, tol, states);
+      }
+      met = grid_meet(bar, round_no);
+    }
+    if (!met) break;
+    if (blockIdx.x == 0)
+      for (int m = threadIdx.x; m < count; m += blockDim.x) if (flags[m]) sweep_end(states, m, tol);
+    met = grid_meet(bar, round_no);
+    bool busy = false;
+    for (int m = 0; m < count; ++m) busy = busy || (flags[m] && !*reinterpret_cast<volatile int*>(&states[m].done));
+    if (!busy) return;
+  }
+  if (!met && blockIdx.x == 0)
+    for (int m = threadIdx.x; m < count; m += blockDim.x) if (flags[m]) states[m].status = AB_ERR_TIMEOUT;
+}
+
+template <int PB, int kCl>
 size_t jacobi_smem_bytes(int s) {
   const int s4 = (s + 3) >> 2;
   const int ldp = (((s4 + kCl - 1) / kCl) * 4) + 4;
@@ -348,9 +414,11 @@ size_t jacobi_smem_bytes(int s) {
 
 // lam[i] = |row i of X|, perm = indices by descending lam (ties by index).  One CTA per matrix.
 __global__ void __launch_bounds__(256)
-norms_sort_kernel(const float* __restrict__ Xall, int s, float* __restrict__ lam_all, int* __restrict__ perm_all) {
+norms_sort_kernel(const float* __restrict__ Xall, int s, float* __restrict__ lam_all, int* __restrict__ perm_all,
+                  const int* __restrict__ flags) {
   extern __shared__ float lam_s[];
   const int mat = blockIdx.x;
+  if (flags && flags[mat] == 0) return;
   const float* X = Xall + (size_t)mat * s * s;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int i = warp; i < s; i += 8) {
@@ -437,7 +505,8 @@ complete_basis_kernel(float* __restrict__ rows_all, const float* __restrict__ la
 // the rows orthogonal but let their norms wander by ~1e-6)
 __global__ void __launch_bounds__(256)
 gather_rows_kernel(const float* __restrict__ Vt, const int* __restrict__ perm, int s, int r_cap,
-                   float* __restrict__ Vr) {
+                   float* __restrict__ Vr, const int* __restrict__ flag) {
+  if (flag && *flag == 0) return;
   __shared__ double red[8];
   const int k = blockIdx.x;
   if (k >= r_cap) return;
@@ -564,13 +633,17 @@ struct Layout {
   std::map<int, std::vector<int>> groups;     // s -> item indices
   std::map<int, float*> X, Vt;
   std::map<int, JState*> st;
-  std::map<int, void*> jobs;                  // short side up to kEigSmallMax: EigJobs, scratch of the eigensolver,
-  std::map<int, double*> eig;                 //   fallback flags and the in-shared-memory Jacobi's scratch
-  std::map<int, int*> flags;
+  std::map<int, void*> jobs;                  // short side up to kEigSmallMax: the in-shared-memory Jacobi's scratch
+  std::map<int, double*> eig;                 // direct solver: its scratch, EigJobs, fallback flags (and behind the flags of
+  std::map<int, int*> flags;                  //   a group two words on which the blocks of the fallback meet)
   std::map<int, EigJob*> ejobs;
   std::vector<ItemWs> item;
   size_t bytes;
 };
+
+// Matrices of one order that are solved (and hold scratch) at the same time: two or three of the large ones fill the
+// device in the reduction, a dozen in the steps behind it.
+int eig_chunk(int s) { return s <= kEigSmallMax ? 1 << 20 : 12; }
 
 Layout make_layout(const SvdItem* items, int L, void* ws) {
   Layout lo;
@@ -581,11 +654,11 @@ Layout make_layout(const SvdItem* items, int L, void* ws) {
     lo.X[g.first] = ar.take_n<float>(cnt * s * s);
     lo.Vt[g.first] = ar.take_n<float>(cnt * s * s);
     lo.st[g.first] = ar.take_n<JState>(cnt);
-    if (g.first <= kEigSmallMax) {
-      lo.jobs[g.first] = ar.take_n<char>(rows_jacobi_scratch_bytes((int)cnt));
+    if (g.first <= kEigSmallMax) lo.jobs[g.first] = ar.take_n<char>(rows_jacobi_scratch_bytes((int)cnt));
+    if (g.first <= eig_max()) {
       lo.ejobs[g.first] = ar.take_n<EigJob>(cnt);
-      lo.flags[g.first] = ar.take_n<int>(cnt);
-      lo.eig[g.first] = ar.take_n<double>(cnt * eig_ws_doubles(g.first));
+      lo.flags[g.first] = ar.take_n<int>(cnt + 2);
+      lo.eig[g.first] = ar.take_n<double>(std::min(cnt, (size_t)eig_chunk(g.first)) * eig_ws_doubles(g.first));
     }
   }
   lo.item.resize(L);
@@ -650,6 +723,29 @@ int run_jacobi(float* X, float* Vt, JState* st, int s, int nb, int count, cudaSt
   return run_jacobi_cl<PB, 1>(X, Vt, st, s, nb, count, stream);
 }
 
+template <int PB>
+int run_jacobi_fallback(float* X, float* Vt, JState* st, int* flags, int s, int nb, int count, cudaStream_t stream) {
+  const size_t smem = jacobi_smem_bytes<PB, 1>(s);
+  if (smem > 227 * 1024) return AB_ERR_UNSUPPORTED;
+  AB_CUDA_OK(cudaFuncSetAttribute(jacobi_sweeps_kernel<PB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  int per_sm = 0;
+  AB_CUDA_OK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, jacobi_sweeps_kernel<PB>, 256, smem));
+  const int sms = sm_count();
+  if (sms <= 0 || per_sm <= 0) return AB_ERR_CUDA;
+  const int pairs = (nb + 1) / 2;
+  const unsigned grid = (unsigned)std::min<long long>((long long)pairs * count, (long long)per_sm * sms);
+  float tol = jacobi_tol(s);
+  unsigned* bar = reinterpret_cast<unsigned*>(flags + count);
+  const int* cflags = flags;
+  void* args[] = {&X, &Vt, &s, &nb, &count, &tol, &st, &cflags, &bar};
+  AB_CUDA_OK(cudaLaunchCooperativeKernel(jacobi_sweeps_kernel<PB>, dim3(grid), dim3(256), args, smem, stream));
+  AB_LAUNCH_OK();
+  return AB_OK;
+}
+
+// Whether a group of `count` matrices of short side s goes to the direct solver (its fallback has to fit as well).
+bool direct(int s, int count) { return s <= kEigSmallMax ? rows_jacobi_fits(count, s) : s <= eig_max(); }
+
 }  // namespace
 
 size_t svd_batch_ws(const SvdItem* items, int L) {
@@ -675,39 +771,51 @@ int svd_batch(const SvdItem* items, int L, float sigma_cutoff, void* ws, size_t 
   for (auto& g : lo.groups) {
     const int s = g.first, count = (int)g.second.size();
     Plan p = make_plan(items[g.second[0]]);
-    if (s <= kEigSmallMax && rows_jacobi_fits(count, s)) {
-      // The direct solver leaves the leading eigenvectors as unit rows in descending order in Vt.  A flagged matrix
-      // goes through the Jacobi kernel that keeps it in shared memory (the rows of G rotated until orthogonal are
-      // lambda_i v_i^T), which returns at once for the others.
+    float* lam = lo.item[g.second[0]].lam;
+    int* perm = lo.item[g.second[0]].perm;
+    if (direct(s, count)) {
+      // The direct solver leaves the leading eigenvectors as unit rows in descending order in Vr (for a group that may
+      // fall back to the Jacobi in shared memory: in Vt, where that leaves its rows).  Flagged matrices go on to the
+      // Jacobi route of their size, whose kernels return at once for the others.
+      const bool small = s <= kEigSmallMax;
+      const int chunk = std::min(count, eig_chunk(s));
       std::vector<EigJob> ej((size_t)count);
       for (int j = 0; j < count; ++j) {
         EigJob& q = ej[j];
-        q.X = lo.X[s] + (size_t)j * s * s; q.gram = 0; q.s = s; q.need = make_plan(items[g.second[j]]).r_cap;
-        q.rows = lo.Vt[s] + (size_t)j * s * s; q.vals = nullptr; q.flag = lo.flags[s] + j;
-        eig_bind(q, lo.eig[s] + (size_t)j * eig_ws_doubles(s));
+        const int idx = g.second[j];
+        q.X = lo.X[s] + (size_t)j * s * s; q.gram = 0; q.s = s; q.need = make_plan(items[idx]).r_cap;
+        q.rows = small ? lo.Vt[s] + (size_t)j * s * s : lo.item[idx].Vr; q.vals = nullptr; q.flag = lo.flags[s] + j;
+        eig_bind(q, lo.eig[s] + (size_t)(j % chunk) * eig_ws_doubles(s));
       }
       AB_CUDA_OK(cudaMemsetAsync(lo.st[s], 0, sizeof(JState) * count, stream));
-      AB_CUDA_OK(cudaMemsetAsync(lo.flags[s], 0, sizeof(int) * count, stream));
+      AB_CUDA_OK(cudaMemsetAsync(lo.flags[s], 0, sizeof(int) * (count + 2), stream));
       AB_CUDA_OK(cudaMemcpyAsync(lo.ejobs[s], ej.data(), ej.size() * sizeof(EigJob), cudaMemcpyHostToDevice, stream));
-      AB_TRY(eig_direct(lo.ejobs[s], count, s, &lo.st[s]->status, stream));
-      AB_TRY(rows_jacobi(lo.X[s], lo.Vt[s], lo.item[g.second[0]].lam, &lo.st[s]->status, sizeof(JState), lo.flags[s], count,
-                         s, lo.jobs[s], stream));
-      int r_need = 0;
-      for (int idx : g.second) r_need = std::max(r_need, make_plan(items[idx]).r_cap);
-      complete_basis_kernel<<<count, 256, 2 * (size_t)s * sizeof(float), stream>>>(lo.Vt[s], lo.item[g.second[0]].lam,
-                                                                                  lo.flags[s], s, r_need);
-      AB_LAUNCH_OK();
+      for (int j = 0; j < count; j += chunk)
+        AB_TRY(eig_direct(ej.data() + j, lo.ejobs[s] + j, std::min(chunk, count - j), s, &lo.st[s][j].status, stream));
+      if (small) {
+        AB_TRY(rows_jacobi(lo.X[s], lo.Vt[s], lam, &lo.st[s]->status, sizeof(JState), lo.flags[s], count, s, lo.jobs[s], stream));
+        int r_need = 0;
+        for (int idx : g.second) r_need = std::max(r_need, make_plan(items[idx]).r_cap);
+        complete_basis_kernel<<<count, 256, 2 * (size_t)s * sizeof(float), stream>>>(lo.Vt[s], lam, lo.flags[s], s, r_need);
+        AB_LAUNCH_OK();
+      } else {
+        init_state_kernel<<<dim3(64, (unsigned)count), 256, 0, stream>>>(lo.Vt[s], lo.st[s], s, lo.flags[s]);
+        AB_LAUNCH_OK();
+        AB_TRY(run_jacobi_fallback<32>(lo.X[s], lo.Vt[s], lo.st[s], lo.flags[s], s, p.nb, count, stream));
+        norms_sort_kernel<<<count, 256, (size_t)s * sizeof(float), stream>>>(lo.X[s], s, lam, perm, lo.flags[s]);
+        AB_LAUNCH_OK();
+      }
       continue;
     }
     dim3 ig(64, (unsigned)count);
-    init_state_kernel<<<ig, 256, 0, stream>>>(lo.Vt[s], lo.st[s], s, count);
+    init_state_kernel<<<ig, 256, 0, stream>>>(lo.Vt[s], lo.st[s], s, nullptr);
     AB_LAUNCH_OK();
     int rc;
     if (p.pb == 32) rc = run_jacobi<32>(lo.X[s], lo.Vt[s], lo.st[s], s, p.nb, count, stream);
     else rc = run_jacobi<16>(lo.X[s], lo.Vt[s], lo.st[s], s, p.nb, count, stream);
     AB_TRY(rc);
     norms_sort_kernel<<<count, 256, (size_t)s * sizeof(float), stream>>>(
-        lo.X[s], s, lo.item[g.second[0]].lam, lo.item[g.second[0]].perm);
+        lo.X[s], s, lam, perm, nullptr);
     AB_LAUNCH_OK();
   }
   // 3. per matrix: leading vectors, long-side product, sigma, rank rule, factors
@@ -719,10 +827,11 @@ int svd_batch(const SvdItem* items, int L, float sigma_cutoff, void* ws, size_t 
       Plan p = make_plan(it);
       ItemWs w = lo.item[i];
       float* Vt = lo.Vt[s] + j * (size_t)s * s;
-      if (s <= kEigSmallMax && rows_jacobi_fits((int)g.second.size(), s)) {
+      const bool solved = direct(s, (int)g.second.size());
+      if (solved && s <= kEigSmallMax) {
         w.Vr = Vt;                  // unit rows in order already
       } else {
-        gather_rows_kernel<<<p.r_cap, 256, 0, stream>>>(Vt, w.perm, s, p.r_cap, w.Vr);
+        gather_rows_kernel<<<p.r_cap, 256, 0, stream>>>(Vt, w.perm, s, p.r_cap, w.Vr, solved ? lo.flags[s] + j : nullptr);
         AB_LAUNCH_OK();
       }
       int64_t yt, yk;   // Ylong(k,t) = Y[t*yt + k*yk]

@@ -904,7 +904,7 @@ int sync_factored(const ab_sync_desc* d, int L, int K, float sigma_cutoff, int d
   AB_TRY(gemm_simt_batched(w.descs + 2 * L, L, rmax, rmax, st));                            // M
   int side_rc = AB_OK;
   if (side && cudaEventRecord(fork, st) != cudaSuccess) side_rc = AB_ERR_CUDA;
-  AB_TRY(eig_direct(w.ejobs, L, rmax, w.tc_status + 3, st));                                                 // SVD of M: right vectors, sigma
+  AB_TRY(eig_direct(ej.data(), w.ejobs, L, rmax, w.tc_status + 3, st));                                                 // SVD of M: right vectors, sigma
   AB_TRY(launch_jacobi(w.jobs, L, rmax, tol, st));                                          // of flagged matrices, from M
   if (side) {
     if (side_rc == AB_OK && cudaStreamWaitEvent(side, fork, 0) != cudaSuccess) side_rc = AB_ERR_CUDA;

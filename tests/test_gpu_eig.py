@@ -33,7 +33,8 @@ def spectrum(kind, s):
 
 
 @pytest.mark.parametrize("kind", ["random", "clustered", "equal", "low_rank", "zero_columns", "diagonal"])
-@pytest.mark.parametrize("s", [1, 2, 3, 31, 32, 33, 64, 65, 97, 128, 129, 160, 192, 193, 225, 256])
+@pytest.mark.parametrize("s", [1, 2, 3, 31, 32, 33, 64, 65, 97, 128, 129, 160, 192, 193, 225, 256,
+                               257, 512, 513, 765, 768, 769, 1024, 1025, 1184])
 def test_split_by_order_and_spectrum(ab, s, kind):
     rng = np.random.default_rng(1000 * s + len(kind))
     m, n = s + 40, s
