@@ -324,21 +324,20 @@ chain_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant__ C
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
-    // One thread feeds the tensor pipe; its own instruction count per MMA is kept small: the descriptors of
-    // slot 0 are built once, a slot is an addition, a K step is an addition (32 bytes along a K-major row,
-    // 2048 bytes -- 16 rows -- down an MN-major tile), and the four K steps are unrolled.  (Measured: a second
-    // issuing thread, one per block of a unit, changes nothing -- 100.7 against 102.2 us for a ViT forward:
-    // the pipe itself takes about 200 cycles per 128 x 256 x 16 MMA here.)
-    if (lane == 0) {
+    // The descriptors of slot 0 are built once, a slot is an addition, a K step is an addition (32 bytes along a K-major
+    // row, 2048 bytes -- 16 rows -- down an MN-major tile), and the four K steps are unrolled.  The whole warp walks the
+    // loop and one elected lane issues (see elect_one).
+    {
+      const uint32_t tmem = uniform(tmem_base);
       const uint32_t idesc1 = instr_desc_bf16(128, p.r, 0, p.f1_mn);
       const uint32_t idesc2 = instr_desc_bf16(128, kChunk, 0, p.f2_mn);
-      const uint32_t s_base = smem_u32(smem);
+      const uint32_t s_base = uniform(smem_u32(smem));
       const uint64_t dA1 = smem_desc_sw128(s_base, 16);                          // In tile of block 0, slot 0
       const uint64_t dF1 = p.f1_mn ? smem_desc_sw128(s_base + p.max_blocks * kAtomBytes, kF1AtomBytes)
                                    : smem_desc_sw128(s_base + p.max_blocks * kAtomBytes, 16);
       const uint64_t f1_step = p.f1_mn ? (2048u >> 4) : 2u;
       const uint64_t slot_step = (uint64_t)(p.slot_bytes >> 4);
-      const uint64_t dS = smem_desc_sw128(smem_u32(S0), 16);                     // S tile 0 of block 0
+      const uint64_t dS = smem_desc_sw128(uniform(smem_u32(S0)), 16);                     // S tile 0 of block 0
       const uint64_t dF2 = p.f2_mn ? smem_desc_sw128(s_base, kF1AtomBytes) : smem_desc_sw128(s_base, 16);
       const uint64_t f2_step = p.f2_mn ? (2048u >> 4) : 2u;
       const uint64_t blk_step = (uint64_t)(kAtomBytes >> 4);
@@ -351,59 +350,67 @@ chain_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant__ C
         const int nt = un.nt;
         int kr = rot1;
         for (int ks = 0; ks < p.nk1; ++ks) {
-          if (!mbar_wait(&bars->full[slot1], ph1, lim)) { raise_timeout(bars, p.status); ok = false; break; }
+          if (!mbar_wait_warp(&bars->full[slot1], ph1, lim)) { raise_timeout(bars, p.status); ok = false; break; }
           tc_fence_after();
           const uint64_t da0 = dA1 + slot_step * slot1, db0 = dF1 + slot_step * slot1;
           const int ksteps = p.cv.on ? (p.cv.in_ch - (kr % p.cv.cslabs) * 64 + 15) >> 4 : (p.K1 - kr * 64 + 15) >> 4;
           const uint32_t acc0 = ks != 0;
-          if (nt == 2) {
+          if (elect_one()) {
+            if (nt == 2) {
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk) {
               if (kk < ksteps) {
-                tc_mma_bf16(tmem_base, da0 + 2 * kk, db0 + f1_step * kk, idesc1, kk ? 1u : acc0);
-                tc_mma_bf16(tmem_base + 256, da0 + blk_step + 2 * kk, db0 + f1_step * kk, idesc1, kk ? 1u : acc0);
+                tc_mma_bf16(tmem, da0 + 2 * kk, db0 + f1_step * kk, idesc1, kk ? 1u : acc0);
+                tc_mma_bf16(tmem + 256, da0 + blk_step + 2 * kk, db0 + f1_step * kk, idesc1, kk ? 1u : acc0);
               }
             }
           } else {
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk)
-              if (kk < ksteps) tc_mma_bf16(tmem_base, da0 + 2 * kk, db0 + f1_step * kk, idesc1, kk ? 1u : acc0);
+              if (kk < ksteps) tc_mma_bf16(tmem, da0 + 2 * kk, db0 + f1_step * kk, idesc1, kk ? 1u : acc0);
           }
-          tc_commit(&bars->empty[slot1]);
+            tc_commit(&bars->empty[slot1]);
+          }
+          __syncwarp();
           if (++slot1 == p.ns) { slot1 = 0; ph1 ^= 1; }
           if (++kr == p.nk1) kr = 0;
         }
         if (!ok) break;
-        tc_commit(&bars->t_full);
+        if (elect_one()) tc_commit(&bars->t_full);
+        __syncwarp();
         if (p.nchunks > 0) {
-          if (!mbar_wait(&bars->s_ready, u & 1, lim)) { raise_timeout(bars, p.status); ok = false; break; }
+          if (!mbar_wait_warp(&bars->s_ready, u & 1, lim)) { raise_timeout(bars, p.status); ok = false; break; }
           tc_fence_after();
         }
         for (int c = 0; c < p.nchunks && ok; ++c) {
           for (int tt = 0; tt < nt && ok; ++tt) {
             const int b = (nt == 2) ? tt : (c & 1);
-            if (!mbar_wait(&bars->acc_empty[b], ((b ? q1 : q0) & 1) ^ 1, lim)) { raise_timeout(bars, p.status); ok = false; break; }
+            if (!mbar_wait_warp(&bars->acc_empty[b], ((b ? q1 : q0) & 1) ^ 1, lim)) { raise_timeout(bars, p.status); ok = false; break; }
             tc_fence_after();
-            const uint32_t tacc = tmem_base + kChunk * b;
+            const uint32_t tacc = tmem + kChunk * b;
             const uint64_t dSb = dS + blk_step * (uint64_t)(tt * p.natoms);
             for (int j = 0; j < p.natoms; ++j) {
               const int idx = i2 + j, slot = idx % p.ns2, ph = (idx / p.ns2) & 1;
-              if (!mbar_wait(&bars->full2[slot], ph, lim)) { raise_timeout(bars, p.status); ok = false; break; }
+              if (!mbar_wait_warp(&bars->full2[slot], ph, lim)) { raise_timeout(bars, p.status); ok = false; break; }
               tc_fence_after();
               const uint64_t da = dSb + blk_step * j;
               const uint64_t db = dF2 + (uint64_t)(kAtom2Bytes >> 4) * slot;
               const int ksteps = (p.r - j * 64) >> 4;
               const uint32_t acc0 = j != 0;
+              if (elect_one()) {
 #pragma unroll
-              for (int kk = 0; kk < 4; ++kk)
-                if (kk < ksteps) tc_mma_bf16(tacc, da + 2 * kk, db + f2_step * kk, idesc2, kk ? 1u : acc0);
-              if (tt == nt - 1) tc_commit(&bars->empty2[slot]);     // the last block of the unit is done with this tile
+                for (int kk = 0; kk < 4; ++kk)
+                  if (kk < ksteps) tc_mma_bf16(tacc, da + 2 * kk, db + f2_step * kk, idesc2, kk ? 1u : acc0);
+                if (tt == nt - 1) tc_commit(&bars->empty2[slot]);     // the last block of the unit is done with this tile
+              }
+              __syncwarp();
             }
-            if (ok) { tc_commit(&bars->acc_full[b]); if (b) ++q1; else ++q0; }
+            if (ok) { if (elect_one()) tc_commit(&bars->acc_full[b]); __syncwarp(); if (b) ++q1; else ++q0; }
           }
           i2 += p.natoms;
         }
-        if (ok) tc_commit(&bars->unit_done);
+        if (ok && elect_one()) tc_commit(&bars->unit_done);
+        __syncwarp();
         g += un.adv;
       }
     }
@@ -548,6 +555,32 @@ chain_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant__ C
   }
 }
 
+// The MMA warp of both gradient kernels: nk slabs of 64, two 128-row accumulators sharing every slab of `small`.
+__device__ __forceinline__ void grad_mma_loop(Bars* bars, uint8_t* ring, int nk, int ns, int slot_bytes, int r, uint32_t tmem_base,
+                                              int* status) {
+  const uint32_t idesc = instr_desc_bf16(128, r, 1, 1), tmem = uniform(tmem_base);
+  const uint64_t d0 = smem_desc_sw128(uniform(smem_u32(ring)), 8192), slot_step = (uint64_t)(slot_bytes >> 4);
+  int slot = 0, ph = 0;
+  for (int i = 0; i < nk; ++i) {
+    if (!mbar_wait_warp(&bars->full[slot], ph)) { raise_timeout(bars, status); return; }
+    tc_fence_after();
+    const uint64_t d = d0 + slot_step * slot;
+    if (elect_one()) {
+#pragma unroll
+      for (int kk = 0; kk < 4; ++kk) {
+        const uint64_t da = d + 128 * kk, db = da + (32768 >> 4);
+        tc_mma_bf16(tmem, da, db, idesc, (i | kk) != 0);
+        tc_mma_bf16(tmem + 256, da + (16384 >> 4), db, idesc, (i | kk) != 0);
+      }
+      tc_commit(&bars->empty[slot]);
+    }
+    __syncwarp();
+    if (++slot == ns) { slot = 0; ph ^= 1; }
+  }
+  if (elect_one()) tc_commit(&bars->t_full);
+  __syncwarp();
+}
+
 // ---------------------------------------------------------------------------------------------
 // grad kernel: partial[slice][p][j] = sum_{k in slice} act[k][p] * small[k][j]
 struct GradJob {
@@ -627,23 +660,7 @@ grad_kernel(const __grid_constant__ CUtensorMap tmAct0, const __grid_constant__ 
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      const uint32_t idesc = instr_desc_bf16(128, p.r, 1, 1);
-      bool ok = true;
-      for (int i = 0; i < nk; ++i) {
-        const int slot = i % p.ns, ph = (i / p.ns) & 1;
-        if (!mbar_wait(&bars->full[slot], ph)) { raise_timeout(bars, p.status); ok = false; break; }
-        tc_fence_after();
-        const uint32_t sa = smem_u32(ring + (size_t)slot * p.slot_bytes);
-        for (int kk = 0; kk < 4; ++kk) {
-          const uint64_t db = smem_desc_sw128(sa + 32768 + kk * 2048, 8192);
-          tc_mma_bf16(tmem_base, smem_desc_sw128(sa + kk * 2048, 8192), db, idesc, (i | kk) != 0);
-          tc_mma_bf16(tmem_base + 256, smem_desc_sw128(sa + 16384 + kk * 2048, 8192), db, idesc, (i | kk) != 0);
-        }
-        tc_commit(&bars->empty[slot]);
-      }
-      if (ok) tc_commit(&bars->t_full);
-    }
+    grad_mma_loop(bars, ring, nk, p.ns, p.slot_bytes, p.r, tmem_base, p.status);
   } else {
     const int q = warp & 3;
     const int row = q * 32 + lane;
@@ -760,23 +777,7 @@ conv_grad_kernel(const __grid_constant__ CUtensorMap tmX4, const __grid_constant
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      const uint32_t idesc = instr_desc_bf16(128, p.r, 1, 1);
-      bool ok = true;
-      for (int i = 0; i < nk; ++i) {
-        const int slot = i % p.ns, ph = (i / p.ns) & 1;
-        if (!mbar_wait(&bars->full[slot], ph)) { raise_timeout(bars, p.status); ok = false; break; }
-        tc_fence_after();
-        const uint32_t sa = smem_u32(ring + (size_t)slot * p.slot_bytes);
-        for (int kk = 0; kk < 4; ++kk) {
-          const uint64_t db = smem_desc_sw128(sa + 32768 + kk * 2048, 8192);
-          tc_mma_bf16(tmem_base, smem_desc_sw128(sa + kk * 2048, 8192), db, idesc, (i | kk) != 0);
-          tc_mma_bf16(tmem_base + 256, smem_desc_sw128(sa + 16384 + kk * 2048, 8192), db, idesc, (i | kk) != 0);
-        }
-        tc_commit(&bars->empty[slot]);
-      }
-      if (ok) tc_commit(&bars->t_full);
-    }
+    grad_mma_loop(bars, ring, nk, p.ns, p.slot_bytes, p.r, tmem_base, p.status);
   } else {
     const int q = warp & 3;
     const int row = q * 32 + lane;

@@ -148,37 +148,39 @@ gemm_tc_kernel(const TcProblemDev* __restrict__ probs, int nprobs, int ntiles, i
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      int i = 0, it = 0;
+    {
+      int slot = 0, ph = 0, it = 0;
       bool ok = true;
+      const uint32_t sbase = uniform(smem_u32(ring)), tmem = uniform(tmem_base);
       for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, ++it) {
         const TileInfo ti = decode_tile(probs, nprobs, tile);
-        const TcProblemDev* P = ti.P;
-        const int a_mn = P->a_mn, b_mn = P->b_mn;
-        const uint32_t idesc = instr_desc_bf16(kBM, ti.nmma, a_mn, b_mn);
+        const int nterms = (int)uniform(ti.P->nterms), nslab = (int)uniform(ti.nslab), klen = (int)uniform(ti.k_end - ti.k_begin);
+        const int a_mn = (int)uniform(ti.P->a_mn), b_mn = (int)uniform(ti.P->b_mn);
+        const uint32_t idesc = instr_desc_bf16(kBM, (int)uniform(ti.nmma), a_mn, b_mn);
+        const uint64_t da0 = smem_desc_sw128(sbase, a_mn ? 8192 : 16), db0 = smem_desc_sw128(sbase + kAStage, b_mn ? 8192 : 16);
+        const uint64_t as = a_mn ? 128u : 2u, bs = b_mn ? 128u : 2u;      // 16 of the reduction, in 16-byte units
         const int b = it & 1;
-        if (!mbar_wait(&bars->acc_empty[b], ((it >> 1) & 1) ^ 1)) { tc_raise(bars, status); ok = false; break; }
+        if (!mbar_wait_warp(&bars->acc_empty[b], ((it >> 1) & 1) ^ 1)) { tc_raise(bars, status); ok = false; break; }
         tc_fence_after();
-        const uint32_t tacc = tmem_base + 256 * b;
-        int first = 1;
-        for (int tix = 0; tix < P->nterms && ok; ++tix) {
-          for (int ks = 0; ks < ti.nslab; ++ks, ++i) {
-            const int slot = i % kStages, ph = (i / kStages) & 1;
-            if (!mbar_wait(&bars->full[slot], ph)) { tc_raise(bars, status); ok = false; break; }
+        const uint32_t tacc = tmem + 256 * b;
+        for (int tix = 0; tix < nterms && ok; ++tix) {
+          for (int ks = 0; ks < nslab; ++ks) {
+            if (!mbar_wait_warp(&bars->full[slot], ph)) { tc_raise(bars, status); ok = false; break; }
             tc_fence_after();
-            const uint32_t sa = smem_u32(ring + (size_t)slot * kStage), sb = sa + kAStage;
-            int ksteps = (ti.k_end - (ti.k_begin + ks * kBK) + 15) >> 4;
-            if (ksteps > 4) ksteps = 4;
-            for (int kk = 0; kk < ksteps; ++kk) {
-              const uint64_t da = a_mn ? smem_desc_sw128(sa + kk * 2048, 8192) : smem_desc_sw128(sa, 16) + 2 * kk;
-              const uint64_t db = b_mn ? smem_desc_sw128(sb + kk * 2048, 8192) : smem_desc_sw128(sb, 16) + 2 * kk;
-              tc_mma_bf16(tacc, da, db, idesc, first ? 0u : 1u);
-              first = 0;
+            const uint64_t da = da0 + (uint64_t)(slot * (kStage >> 4)), db = db0 + (uint64_t)(slot * (kStage >> 4));
+            const int ksteps = (klen - ks * kBK + 15) >> 4;
+            if (elect_one()) {
+#pragma unroll
+              for (int kk = 0; kk < 4; ++kk)
+                if (kk < ksteps) tc_mma_bf16(tacc, da + as * kk, db + bs * kk, idesc, (tix | ks | kk) ? 1u : 0u);
+              tc_commit(&bars->empty[slot]);
             }
-            tc_commit(&bars->empty[slot]);
+            __syncwarp();
+            if (++slot == kStages) { slot = 0; ph ^= 1; }
           }
         }
-        if (ok) tc_commit(&bars->acc_full[b]);
+        if (ok && elect_one()) tc_commit(&bars->acc_full[b]);
+        __syncwarp();
       }
     }
   } else {

@@ -115,6 +115,21 @@ __device__ __forceinline__ void tc_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
                : "memory");
 }
+// True in one lane of a converged warp.  MMAs are issued under this by a warp whose control flow is uniform, not under
+// a lane comparison: the compiler then knows that they run in one thread and keeps descriptors in uniform registers.
+// Under "lane == 0" every MMA waits for moves from vector registers: 165 to 200 cycles an MMA whatever its width, against
+// 51 (N = 64), 65 (N = 128) and about 130 (N = 256).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.b32 %0, 1, 0, q;\n\t}" : "=r"(p));
+  return p != 0;
+}
+// A value that is the same in all lanes, known to the compiler as such.
+__device__ __forceinline__ uint32_t uniform(uint32_t x) { return __shfl_sync(0xffffffffu, x, 0); }
+// The whole warp waits; the verdict is a vote, on which the compiler branches uniformly.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, uint64_t limit_ns = kWaitLimitNs) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, limit_ns));
+}
 // D[tmem] (+)= A[smem] * B[smem], bf16 inputs, fp32 accumulate; one thread issues.
 __device__ __forceinline__ void tc_mma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
                                             uint32_t accumulate) {
