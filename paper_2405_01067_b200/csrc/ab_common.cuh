@@ -74,22 +74,11 @@ int gemm_simt(const void* A, int a_dt, int64_t sAm, int64_t sAk,
               void* C, int c_dt, int64_t ldc,
               int64_t M, int64_t N, int64_t K, cudaStream_t st);
 
-// Batched form for the small products of the factored group sync: problem z of the batch is
-// described by one GemmDesc in device memory.  fp32 operands; optional diagonal scalings
-//   C[i,j] = rs(i) * cs(j) * sum_k A(i,k) * ks(k) * B(k,j)
-// where each of rs/cs/ks is derived from a vector v sorted in descending order:
-//   mode 0: 1,  mode 1: sqrt(v),  mode 2: 1/sqrt(v);  entries with v <= thr * v[0] count as 0.
-// Rows >= *live_rows and columns >= *live_cols (device ints, optional) are written as zero.
+// One fp32 problem of the register-tiled kernel.
 struct GemmDesc {
   const float* A; const float* B; void* C;
   int64_t sAm, sAk, sBk, sBn, ldc;
   int M, N, K;
-  int c_bf16;
-  const float* row_vec; const float* col_vec; const float* k_vec;
-  int row_mode, col_mode, k_mode;
-  float thr;
-  const int* live_rows; const int* live_cols;
-  int upper_only;   // 1: tiles entirely below the diagonal are skipped (symmetric result, upper part used)
   // Operand prologue that averages group copies (0 / 1 copies: plain operand).  Copy c of A starts a_cstride
   // elements after copy c - 1; the loader adds the copies in ascending c in fp32 and scales by copy_inv, the
   // arithmetic of the group mean.  The CTAs of the first tile column / row also write the averaged operand out.
@@ -99,7 +88,6 @@ struct GemmDesc {
   float* a_mean_out;   // optional, M x K row-major
   float* b_mean_out;   // optional, K x N row-major
 };
-int gemm_simt_batched(const GemmDesc* d_descs, int count, int max_M, int max_N, cudaStream_t st);
 // W = mean_k(A_k) mean_k(B_k) in one kernel (the mean as the product's operand prologue); Abar, Bbar optional outputs.
 int recombine_mean_simt(const float* A_copies, int64_t strideA, const float* B_copies, int64_t strideB, int K,
                         float* W, float* Abar, float* Bbar, int m, int n, int r, cudaStream_t st);
@@ -128,10 +116,33 @@ size_t gemm_tc_table_bytes(int count);
 // table_dev: device memory of gemm_tc_table_bytes(count); status: device int that receives AB_ERR_TIMEOUT
 // if a bounded wait ran out (never cleared here).
 int gemm_tc_batched(const TcProblem* probs, int count, void* table_dev, int* status, cudaStream_t st);
-struct SplitJob { const float* src; int64_t ld_src; int rows, cols; bf16 *hi, *mid, *lo; int64_t ld_dst; int64_t first_block; };
-int64_t split_job_blocks(int rows, int cols);
-int split3_batched(const SplitJob* d_jobs, int njobs, int64_t total_blocks, cudaStream_t st);
 int sum_slices(const float* part, float* out, int64_t count, int64_t slice_stride, int slices, cudaStream_t st);
+
+// ---- batched fp32-accurate products with the split in the loader (ab_gemm_split.cu) --------------------------
+// C[i,j] = rs(i) cs(j) sum_k A(i,k) B(j,k).  A(i,k) at A[i * lda + k] (a_mn 0) or A[k * lda + i] (a_mn 1), B(j,k)
+// likewise.  rs, cs from a vector v sorted in descending order: mode 0: 1, 1: sqrt(v), 2: 1/sqrt(v), entries v <= thr v[0]
+// count as 0.  Rows >= *live_rows and columns >= *live_cols (device ints, optional) are written as zero.  K >= 1.
+struct SplitGemm {
+  const void* A; const void* B; void* C;
+  int64_t lda, ldb, ldc;
+  int M, N, K;
+  int a_mn, b_mn;
+  int c_bf16;
+  int upper_only;           // 1: tiles entirely below the diagonal are skipped
+  const float* row_vec; const float* col_vec;
+  int row_mode, col_mode;
+  float thr;
+  const int* live_rows; const int* live_cols;
+  int first_tile;           // set by gemm_split_plan
+};
+struct SplitBatch { int count, tiles, bn; };
+SplitBatch gemm_split_plan(SplitGemm* probs, int count);      // fills first_tile; the table then goes to the device
+int gemm_split_batched(const SplitGemm* d_probs, const SplitBatch& b, int* status, cudaStream_t st);   // fp32 operands
+int gemm_split_one(SplitGemm p, bool src_bf16, int* status, cudaStream_t st);    // one problem; clears *status first
+
+// Copies a host table to the device in pieces the runtime stages without waiting for the stream (a pageable copy of
+// more than 64 KB waits until the stream has drained).
+int upload_async(void* dst, const void* src, size_t bytes, cudaStream_t st);
 
 // ---- dense layer of the full-rank phases (ab_dense.cu) ------------------------------------------
 size_t dense_forward_ws(int64_t N, int m, int n);

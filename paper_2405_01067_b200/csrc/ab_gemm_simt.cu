@@ -5,8 +5,8 @@
 //    slabs staged in shared memory, 4x4 accumulators per thread.  Each 16-term partial dot
 //    product is formed in fp32 and added to a running fp64 sum, so long reductions keep ~1e-7
 //    relative accuracy; the order of additions is fixed by the shape alone.
-//  - gemm_simt_batched_kernel: many fp32 GEMMs per launch with diagonal scalings and live-rank
-//    masks (the group synchronisation's products), register-tiled 8x8 and double-buffered.
+//  - gemm_simt_one_kernel: large all-fp32 problems, register-tiled 8x8 and double-buffered; also the recombination with
+//    the group mean in its loader.
 #include "ab_common.cuh"
 
 namespace ab {
@@ -96,15 +96,8 @@ int launch(const void* A, int64_t sAm, int64_t sAk, const void* B, int64_t sBk, 
   return AB_OK;
 }
 
-__device__ __forceinline__ float diag_scale(const float* v, int idx, int mode, float thr) {
-  if (mode == 0 || v == nullptr) return 1.f;
-  const float x = v[idx];
-  if (!(x > thr * v[0]) || !(x > 0.f)) return 0.f;
-  return mode == 1 ? sqrtf(x) : 1.f / sqrtf(x);
-}
-
-// ---- batched fp32 GEMM with diagonal scalings ---------------------------------------------------
-// One descriptor per blockIdx.z.  BM_ x BN_ output tile, 8 x 8 accumulators per thread (two 4-wide
+// ---- register-tiled fp32 GEMM --------------------------------------------------------------------
+// BM_ x BN_ output tile, 8 x 8 accumulators per thread (two 4-wide
 // groups half a tile apart, so the float4 operand reads from shared memory are conflict-free and an
 // 8 x 8 update needs four of them: the FMA pipe, not the shared-memory port, is the limit), 16-deep k
 // slabs double-buffered: the next slab's global loads are issued before the current slab's FMAs and
@@ -140,8 +133,7 @@ struct TileIo {
     const bool al = (reinterpret_cast<uintptr_t>(p) & 15u) == 0;
     vec = al && (along_k ? (sk == 1 && (sr & 3) == 0) : (sr == 1 && (sk & 3) == 0));
   }
-  __device__ __forceinline__ void fetch(float4 (&v)[F], int64_t r0, int R, int64_t k0, int K, const float* kvec,
-                                        int kmode, float thr, int tid) const {
+  __device__ __forceinline__ void fetch(float4 (&v)[F], int64_t r0, int R, int64_t k0, int K, int tid) const {
 #pragma unroll
     for (int e = 0; e < F; ++e) {
       const int f = tid + e * NT;
@@ -159,10 +151,6 @@ struct TileIo {
           for (int j = 0; j < 4; ++j) t[j] = (gr < R && gk + j < K) ? p[j * s_k] : 0.f;
           if (copies > 1 && gr < R) add_copies(t, p, false, s_k, (int)(K - gk < 4 ? (K - gk < 0 ? 0 : K - gk) : 4));
         }
-        if (kvec) {
-#pragma unroll
-          for (int j = 0; j < 4; ++j) if (gk + j < K) t[j] *= diag_scale(kvec, (int)(gk + j), kmode, thr);
-        }
       } else {
         const int r4 = f % (R_ / 4), kk = f / (R_ / 4);
         const int64_t gr = r0 + 4 * r4, gk = k0 + kk;
@@ -175,11 +163,6 @@ struct TileIo {
 #pragma unroll
           for (int j = 0; j < 4; ++j) t[j] = (gr + j < R && gk < K) ? p[j * s_r] : 0.f;
           if (copies > 1 && gk < K) add_copies(t, p, false, s_r, (int)(R - gr < 4 ? (R - gr < 0 ? 0 : R - gr) : 4));
-        }
-        if (kvec && gk < K) {
-          const float sc = diag_scale(kvec, (int)gk, kmode, thr);
-#pragma unroll
-          for (int j = 0; j < 4; ++j) t[j] *= sc;
         }
       }
       v[e] = make_float4(t[0], t[1], t[2], t[3]);
@@ -226,7 +209,6 @@ __device__ __forceinline__ void gemm_tile_8x8(const GemmDesc& d) {
   constexpr int NT = (BM_ / 8) * (BN_ / 8);
   const int64_t m0 = (int64_t)blockIdx.y * BM_, n0 = (int64_t)blockIdx.x * BN_;
   if (m0 >= d.M || n0 >= d.N) return;
-  if (d.upper_only && n0 + BN_ <= m0) return;
   __shared__ __align__(16) float As[2][BK][BM_ + 4];
   __shared__ __align__(16) float Bs[2][BK][BN_ + 4];
   const int tid = threadIdx.x;
@@ -247,8 +229,8 @@ __device__ __forceinline__ void gemm_tile_8x8(const GemmDesc& d) {
     for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
 
   const int nk = (d.K + BK - 1) / BK;
-  ioA.fetch(va, m0, d.M, 0, d.K, d.k_vec, d.k_mode, d.thr, tid);
-  ioB.fetch(vb, n0, d.N, 0, d.K, nullptr, 0, 0.f, tid);
+  ioA.fetch(va, m0, d.M, 0, d.K, tid);
+  ioB.fetch(vb, n0, d.N, 0, d.K, tid);
   if (emit_a) ioA.emit(d.a_mean_out, d.K, 1, va, m0, d.M, 0, d.K, tid);
   if (emit_b) ioB.emit(d.b_mean_out, 1, d.N, vb, n0, d.N, 0, d.K, tid);
   ioA.stash(As[0], va, tid);
@@ -258,8 +240,8 @@ __device__ __forceinline__ void gemm_tile_8x8(const GemmDesc& d) {
     const int cur = kt & 1;
     const bool more = kt + 1 < nk;
     if (more) {
-      ioA.fetch(va, m0, d.M, (int64_t)(kt + 1) * BK, d.K, d.k_vec, d.k_mode, d.thr, tid);
-      ioB.fetch(vb, n0, d.N, (int64_t)(kt + 1) * BK, d.K, nullptr, 0, 0.f, tid);
+      ioA.fetch(va, m0, d.M, (int64_t)(kt + 1) * BK, d.K, tid);
+      ioB.fetch(vb, n0, d.N, (int64_t)(kt + 1) * BK, d.K, tid);
       if (emit_a) ioA.emit(d.a_mean_out, d.K, 1, va, m0, d.M, (int64_t)(kt + 1) * BK, d.K, tid);
       if (emit_b) ioB.emit(d.b_mean_out, 1, d.N, vb, n0, d.N, (int64_t)(kt + 1) * BK, d.K, tid);
     }
@@ -283,56 +265,31 @@ __device__ __forceinline__ void gemm_tile_8x8(const GemmDesc& d) {
     __syncthreads();
   }
 
-  const int live_r = d.live_rows ? *d.live_rows : d.M;
-  const int live_c = d.live_cols ? *d.live_cols : d.N;
   const bool c_vec = (d.ldc & 3) == 0 && (reinterpret_cast<uintptr_t>(d.C) & 15u) == 0;
-  float cs[8];
-#pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    const int64_t gn = n0 + (j < 4 ? tx * 4 + j : BN_ / 2 + tx * 4 + (j - 4));
-    cs[j] = (gn < d.N && gn < live_c) ? diag_scale(d.col_vec, (int)gn, d.col_mode, d.thr) : 0.f;
-  }
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     const int64_t gm = m0 + (i < 4 ? ty * 4 + i : BM_ / 2 + ty * 4 + (i - 4));
     if (gm >= d.M) continue;
-    const float rs = gm < live_r ? diag_scale(d.row_vec, (int)gm, d.row_mode, d.thr) : 0.f;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int64_t gn = n0 + (h == 0 ? tx * 4 : BN_ / 2 + tx * 4);
       float v[4];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) v[j] = acc[i][4 * h + j] * rs * cs[4 * h + j];
+      for (int j = 0; j < 4; ++j) v[j] = acc[i][4 * h + j];
       if (c_vec && gn + 3 < d.N) {
-        if (d.c_bf16) {
-          __nv_bfloat162 lo = __floats2bfloat162_rn(v[0], v[1]), hi = __floats2bfloat162_rn(v[2], v[3]);
-          uint2 pk;
-          pk.x = *reinterpret_cast<uint32_t*>(&lo);
-          pk.y = *reinterpret_cast<uint32_t*>(&hi);
-          *reinterpret_cast<uint2*>(static_cast<bf16*>(d.C) + gm * d.ldc + gn) = pk;
-        } else {
-          *reinterpret_cast<float4*>(static_cast<float*>(d.C) + gm * d.ldc + gn) = make_float4(v[0], v[1], v[2], v[3]);
-        }
+        *reinterpret_cast<float4*>(static_cast<float*>(d.C) + gm * d.ldc + gn) = make_float4(v[0], v[1], v[2], v[3]);
       } else {
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           if (gn + j >= d.N) continue;
-          if (d.c_bf16) static_cast<bf16*>(d.C)[gm * d.ldc + gn + j] = __float2bfloat16_rn(v[j]);
-          else static_cast<float*>(d.C)[gm * d.ldc + gn + j] = v[j];
+          static_cast<float*>(d.C)[gm * d.ldc + gn + j] = v[j];
         }
       }
     }
   }
 }
 
-template <int BM_, int BN_>
-__global__ void __launch_bounds__((BM_ / 8) * (BN_ / 8), 512 / ((BM_ / 8) * (BN_ / 8)))
-gemm_simt_batched_kernel(const GemmDesc* __restrict__ descs) {
-  const GemmDesc d = descs[blockIdx.z];
-  gemm_tile_8x8<BM_, BN_>(d);
-}
-
-// The same tile code for one problem whose descriptor travels as a kernel argument.
+// The descriptor travels as a kernel argument.
 template <int BM_, int BN_>
 __global__ void __launch_bounds__((BM_ / 8) * (BN_ / 8), 512 / ((BM_ / 8) * (BN_ / 8)))
 gemm_simt_one_kernel(const __grid_constant__ GemmDesc d) {
@@ -348,38 +305,14 @@ int launch_one(const GemmDesc& d, cudaStream_t st) {
   return AB_OK;
 }
 
-template <int BM_, int BN_>
-int launch_batched(const GemmDesc* d_descs, int count, int max_M, int max_N, cudaStream_t st) {
-  dim3 grid((unsigned)((max_N + BN_ - 1) / BN_), (unsigned)((max_M + BM_ - 1) / BM_), (unsigned)count);
-  if (grid.y > 65535u || grid.z > 65535u) return AB_ERR_UNSUPPORTED;
-  gemm_simt_batched_kernel<BM_, BN_><<<grid, (BM_ / 8) * (BN_ / 8), 0, st>>>(d_descs);
-  AB_LAUNCH_OK();
-  return AB_OK;
-}
-
 }  // namespace
-
-// Tile edges of 128 for the long dimensions (m, n), 64 for the rank-sized ones.
-int gemm_simt_batched(const GemmDesc* d_descs, int count, int max_M, int max_N, cudaStream_t st) {
-  if (count <= 0 || max_M <= 0 || max_N <= 0) return AB_OK;
-  const bool bigM = max_M >= 512, bigN = max_N >= 512;
-  if (bigM && bigN) return launch_batched<128, 128>(d_descs, count, max_M, max_N, st);
-  if (bigM) return launch_batched<128, 64>(d_descs, count, max_M, max_N, st);
-  if (bigN) return launch_batched<64, 128>(d_descs, count, max_M, max_N, st);
-  return launch_batched<64, 64>(d_descs, count, max_M, max_N, st);
-}
 
 int recombine_mean_simt(const float* A_copies, int64_t strideA, const float* B_copies, int64_t strideB, int K,
                         float* W, float* Abar, float* Bbar, int m, int n, int r, cudaStream_t st) {
   GemmDesc d;
   d.A = A_copies; d.B = B_copies; d.C = W;
   d.sAm = r; d.sAk = 1; d.sBk = n; d.sBn = 1; d.ldc = n;
-  d.M = m; d.N = n; d.K = r; d.c_bf16 = 0;
-  d.row_vec = d.col_vec = d.k_vec = nullptr;
-  d.row_mode = d.col_mode = d.k_mode = 0;
-  d.thr = 0.f;
-  d.live_rows = d.live_cols = nullptr;
-  d.upper_only = 0;
+  d.M = m; d.N = n; d.K = r;
   d.a_copies = d.b_copies = K; d.a_cstride = strideA; d.b_cstride = strideB; d.copy_inv = 1.0f / (float)K;
   d.a_mean_out = Abar; d.b_mean_out = Bbar;
   const bool bigM = m >= 512, bigN = n >= 512;
@@ -402,12 +335,7 @@ int gemm_simt(const void* A, int a_dt, int64_t sAm, int64_t sAk,
     GemmDesc d;
     d.A = static_cast<const float*>(A); d.B = static_cast<const float*>(B); d.C = C;
     d.sAm = sAm; d.sAk = sAk; d.sBk = sBk; d.sBn = sBn; d.ldc = ldc;
-    d.M = (int)M; d.N = (int)N; d.K = (int)K; d.c_bf16 = 0;
-    d.row_vec = d.col_vec = d.k_vec = nullptr;
-    d.row_mode = d.col_mode = d.k_mode = 0;
-    d.thr = 0.f;
-    d.live_rows = d.live_cols = nullptr;
-    d.upper_only = 0;
+    d.M = (int)M; d.N = (int)N; d.K = (int)K;
     d.a_copies = d.b_copies = 1; d.a_cstride = d.b_cstride = 0; d.copy_inv = 1.f; d.a_mean_out = d.b_mean_out = nullptr;
     const bool bigM = M >= 512, bigN = N >= 512;
     if (bigM && bigN) return launch_one<128, 128>(d, st);

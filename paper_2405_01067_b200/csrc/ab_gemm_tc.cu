@@ -284,55 +284,6 @@ gemm_tc_kernel(const TcProblemDev* __restrict__ probs, int nprobs, int ntiles, i
   }
 }
 
-// ---------------------------------------------------------------------------------------------
-// fp32 -> three bf16 pieces: hi = bf16(x), mid = bf16(x - hi), lo = bf16(x - hi - mid); hi + mid + lo = x to
-// 2^-24 (the subtractions are exact).  One job per matrix, all jobs in one launch.
-__global__ void __launch_bounds__(256)
-split3_kernel(const SplitJob* __restrict__ jobs, int njobs) {
-  int lo = 0, hi = njobs - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (jobs[mid].first_block <= (int64_t)blockIdx.x) lo = mid; else hi = mid - 1;
-  }
-  const SplitJob j = jobs[lo];
-  // four consecutive elements of a row per thread when the rows allow 16-byte loads and 8-byte stores
-  const bool vec = (j.cols & 3) == 0 && (j.ld_src & 3) == 0 && (j.ld_dst & 3) == 0 &&
-                   ((reinterpret_cast<uintptr_t>(j.src) & 15u) == 0) && ((reinterpret_cast<uintptr_t>(j.hi) & 7u) == 0) &&
-                   ((reinterpret_cast<uintptr_t>(j.mid) & 7u) == 0) && ((reinterpret_cast<uintptr_t>(j.lo) & 7u) == 0);
-  const unsigned cols4 = (unsigned)(j.cols + 3) >> 2;
-  const unsigned total4 = (unsigned)j.rows * cols4;
-  const unsigned i = (unsigned)((int64_t)blockIdx.x - j.first_block) * 256u + threadIdx.x;
-  if (i >= total4) return;
-  const unsigned r = i / cols4, c = (i - r * cols4) * 4u;
-  float x[4];
-  const float* src = j.src + (int64_t)r * j.ld_src + c;
-  if (vec) {
-    const float4 q = *reinterpret_cast<const float4*>(src);
-    x[0] = q.x; x[1] = q.y; x[2] = q.z; x[3] = q.w;
-  } else {
-#pragma unroll
-    for (int e = 0; e < 4; ++e) x[e] = (c + e < (unsigned)j.cols) ? src[e] : 0.f;
-  }
-  bf16 h[4], m[4], l[4];
-#pragma unroll
-  for (int e = 0; e < 4; ++e) {
-    h[e] = __float2bfloat16_rn(x[e]);
-    const float r1 = x[e] - __bfloat162float(h[e]);
-    m[e] = __float2bfloat16_rn(r1);
-    l[e] = __float2bfloat16_rn(r1 - __bfloat162float(m[e]));
-  }
-  const int64_t o = (int64_t)r * j.ld_dst + c;
-  if (vec) {
-    *reinterpret_cast<uint2*>(j.hi + o) = *reinterpret_cast<const uint2*>(h);
-    *reinterpret_cast<uint2*>(j.mid + o) = *reinterpret_cast<const uint2*>(m);
-    *reinterpret_cast<uint2*>(j.lo + o) = *reinterpret_cast<const uint2*>(l);
-  } else {
-#pragma unroll
-    for (int e = 0; e < 4; ++e)
-      if (c + e < (unsigned)j.cols) { j.hi[o + e] = h[e]; j.mid[o + e] = m[e]; j.lo[o + e] = l[e]; }
-  }
-}
-
 // out[i] = sum over slices of part[s][i], ascending s (fixed order); partials are rows_pad x ld, out is rows x ld
 __global__ void __launch_bounds__(256)
 sum_slices_kernel(const float* __restrict__ part, float* __restrict__ out, int64_t count, int64_t slice_stride, int slices) {
@@ -344,16 +295,6 @@ sum_slices_kernel(const float* __restrict__ part, float* __restrict__ out, int64
 }
 
 }  // namespace
-
-int64_t split_job_blocks(int rows, int cols) { return ((int64_t)rows * ((cols + 3) / 4) + 255) / 256; }
-
-int split3_batched(const SplitJob* d_jobs, int njobs, int64_t total_blocks, cudaStream_t st) {
-  if (njobs <= 0 || total_blocks <= 0) return AB_OK;
-  if (total_blocks > ((int64_t)1 << 30)) return AB_ERR_UNSUPPORTED;
-  split3_kernel<<<(unsigned)total_blocks, 256, 0, st>>>(d_jobs, njobs);
-  AB_LAUNCH_OK();
-  return AB_OK;
-}
 
 int sum_slices(const float* part, float* out, int64_t count, int64_t slice_stride, int slices, cudaStream_t st) {
   if (count <= 0) return AB_OK;

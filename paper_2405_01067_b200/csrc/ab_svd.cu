@@ -789,7 +789,7 @@ int svd_batch(const SvdItem* items, int L, float sigma_cutoff, void* ws, size_t 
       }
       AB_CUDA_OK(cudaMemsetAsync(lo.st[s], 0, sizeof(JState) * count, stream));
       AB_CUDA_OK(cudaMemsetAsync(lo.flags[s], 0, sizeof(int) * (count + 2), stream));
-      AB_CUDA_OK(cudaMemcpyAsync(lo.ejobs[s], ej.data(), ej.size() * sizeof(EigJob), cudaMemcpyHostToDevice, stream));
+      AB_TRY(upload_async(lo.ejobs[s], ej.data(), ej.size() * sizeof(EigJob), stream));
       for (int j = 0; j < count; j += chunk)
         AB_TRY(eig_direct(ej.data() + j, lo.ejobs[s] + j, std::min(chunk, count - j), s, &lo.st[s][j].status, stream));
       if (small) {

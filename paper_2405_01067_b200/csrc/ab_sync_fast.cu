@@ -528,24 +528,35 @@ __global__ void __launch_bounds__(kCThreads, 1) chol_inv_kernel(const CholJob* _
 
 size_t chol_smem_bytes(int r) { return sizeof(float) * ((size_t)r * (r + 1) + r) + 64; }
 
-// r' = #{ i < r : sigma_i >= cutoff * sigma_0 } (at least 1); folds the three solver statuses.
-__global__ void fast_rank_rule_kernel(const float* const* __restrict__ sigma, const int* __restrict__ rs,
-                                      float cutoff, int* const* __restrict__ r_out,
-                                      const int* __restrict__ jstatus, int* __restrict__ dev_status, int L) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+// r' = #{ i < r : sigma_i >= cutoff * sigma_0 } (at least 1); folds the three solver statuses.  A warp per matrix (one
+// thread per matrix walked its values one load after the other: 31 us for 72 matrices of rank 192).
+__global__ void __launch_bounds__(128)
+fast_rank_rule_kernel(const float* const* __restrict__ sigma, const int* __restrict__ rs,
+                      float cutoff, int* const* __restrict__ r_out,
+                      const int* __restrict__ jstatus, int* __restrict__ dev_status, int L) {
+  const int i = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (i >= L) return;
   const float* sg = sigma[i];
   const int r = rs[i];
-  float top = 0.f;
-  for (int k = 0; k < r; ++k) top = fmaxf(top, sg[k]);
+  float v[8], top = 0.f;               // r <= 256
+#pragma unroll
+  for (int e = 0; e < 8; ++e) {
+    v[e] = lane + 32 * e < r ? sg[lane + 32 * e] : 0.f;
+    top = fmaxf(top, v[e]);
+  }
+  top = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(top)));
   int keep = 0;
-  for (int k = 0; k < r; ++k) keep += (sg[k] >= cutoff * top) ? 1 : 0;
-  if (keep < 1) keep = 1;
+#pragma unroll
+  for (int e = 0; e < 8; ++e) keep += (lane + 32 * e < r && v[e] >= cutoff * top) ? 1 : 0;
+  keep = max(1, __reduce_add_sync(0xffffffffu, keep));
+  int low = 0;                         // a kept value below the accuracy domain
+#pragma unroll
+  for (int e = 0; e < 8; ++e) low |= (lane + 32 * e < keep && v[e] < kFDomainRel * top && v[e] > kFZeroRel * top) ? 1 : 0;
+  low = __any_sync(0xffffffffu, low);
+  if (lane != 0) return;
   *r_out[i] = keep;
   if (dev_status) {
-    int st = AB_OK;
-    for (int k = 0; k < keep; ++k)
-      if (sg[k] < kFDomainRel * top && sg[k] > kFZeroRel * top) st = AB_ERR_ACCURACY;
+    int st = low ? AB_ERR_ACCURACY : AB_OK;
     for (int j = 0; j < 3; ++j) if (jstatus[3 * i + j] == AB_ERR_ACCURACY) st = AB_ERR_ACCURACY;
     for (int j = 0; j < 3; ++j)          // a solver that did not converge outranks the accuracy note
       if (jstatus[3 * i + j] != AB_OK && jstatus[3 * i + j] != AB_ERR_ACCURACY) st = jstatus[3 * i + j];
@@ -561,19 +572,28 @@ __global__ void fold_tc_status_kernel(const int* __restrict__ tc_status, int* __
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < L; i += gridDim.x * blockDim.x) dev_status[i] = bad;
 }
 
-// The long index of a Gram product is cut into slices of about kGramSlice (at most kGramMaxParts).
-constexpr int kGramSlice = 768, kGramMaxParts = 8;
-int gram_parts(int len) { return std::max(1, std::min(kGramMaxParts, (len + kGramSlice - 1) / kGramSlice)); }
-int gram_k0(int len, int parts, int q) {      // start of slice q (a multiple of 16), len for q == parts
-  if (q >= parts) return len;
-  const int per = (((len + parts - 1) / parts) + 15) / 16 * 16;
-  return std::min(len, q * per);
+// The long index of a Gram product is cut into slices, whose partial sums the Cholesky kernel adds in ascending
+// order: short enough that the slices of all matrices give every SM a tile, at least 128 (two slabs; a lone
+// 512 x 4608 layer of rank 64 then takes 19 CTAs instead of two), at most 768, at most kGramMaxParts of them.
+constexpr int kGramMaxParts = 16;
+int gram_slice(const ab_sync_desc* d, int L) {
+  int64_t work = 0;                     // tiles x length
+  for (int i = 0; i < L; ++i) {
+    const int64_t t = (d[i].r + 127) / 128;
+    work += t * (t + 1) / 2 * ((int64_t)d[i].m + d[i].n);
+  }
+  const int64_t per = (work / std::max(sm_count(), 1) + 63) / 64 * 64;
+  return (int)std::max<int64_t>(128, std::min<int64_t>(768, per));
 }
+int gram_per(int len, int slice) {      // length of a part, a multiple of 64
+  const int parts = std::max(1, std::min(kGramMaxParts, (len + slice - 1) / slice));
+  return ((len + parts - 1) / parts + 63) / 64 * 64;
+}
+int gram_parts(int len, int slice) { const int per = gram_per(len, slice); return (len + per - 1) / per; }
 
 struct FastWs {
   std::vector<float*> Abar, Bbar, GA, GB, RA, RB, IA, IB, M, Vs, Y1, ZA, ZB;
-  GemmDesc* descs;      // 9 L
-  GemmDesc* gram_descs; // up to 2 kGramMaxParts L
+  SplitGemm* gemms;     // the products of all launches, one after the other: up to (2 kGramMaxParts + 7) L
   CholJob* cjobs;       // 2 L
   AvgJob* ajobs;        // 2 L
   JacobiJob* jobs;      // L
@@ -582,20 +602,15 @@ struct FastWs {
   const float** sig_ptrs;
   int** rout_ptrs;
   int* rs;
-  // tensor-core route of the long products: bf16 pieces (hi, mid, lo) of Abar, Bbar, Z_A, Z_B
-  SplitJob* sjobs;      // 4 L
-  std::vector<bf16*> Asp, Bsp, ZAsp, ZBsp;    // each: three pieces one after the other
-  void* tc_table[3];    // problem tables of the three tensor-core launches
-  int* tc_status;       // 64, and behind them one fallback flag per matrix (see EigJob)
+  int* tc_status;       // 64 (what the products' and the eigensolver's waits report), and behind them one fallback flag per matrix (see EigJob)
   std::vector<double*> eig;   // scratch of the eigensolver
   size_t bytes;
 };
 
-int r8(int v) { return (v + 7) & ~7; }
-
 FastWs fast_layout(const ab_sync_desc* d, int L, void* ws) {
   FastWs w;
   Arena ar(ws, 0);
+  const int slice = gram_slice(d, L);
   auto each = [&](std::vector<float*>& v, auto count) {
     v.resize(L);
     for (int i = 0; i < L; ++i) v[i] = ar.take_n<float>(count(d[i]));
@@ -603,12 +618,13 @@ FastWs fast_layout(const ab_sync_desc* d, int L, void* ws) {
   each(w.Abar, [](const ab_sync_desc& x) { return (size_t)x.m * x.r; });
   each(w.Bbar, [](const ab_sync_desc& x) { return (size_t)x.r * x.n; });
   auto rr = [](const ab_sync_desc& x) { return (size_t)x.r * x.r; };
-  each(w.GA, [](const ab_sync_desc& x) { return (size_t)gram_parts(x.m) * x.r * x.r; });
-  each(w.GB, [](const ab_sync_desc& x) { return (size_t)gram_parts(x.n) * x.r * x.r; });
+  each(w.GA, [=](const ab_sync_desc& x) { return (size_t)gram_parts(x.m, slice) * x.r * x.r; });
+  each(w.GB, [=](const ab_sync_desc& x) { return (size_t)gram_parts(x.n, slice) * x.r * x.r; });
   each(w.RA, rr); each(w.RB, rr); each(w.IA, rr); each(w.IB, rr);
   each(w.M, rr); each(w.Vs, rr); each(w.Y1, rr); each(w.ZA, rr); each(w.ZB, rr);
-  w.descs = ar.take_n<GemmDesc>((size_t)9 * L);
-  w.gram_descs = ar.take_n<GemmDesc>((size_t)2 * kGramMaxParts * L);
+  size_t ngemm = (size_t)7 * L;
+  for (int i = 0; i < L; ++i) ngemm += gram_parts(d[i].m, slice) + gram_parts(d[i].n, slice);
+  w.gemms = ar.take_n<SplitGemm>(ngemm);
   w.cjobs = ar.take_n<CholJob>((size_t)2 * L);
   w.ajobs = ar.take_n<AvgJob>((size_t)2 * L);
   w.jobs = ar.take_n<JacobiJob>((size_t)L);
@@ -617,18 +633,6 @@ FastWs fast_layout(const ab_sync_desc* d, int L, void* ws) {
   w.sig_ptrs = ar.take_n<const float*>(L);
   w.rout_ptrs = ar.take_n<int*>(L);
   w.rs = ar.take_n<int>(L);
-  w.sjobs = ar.take_n<SplitJob>((size_t)4 * L);
-  auto each_bf = [&](std::vector<bf16*>& v, auto count) {
-    v.resize(L);
-    for (int i = 0; i < L; ++i) v[i] = ar.take_n<bf16>(3 * count(d[i]));
-  };
-  each_bf(w.Asp, [](const ab_sync_desc& x) { return (size_t)x.m * r8(x.r); });
-  each_bf(w.Bsp, [](const ab_sync_desc& x) { return (size_t)x.r * r8(x.n); });
-  each_bf(w.ZAsp, [](const ab_sync_desc& x) { return (size_t)x.r * r8(x.r); });
-  each_bf(w.ZBsp, [](const ab_sync_desc& x) { return (size_t)x.r * r8(x.r); });
-  w.tc_table[0] = ar.take(gemm_tc_table_bytes(2 * L));
-  w.tc_table[1] = ar.take(gemm_tc_table_bytes(2 * L));
-  w.tc_table[2] = ar.take(gemm_tc_table_bytes(L));
   w.tc_status = ar.take_n<int>(64 + (size_t)L);
   w.eig.resize(L);
   for (int i = 0; i < L; ++i) w.eig[i] = ar.take_n<double>(eig_ws_doubles(d[i].r));
@@ -636,24 +640,12 @@ FastWs fast_layout(const ab_sync_desc* d, int L, void* ws) {
   return w;
 }
 
-TcOperand pieces3(const bf16* base, size_t piece_elems, int64_t ld, bool mn) {
-  TcOperand o;
-  for (int k = 0; k < 3; ++k) o.p[k] = base + k * piece_elems;
-  o.pieces = 3; o.ld = ld; o.mn = mn;
-  return o;
-}
-
-GemmDesc mk(const float* A, int64_t sAm, int64_t sAk, const float* B, int64_t sBk, int64_t sBn, void* C, int64_t ldc,
-            int M, int N, int K) {
-  GemmDesc g;
-  g.A = A; g.B = B; g.C = C; g.sAm = sAm; g.sAk = sAk; g.sBk = sBk; g.sBn = sBn; g.ldc = ldc;
-  g.M = M; g.N = N; g.K = K; g.c_bf16 = 0;
-  g.row_vec = g.col_vec = g.k_vec = nullptr;
-  g.row_mode = g.col_mode = g.k_mode = 0;
+SplitGemm product(const void* A, int64_t lda, int a_mn, const void* B, int64_t ldb, int b_mn, void* C, int64_t ldc, int M, int N,
+                  int K) {
+  SplitGemm g;
+  std::memset(&g, 0, sizeof(g));
+  g.A = A; g.lda = lda; g.a_mn = a_mn; g.B = B; g.ldb = ldb; g.b_mn = b_mn; g.C = C; g.ldc = ldc; g.M = M; g.N = N; g.K = K;
   g.thr = kEigThr;
-  g.live_rows = g.live_cols = nullptr;
-  g.upper_only = 0;
-  g.a_copies = g.b_copies = 1; g.a_cstride = g.b_cstride = 0; g.copy_inv = 1.f; g.a_mean_out = g.b_mean_out = nullptr;
   return g;
 }
 
@@ -699,7 +691,7 @@ int rows_jacobi(const float* X, float* rows, float* norms, int* status, size_t s
     int* stj = reinterpret_cast<int*>(reinterpret_cast<char*>(status) + (size_t)j * status_stride_bytes);
     jb[j] = JacobiJob{X + (size_t)j * s * s, rows + (size_t)j * s * s, norms + (size_t)j * s, stj, flags + j, s, s};
   }
-  AB_CUDA_OK(cudaMemcpyAsync(scratch, jb.data(), jb.size() * sizeof(JacobiJob), cudaMemcpyHostToDevice, st));
+  AB_TRY(upload_async(scratch, jb.data(), jb.size() * sizeof(JacobiJob), st));
   return launch_jacobi(static_cast<const JacobiJob*>(scratch), count, s, rows_jacobi_tol(s), st);
 }
 
@@ -717,27 +709,16 @@ int sync_factored(const ab_sync_desc* d, int L, int K, float sigma_cutoff, int d
                   void* ws, size_t ws_bytes, cudaStream_t st) {
   FastWs w = fast_layout(d, L, ws);
   if (w.bytes > ws_bytes) return AB_ERR_WORKSPACE;
+  if (!gemm_tc_available()) return AB_ERR_UNSUPPORTED;
   const int out_bf16 = (dt == AB_BF16) ? 1 : 0;
-  int rmax = 0, mmax = 0, nmax = 0;
-  for (int i = 0; i < L; ++i) {
-    rmax = std::max(rmax, d[i].r); mmax = std::max(mmax, d[i].m); nmax = std::max(nmax, d[i].n);
-  }
-  // The long products (Gram matrices, A', B', W) run on the tensor cores as six-term bf16 products when
-  // every output can be stored by 16-byte rows; otherwise on the fp32 pipes.
-  bool use_tc = gemm_tc_available();
-  for (int i = 0; i < L && use_tc; ++i) {
-    const int q = out_bf16 ? 8 : 4;
-    use_tc = d[i].r % 4 == 0 && d[i].r % q == 0 && d[i].n % q == 0 && aligned(d[i].A_out, 16) && aligned(d[i].B_out, 16) &&
-             (!d[i].W_out || (d[i].n % 4 == 0 && aligned(d[i].W_out, 16)));
-  }
-  std::vector<SplitJob> sj((size_t)4 * L);
-  std::vector<TcProblem> tp_gram, tp_out, tp_w;
-  int64_t split_blocks[2] = {0, 0};
-  // ---- host-built tables: 9 GEMM descriptors, 2 Cholesky jobs and 1 Jacobi job per matrix, copied in one go each
-  std::vector<GemmDesc> g((size_t)9 * L);
+  const int slice = gram_slice(d, L);
+  int rmax = 0;
+  bool any_w = false;
+  for (int i = 0; i < L; ++i) { rmax = std::max(rmax, d[i].r); any_w = any_w || d[i].W_out != nullptr; }
+  // ---- host-built tables, uploaded together.  The products, by launch:
+  enum { kGram, kM, kZ1, kZ2, kOut, kW, kLaunches };
+  std::vector<SplitGemm> g[kLaunches];
   std::vector<CholJob> cj((size_t)2 * L);
-  std::vector<GemmDesc> gg;
-  gg.reserve((size_t)2 * kGramMaxParts * L);
   std::vector<JacobiJob> jb((size_t)L);
   std::vector<EigJob> ej((size_t)L);
   std::vector<const float*> sigp(L);
@@ -746,84 +727,36 @@ int sync_factored(const ab_sync_desc* d, int L, int K, float sigma_cutoff, int d
   for (int i = 0; i < L; ++i) {
     const int m = d[i].m, n = d[i].n, r = d[i].r;
     float *Ab = w.Abar[i], *Bb = w.Bbar[i];
-    // (slots 0 .. 2L of this table are unused: the Gram products G_A = Abar^T Abar and
-    // G_B = Bbar Bbar^T have a table of their own, one entry per slice of the long index)
-    g[0 * L + i] = mk(nullptr, 0, 0, nullptr, 0, 0, nullptr, 0, 0, 0, 0);
-    g[1 * L + i] = g[0 * L + i];
-    // batch 1 (L): M = R_A R_B^T
-    g[2 * L + i] = mk(w.RA[i], r, 1, w.RB[i], 1, r, w.M[i], r, r, r, r);
-    // batch 2 (2L): Y1 = M Vs^T ;  Z_B = diag(sqrt sig) Vs R_B^-T
-    g[3 * L + i] = mk(w.M[i], r, 1, w.Vs[i], 1, r, w.Y1[i], r, r, r, r);
-    GemmDesc& gzb = g[4 * L + i];
-    gzb = mk(w.Vs[i], r, 1, w.IB[i], 1, r, w.ZB[i], r, r, r, r);
-    gzb.row_vec = d[i].sigma; gzb.row_mode = 1;
-    // batch 3 (L): Z_A = R_A^-1 Y1 diag(sig^-1/2)
-    GemmDesc& gza = g[5 * L + i];
-    gza = mk(w.IA[i], r, 1, w.Y1[i], r, 1, w.ZA[i], r, r, r, r);
-    gza.col_vec = d[i].sigma; gza.col_mode = 2;
-    // batch 4 (L): A' = Abar Z_A (columns >= r' zero);  batch 5 (L): B' = Z_B Bbar (rows >= r' zero)
-    GemmDesc& ga = g[6 * L + i];
-    ga = mk(Ab, r, 1, w.ZA[i], r, 1, d[i].A_out, r, m, r, r);
-    ga.c_bf16 = out_bf16; ga.live_cols = d[i].r_out;
-    GemmDesc& gb = g[7 * L + i];
-    gb = mk(w.ZB[i], r, 1, Bb, n, 1, d[i].B_out, n, r, n, r);
-    gb.c_bf16 = out_bf16; gb.live_rows = d[i].r_out;
-    // batch 6 (L, optional): W = Abar Bbar
-    g[8 * L + i] = mk(Ab, r, 1, Bb, n, 1, d[i].W_out, n, d[i].W_out ? m : 0, d[i].W_out ? n : 0, r);
-    const int pa = use_tc ? 1 : gram_parts(m), pb = use_tc ? 1 : gram_parts(n);
-    if (use_tc) {
-      const int rr8 = r8(r), n8 = r8(n);
-      const size_t ea = (size_t)m * rr8, eb = (size_t)r * n8, ez = (size_t)r * rr8;
-      sj[2 * i] = SplitJob{Ab, r, m, r, w.Asp[i], w.Asp[i] + ea, w.Asp[i] + 2 * ea, rr8, 0};
-      sj[2 * i + 1] = SplitJob{Bb, n, r, n, w.Bsp[i], w.Bsp[i] + eb, w.Bsp[i] + 2 * eb, n8, 0};
-      sj[2 * L + 2 * i] = SplitJob{w.ZA[i], r, r, r, w.ZAsp[i], w.ZAsp[i] + ez, w.ZAsp[i] + 2 * ez, rr8, 0};
-      sj[2 * L + 2 * i + 1] = SplitJob{w.ZB[i], r, r, r, w.ZBsp[i], w.ZBsp[i] + ez, w.ZBsp[i] + 2 * ez, rr8, 0};
-      for (int h = 0; h < 2; ++h) {
-        sj[2 * i + h].first_block = split_blocks[0];
-        split_blocks[0] += split_job_blocks(sj[2 * i + h].rows, sj[2 * i + h].cols);
-        sj[2 * L + 2 * i + h].first_block = split_blocks[1];
-        split_blocks[1] += split_job_blocks(r, r);
-      }
-      const TcOperand A_k = pieces3(w.Asp[i], ea, rr8, false), A_t = pieces3(w.Asp[i], ea, rr8, true);
-      const TcOperand B_k = pieces3(w.Bsp[i], eb, n8, false), B_t = pieces3(w.Bsp[i], eb, n8, true);
-      TcProblem q;
-      q.ksplit = 1; q.live_rows = q.live_cols = nullptr; q.c_f32 = true;
-      // G_A = Abar^T Abar: both operands are Abar as it lies, (reduction index m) x r
-      q.A = A_t; q.B = A_t; q.C = w.GA[i]; q.ldc = r; q.M = r; q.N = r; q.K = m;
-      tp_gram.push_back(q);
-      // G_B = Bbar Bbar^T: both operands Bbar, r x (reduction index n)
-      q.A = B_k; q.B = B_k; q.C = w.GB[i]; q.ldc = r; q.M = r; q.N = r; q.K = n;
-      tp_gram.push_back(q);
-      // A' = Abar Z_A (columns at or beyond r' zero), B' = Z_B Bbar (rows at or beyond r' zero)
-      q.c_f32 = !out_bf16;
-      q.A = A_k; q.B = pieces3(w.ZAsp[i], ez, rr8, true); q.C = d[i].A_out; q.ldc = r; q.M = m; q.N = r; q.K = r;
-      q.live_cols = d[i].r_out;
-      tp_out.push_back(q);
-      q.A = pieces3(w.ZBsp[i], ez, rr8, false); q.B = B_t; q.C = d[i].B_out; q.ldc = n; q.M = r; q.N = n; q.K = r;
-      q.live_cols = nullptr; q.live_rows = d[i].r_out;
-      tp_out.push_back(q);
-      if (d[i].W_out) {     // W = Abar Bbar
-        q.c_f32 = true; q.live_rows = nullptr;
-        q.A = A_k; q.B = B_t; q.C = d[i].W_out; q.ldc = n; q.M = m; q.N = n; q.K = r;
-        tp_w.push_back(q);
-      }
+    // G_A = Abar^T Abar, G_B = Bbar Bbar^T, upper tiles only, in slices of the long index
+    const int pa = gram_parts(m, slice), pb = gram_parts(n, slice);
+    for (int q = 0; q < pa; ++q) {
+      const int per = gram_per(m, slice), k0 = q * per, k1 = std::min(m, k0 + per);
+      const float* src = Ab + (size_t)k0 * r;
+      g[kGram].push_back(product(src, r, 1, src, r, 1, w.GA[i] + (size_t)q * r * r, r, r, r, k1 - k0));
+      g[kGram].back().upper_only = 1;
     }
+    for (int q = 0; q < pb; ++q) {
+      const int per = gram_per(n, slice), k0 = q * per, k1 = std::min(n, k0 + per);
+      g[kGram].push_back(product(Bb + k0, n, 0, Bb + k0, n, 0, w.GB[i] + (size_t)q * r * r, r, r, r, k1 - k0));
+      g[kGram].back().upper_only = 1;
+    }
+    // M = R_A R_B^T
+    g[kM].push_back(product(w.RA[i], r, 0, w.RB[i], r, 0, w.M[i], r, r, r, r));
+    // Y1 = M Vs^T;  Z_B = diag(sqrt sig) Vs R_B^-T
+    g[kZ1].push_back(product(w.M[i], r, 0, w.Vs[i], r, 0, w.Y1[i], r, r, r, r));
+    g[kZ1].push_back(product(w.Vs[i], r, 0, w.IB[i], r, 0, w.ZB[i], r, r, r, r));
+    g[kZ1].back().row_vec = d[i].sigma; g[kZ1].back().row_mode = 1;
+    // Z_A = R_A^-1 Y1 diag(sig^-1/2)
+    g[kZ2].push_back(product(w.IA[i], r, 0, w.Y1[i], r, 1, w.ZA[i], r, r, r, r));
+    g[kZ2].back().col_vec = d[i].sigma; g[kZ2].back().col_mode = 2;
+    // A' = Abar Z_A (columns at or beyond r' zero), B' = Z_B Bbar (rows at or beyond r' zero)
+    g[kOut].push_back(product(Ab, r, 0, w.ZA[i], r, 1, d[i].A_out, r, m, r, r));
+    g[kOut].back().c_bf16 = out_bf16; g[kOut].back().live_cols = d[i].r_out;
+    g[kOut].push_back(product(w.ZB[i], r, 0, Bb, n, 1, d[i].B_out, n, r, n, r));
+    g[kOut].back().c_bf16 = out_bf16; g[kOut].back().live_rows = d[i].r_out;
+    if (d[i].W_out) g[kW].push_back(product(Ab, r, 0, Bb, n, 1, d[i].W_out, n, m, n, r));      // W = Abar Bbar
     cj[i] = CholJob{w.GA[i], pa, w.RA[i], w.IA[i], w.jstatus + 3 * i, r};
     cj[L + i] = CholJob{w.GB[i], pb, w.RB[i], w.IB[i], w.jstatus + 3 * i + 1, r};
-    // Gram matrices in slices of the long index (equal work per CTA, partial sums added by the
-    // Cholesky kernel in ascending slice order), upper tiles only
-    for (int q = 0; q < pa && !use_tc; ++q) {
-      const int k0 = gram_k0(m, pa, q), k1 = gram_k0(m, pa, q + 1);
-      GemmDesc x = mk(Ab + (size_t)k0 * r, 1, r, Ab + (size_t)k0 * r, r, 1, w.GA[i] + (size_t)q * r * r, r, r, r, k1 - k0);
-      x.upper_only = 1;
-      gg.push_back(x);
-    }
-    for (int q = 0; q < pb && !use_tc; ++q) {
-      const int k0 = gram_k0(n, pb, q), k1 = gram_k0(n, pb, q + 1);
-      GemmDesc x = mk(Bb + k0, n, 1, Bb + k0, 1, n, w.GB[i] + (size_t)q * r * r, r, r, r, k1 - k0);
-      x.upper_only = 1;
-      gg.push_back(x);
-    }
     int* flag = w.tc_status + 64 + i;
     jb[i] = JacobiJob{w.M[i], w.Vs[i], d[i].sigma, w.jstatus + 3 * i + 2, flag, r, r};
     EigJob& q = ej[i];
@@ -831,7 +764,9 @@ int sync_factored(const ab_sync_desc* d, int L, int K, float sigma_cutoff, int d
     eig_bind(q, w.eig[i]);
     sigp[i] = d[i].sigma; routp[i] = d[i].r_out; rs[i] = r;
   }
-  // All tables sit back to back in the workspace (descs ... rs): one host image, one copy.
+  // All tables sit back to back in the workspace (gemms ... rs): one host image.
+  SplitBatch batch[kLaunches];
+  const SplitGemm* table[kLaunches];
   std::vector<AvgJob> aj((size_t)2 * L);
   int64_t avg_blocks = 0;            // flat grid of the batched mean: one 16-byte group per thread
   for (int i = 0; i < L; ++i) {
@@ -843,14 +778,19 @@ int sync_factored(const ab_sync_desc* d, int L, int K, float sigma_cutoff, int d
     }
   }
   {
-    char* base = reinterpret_cast<char*>(w.descs);
-    const size_t span = (size_t)(reinterpret_cast<char*>(w.sjobs + 4 * L) - base);
+    char* base = reinterpret_cast<char*>(w.gemms);
+    const size_t span = (size_t)(reinterpret_cast<char*>(w.rs + L) - base);
     std::vector<char> img(span, 0);
     auto put = [&](const void* dev_ptr, const void* src, size_t bytes) {
       std::memcpy(img.data() + (reinterpret_cast<const char*>(dev_ptr) - base), src, bytes);
     };
-    put(w.descs, g.data(), g.size() * sizeof(GemmDesc));
-    put(w.gram_descs, gg.data(), gg.size() * sizeof(GemmDesc));
+    SplitGemm* at = w.gemms;
+    for (int k = 0; k < kLaunches; ++k) {
+      batch[k] = gemm_split_plan(g[k].data(), (int)g[k].size());
+      table[k] = at;
+      put(at, g[k].data(), g[k].size() * sizeof(SplitGemm));
+      at += g[k].size();
+    }
     put(w.cjobs, cj.data(), cj.size() * sizeof(CholJob));
     put(w.ajobs, aj.data(), aj.size() * sizeof(AvgJob));
     put(w.jobs, jb.data(), jb.size() * sizeof(JacobiJob));
@@ -858,15 +798,12 @@ int sync_factored(const ab_sync_desc* d, int L, int K, float sigma_cutoff, int d
     put(w.sig_ptrs, sigp.data(), L * sizeof(float*));
     put(w.rout_ptrs, routp.data(), L * sizeof(int*));
     put(w.rs, rs.data(), L * sizeof(int));
-    put(w.sjobs, sj.data(), sj.size() * sizeof(SplitJob));
-    AB_CUDA_OK(cudaMemcpyAsync(base, img.data(), span, cudaMemcpyHostToDevice, st));
+    AB_TRY(upload_async(base, img.data(), span, st));
   }
 
   // ---- a7: means of the K copies (fp32), all matrices in one launch
   AB_TRY(group_average_batched(w.ajobs, 2 * L, K, dt, avg_blocks, st));
   const float tol = rows_jacobi_tol(rmax);
-  bool any_w = false;
-  for (int i = 0; i < L; ++i) any_w = any_w || d[i].W_out != nullptr;
   // a8 (optional): forked off where the Jacobi kernel starts (the kernels before it fill every SM
   // themselves), joined at the end
   cudaStream_t side = any_w ? side_stream() : nullptr;
@@ -888,41 +825,30 @@ int sync_factored(const ab_sync_desc* d, int L, int K, float sigma_cutoff, int d
   } evs;
   if (side && !evs.create()) side = nullptr;
   cudaEvent_t fork = evs.fork, join = evs.join;
-  auto product_w = [&](cudaStream_t s2) -> int {
-    if (use_tc) return gemm_tc_batched(tp_w.data(), (int)tp_w.size(), w.tc_table[2], w.tc_status + 2, s2);
-    return gemm_simt_batched(w.descs + 8 * L, L, mmax, nmax, s2);
-  };
-  AB_CUDA_OK(cudaMemsetAsync(w.tc_status, 0, (64 + (size_t)L) * sizeof(int), st));          // launch status and flags
-  if (use_tc) AB_TRY(split3_batched(w.sjobs, 2 * L, split_blocks[0], st));                  // pieces of Abar, Bbar
-  if (any_w && !side) AB_TRY(product_w(st));
-  if (use_tc) AB_TRY(gemm_tc_batched(tp_gram.data(), (int)tp_gram.size(), w.tc_table[0], w.tc_status, st));
-  else AB_TRY(gemm_simt_batched(w.gram_descs, (int)gg.size(), rmax, rmax, st));             // Gram slices
+  auto run = [&](int k, int* status, cudaStream_t s2) -> int { return gemm_split_batched(table[k], batch[k], status, s2); };
+  AB_CUDA_OK(cudaMemsetAsync(w.tc_status, 0, (64 + (size_t)L) * sizeof(int), st));          // wait reports and flags
+  if (any_w && !side) AB_TRY(run(kW, w.tc_status + 2, st));
+  AB_TRY(run(kGram, w.tc_status, st));
   const size_t csm = chol_smem_bytes(rmax);
   AB_CUDA_OK(cudaFuncSetAttribute(chol_inv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csm));
   chol_inv_kernel<<<2 * L, kCThreads, csm, st>>>(w.cjobs);                                  // R_A, R_B and inverses
   AB_LAUNCH_OK();
-  AB_TRY(gemm_simt_batched(w.descs + 2 * L, L, rmax, rmax, st));                            // M
+  AB_TRY(run(kM, w.tc_status, st));
   int side_rc = AB_OK;
   if (side && cudaEventRecord(fork, st) != cudaSuccess) side_rc = AB_ERR_CUDA;
   AB_TRY(eig_direct(ej.data(), w.ejobs, L, rmax, w.tc_status + 3, st));                                                 // SVD of M: right vectors, sigma
   AB_TRY(launch_jacobi(w.jobs, L, rmax, tol, st));                                          // of flagged matrices, from M
   if (side) {
     if (side_rc == AB_OK && cudaStreamWaitEvent(side, fork, 0) != cudaSuccess) side_rc = AB_ERR_CUDA;
-    if (side_rc == AB_OK) side_rc = product_w(side);
+    if (side_rc == AB_OK) side_rc = run(kW, w.tc_status + 2, side);
     if (side_rc == AB_OK && cudaEventRecord(join, side) != cudaSuccess) side_rc = AB_ERR_CUDA;
   }
-  fast_rank_rule_kernel<<<(L + 127) / 128, 128, 0, st>>>(w.sig_ptrs, w.rs, sigma_cutoff, w.rout_ptrs, w.jstatus,
+  fast_rank_rule_kernel<<<(L + 3) / 4, 128, 0, st>>>(w.sig_ptrs, w.rs, sigma_cutoff, w.rout_ptrs, w.jstatus,
                                                          dev_status, L);
   AB_LAUNCH_OK();
-  AB_TRY(gemm_simt_batched(w.descs + 3 * L, 2 * L, rmax, rmax, st));                        // Y1, Z_B
-  AB_TRY(gemm_simt_batched(w.descs + 5 * L, L, rmax, rmax, st));                            // Z_A
-  if (use_tc) {
-    AB_TRY(split3_batched(w.sjobs + 2 * L, 2 * L, split_blocks[1], st));                    // pieces of Z_A, Z_B
-    AB_TRY(gemm_tc_batched(tp_out.data(), (int)tp_out.size(), w.tc_table[1], w.tc_status + 1, st));   // A', B'
-  } else {
-    AB_TRY(gemm_simt_batched(w.descs + 6 * L, L, mmax, rmax, st));                          // A'
-    AB_TRY(gemm_simt_batched(w.descs + 7 * L, L, rmax, nmax, st));                          // B'
-  }
+  AB_TRY(run(kZ1, w.tc_status, st));
+  AB_TRY(run(kZ2, w.tc_status, st));
+  AB_TRY(run(kOut, w.tc_status + 1, st));
   if (side) {
     if (side_rc == AB_OK && cudaStreamWaitEvent(st, join, 0) != cudaSuccess) side_rc = AB_ERR_CUDA;
     if (side_rc != AB_OK) { (void)cudaGetLastError(); return side_rc; }
