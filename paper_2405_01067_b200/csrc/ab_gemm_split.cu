@@ -12,8 +12,7 @@
 // through tensor maps, and the r x r products ran on the fp32 pipes.  Here the converter warps read the operand as it
 // lies, and write the pieces straight into the swizzled tiles that the MMAs read: no pieces in memory, no tensor
 // maps to encode and upload, one launch where there were three.  Per slab of 64 of the reduction the conversion runs
-// beside the 24 MMAs (1570 cycles at 128 columns) of the slab before it, and one operand's next loads are in flight while the
-// other operand is converted.
+// beside the 24 MMAs (1570 cycles at 128 columns) of the slab before it.
 //
 // Persistent CTAs: CTA b takes tiles b, b + grid, ... of all problems of the launch.  Warps 0..7 convert, warps
 // 8..11 empty the accumulators (two pairs, used in turn), warp 12 issues the MMAs, warp 13 finds the tiles' problems
@@ -252,16 +251,13 @@ __device__ __forceinline__ void gemm_split_body(const SplitGemm* probs, int npro
       if (!split_warp_wait(bars, &bars->empty[slot], ph, status)) break;
       uint8_t* dst = smem + (size_t)slot * C::kStage;
       store_slab<kM, kBf16>(a, dst + ca.soff, (ca.mn ? SA::kStepMn : SA::kStepK) * 128);
-      uint8_t* dst_b = dst + C::kPieces * C::kABytes + cb.soff;
-      const uint32_t step_b = (cb.mn ? SB::kStepMn : SB::kStepK) * 128;
-      if (k0 >= K) more = open();                        // both operands of the old tile are in registers
-      if (more) ca.load(a, min(64, K - k0));
-      store_slab<BN, kBf16>(b, dst_b, step_b);
-      if (more) { cb.load(b, min(64, K - k0)); k0 += 64; }
-      fence_proxy_async_smem();
+      store_slab<BN, kBf16>(b, dst + C::kPieces * C::kABytes + cb.soff, (cb.mn ? SB::kStepMn : SB::kStepK) * 128);
+      fence_proxy_async_smem();                          // before the next loads: it waits for what is in flight
       __syncwarp();
       if (lane == 0) mbar_arrive(&bars->full[slot]);
       if (++slot == C::kStages) { slot = 0; ph ^= 1; }
+      if (k0 >= K) more = open();
+      if (more) { ca.load(a, min(64, K - k0)); cb.load(b, min(64, K - k0)); k0 += 64; }
     }
   } else if (warp >= kMmaWarp) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsMma));
@@ -408,28 +404,37 @@ __device__ __forceinline__ void gemm_split_body(const SplitGemm* probs, int npro
 #pragma unroll
         for (int j = 0; j < 4; ++j) cs[j] = col + j < live_c ? split_diag(col_vec, col + j, col_mode, thr) : 0.f;
         const bool plain = cs[0] == 1.f && cs[1] == 1.f && cs[2] == 1.f && cs[3] == 1.f;
-        const int nrows = min(32, M - (m0 + qw * 32)), ncol = N - col;
-        const int64_t off0 = (int64_t)(m0 + qw * 32 + (lane >> 3)) * ldc + col;
+        const int nrows = min(32, M - (m0 + qw * 32)), ncol = N - col, r0 = lane >> 3;
+        const int64_t off0 = (int64_t)(m0 + qw * 32 + r0) * ldc + col;
+        float4 q[8];
 #pragma unroll
-        for (int rr = 0; rr < 8; ++rr) {
-          const int rw = rr * 4 + (lane >> 3);
-          if (rw >= nrows || ncol <= 0) continue;
-          float4 q = *reinterpret_cast<const float4*>(mystg + rw * 128 + ((ch ^ (rw & 7)) << 4));
-          if (!plain) {
-            q.x = cs[0] == 0.f ? 0.f : q.x * cs[0]; q.y = cs[1] == 0.f ? 0.f : q.y * cs[1];
-            q.z = cs[2] == 0.f ? 0.f : q.z * cs[2]; q.w = cs[3] == 0.f ? 0.f : q.w * cs[3];
+        for (int rr = 0; rr < 8; ++rr) q[rr] = *reinterpret_cast<const float4*>(mystg + (rr * 4 + r0) * 128 + ((ch ^ ((rr * 4 + r0) & 7)) << 4));
+        if (!plain) {
+#pragma unroll
+          for (int rr = 0; rr < 8; ++rr) {
+            q[rr].x = cs[0] == 0.f ? 0.f : q[rr].x * cs[0]; q[rr].y = cs[1] == 0.f ? 0.f : q[rr].y * cs[1];
+            q[rr].z = cs[2] == 0.f ? 0.f : q[rr].z * cs[2]; q[rr].w = cs[3] == 0.f ? 0.f : q[rr].w * cs[3];
           }
-          const int64_t off = off0 + rr * 4 * ldc;
-          if (cvec && ncol >= 4) {
-            if (c_bf16) {
-              __nv_bfloat162 lo = __floats2bfloat162_rn(q.x, q.y), hi = __floats2bfloat162_rn(q.z, q.w);
-              *reinterpret_cast<uint2*>(static_cast<bf16*>(Cp) + off) =
-                  make_uint2(*reinterpret_cast<uint32_t*>(&lo), *reinterpret_cast<uint32_t*>(&hi));
-            } else {
-              *reinterpret_cast<float4*>(static_cast<float*>(Cp) + off) = q;
+        }
+        if (cvec && nrows == 32 && n0 + c0 + 32 <= N) {          // a whole piece: no checks between the stores
+          if (c_bf16) {
+            uint2* o = reinterpret_cast<uint2*>(static_cast<bf16*>(Cp) + off0);
+#pragma unroll
+            for (int rr = 0; rr < 8; ++rr) {
+              __nv_bfloat162 lo = __floats2bfloat162_rn(q[rr].x, q[rr].y), hi = __floats2bfloat162_rn(q[rr].z, q[rr].w);
+              o[rr * ldc] = make_uint2(*reinterpret_cast<uint32_t*>(&lo), *reinterpret_cast<uint32_t*>(&hi));
             }
           } else {
-            const float x[4] = {q.x, q.y, q.z, q.w};
+            float4* o = reinterpret_cast<float4*>(static_cast<float*>(Cp) + off0);
+#pragma unroll
+            for (int rr = 0; rr < 8; ++rr) o[rr * ldc] = q[rr];      // 4 rows of 4-value groups: ldc groups on
+          }
+        } else {
+#pragma unroll
+          for (int rr = 0; rr < 8; ++rr) {
+            if (rr * 4 + r0 >= nrows) continue;
+            const float x[4] = {q[rr].x, q[rr].y, q[rr].z, q[rr].w};
+            const int64_t off = off0 + rr * 4 * ldc;
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
               if (j >= ncol) continue;
