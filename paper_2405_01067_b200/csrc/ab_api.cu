@@ -77,6 +77,9 @@ int general_forward(const void* x, const void* A, const void* B, void* y, void* 
   int* status = ar.take_n<int>(64);
   float* T = ar.take_n<float>((size_t)N * r);
   if (!ws || !ar.fits()) return AB_ERR_WORKSPACE;
+  if (dt == AB_F32 && layer_small_ok(N, m, n, r))
+    return layer_small_forward(static_cast<const float*>(x), static_cast<const float*>(A), static_cast<const float*>(B),
+                               static_cast<float*>(y), static_cast<float*>(T_save), N, m, n, r, ldA, ldB, status, st);
   AB_CUDA_OK(cudaMemsetAsync(status, 0, sizeof(int), st));
   AB_TRY(gemm_simt(x, dt, n, 1, B, dt, 1, ldB, T, AB_F32, r, N, r, n, st));        // T = x B^T
   if (T_save) AB_TRY(cast_f32_to(T, T_save, dt, N * r, st));
@@ -92,6 +95,10 @@ int general_backward(const void* x, const void* dY, const void* A, const void* B
   float* T = ar.take_n<float>((size_t)N * r);
   float* dT = ar.take_n<float>((size_t)N * r);
   if (!ws || !ar.fits()) return AB_ERR_WORKSPACE;
+  if (dt == AB_F32 && layer_small_ok(N, m, n, r))
+    return layer_small_backward(static_cast<const float*>(x), static_cast<const float*>(dY), static_cast<const float*>(A),
+                                static_cast<const float*>(B), static_cast<const float*>(T_saved), static_cast<float*>(dX), dA, dB, N,
+                                m, n, r, ldA, ldB, T, dT, status, st);
   AB_CUDA_OK(cudaMemsetAsync(status, 0, sizeof(int), st));
   AB_TRY(gemm_simt(dY, dt, m, 1, A, dt, ldA, 1, dT, AB_F32, r, N, r, m, st));      // dT = dY A
   if (dX) AB_TRY(gemm_simt(dT, AB_F32, r, 1, B, dt, ldB, 1, dX, dt, n, N, n, r, st));   // dX = dT B

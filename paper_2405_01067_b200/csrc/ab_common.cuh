@@ -161,6 +161,14 @@ int chain_tc_backward(const void* x, const void* dY, const void* A, const void* 
                       int64_t N, int m, int n, int r, int ldA, int ldB,
                       void* ws, size_t ws_bytes, cudaStream_t st);
 
+// ---- small fp32 layers (ab_layer_small.cu) -------------------------------------------------------
+bool layer_small_ok(int64_t N, int m, int n, int r);
+int layer_small_forward(const float* x, const float* A, const float* B, float* y, float* T_save, int64_t N, int m, int n, int r,
+                        int ldA, int ldB, int* status, cudaStream_t st);
+int layer_small_backward(const float* x, const float* dY, const float* A, const float* B, const float* T_saved, float* dX, float* dA,
+                         float* dB, int64_t N, int m, int n, int r, int ldA, int ldB, float* wsT, float* wsdT, int* status,
+                         cudaStream_t st);
+
 // 3 x 3 convolution with the factorised weight on NHWC activations, im2col rows never formed (ab_chain_tc.cu)
 bool conv_tc_supported(int B, int H, int W, int C, int m, int r, int ldA, int ldB, int dt,
                        const void* x, const void* A, const void* Bf);
