@@ -77,9 +77,15 @@ int general_forward(const void* x, const void* A, const void* B, void* y, void* 
   int* status = ar.take_n<int>(64);
   float* T = ar.take_n<float>((size_t)N * r);
   if (!ws || !ar.fits()) return AB_ERR_WORKSPACE;
-  if (dt == AB_F32 && layer_small_ok(N, m, n, r))
-    return layer_small_forward(static_cast<const float*>(x), static_cast<const float*>(A), static_cast<const float*>(B),
-                               static_cast<float*>(y), static_cast<float*>(T_save), N, m, n, r, ldA, ldB, status, st);
+  if (dt == AB_F32) {
+    const float *x32 = static_cast<const float*>(x), *A32 = static_cast<const float*>(A), *B32 = static_cast<const float*>(B);
+    float* T32 = T_save ? static_cast<float*>(T_save) : T;
+    if (layer_small_ok(N, m, n, r))
+      return layer_small_chain(x32, N, n, B32, ldB, 1, A32, ldA, 1, static_cast<float*>(y), m, static_cast<float*>(T_save), r, status, st);
+    AB_CUDA_OK(cudaMemsetAsync(status, 0, sizeof(int), st));
+    AB_TRY(gemm_simt(x, dt, n, 1, B, dt, 1, ldB, T32, AB_F32, r, N, r, n, st));       // T = x B^T
+    return gemm_simt(T32, AB_F32, r, 1, A, dt, 1, ldA, y, dt, m, N, m, r, st);        // y = T A^T
+  }
   AB_CUDA_OK(cudaMemsetAsync(status, 0, sizeof(int), st));
   AB_TRY(gemm_simt(x, dt, n, 1, B, dt, 1, ldB, T, AB_F32, r, N, r, n, st));        // T = x B^T
   if (T_save) AB_TRY(cast_f32_to(T, T_save, dt, N * r, st));
@@ -95,10 +101,39 @@ int general_backward(const void* x, const void* dY, const void* A, const void* B
   float* T = ar.take_n<float>((size_t)N * r);
   float* dT = ar.take_n<float>((size_t)N * r);
   if (!ws || !ar.fits()) return AB_ERR_WORKSPACE;
-  if (dt == AB_F32 && layer_small_ok(N, m, n, r))
-    return layer_small_backward(static_cast<const float*>(x), static_cast<const float*>(dY), static_cast<const float*>(A),
-                                static_cast<const float*>(B), static_cast<const float*>(T_saved), static_cast<float*>(dX), dA, dB, N,
-                                m, n, r, ldA, ldB, T, dT, status, st);
+  if (dt == AB_F32) {
+    const float *x32 = static_cast<const float*>(x), *y32 = static_cast<const float*>(dY), *A32 = static_cast<const float*>(A),
+                *B32 = static_cast<const float*>(B);
+    const bool fused = layer_small_ok(N, m, n, r);
+    int* clear = status;              // the first kernel of the call clears the status word
+    if (!fused) { AB_CUDA_OK(cudaMemsetAsync(status, 0, sizeof(int), st)); clear = nullptr; }
+    if (dX || dB) {                   // dT = dY A, dX = dT B
+      if (fused) {
+        AB_TRY(layer_small_chain(y32, N, m, A32, 1, ldA, B32, 1, ldB, static_cast<float*>(dX), n, dB ? dT : nullptr, r, clear, st));
+        clear = nullptr;
+      } else {
+        AB_TRY(gemm_simt(dY, dt, m, 1, A, dt, ldA, 1, dT, AB_F32, r, N, r, m, st));
+        if (dX) AB_TRY(gemm_simt(dT, AB_F32, r, 1, B, dt, ldB, 1, dX, dt, n, N, n, r, st));
+      }
+    }
+    const float* Ts = static_cast<const float*>(T_saved);
+    if (dA && !Ts) {
+      if (fused) {
+        AB_TRY(layer_small_chain(x32, N, n, B32, ldB, 1, nullptr, 0, 0, nullptr, 0, T, r, clear, st));
+        clear = nullptr;
+      } else {
+        AB_TRY(gemm_simt(x, dt, n, 1, B, dt, 1, ldB, T, AB_F32, r, N, r, n, st));
+      }
+      Ts = T;
+    }
+    SmallProduct g[2];                // dA = dY^T T, dB = dT^T x: one launch
+    int ng = 0;
+    if (dA) g[ng++] = SmallProduct{y32, 1, m, Ts, 1, r, dA, r, m, r};
+    if (dB) g[ng++] = SmallProduct{dT, 1, r, x32, 1, n, dB, n, r, n};
+    if (ng > 0) { AB_TRY(gemm_small(g, ng, N, clear, st)); clear = nullptr; }
+    if (clear) AB_CUDA_OK(cudaMemsetAsync(status, 0, sizeof(int), st));
+    return AB_OK;
+  }
   AB_CUDA_OK(cudaMemsetAsync(status, 0, sizeof(int), st));
   AB_TRY(gemm_simt(dY, dt, m, 1, A, dt, ldA, 1, dT, AB_F32, r, N, r, m, st));      // dT = dY A
   if (dX) AB_TRY(gemm_simt(dT, AB_F32, r, 1, B, dt, ldB, 1, dX, dt, n, N, n, r, st));   // dX = dT B

@@ -161,13 +161,16 @@ int chain_tc_backward(const void* x, const void* dY, const void* A, const void* 
                       int64_t N, int m, int n, int r, int ldA, int ldB,
                       void* ws, size_t ws_bytes, cudaStream_t st);
 
-// ---- small fp32 layers (ab_layer_small.cu) -------------------------------------------------------
+// ---- small fp32 products and layers (ab_layer_small.cu) -----------------------------------------
+// C[p][q] = sum over k of U[p * u_p + k * u_k] V[q * v_q + k * v_k], row stride ldc; sums of 16 products in fp32, those
+// in fp64.  One or two products with the same reduction length in one launch; status: cleared if not null.
+struct SmallProduct { const float* U; int64_t u_p, u_k; const float* V; int64_t v_q, v_k; float* C; int64_t ldc; int P, Q; };
+int gemm_small(const SmallProduct* jobs, int njobs, int64_t K, int* status, cudaStream_t st);
+// S = In F1^T, Out = S F2^T (Out null: only S; S null: not stored) for a layer small enough to be latency-bound;
+// F1(j, k) at F1[j * f1_j + k * f1_k], F2(p, j) at F2[p * f2_p + j * f2_j]
 bool layer_small_ok(int64_t N, int m, int n, int r);
-int layer_small_forward(const float* x, const float* A, const float* B, float* y, float* T_save, int64_t N, int m, int n, int r,
-                        int ldA, int ldB, int* status, cudaStream_t st);
-int layer_small_backward(const float* x, const float* dY, const float* A, const float* B, const float* T_saved, float* dX, float* dA,
-                         float* dB, int64_t N, int m, int n, int r, int ldA, int ldB, float* wsT, float* wsdT, int* status,
-                         cudaStream_t st);
+int layer_small_chain(const float* In, int64_t N, int K1, const float* F1, int64_t f1_j, int64_t f1_k, const float* F2, int64_t f2_p,
+                      int64_t f2_j, float* Out, int P, float* S, int r, int* status, cudaStream_t st);
 
 // 3 x 3 convolution with the factorised weight on NHWC activations, im2col rows never formed (ab_chain_tc.cu)
 bool conv_tc_supported(int B, int H, int W, int C, int m, int r, int ldA, int ldB, int dt,

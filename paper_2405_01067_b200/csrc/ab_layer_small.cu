@@ -3,11 +3,14 @@
 //
 //   small_chain_kernel:  S = In F1^T,  Out = S F2^T  for a few rows per CTA, S in shared memory (forward: T and y;
 //                        backward: dT and dX with A and B read the other way round)
-//   small_grad_kernel:   dA = dY^T T and dB = dT^T x in one launch, 32 x 32 tiles, the rows cut over a cluster
+//   small_gemm_kernel:   dA = dY^T T and dB = dT^T x in one launch, 32 x 32 tiles, the rows cut over a cluster; also
+//                        every other fp32 product that is too small for the register-tiled kernel
 //
 // Sums: 16 products in fp32, those sums in fp64, in an order fixed by the shape, as in the general kernel.
 // What bounds both at the small sizes is latency: a launch, a trip to L2 for the first values, then the factors streamed once per
-// CTA (96 KB, about 1 us).  64 x 512 -> 256, rank 32, forward and backward: 70 us of kernels -> three kernels.
+// CTA (96 KB, about 1 us).  64 x 512 -> 256, rank 32, forward and backward: 82 -> 27 us, seven kernels -> three.
+// The tiled product against the general kernel it replaces for fp32 (64 x 64 tiles, one CTA walking the whole reduction):
+// 64 x 64, rank 16, 4096 rows, forward and backward 538 -> 52 us; 1000 x 1000, rank 250, 1000 rows 362 -> 270 us.
 #include <cooperative_groups.h>
 
 #include "ab_common.cuh"
@@ -165,13 +168,13 @@ small_chain_kernel(const SmallChain p) {
   }
 }
 
-// C[p][q] = sum over rows k of U[k][p] V[k][q] for two problems at once.
-struct SmallGradJob { const float* U; const float* V; float* C; int P, Q, tiles_q, tiles; };
-struct SmallGrad { SmallGradJob job[2]; int64_t N; int* status; };
+// C[p][q] = sum over k of U(p, k) V(q, k) for up to two problems with the same k at once; U(p, k) at U[p * u_p + k * u_k],
+// V likewise.  32 x 32 tiles; the reduction is cut over the CTAs of a cluster, in each over its eight warps.
+struct SmallGemm { SmallProduct job[2]; int64_t K; int tiles0, tiles_q[2]; int* status; };
 
-constexpr int kGt = 32, kGk = 128;                 // tile edge, rows per slab: 16 for each of the eight warps
+constexpr int kGt = 32, kGk = 128;                 // tile edge, reduction per slab: 16 for each of the eight warps
 __global__ void __launch_bounds__(kThreads)
-small_grad_kernel(const SmallGrad p) {
+small_gemm_kernel(const __grid_constant__ SmallGemm p) {
   __shared__ __align__(16) float us[kGk][kGt + 4], vs[kGk][kGt + 4];
   extern __shared__ __align__(16) double gred[];     // 8 warps x 1024
   cg::cluster_group cluster = cg::this_cluster();
@@ -181,31 +184,45 @@ small_grad_kernel(const SmallGrad p) {
   tc::dep_launch();
   if (p.status && blockIdx.x == 0 && tid == 0) *p.status = 0;
   int t = blockIdx.x / C;
-  const int jb = t >= p.job[0].tiles ? 1 : 0;
-  const SmallGradJob& job = p.job[jb];
-  if (jb) t -= p.job[0].tiles;
-  const int p0 = (t / job.tiles_q) * kGt, q0 = (t % job.tiles_q) * kGt;
-  // this CTA's rows: whole 16-row groups
-  const int64_t n16 = (p.N + 15) / 16;
+  const int jb = t >= p.tiles0 ? 1 : 0;
+  const SmallProduct& job = p.job[jb];
+  if (jb) t -= p.tiles0;
+  const int p0 = (t / p.tiles_q[jb]) * kGt, q0 = (t % p.tiles_q[jb]) * kGt;
+  // this CTA's part of the reduction: whole groups of 16
+  const int64_t n16 = (p.K + 15) / 16;
   const int64_t k_begin = n16 * rank / C * 16;
   int64_t k_end = n16 * (rank + 1) / C * 16;
-  if (k_end > p.N) k_end = p.N;
+  if (k_end > p.K) k_end = p.K;
   const int ty = lane >> 2, tx = lane & 3;
   double acc[4][8];
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
     for (int j = 0; j < 8; ++j) acc[i][j] = 0.0;
-  float fu[16], fv[16];                              // a column of the slab per lane, 16 rows per thread
-  auto fetch = [&](int64_t k0) {
+  // lane: a row of U and one of V; 16 of the reduction per warp and slab
+  const float* up = job.U + (int64_t)(p0 + lane) * job.u_p;
+  const float* vp = job.V + (int64_t)(q0 + lane) * job.v_q;
+  const bool uin = p0 + lane < job.P, vin = q0 + lane < job.Q;
+  const bool uvec = job.u_k == 1 && job.u_p % 4 == 0 && (reinterpret_cast<uintptr_t>(job.U) & 15u) == 0;
+  const bool vvec = job.v_k == 1 && job.v_q % 4 == 0 && (reinterpret_cast<uintptr_t>(job.V) & 15u) == 0;
+  float fu[16], fv[16];
+  auto load16 = [](float (&f)[16], const float* b, int64_t step, bool in, bool vec, int64_t k, int64_t kend) {
+    if (vec && in && k + 16 <= kend) {
 #pragma unroll
-    for (int e = 0; e < 16; ++e) {
-      const int64_t k = k0 + warp * 16 + e;
-      fu[e] = (k < k_end && p0 + lane < job.P) ? job.U[k * job.P + p0 + lane] : 0.f;
-      fv[e] = (k < k_end && q0 + lane < job.Q) ? job.V[k * job.Q + q0 + lane] : 0.f;
+      for (int e = 0; e < 4; ++e) {
+        const float4 q = *reinterpret_cast<const float4*>(b + k + 4 * e);
+        f[4 * e] = q.x; f[4 * e + 1] = q.y; f[4 * e + 2] = q.z; f[4 * e + 3] = q.w;
+      }
+    } else {
+#pragma unroll
+      for (int e = 0; e < 16; ++e) f[e] = (in && k + e < kend) ? b[(k + e) * step] : 0.f;
     }
   };
-  // a warp multiplies the rows it has fetched itself: no barrier inside the loop
+  auto fetch = [&](int64_t k0) {
+    load16(fu, up, job.u_k, uin, uvec, k0 + warp * 16, k_end);
+    load16(fv, vp, job.v_k, vin, vvec, k0 + warp * 16, k_end);
+  };
+  // a warp multiplies what it has fetched itself: no barrier inside the loop
   if (k_begin < k_end) fetch(k_begin);
   for (int64_t k0 = k_begin; k0 < k_end; k0 += kGk) {
 #pragma unroll
@@ -253,7 +270,7 @@ small_grad_kernel(const SmallGrad p) {
     double s = 0.0;
     for (int c = 0; c < C; ++c) s += C > 1 ? cluster.map_shared_rank(gred, c)[e] : gred[e];
     const int pp = p0 + (e >> 5), qq = q0 + (e & 31);
-    if (pp < job.P && qq < job.Q) job.C[(int64_t)pp * job.Q + qq] = (float)s;
+    if (pp < job.P && qq < job.Q) job.C[(int64_t)pp * job.ldc + qq] = (float)s;
   }
   if (C > 1) cluster.sync();                          // nobody leaves while a peer reads its sums
 }
@@ -303,65 +320,43 @@ int run_chain(const SmallChain& p, cudaStream_t st) {
 
 }  // namespace
 
-// Where a product gives the register-tiled kernel enough tiles to fill the device twice, that one is the better;
-// the row blocks also have to fit shared memory.
+int gemm_small(const SmallProduct* jobs, int njobs, int64_t K, int* status, cudaStream_t st) {
+  SmallGemm g;
+  int64_t tiles = 0;
+  for (int i = 0; i < 2; ++i) {
+    g.job[i] = jobs[i < njobs ? i : 0];
+    g.tiles_q[i] = (g.job[i].Q + kGt - 1) / kGt;
+    const int64_t t = (int64_t)((g.job[i].P + kGt - 1) / kGt) * g.tiles_q[i];
+    if (i < njobs) tiles += t;
+    if (i == 0) g.tiles0 = (int)t;
+  }
+  if (tiles <= 0 || tiles > ((int64_t)1 << 27)) return tiles <= 0 ? AB_OK : AB_ERR_UNSUPPORTED;
+  g.K = K;
+  g.status = status;
+  // the reduction cut over a cluster while each CTA keeps a slab and the device has room for two CTAs an SM
+  const int sms = sm_count() > 0 ? sm_count() : 1;
+  int C = 1;
+  while (C < 8 && K / (2 * C) >= kGk && tiles * 2 * C <= 2LL * sms) C *= 2;
+  return launch_small(small_gemm_kernel, (unsigned)(tiles * C), C, sizeof(double) * 8 * 1024, st, g);
+}
+
+// The fused chain streams both factors once per CTA of a few rows, from L2 by single values: it wins where that is little (measured,
+// square layers of width w, forward and backward, us fused / one product at a time: r 8, w 1024, 1000 rows 48 / 128; r 32,
+// w 256, 64 rows 28 / 39, 4096 rows 88 / 121) and loses beyond (r 32, w 64, 4096 rows 62 / 52; r 64, w 256, 1000 rows 60 / 52;
+// r 32, w 1024, 64 rows 54 / 39; r 256, w 256, 64 rows 210 / 43).
 bool layer_small_ok(int64_t N, int m, int n, int r) {
-  const int64_t wide = m > n ? m : n;
-  if (((N + 63) / 64) * ((wide + 63) / 64) >= 296) return false;
+  const int64_t work = (int64_t)r * (m > n ? m : n);
+  if (!(work <= 8192 && (N <= 1024 || r < 32 || work > 4096)) && !(work <= 16384 && N <= 300)) return false;
   const int R = rows_per_cta(N);
   return chain_smem(R, n, r) <= 200 * 1024 && chain_smem(R, m, r) <= 200 * 1024;
 }
 
-int layer_small_forward(const float* x, const float* A, const float* B, float* y, float* T_save, int64_t N, int m, int n, int r,
-                        int ldA, int ldB, int* status, cudaStream_t st) {
+int layer_small_chain(const float* In, int64_t N, int K1, const float* F1, int64_t f1_j, int64_t f1_k, const float* F2, int64_t f2_p,
+                      int64_t f2_j, float* Out, int P, float* S, int r, int* status, cudaStream_t st) {
   SmallChain p;
-  p.In = x; p.K1 = n; p.F1 = B; p.f1_j = ldB; p.f1_k = 1; p.F2 = A; p.f2_p = ldA; p.f2_j = 1; p.Out = y; p.P = m; p.S = T_save;
-  p.N = N; p.r = r; p.status = status;
+  p.In = In; p.K1 = K1; p.F1 = F1; p.f1_j = f1_j; p.f1_k = f1_k; p.F2 = F2; p.f2_p = f2_p; p.f2_j = f2_j; p.Out = Out; p.P = P;
+  p.S = S; p.N = N; p.r = r; p.status = status;
   return run_chain(p, st);
-}
-
-int layer_small_backward(const float* x, const float* dY, const float* A, const float* B, const float* T_saved, float* dX, float* dA,
-                         float* dB, int64_t N, int m, int n, int r, int ldA, int ldB, float* wsT, float* wsdT, int* status,
-                         cudaStream_t st) {
-  int* clear = status;                // the first kernel of the call clears the status word
-  if (dX || dB) {
-    SmallChain p;
-    p.In = dY; p.K1 = m; p.F1 = A; p.f1_j = 1; p.f1_k = ldA; p.F2 = B; p.f2_p = 1; p.f2_j = ldB; p.Out = dX; p.P = n;
-    p.S = dB ? wsdT : nullptr; p.N = N; p.r = r; p.status = clear;
-    AB_TRY(run_chain(p, st));
-    clear = nullptr;
-  }
-  const float* T = T_saved;
-  if (dA && !T) {
-    SmallChain p;
-    p.In = x; p.K1 = n; p.F1 = B; p.f1_j = ldB; p.f1_k = 1; p.F2 = nullptr; p.f2_p = p.f2_j = 0; p.Out = nullptr; p.P = 0;
-    p.S = wsT; p.N = N; p.r = r; p.status = clear;
-    AB_TRY(run_chain(p, st));
-    clear = nullptr;
-    T = wsT;
-  }
-  if (dA || dB) {
-    SmallGrad g;
-    auto job = [](const float* U, const float* V, float* C, int P, int Q) {
-      SmallGradJob j;
-      j.U = U; j.V = V; j.C = C; j.P = P; j.Q = Q; j.tiles_q = (Q + kGt - 1) / kGt; j.tiles = ((P + kGt - 1) / kGt) * j.tiles_q;
-      return j;
-    };
-    const SmallGradJob ja = job(dY, T, dA, m, r), jb = job(wsdT, x, dB, r, n);
-    g.job[0] = dA ? ja : jb;
-    g.job[1] = jb;
-    if (!(dA && dB)) g.job[1].tiles = 0;
-    g.N = N;
-    g.status = clear;
-    const int tiles = g.job[0].tiles + g.job[1].tiles, sms = sm_count() > 0 ? sm_count() : 1;
-    // the rows cut over a cluster while that leaves each CTA 256 of them and the device room for the clusters
-    int C = 1;
-    while (C < 8 && N / (2 * C) >= 256 && (long long)tiles * 2 * C <= 2LL * sms) C *= 2;
-    AB_TRY(launch_small(small_grad_kernel, (unsigned)(tiles * C), C, sizeof(double) * 8 * 1024, st, g));
-    clear = nullptr;
-  }
-  if (clear) AB_CUDA_OK(cudaMemsetAsync(status, 0, sizeof(int), st));    // nothing was asked for
-  return AB_OK;
 }
 
 }  // namespace ab
