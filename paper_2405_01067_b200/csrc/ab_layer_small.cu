@@ -169,14 +169,24 @@ small_chain_kernel(const SmallChain p) {
 }
 
 // C[p][q] = sum over k of U(p, k) V(q, k) for up to two problems with the same k at once; U(p, k) at U[p * u_p + k * u_k],
-// V likewise.  32 x 32 tiles; the reduction is cut over the CTAs of a cluster, in each over its eight warps.
+// V likewise.  32 x 32 tiles; the reduction is cut over the CTAs of a cluster, in each over its eight warps.  A warp
+// fetches the 16 x 32 values of each operand that it multiplies itself, so no barrier is inside the loop.
+//   kMany false: the next slab waits in registers (one CTA per SM; what counts is the latency of a lone tile)
+//   kMany true : asynchronous copies into a second buffer, lanes along the index that is contiguous in memory; two CTAs
+//                per SM hide each other's waits (768 x 768 x 3072: 290 -> 154 us, but a 256 x 64 layer of 1000 rows 51 -> 61 us)
 struct SmallGemm { SmallProduct job[2]; int64_t K; int tiles0, tiles_q[2]; int* status; };
 
 constexpr int kGt = 32, kGk = 128;                 // tile edge, reduction per slab: 16 for each of the eight warps
-__global__ void __launch_bounds__(kThreads)
+static_assert(sizeof(float) * 4 * kGk * (kGt + 4) >= sizeof(double) * 8 * 1024, "");
+template <bool kMany>
+__global__ void __launch_bounds__(kThreads, kMany ? 2 : 1)
 small_gemm_kernel(const __grid_constant__ SmallGemm p) {
-  __shared__ __align__(16) float us[kGk][kGt + 4], vs[kGk][kGt + 4];
-  extern __shared__ __align__(16) double gred[];     // 8 warps x 1024
+  // two slabs of both operands; afterwards the eight warps' sums (8 x 1024 doubles) lie over them
+  extern __shared__ __align__(16) unsigned char gsm[];
+  typedef float Slab[kGk][kGt + 4];
+  Slab* us = reinterpret_cast<Slab*>(gsm);
+  Slab* vs = us + 2;
+  double* gred = reinterpret_cast<double*>(gsm);
   cg::cluster_group cluster = cg::this_cluster();
   const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -199,13 +209,40 @@ small_gemm_kernel(const __grid_constant__ SmallGemm p) {
   for (int i = 0; i < 4; ++i)
 #pragma unroll
     for (int j = 0; j < 8; ++j) acc[i][j] = 0.0;
-  // lane: a row of U and one of V; 16 of the reduction per warp and slab
+  struct Source { const float* p; int64_t step; int row, k, drow, dk; };     // value e of a lane: row + e drow, k + e dk
+  auto source = [&](const float* b, int64_t s_row, int64_t s_k, int row0) {
+    Source o;
+    if (s_k == 1) { o.row = lane >> 4; o.k = lane & 15; o.drow = 2; o.dk = 0; o.step = 2 * s_row; }
+    else { o.row = lane; o.k = 0; o.drow = 0; o.dk = 1; o.step = s_k; }
+    o.p = b + (int64_t)(row0 + o.row) * s_row + (int64_t)(warp * 16 + o.k) * s_k;
+    return o;
+  };
+  const Source su = source(job.U, job.u_p, job.u_k, p0), sv = source(job.V, job.v_q, job.v_k, q0);
+  auto fetch_one = [&](const Source& o, int64_t s_k, int rows, Slab& dst, int64_t k0) {
+    const float* g = o.p + k0 * s_k;
+    const int left = (int)(k_end - k0 < (int64_t)kGk ? k_end - k0 : (int64_t)kGk) - warp * 16;      // of the reduction
+#pragma unroll
+    for (int e = 0; e < 16; ++e) {
+      const int row = o.row + e * o.drow, k = o.k + e * o.dk;
+      const int bytes = (row < rows && k < left) ? 4 : 0;                  // nothing read: zero
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(tc::smem_u32(&dst[warp * 16 + k][row])),
+                   "l"(bytes ? g + e * o.step : job.U), "r"(bytes)
+                   : "memory");
+    }
+  };
+  auto fetch = [&](int64_t k0, int buf) {
+    if (k0 < k_end) {
+      fetch_one(su, job.u_k, job.P - p0, us[buf], k0);
+      fetch_one(sv, job.v_k, job.Q - q0, vs[buf], k0);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  float fu[16], fv[16];
   const float* up = job.U + (int64_t)(p0 + lane) * job.u_p;
   const float* vp = job.V + (int64_t)(q0 + lane) * job.v_q;
   const bool uin = p0 + lane < job.P, vin = q0 + lane < job.Q;
   const bool uvec = job.u_k == 1 && job.u_p % 4 == 0 && (reinterpret_cast<uintptr_t>(job.U) & 15u) == 0;
   const bool vvec = job.v_k == 1 && job.v_q % 4 == 0 && (reinterpret_cast<uintptr_t>(job.V) & 15u) == 0;
-  float fu[16], fv[16];
   auto load16 = [](float (&f)[16], const float* b, int64_t step, bool in, bool vec, int64_t k, int64_t kend) {
     if (vec && in && k + 16 <= kend) {
 #pragma unroll
@@ -218,17 +255,24 @@ small_gemm_kernel(const __grid_constant__ SmallGemm p) {
       for (int e = 0; e < 16; ++e) f[e] = (in && k + e < kend) ? b[(k + e) * step] : 0.f;
     }
   };
-  auto fetch = [&](int64_t k0) {
+  auto fetch_regs = [&](int64_t k0) {
     load16(fu, up, job.u_k, uin, uvec, k0 + warp * 16, k_end);
     load16(fv, vp, job.v_k, vin, vvec, k0 + warp * 16, k_end);
   };
-  // a warp multiplies what it has fetched itself: no barrier inside the loop
-  if (k_begin < k_end) fetch(k_begin);
+  if constexpr (kMany) fetch(k_begin, 0);
+  else if (k_begin < k_end) fetch_regs(k_begin);
+  int buf = 0;
   for (int64_t k0 = k_begin; k0 < k_end; k0 += kGk) {
+    if constexpr (kMany) {
+      fetch(k0 + kGk, buf ^ 1);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+      __syncwarp();
+    } else {
 #pragma unroll
-    for (int e = 0; e < 16; ++e) { us[warp * 16 + e][lane] = fu[e]; vs[warp * 16 + e][lane] = fv[e]; }
-    __syncwarp();
-    if (k0 + kGk < k_end) fetch(k0 + kGk);
+      for (int e = 0; e < 16; ++e) { us[0][warp * 16 + e][lane] = fu[e]; vs[0][warp * 16 + e][lane] = fv[e]; }
+      __syncwarp();
+      if (k0 + kGk < k_end) fetch_regs(k0 + kGk);
+    }
     float part[4][8];
 #pragma unroll
     for (int i = 0; i < 4; ++i)
@@ -237,8 +281,8 @@ small_gemm_kernel(const __grid_constant__ SmallGemm p) {
     if (k0 + warp * 16 < k_end) {
 #pragma unroll 4
       for (int e = 0; e < 16; ++e) {
-        const float4 a = *reinterpret_cast<const float4*>(&us[warp * 16 + e][ty * 4]);
-        const float4 b0 = *reinterpret_cast<const float4*>(&vs[warp * 16 + e][tx * 8]), b1 = *reinterpret_cast<const float4*>(&vs[warp * 16 + e][tx * 8 + 4]);
+        const float4 a = *reinterpret_cast<const float4*>(&us[buf][warp * 16 + e][ty * 4]);
+        const float4 b0 = *reinterpret_cast<const float4*>(&vs[buf][warp * 16 + e][tx * 8]), b1 = *reinterpret_cast<const float4*>(&vs[buf][warp * 16 + e][tx * 8 + 4]);
         const float av[4] = {a.x, a.y, a.z, a.w}, bv[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
 #pragma unroll
         for (int i = 0; i < 4; ++i)
@@ -251,7 +295,10 @@ small_gemm_kernel(const __grid_constant__ SmallGemm p) {
 #pragma unroll
       for (int j = 0; j < 8; ++j) acc[i][j] += (double)part[i][j];
     __syncwarp();
+    if constexpr (kMany) buf ^= 1;
   }
+  if constexpr (kMany) asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncthreads();
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
@@ -337,7 +384,9 @@ int gemm_small(const SmallProduct* jobs, int njobs, int64_t K, int* status, cuda
   const int sms = sm_count() > 0 ? sm_count() : 1;
   int C = 1;
   while (C < 8 && K / (2 * C) >= kGk && tiles * 2 * C <= 2LL * sms) C *= 2;
-  return launch_small(small_gemm_kernel, (unsigned)(tiles * C), C, sizeof(double) * 8 * 1024, st, g);
+  const size_t sm = sizeof(float) * 4 * kGk * (kGt + 4);
+  if (tiles * C > sms) return launch_small(small_gemm_kernel<true>, (unsigned)(tiles * C), C, sm, st, g);
+  return launch_small(small_gemm_kernel<false>, (unsigned)(tiles * C), C, sm, st, g);
 }
 
 // The fused chain streams both factors once per CTA of a few rows, from L2 by single values: it wins where that is little (measured,
