@@ -33,9 +33,7 @@ constexpr int kSmemLimit = 227 * 1024;
 constexpr int kTmemCols = 512;
 constexpr int kEpiThreads = 128;
 
-constexpr int kEpiWarps = 4;                         // 4 or 8: one or two warps per quarter of the TMEM lanes
-constexpr int kWarpsPerQuarter = kEpiWarps / 4;
-constexpr int kPiecesPerWarp = 4 / kWarpsPerQuarter;  // 64-column pieces of a 256-column chunk per warp
+constexpr int kEpiWarps = 4;                         // one per quarter of the TMEM lanes
 constexpr int kStgTiles = 2;                         // staging tiles per epilogue warp
 constexpr int kChainThreads = 32 * (2 + kEpiWarps);
 constexpr int kGroupRows = 32;                   // rows are dealt to CTAs, loaded and stored in groups of 32
@@ -120,14 +118,14 @@ __device__ __forceinline__ bool epi_wait(Bars* b, uint64_t* bar, uint32_t parity
   return *reinterpret_cast<volatile int*>(&b->epi_abort) == 0;
 }
 
-// one warp waits; the verdict is uniform over the warp
+// one warp waits; the verdict is a vote, on which the compiler branches uniformly
 __device__ __forceinline__ bool warp_wait(Bars* b, uint64_t* bar, uint32_t parity, unsigned long long limit, int* status) {
   int ok = 1;
   if ((threadIdx.x & 31) == 0) {          // one lane polls; the others rest at the shuffle
     ok = mbar_wait(bar, parity, limit) ? 1 : 0;
     if (!ok) raise_timeout(b, status);
   }
-  return __shfl_sync(0xffffffffu, ok, 0) != 0;
+  return __all_sync(0xffffffffu, ok);
 }
 
 __device__ __forceinline__ void store_bf16x16_swizzled(uint8_t* row_base, int row, int c0, const uint32_t* v) {
@@ -200,7 +198,7 @@ __device__ __forceinline__ void store_partial_group(const uint8_t* buf, bf16* ds
 //
 // Warps (192 threads): 0 = TMA producer, 1 = MMA issuer and TMEM owner, 2..5 = epilogue.  An epilogue
 // warp may read the quarter of the TMEM lanes given by its index modulo 4, i.e. the 32 rows of one group.
-// Each warp converts its 32 x 64 pieces into staging tiles of its own (two, used in turn) and stores them
+// Each warp converts its 32 x 64 pieces, two at a time, into two staging tiles of its own and stores them
 // with TMA stores of its own: no barrier spans the epilogue warps.  (Measured: two warps per quarter with
 // one staging tile each are slower, 129 against 110 us for a ViT forward; more pollers, no more overlap.)
 //
@@ -227,7 +225,7 @@ chain_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant__ C
   uint8_t* stg = S0 + (size_t)p.max_blocks * p.natoms * kAtomBytes;
   Bars* bars = reinterpret_cast<Bars*>(stg + kEpiWarps * kStgTiles * kGroupBytes);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = (int)uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
   // items are dealt in runs of p.deal (1, or 4 = whole 128-row blocks when every CTA gets at least two blocks:
   // a block costs the same whether full or not, so whole blocks waste none, and the CTAs with one block fewer
   // leave their SMs to the kernel that follows)
@@ -264,60 +262,72 @@ chain_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant__ C
   const unsigned long long lim = p.wait_ns;
 
   if (warp == 0) {
-    // ------------------------------------------------------------ TMA producer
-    if (lane == 0 && !p.stall_selftest) {
-      int i1 = 0, i2 = 0, u = 0;
+    // ------------------------------------------------------------ TMA producer (one elected lane, as the MMA issuer)
+    if (!p.stall_selftest) {
+      int u = 0;
+      int slot1 = 0, ph1 = 1, slot2 = 0, ph2 = 1;       // ring positions; parity of the next wait for an empty slot
       bool ok = true;
       for (int g = g_begin; g < g_end && ok; ++u) {
         const Unit un = make_unit(p, g, g_end);
         const int nt = un.nt;
         // the shared memory of the last unit is free once its MMAs are done and its stores have been read
-        if (u > 0 && !mbar_wait(&bars->unit_done, (u - 1) & 1, lim)) { raise_timeout(bars, p.status); ok = false; break; }
-        for (int ks = 0; ks < p.nk1 && ok; ++ks, ++i1) {
-          const int slot = i1 % p.ns, ph = (i1 / p.ns) & 1;
-          if (!mbar_wait(&bars->empty[slot], ph ^ 1, lim)) { raise_timeout(bars, p.status); ok = false; break; }
-          uint8_t* dst = smem + (size_t)slot * p.slot_bytes;
-          const int kr = (ks + rot1) % p.nk1;
-          uint8_t* f1 = dst + p.max_blocks * kAtomBytes;
-          if (!p.cv.on) {
-            mbar_arrive_expect_tx(&bars->full[slot], nt * kAtomBytes + p.f1_bytes);
-            // a block at the end of the run is loaded whole as well: the rows past the run are a neighbour's
-            // (or zeros past the last row) and cost less than four separate 32-row loads
-            for (int tt = 0; tt < nt; ++tt)
-              tma_load_2d(dst + tt * kAtomBytes, &tmIn, &bars->full[slot], kr * 64, un.row0[tt]);
-            if (p.f1_mn)
-              for (int a = 0; a < p.natoms; ++a) tma_load_2d(f1 + a * kF1AtomBytes, &tmF1, &bars->full[slot], a * 64, kr * 64);
-            else
-              tma_load_2d(f1, &tmF1, &bars->full[slot], kr * 64, 0);
-          } else {
-            // slab kr = (tap, 64 channels): the tile's box of the activation, shifted by the tap
-            const int tap = kr / p.cv.cslabs, cs = kr - tap * p.cv.cslabs;
-            const int dy = (tap / 3 - 1) * p.cv.sign, dx = (tap % 3 - 1) * p.cv.sign;
-            mbar_arrive_expect_tx(&bars->full[slot], nt * p.cv.box_rows * 128 + p.f1_bytes);
-            for (int tt = 0; tt < nt; ++tt)
-              tma_load_4d(dst + tt * kAtomBytes, &tmIn4, &bars->full[slot], cs * 64, dx, un.y0[tt] + dy, un.b0[tt]);
-            const int fcol = tap * p.cv.tap_stride + p.cv.f1_col_off;
-            if (p.f1_mn)
-              for (int a = 0; a < p.natoms; ++a)
-                tma_load_2d(f1 + a * kF1AtomBytes, &tmF1, &bars->full[slot], fcol + a * 64, cs * 64);
-            else
-              tma_load_2d(f1, &tmF1, &bars->full[slot], fcol + cs * 64, 0);
+        if (u > 0 && !mbar_wait_warp(&bars->unit_done, (u - 1) & 1, lim)) { raise_timeout(bars, p.status); ok = false; break; }
+        int kr = rot1;
+        int tap = p.cv.on ? rot1 / p.cv.cslabs : 0, cs = p.cv.on ? rot1 - tap * p.cv.cslabs : 0;
+        const uint32_t tx1 = (p.cv.on ? nt * p.cv.box_rows * 128 : nt * kAtomBytes) + p.f1_bytes;
+        for (int ks = 0; ks < p.nk1; ++ks) {
+          if (!mbar_wait_warp(&bars->empty[slot1], ph1, lim)) { raise_timeout(bars, p.status); ok = false; break; }
+          if (elect_one()) {
+            uint8_t* dst = smem + (size_t)slot1 * p.slot_bytes;
+            uint8_t* f1 = dst + p.max_blocks * kAtomBytes;
+            uint64_t* bar = &bars->full[slot1];
+            mbar_arrive_expect_tx(bar, tx1);
+            if (!p.cv.on) {
+              // a block at the end of the run is loaded whole as well: the rows past the run are a neighbour's
+              // (or zeros past the last row) and cost less than four separate 32-row loads
+              for (int tt = 0; tt < nt; ++tt) tma_load_2d(dst + tt * kAtomBytes, &tmIn, bar, kr * 64, un.row0[tt]);
+              if (p.f1_mn)
+                for (int a = 0; a < p.natoms; ++a) tma_load_2d(f1 + a * kF1AtomBytes, &tmF1, bar, a * 64, kr * 64);
+              else
+                tma_load_2d(f1, &tmF1, bar, kr * 64, 0);
+            } else {
+              // slab kr = (tap, 64 channels): the tile's box of the activation, shifted by the tap
+              const int ty = tap / 3, dy = (ty - 1) * p.cv.sign, dx = (tap - 3 * ty - 1) * p.cv.sign;
+              for (int tt = 0; tt < nt; ++tt)
+                tma_load_4d(dst + tt * kAtomBytes, &tmIn4, bar, cs * 64, dx, un.y0[tt] + dy, un.b0[tt]);
+              const int fcol = tap * p.cv.tap_stride + p.cv.f1_col_off;
+              if (p.f1_mn)
+                for (int a = 0; a < p.natoms; ++a) tma_load_2d(f1 + a * kF1AtomBytes, &tmF1, bar, fcol + a * 64, cs * 64);
+              else
+                tma_load_2d(f1, &tmF1, bar, fcol + cs * 64, 0);
+            }
           }
+          __syncwarp();
+          if (++slot1 == p.ns) { slot1 = 0; ph1 ^= 1; }
+          if (++cs == p.cv.cslabs) { cs = 0; ++tap; }
+          if (++kr == p.nk1) { kr = 0; tap = 0; cs = 0; }
         }
+        if (!ok) break;
         // the second product's slots lie over the first product's: wait until its MMAs have read them
-        if (ok && !mbar_wait(&bars->t_full, u & 1, lim)) { raise_timeout(bars, p.status); ok = false; }
+        if (!mbar_wait_warp(&bars->t_full, u & 1, lim)) { raise_timeout(bars, p.status); ok = false; break; }
+        int col0 = rot2 * kChunk;
         for (int c = 0; c < p.nchunks && ok; ++c) {
-          const int col0 = ((c + rot2) % p.nchunks) * kChunk;
-          for (int j = 0; j < p.natoms; ++j, ++i2) {
-            const int slot = i2 % p.ns2, ph = (i2 / p.ns2) & 1;
-            if (!mbar_wait(&bars->empty2[slot], ph ^ 1, lim)) { raise_timeout(bars, p.status); ok = false; break; }
-            uint8_t* d = ring + (size_t)slot * kAtom2Bytes;
-            mbar_arrive_expect_tx(&bars->full2[slot], kAtom2Bytes);
-            if (p.f2_mn)
-              for (int b = 0; b < 4; ++b) tma_load_2d(d + b * kF1AtomBytes, &tmF2, &bars->full2[slot], col0 + 64 * b, j * 64);
-            else
-              tma_load_2d(d, &tmF2, &bars->full2[slot], j * 64, col0);
+          for (int j = 0; j < p.natoms; ++j) {
+            if (!mbar_wait_warp(&bars->empty2[slot2], ph2, lim)) { raise_timeout(bars, p.status); ok = false; break; }
+            if (elect_one()) {
+              uint8_t* d = ring + (size_t)slot2 * kAtom2Bytes;
+              uint64_t* bar = &bars->full2[slot2];
+              mbar_arrive_expect_tx(bar, kAtom2Bytes);
+              if (p.f2_mn)
+                for (int b = 0; b < 4; ++b) tma_load_2d(d + b * kF1AtomBytes, &tmF2, bar, col0 + 64 * b, j * 64);
+              else
+                tma_load_2d(d, &tmF2, bar, j * 64, col0);
+            }
+            __syncwarp();
+            if (++slot2 == p.ns2) { slot2 = 0; ph2 ^= 1; }
           }
+          col0 += kChunk;
+          if (col0 >= p.nchunks * kChunk) col0 = 0;
         }
         g += un.adv;
       }
@@ -341,19 +351,19 @@ chain_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant__ C
       const uint64_t dF2 = p.f2_mn ? smem_desc_sw128(s_base, kF1AtomBytes) : smem_desc_sw128(s_base, 16);
       const uint64_t f2_step = p.f2_mn ? (2048u >> 4) : 2u;
       const uint64_t blk_step = (uint64_t)(kAtomBytes >> 4);
-      int i2 = 0, u = 0;
-      int slot1 = 0, ph1 = 0;                  // first-product ring position
+      int u = 0;
+      int slot1 = 0, ph1 = 0, slot2 = 0, ph2 = 0;                  // ring positions
       int q0 = 0, q1 = 0;                      // uses of each accumulator so far
       bool ok = true;
       for (int g = g_begin; g < g_end && ok; ++u) {
         const Unit un = make_unit(p, g, g_end);
         const int nt = un.nt;
-        int kr = rot1;
+        int kr = rot1, cs = p.cv.on ? rot1 % p.cv.cslabs : 0;
         for (int ks = 0; ks < p.nk1; ++ks) {
           if (!mbar_wait_warp(&bars->full[slot1], ph1, lim)) { raise_timeout(bars, p.status); ok = false; break; }
           tc_fence_after();
           const uint64_t da0 = dA1 + slot_step * slot1, db0 = dF1 + slot_step * slot1;
-          const int ksteps = p.cv.on ? (p.cv.in_ch - (kr % p.cv.cslabs) * 64 + 15) >> 4 : (p.K1 - kr * 64 + 15) >> 4;
+          const int ksteps = p.cv.on ? (p.cv.in_ch - cs * 64 + 15) >> 4 : (p.K1 - kr * 64 + 15) >> 4;
           const uint32_t acc0 = ks != 0;
           if (elect_one()) {
             if (nt == 2) {
@@ -373,7 +383,8 @@ chain_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant__ C
           }
           __syncwarp();
           if (++slot1 == p.ns) { slot1 = 0; ph1 ^= 1; }
-          if (++kr == p.nk1) kr = 0;
+          if (++cs == p.cv.cslabs) cs = 0;
+          if (++kr == p.nk1) { kr = 0; cs = 0; }
         }
         if (!ok) break;
         if (elect_one()) tc_commit(&bars->t_full);
@@ -383,14 +394,15 @@ chain_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant__ C
           tc_fence_after();
         }
         for (int c = 0; c < p.nchunks && ok; ++c) {
+          int slot = slot2, ph = ph2;          // every block of the unit walks the same tiles
           for (int tt = 0; tt < nt && ok; ++tt) {
             const int b = (nt == 2) ? tt : (c & 1);
+            slot = slot2; ph = ph2;
             if (!mbar_wait_warp(&bars->acc_empty[b], ((b ? q1 : q0) & 1) ^ 1, lim)) { raise_timeout(bars, p.status); ok = false; break; }
             tc_fence_after();
             const uint32_t tacc = tmem + kChunk * b;
             const uint64_t dSb = dS + blk_step * (uint64_t)(tt * p.natoms);
             for (int j = 0; j < p.natoms; ++j) {
-              const int idx = i2 + j, slot = idx % p.ns2, ph = (idx / p.ns2) & 1;
               if (!mbar_wait_warp(&bars->full2[slot], ph, lim)) { raise_timeout(bars, p.status); ok = false; break; }
               tc_fence_after();
               const uint64_t da = dSb + blk_step * j;
@@ -404,10 +416,11 @@ chain_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant__ C
                 if (tt == nt - 1) tc_commit(&bars->empty2[slot]);     // the last block of the unit is done with this tile
               }
               __syncwarp();
+              if (++slot == p.ns2) { slot = 0; ph ^= 1; }
             }
             if (ok) { if (elect_one()) tc_commit(&bars->acc_full[b]); __syncwarp(); if (b) ++q1; else ++q0; }
           }
-          i2 += p.natoms;
+          slot2 = slot; ph2 = ph;
         }
         if (ok && elect_one()) tc_commit(&bars->unit_done);
         __syncwarp();
@@ -415,13 +428,11 @@ chain_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant__ C
       }
     }
   } else {
-    // ------------------------------------------------------------ epilogue (warps 2..9)
+    // ------------------------------------------------------------ epilogue (warps 2..5)
     const int qw = warp & 3;                // TMEM lane quarter this warp may read = the 32-row group it serves
-    const int hw = (warp - 2) >> 2;         // which of the warps of that quarter
     const int row = qw * 32 + lane;         // row of the 128-row block
     const uint32_t lane_base = (uint32_t)(qw * 32) << 16;
     uint8_t* mystg = stg + (size_t)(warp - 2) * kStgTiles * kGroupBytes;
-    int nst = 0;                            // stores issued from this warp's staging tiles
     int q0 = 0, q1 = 0;
     int u = 0;
     bool ok = true;
@@ -431,11 +442,10 @@ chain_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant__ C
       ok = warp_wait(bars, &bars->t_full, u & 1, lim, p.status);
       if (!ok) break;
       tc_fence_after();
-      // S of every block of the unit: the two warps of a quarter take alternate 64-column tiles
+      // S of every block of the unit
       for (int tt = 0; tt < nt; ++tt) {
         uint8_t* Sb = S0 + (size_t)tt * p.natoms * kAtomBytes;
         for (int j = 0; j < p.natoms; ++j) {
-          if (((tt * p.natoms + j) % kWarpsPerQuarter) != hw) continue;
           const int c0 = j * 64;
           uint32_t v[4][16];
 #pragma unroll
@@ -451,93 +461,105 @@ chain_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant__ C
       fence_proxy_async_smem();
       __syncwarp();
       if (lane == 0) mbar_arrive(&bars->s_ready);
-      if (p.save_s) {                        // this warp's tiles, this warp's 32 rows, if the block has them
+      if (p.save_s) {                        // this warp's 32 rows, if the block has them
         for (int tt = 0; tt < nt; ++tt) {
-          const int grows = un.nrows[tt] - qw * kGroupRows;      // rows of this warp's group in the block
+          const int grows = (int)uniform(un.nrows[tt] - qw * kGroupRows);      // rows of this warp's group in the block
           if (grows <= 0) continue;
           const int grow0 = un.row0[tt] + qw * kGroupRows;
           for (int j = 0; j < p.natoms; ++j) {
-            if (((tt * p.natoms + j) % kWarpsPerQuarter) != hw) continue;
             const uint8_t* src = S0 + ((size_t)tt * p.natoms + j) * kAtomBytes + qw * kGroupBytes;
             if (grows >= kGroupRows) {
-              if (lane == 0) tma_store_2d(&tmS, src, j * 64 + p.cv.s_col_off, grow0);
+              if (elect_one()) tma_store_2d(&tmS, src, j * 64 + p.cv.s_col_off, grow0);
+              __syncwarp();
             } else {
               store_partial_group(src, p.s_ptr + (int64_t)grow0 * p.s_ld + p.cv.s_col_off + j * 64, p.s_ld, grows,
                                   p.s_cols - j * 64);
             }
           }
         }
-        if (lane == 0) tma_store_commit();
+        if (elect_one()) tma_store_commit();
+        __syncwarp();
       }
+      int col0 = rot2 * kChunk;
       for (int c = 0; c < p.nchunks && ok; ++c) {
-        const int col0 = ((c + rot2) % p.nchunks) * kChunk + hw * (64 * kPiecesPerWarp);
         for (int tt = 0; tt < nt && ok; ++tt) {
           const int b = (nt == 2) ? tt : (c & 1);
           ok = warp_wait(bars, &bars->acc_full[b], (b ? q1 : q0) & 1, lim, p.status);
           if (!ok) break;
           if (b) ++q1; else ++q0;
           tc_fence_after();
-          const int grows = un.nrows[tt] - qw * kGroupRows;   // rows of this warp's group in the block
-          const bool rows_live = grows > 0;
+          const int grows = (int)uniform(un.nrows[tt] - qw * kGroupRows);   // rows of this warp's group in the block
           const int grow0 = un.row0[tt] + qw * kGroupRows;
-          const uint32_t tacc = tmem_base + kChunk * b + lane_base + hw * (64 * kPiecesPerWarp);
-          // the warp's 64-column pieces: each is read from TMEM and rounded to bf16 pairs at once (32
-          // registers a piece); they are staged and stored after the accumulator has been handed back
-          uint32_t w[kPiecesPerWarp][32];
+          const uint32_t tacc = tmem_base + kChunk * b + lane_base;
+          const int npairs = grows > 0 ? min(2, (p.P - col0 + 127) >> 7) : 0;     // 128-column pairs of pieces this warp stores
+          // two 64-column pieces at a time: TMEM -> registers (bf16 pairs) while the stores of the pair before them still
+          // read the staging tiles; the accumulator is handed back as soon as its last piece is in registers
 #pragma unroll
-          for (int pc = 0; pc < kPiecesPerWarp; ++pc) {
-            if (rows_live && col0 + pc * 64 < p.P) {
-              uint32_t v[4][16];
+          for (int pr = 0; pr < 2; ++pr) {
+            uint32_t w[2][32];
+            if (pr < npairs) {
 #pragma unroll
-              for (int gq = 0; gq < 4; ++gq) tmem_ld16_nowait(tacc + pc * 64 + gq * 16, v[gq]);
-              tmem_wait_ld();
+              for (int h = 0; h < 2; ++h) {
+                uint32_t v[4][16];
 #pragma unroll
-              for (int gq = 0; gq < 4; ++gq)
+                for (int gq = 0; gq < 4; ++gq) tmem_ld16_nowait(tacc + pr * 128 + h * 64 + gq * 16, v[gq]);
+                tmem_wait_ld();
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                  __nv_bfloat162 h2 = __floats2bfloat162_rn(__uint_as_float(v[gq][2 * i]), __uint_as_float(v[gq][2 * i + 1]));
-                  w[pc][gq * 8 + i] = *reinterpret_cast<uint32_t*>(&h2);
-                }
+                for (int gq = 0; gq < 4; ++gq)
+#pragma unroll
+                  for (int e = 0; e < 8; ++e) {
+                    __nv_bfloat162 h2 = __floats2bfloat162_rn(__uint_as_float(v[gq][2 * e]), __uint_as_float(v[gq][2 * e + 1]));
+                    w[h][gq * 8 + e] = *reinterpret_cast<uint32_t*>(&h2);
+                  }
+              }
             }
-          }
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&bars->acc_empty[b]);
-#pragma unroll
-          for (int pc = 0; pc < kPiecesPerWarp; ++pc) {
-            if (!(rows_live && col0 + pc * 64 < p.P)) continue;
-            uint8_t* buf = mystg + (nst % kStgTiles) * kGroupBytes;
-            ++nst;
-            if (lane == 0) tma_store_wait_read<kStgTiles - 1>();   // the store that last read this staging tile
+            if (pr == (npairs == 2 ? 1 : 0)) {
+              tc_fence_before();
+              __syncwarp();
+              if (lane == 0) mbar_arrive(&bars->acc_empty[b]);
+            }
+            if (pr >= npairs) continue;
+            if (elect_one()) tma_store_wait_read<0>();     // the stores that last read the staging tiles
             __syncwarp();
-            uint8_t* rowp = buf + lane * 128;
+            const int pcol = col0 + pr * 128;
 #pragma unroll
-            for (int ch = 0; ch < 8; ++ch)                 // 16-byte chunk ch of the row goes to slot ch ^ (row & 7)
-              *reinterpret_cast<uint4*>(rowp + ((ch ^ (lane & 7)) << 4)) =
-                  make_uint4(w[pc][4 * ch], w[pc][4 * ch + 1], w[pc][4 * ch + 2], w[pc][4 * ch + 3]);
+            for (int h = 0; h < 2; ++h) {
+              uint8_t* rowp = mystg + h * kGroupBytes + lane * 128;
+#pragma unroll
+              for (int ch = 0; ch < 8; ++ch)                 // 16-byte chunk ch of the row goes to slot ch ^ (row & 7)
+                *reinterpret_cast<uint4*>(rowp + ((ch ^ (lane & 7)) << 4)) =
+                    make_uint4(w[h][4 * ch], w[h][4 * ch + 1], w[h][4 * ch + 2], w[h][4 * ch + 3]);
+            }
             fence_proxy_async_smem();
             __syncwarp();
             if (grows >= kGroupRows) {
-              if (lane == 0) {
-                tma_store_2d(&tmOut, buf, col0 + pc * 64, grow0);
+              if (elect_one()) {
+                tma_store_2d(&tmOut, mystg, pcol, grow0);
+                if (pcol + 64 < p.P) tma_store_2d(&tmOut, mystg + kGroupBytes, pcol + 64, grow0);
                 tma_store_commit();
               }
+              __syncwarp();
             } else {        // the last rows of a convolution tile: fewer than 32
-              store_partial_group(buf, p.out_ptr + (int64_t)grow0 * p.P + col0 + pc * 64, p.P, grows, p.P - (col0 + pc * 64));
+              for (int h = 0; h < 2; ++h)
+                if (pcol + 64 * h < p.P)
+                  store_partial_group(mystg + h * kGroupBytes, p.out_ptr + (int64_t)grow0 * p.P + pcol + 64 * h, p.P, grows, p.P - (pcol + 64 * h));
               __syncwarp();
             }
           }
         }
+        col0 += kChunk;
+        if (col0 >= p.nchunks * kChunk) col0 = 0;
       }
       // this warp has read all it will of the unit's accumulators; once its stores have read their
       // shared memory (S tiles and staging) the next unit may overwrite both
       if (ok) {
-        if (lane == 0) { tma_store_wait_read<0>(); mbar_arrive(&bars->unit_done); }
+        if (elect_one()) { tma_store_wait_read<0>(); mbar_arrive(&bars->unit_done); }
         __syncwarp();
       }
       g += un.adv;
     }
-    if (lane == 0) tma_store_wait_all();
+    if (elect_one()) tma_store_wait_all();
+    __syncwarp();
   }
 
   // ------------------------------------------------------------ common exit
