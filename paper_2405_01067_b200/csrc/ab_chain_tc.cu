@@ -629,7 +629,7 @@ grad_kernel(const __grid_constant__ CUtensorMap tmAct0, const __grid_constant__ 
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   uint8_t* ring = smem;
   Bars* bars = reinterpret_cast<Bars*>(ring + (size_t)p.ns * p.slot_bytes);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = (int)uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
 
   // which job, which 128-row chunk of its output, which slice of the N rows
   int tile = blockIdx.x;
@@ -668,18 +668,20 @@ grad_kernel(const __grid_constant__ CUtensorMap tmAct0, const __grid_constant__ 
   clear_status_word(p.clear_status, p.status);
 
   if (warp == 0) {
-    if (lane == 0) {
-      for (int i = 0; i < nk; ++i) {
-        const int slot = i % p.ns, ph = (i / p.ns) & 1;
-        if (!mbar_wait(&bars->empty[slot], ph ^ 1)) { raise_timeout(bars, p.status); break; }
+    int slot = 0, ph = 1;
+    for (int i = 0; i < nk; ++i) {
+      if (!mbar_wait_warp(&bars->empty[slot], ph)) { raise_timeout(bars, p.status); break; }
+      if (elect_one()) {
         uint8_t* dst = ring + (size_t)slot * p.slot_bytes;
+        uint64_t* bar = &bars->full[slot];
         const int k0 = k_begin + i * 64;
         // two 128-row accumulators share every slab of `small`: four 64-wide boxes of act, then small
-        mbar_arrive_expect_tx(&bars->full[slot], (4 + p.natoms) * 8192);
-        for (int a = 0; a < 4; ++a) tma_load_2d(dst + a * 8192, tmAct, &bars->full[slot], chunk * 256 + a * 64, k0);
-        for (int a = 0; a < p.natoms; ++a)
-          tma_load_2d(dst + 32768 + a * 8192, tmSmall, &bars->full[slot], a * 64, k0);
+        mbar_arrive_expect_tx(bar, (4 + p.natoms) * 8192);
+        for (int a = 0; a < 4; ++a) tma_load_2d(dst + a * 8192, tmAct, bar, chunk * 256 + a * 64, k0);
+        for (int a = 0; a < p.natoms; ++a) tma_load_2d(dst + 32768 + a * 8192, tmSmall, bar, a * 64, k0);
       }
+      __syncwarp();
+      if (++slot == p.ns) { slot = 0; ph ^= 1; }
     }
   } else if (warp == 1) {
     grad_mma_loop(bars, ring, nk, p.ns, p.slot_bytes, p.r, tmem_base, p.status);
@@ -751,7 +753,7 @@ conv_grad_kernel(const __grid_constant__ CUtensorMap tmX4, const __grid_constant
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   uint8_t* ring = smem;
   Bars* bars = reinterpret_cast<Bars*>(ring + (size_t)p.ns * p.slot_bytes);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = (int)uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
   int tile = blockIdx.x;
   const int slice = tile % p.slices;
   const int chunk = tile / p.slices;
@@ -784,19 +786,22 @@ conv_grad_kernel(const __grid_constant__ CUtensorMap tmX4, const __grid_constant
   dep_launch();
 
   if (warp == 0) {
-    if (lane == 0) {
-      const int dy = tap / 3 - 1, dx = tap % 3 - 1;
-      for (int i = 0; i < nk; ++i) {
-        const int slot = i % p.ns, ph = (i / p.ns) & 1;
-        if (!mbar_wait(&bars->empty[slot], ph ^ 1)) { raise_timeout(bars, p.status); break; }
+    const int dy = tap / 3 - 1, dx = tap % 3 - 1;
+    int slot = 0, ph = 1;
+    int grp = s_begin / p.spi, ty = s_begin - grp * p.spi;
+    for (int i = 0; i < nk; ++i) {
+      if (!mbar_wait_warp(&bars->empty[slot], ph)) { raise_timeout(bars, p.status); break; }
+      if (elect_one()) {
         uint8_t* dst = ring + (size_t)slot * p.slot_bytes;
-        const int sl = s_begin + i;
-        const int grp = sl / p.spi, ty = sl - grp * p.spi;
+        uint64_t* bar = &bars->full[slot];
         const int b0 = grp * p.kb, y0 = ty * p.bhk;
-        mbar_arrive_expect_tx(&bars->full[slot], (4 + p.natoms) * p.box_rows * 128);
-        for (int a = 0; a < 4; ++a) tma_load_4d(dst + a * 8192, &tmX4, &bars->full[slot], cwin + a * 64, dx, y0 + dy, b0);
-        for (int a = 0; a < p.natoms; ++a) tma_load_4d(dst + 32768 + a * 8192, &tmT4, &bars->full[slot], a * 64, 0, y0, b0);
+        mbar_arrive_expect_tx(bar, (4 + p.natoms) * p.box_rows * 128);
+        for (int a = 0; a < 4; ++a) tma_load_4d(dst + a * 8192, &tmX4, bar, cwin + a * 64, dx, y0 + dy, b0);
+        for (int a = 0; a < p.natoms; ++a) tma_load_4d(dst + 32768 + a * 8192, &tmT4, bar, a * 64, 0, y0, b0);
       }
+      __syncwarp();
+      if (++slot == p.ns) { slot = 0; ph ^= 1; }
+      if (++ty == p.spi) { ty = 0; ++grp; }
     }
   } else if (warp == 1) {
     grad_mma_loop(bars, ring, nk, p.ns, p.slot_bytes, p.r, tmem_base, p.status);

@@ -105,7 +105,7 @@ gemm_tc_kernel(const TcProblemDev* __restrict__ probs, int nprobs, int ntiles, i
   uint8_t* ring = smem;
   uint8_t* stg = smem + kStages * kStage;
   TcBars* bars = reinterpret_cast<TcBars*>(stg + 4 * 2 * kStgBytes);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = (int)uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < kStages; ++i) { mbar_init(&bars->full[i], 1); mbar_init(&bars->empty[i], 1); }
@@ -121,27 +121,31 @@ gemm_tc_kernel(const TcProblemDev* __restrict__ probs, int nprobs, int ntiles, i
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
-    if (lane == 0) {
-      int i = 0;
+    {
+      int slot = 0, ph = 1;
       bool ok = true;
       for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
         const TileInfo ti = decode_tile(probs, nprobs, tile);
         const TcProblemDev* P = ti.P;
-        const int a_mn = P->a_mn, b_mn = P->b_mn;
-        for (int tix = 0; tix < P->nterms && ok; ++tix) {
+        const int a_mn = (int)uniform(P->a_mn), b_mn = (int)uniform(P->b_mn), nterms = (int)uniform(P->nterms), nslab = (int)uniform(ti.nslab);
+        for (int tix = 0; tix < nterms && ok; ++tix) {
           const CUtensorMap* ma = &P->a[P->term_a[tix]];
           const CUtensorMap* mb = &P->b[P->term_b[tix]];
-          for (int ks = 0; ks < ti.nslab; ++ks, ++i) {
-            const int slot = i % kStages, ph = (i / kStages) & 1;
-            if (!mbar_wait(&bars->empty[slot], ph ^ 1)) { tc_raise(bars, status); ok = false; break; }
-            uint8_t* da = ring + (size_t)slot * kStage;
-            uint8_t* db = da + kAStage;
-            const int k0 = ti.k_begin + ks * kBK;
-            mbar_arrive_expect_tx(&bars->full[slot], kStage);
-            if (a_mn) { for (int h = 0; h < 2; ++h) tma_load_2d(da + h * 8192, ma, &bars->full[slot], ti.m0 + 64 * h, k0); }
-            else tma_load_2d(da, ma, &bars->full[slot], k0, ti.m0);
-            if (b_mn) { for (int h = 0; h < 4; ++h) tma_load_2d(db + h * 8192, mb, &bars->full[slot], ti.n0 + 64 * h, k0); }
-            else tma_load_2d(db, mb, &bars->full[slot], k0, ti.n0);
+          for (int ks = 0; ks < nslab; ++ks) {
+            if (!mbar_wait_warp(&bars->empty[slot], ph)) { tc_raise(bars, status); ok = false; break; }
+            if (elect_one()) {
+              uint8_t* da = ring + (size_t)slot * kStage;
+              uint8_t* db = da + kAStage;
+              uint64_t* bar = &bars->full[slot];
+              const int k0 = ti.k_begin + ks * kBK;
+              mbar_arrive_expect_tx(bar, kStage);
+              if (a_mn) { for (int h = 0; h < 2; ++h) tma_load_2d(da + h * 8192, ma, bar, ti.m0 + 64 * h, k0); }
+              else tma_load_2d(da, ma, bar, k0, ti.m0);
+              if (b_mn) { for (int h = 0; h < 4; ++h) tma_load_2d(db + h * 8192, mb, bar, ti.n0 + 64 * h, k0); }
+              else tma_load_2d(db, mb, bar, k0, ti.n0);
+            }
+            __syncwarp();
+            if (++slot == kStages) { slot = 0; ph ^= 1; }
           }
         }
       }
