@@ -6,13 +6,15 @@
 //   forward : In = x,  F1 = B   (r x n), F2 = A   (m x r), Out = y,  S = T
 //   backward: In = dY, F1 = A^T (r x m), F2 = B^T (n x r), Out = dX, S = dT   (A and B read as they lie)
 // grad_kernel: dA = dY^T T and dB^T = x^T dT are reductions over the rows; a CTA owns 256 output rows (a
-// slice of m or of n) and one slice of the N rows, streams 64-row slabs of both operands (both
-// "MN-major": the reduction index is the slow one in memory) and leaves an fp32 partial;
-// reduce_partials_kernel adds the partials in ascending slice order.
+// slice of m or of n) and one slice of the N rows and streams 64-row slabs of both operands (both "MN-major": the reduction
+// index is the slow one in memory).  The slices of a tile form clusters, whose CTAs add their accumulators through
+// distributed shared memory in ascending order; where a tile has more than one cluster, reduce_partials_kernel adds those sums.
 //
 // All operand tiles are TMA boxes of 64 bf16 (128 bytes) x rows with 128-byte swizzle.  Every mbarrier
 // wait gives up after about a second, raises AB_ERR_TIMEOUT in the status word and unwinds to the common
 // exit, where TMEM is released.
+#include <cooperative_groups.h>
+
 #include <cstring>
 #include <mutex>
 
@@ -605,21 +607,87 @@ __device__ __forceinline__ void grad_mma_loop(Bars* bars, uint8_t* ring, int nk,
 
 // ---------------------------------------------------------------------------------------------
 // grad kernel: partial[slice][p][j] = sum_{k in slice} act[k][p] * small[k][j]
+// Where a tile's sums go: element (row, col) to dst[row * ld + col], or, transposed, to dst[col * ld + row].  A tile with
+// several clusters leaves one set of sums per cluster, `stride` elements apart.
+struct GradOut {
+  float* dst;
+  int64_t ld, stride;
+  int rows, cols;
+  int transposed;
+};
 struct GradJob {
-  int P;          // columns of act = rows of the output
-  int chunks;     // ceil(P / 256)
-  float* partial; // [slices][P][r]
+  int chunks;     // 256-row tiles of the output
+  GradOut out;
 };
 struct GradParams {
   GradJob job[2];
-  int njobs;
   int r, natoms, ns, slot_bytes;
-  int slices, rows_per_slice;   // rows_per_slice is a multiple of 64
+  int slices, rows_per_slice;   // slices: CTAs per tile; rows_per_slice is a multiple of 64
   int N;
   int clear_status;
   int job0_independent;   // 1: job 0 reads nothing the kernel before this one in the stream writes (see grad_kernel)
   int* status;
 };
+
+// The end of both gradient kernels: 2 x 128 accumulator rows of r columns -> this CTA's shared memory -> sums over the CTAs
+// of the cluster, in ascending order, each CTA for its share of the rows -> global memory.  Every thread of the
+// CTA comes here, also after a wait that gave up (the outputs are then undefined, the status says so).
+// A row takes r + 4 floats: with r a multiple of 16 eight lanes' 16-byte accesses then fall into different banks.
+__device__ __forceinline__ void grad_finish(uint8_t* ring, uint32_t tmem_base, bool have, int r, int row0, int cluster_index,
+                                            const GradOut& o) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  float* tile = reinterpret_cast<float*>(ring);
+  const int ldt = r + 4, share = 128 / C;
+  float* dst = o.dst + (int64_t)cluster_index * o.stride;
+  for (int mt = 0; mt < 2 && row0 + 128 * mt < o.rows; ++mt) {
+    if (warp >= 2) {
+      const int q = warp & 3, row = q * 32 + lane;
+      const uint32_t t = tmem_base + 256 * mt + ((uint32_t)(q * 32) << 16);
+      for (int c0 = 0; c0 < r; c0 += 16) {
+        float v[16];
+        if (have) tmem_ld16(t + c0, v);
+        else {
+#pragma unroll
+          for (int i = 0; i < 16; ++i) v[i] = 0.f;
+        }
+        float4* d = reinterpret_cast<float4*>(tile + row * ldt + c0);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) d[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+      }
+    }
+    if (C > 1) cluster.sync(); else __syncthreads();
+    const int groups = r >> 2;
+    for (int e = tid; e < share * groups; e += blockDim.x) {
+      const int lr = rank * share + e % share, c = (e / share) * 4;       // neighbouring threads: neighbouring rows
+      float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (C == 8) {
+        float4 v[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = *reinterpret_cast<const float4*>(cluster.map_shared_rank(tile, k) + lr * ldt + c);
+        s = v[0];
+#pragma unroll
+        for (int k = 1; k < 8; ++k) { s.x += v[k].x; s.y += v[k].y; s.z += v[k].z; s.w += v[k].w; }
+      } else {
+        for (int k = 0; k < C; ++k) {
+          const float4 v = *reinterpret_cast<const float4*>((C > 1 ? cluster.map_shared_rank(tile, k) : tile) + lr * ldt + c);
+          s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+        }
+      }
+      const int row = row0 + 128 * mt + lr;
+      if (row >= o.rows || c >= o.cols) continue;
+      if (!o.transposed) {
+        *reinterpret_cast<float4*>(dst + (int64_t)row * o.ld + c) = s;       // cols is a multiple of 4
+      } else {
+        float* d = dst + (int64_t)c * o.ld + row;
+        d[0] = s.x; d[o.ld] = s.y; d[2 * o.ld] = s.z; d[3 * o.ld] = s.w;
+      }
+    }
+    if (C > 1) cluster.sync(); else __syncthreads();     // the tile is reused, or the CTA leaves
+  }
+}
 
 __global__ void __launch_bounds__(192, 1)
 grad_kernel(const __grid_constant__ CUtensorMap tmAct0, const __grid_constant__ CUtensorMap tmSmall0,
@@ -633,6 +701,7 @@ grad_kernel(const __grid_constant__ CUtensorMap tmAct0, const __grid_constant__ 
 
   // which job, which 128-row chunk of its output, which slice of the N rows
   int tile = blockIdx.x;
+  const int cluster_size = (int)cooperative_groups::this_cluster().num_blocks();
   const int slice = tile % p.slices;
   tile /= p.slices;
   int jb = 0;
@@ -685,43 +754,21 @@ grad_kernel(const __grid_constant__ CUtensorMap tmAct0, const __grid_constant__ 
     }
   } else if (warp == 1) {
     grad_mma_loop(bars, ring, nk, p.ns, p.slot_bytes, p.r, tmem_base, p.status);
-  } else {
-    const int q = warp & 3;
-    const int row = q * 32 + lane;
-    const uint32_t lane_base = (uint32_t)(q * 32) << 16;
-    const GradJob& job = p.job[jb];
-    bool ok = true;
-    if (nk > 0) ok = epi_wait(bars, &bars->t_full, 0, p.status);
-    if (ok) {
-      tc_fence_after();
-      for (int mt = 0; mt < 2; ++mt) {
-        const int prow = chunk * 256 + mt * 128 + row;
-        float* out = job.partial + ((size_t)slice * job.P + prow) * p.r;
-        for (int c0 = 0; c0 < p.r; c0 += 16) {
-          float v[16];
-          if (nk > 0) tmem_ld16(tmem_base + mt * 256 + lane_base + c0, v);
-          else {
-#pragma unroll
-            for (int i = 0; i < 16; ++i) v[i] = 0.f;
-          }
-          if (prow < job.P) {
-            float4* o = reinterpret_cast<float4*>(out + c0);
-            o[0] = make_float4(v[0], v[1], v[2], v[3]);
-            o[1] = make_float4(v[4], v[5], v[6], v[7]);
-            o[2] = make_float4(v[8], v[9], v[10], v[11]);
-            o[3] = make_float4(v[12], v[13], v[14], v[15]);
-          }
-        }
-      }
-    }
+  } else if (nk > 0) {
+    if (epi_wait(bars, &bars->t_full, 0, p.status)) tc_fence_after();
   }
-  tc_fence_before();
-  __syncthreads();
-  if (*reinterpret_cast<volatile int*>(&bars->abort_any)) {
+  __syncwarp();
+  __syncthreads();          // the MMAs have read the ring, which now takes the sums
+  const bool failed = *reinterpret_cast<volatile int*>(&bars->abort_any) != 0;
+  if (failed) {             // give copies that are still in flight time to land
     const uint64_t t0 = globaltimer_ns();
     while (globaltimer_ns() - t0 < 200000ull) { }
     __syncthreads();
   }
+  tc_fence_after();
+  grad_finish(ring, tmem_base, nk > 0 && !failed, p.r, chunk * 256, slice / cluster_size, p.job[jb].out);
+  tc_fence_before();
+  __syncthreads();
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem_base, kTmemCols);
@@ -742,7 +789,7 @@ struct ConvGradParams {
   int spi, kb, bhk, box_rows;    // slabs per image (kb == 1) or 1; images per slab; image rows per slab; pixels per box
   int cpt;                       // 256-channel windows per tap
   int slices, slabs_per_slice, nslabs;
-  float* partial;                // [slices][9 C][r]
+  GradOut out;                   // rows: 9 C
   int* status;
 };
 
@@ -755,6 +802,7 @@ conv_grad_kernel(const __grid_constant__ CUtensorMap tmX4, const __grid_constant
   Bars* bars = reinterpret_cast<Bars*>(ring + (size_t)p.ns * p.slot_bytes);
   const int warp = (int)uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
   int tile = blockIdx.x;
+  const int cluster_size = (int)cooperative_groups::this_cluster().num_blocks();
   const int slice = tile % p.slices;
   const int chunk = tile / p.slices;
   const int tap = chunk / p.cpt, cwin = (chunk - tap * p.cpt) * 256;
@@ -805,49 +853,32 @@ conv_grad_kernel(const __grid_constant__ CUtensorMap tmX4, const __grid_constant
     }
   } else if (warp == 1) {
     grad_mma_loop(bars, ring, nk, p.ns, p.slot_bytes, p.r, tmem_base, p.status);
-  } else {
-    const int q = warp & 3;
-    const int row = q * 32 + lane;
-    const uint32_t lane_base = (uint32_t)(q * 32) << 16;
-    bool ok = true;
-    if (nk > 0) ok = epi_wait(bars, &bars->t_full, 0, p.status);
-    if (ok) {
-      tc_fence_after();
-      for (int mt = 0; mt < 2; ++mt) {
-        const int ch = cwin + mt * 128 + row;             // channel within the tap
-        float* out = p.partial + ((size_t)slice * 9 * p.C + (size_t)tap * p.C + ch) * p.r;
-        for (int c0 = 0; c0 < p.r; c0 += 16) {
-          float v[16];
-          if (nk > 0) tmem_ld16(tmem_base + mt * 256 + lane_base + c0, v);
-          else {
-#pragma unroll
-            for (int i = 0; i < 16; ++i) v[i] = 0.f;
-          }
-          if (ch < p.C) {
-            float4* o = reinterpret_cast<float4*>(out + c0);
-            o[0] = make_float4(v[0], v[1], v[2], v[3]);
-            o[1] = make_float4(v[4], v[5], v[6], v[7]);
-            o[2] = make_float4(v[8], v[9], v[10], v[11]);
-            o[3] = make_float4(v[12], v[13], v[14], v[15]);
-          }
-        }
-      }
-    }
+  } else if (nk > 0) {
+    if (epi_wait(bars, &bars->t_full, 0, p.status)) tc_fence_after();
   }
-  tc_fence_before();
+  __syncwarp();
   __syncthreads();
-  if (*reinterpret_cast<volatile int*>(&bars->abort_any)) {
+  const bool failed = *reinterpret_cast<volatile int*>(&bars->abort_any) != 0;
+  if (failed) {
     const uint64_t t0 = globaltimer_ns();
     while (globaltimer_ns() - t0 < 200000ull) { }
     __syncthreads();
   }
+  tc_fence_after();
+  // the tile's rows are channels cwin .. of one tap: rows end with the tap
+  GradOut o = p.out;
+  o.dst += p.out.transposed ? (int64_t)tap * p.C : (int64_t)tap * p.C * p.out.ld;
+  o.rows = p.C;
+  grad_finish(ring, tmem_base, nk > 0 && !failed, p.r, cwin, slice / cluster_size, o);
+  tc_fence_before();
+  __syncthreads();
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem_base, kTmemCols);
   }
 }
 
-// Sums the per-slice partials in ascending slice order (fixed order: identical bits every run).
+// Sums the clusters' partials in ascending order (fixed order: identical bits every run).
 //   blocks [0, nA):  dA[p][j]  = sum_s pA[s][p][j]            (float4 per thread)
 //   blocks [nA, ..): dB[j][q]  = sum_s pB[s][q][j]            (32 x 32 tiles transposed through shared memory)
 __global__ void __launch_bounds__(256)
@@ -912,19 +943,33 @@ __global__ void bounded_wait_selftest_kernel(int* status, unsigned long long lim
 // Launch with programmatic stream serialisation (see dep_wait): only for kernels that call dep_wait()
 // before their first access to global memory.
 template <typename... KArgs, typename... Args>
-cudaError_t launch_dep(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
+cudaError_t launch_dep_cluster(int cluster, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                               Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = cluster; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
+template <typename... KArgs, typename... Args>
+cudaError_t launch_dep(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
+  return launch_dep_cluster(1, kernel, grid, block, smem, st, std::forward<Args>(args)...);
+}
+#define AB_LAUNCH_CLUSTER(...)                             \
+  do {                                                     \
+    if (launch_dep_cluster(__VA_ARGS__) != cudaSuccess) {  \
+      cudaGetLastError();                                  \
+      return AB_ERR_CUDA;                                  \
+    }                                                      \
+  } while (0)
 #define AB_LAUNCH_DEP(...)                         \
   do {                                             \
     if (launch_dep(__VA_ARGS__) != cudaSuccess) {  \
@@ -1006,7 +1051,31 @@ ChainPlan chain_plan(int rp, int max_blocks, bool f1_mn) {
   return pl;
 }
 
-struct GradPlan { int natoms, ns, slot_bytes, slices, rows_per_slice; size_t smem; };
+// How the slabs of a gradient reduction are dealt: clusters of C CTAs, ncl clusters per 256-row tile, per slabs per CTA.  The
+// split with the least time by what was measured: about 0.7 us a slab with the device full, 3 us to fill and empty a CTA, 4 us
+// for a reduction launch and its traffic at 4 TB/s; resident clusters of 8 / 4 / 2 / 1 CTAs: 16 / 36 / 74 / one per SM.
+struct GradSplit { int C, ncl, per; };
+GradSplit grad_split(int64_t slabs, int tiles, int rp) {
+  const int sms = sm_count() > 0 ? sm_count() : 1;
+  GradSplit best = {1, 1, (int)slabs};
+  double best_t = 1e30;
+  for (int C = 1; C <= 8; C *= 2) {
+    if (C > slabs) break;
+    int resident = C == 8 ? sms / 9 : C == 4 ? sms / 4 - 1 : sms / C;
+    if (resident < 1) resident = 1;
+    for (int ncl = 1; ncl <= 32 && (int64_t)C * ncl <= slabs; ++ncl) {
+      const int64_t per = (slabs + (int64_t)C * ncl - 1) / ((int64_t)C * ncl);
+      const int waves = (tiles * ncl + resident - 1) / resident;
+      double t = waves * (0.7 * (double)per + 3.0);
+      if (ncl > 1) t += 4.0 + 2.0 * ncl * tiles * 256.0 * rp * 4.0 / 4e6;
+      if (t < best_t) { best_t = t; best = {C, ncl, (int)per}; }
+    }
+  }
+  return best;
+}
+int tiles256(int v) { return (v + 255) / 256; }
+
+struct GradPlan { int natoms, ns, slot_bytes; GradSplit sp; size_t smem; };
 GradPlan grad_plan(int64_t N, int m, int n, int r) {
   GradPlan pl;
   pl.natoms = (r + 63) / 64;
@@ -1014,28 +1083,31 @@ GradPlan grad_plan(int64_t N, int m, int n, int r) {
   const int fixed = (int)sizeof(Bars) + 1024;
   pl.ns = (kSmemLimit - fixed) / pl.slot_bytes;
   if (pl.ns > kMaxStages) pl.ns = kMaxStages;
-  pl.smem = (size_t)fixed + (size_t)pl.ns * pl.slot_bytes;
-  const int tiles = (m + 255) / 256 + (n + 255) / 256;
-  int slices = (sm_count() > 0 ? sm_count() : 1) / tiles;   // one wave of CTAs
-  if (slices < 1) slices = 1;
-  const int64_t slabs = (N + 63) / 64;
-  if (slices > slabs) slices = (int)slabs;
-  int64_t per = (slabs + slices - 1) / slices;
-  pl.rows_per_slice = (int)(per * 64);
-  pl.slices = (int)((slabs + per - 1) / per);
+  pl.smem = (size_t)fixed + (size_t)pl.ns * pl.slot_bytes;      // the ring also holds 128 x (r + 4) sums: at most 133 KB of it
+  pl.sp = grad_split((N + 63) / 64, tiles256(m) + tiles256(n), pad16(r));
   return pl;
+}
+// floats of the clusters' partial sums of an output of `rows` rows
+size_t grad_partial(const GradSplit& s, int64_t rows, int rp) { return s.ncl > 1 ? (size_t)s.ncl * rows * rp : 0; }
+GradOut grad_out(const GradSplit& sp, float* partial, float* dst, int rows, int r, bool transposed) {
+  GradOut o;
+  const int rp = pad16(r);
+  o.rows = rows;
+  if (sp.ncl > 1) { o.dst = partial; o.ld = rp; o.stride = (int64_t)rows * rp; o.cols = rp; o.transposed = 0; }
+  else { o.dst = dst; o.ld = transposed ? rows : r; o.stride = 0; o.cols = r; o.transposed = transposed ? 1 : 0; }
+  return o;
 }
 
 struct BwdWs { int* status; bf16 *T, *dT; float *pA, *pB; size_t bytes; };
 BwdWs bwd_ws(void* ws, int64_t N, int m, int n, int r) {
-  GradPlan gp = grad_plan(N, m, n, r);
+  const GradSplit sp = grad_plan(N, m, n, r).sp;
   Arena ar(ws, 0);
   BwdWs w;
   w.status = ar.take_n<int>(64);
   w.T = ar.take_n<bf16>((size_t)N * r);
   w.dT = ar.take_n<bf16>((size_t)N * r);
-  w.pA = ar.take_n<float>((size_t)gp.slices * m * pad16(r));
-  w.pB = ar.take_n<float>((size_t)gp.slices * n * pad16(r));
+  w.pA = ar.take_n<float>(grad_partial(sp, m, pad16(r)));
+  w.pB = ar.take_n<float>(grad_partial(sp, n, pad16(r)));
   w.bytes = align_up(ar.used, 256);
   return w;
 }
@@ -1238,36 +1310,37 @@ int chain_tc_backward(const void* x, const void* dY, const void* A, const void* 
     after_chain = true;
   }
   if (dA || dB) {
-    GradPlan gp = grad_plan(N, m, n, r);
-    const int rp = pad16(r);
+    const GradPlan gp = grad_plan(N, m, n, r);     // the same split whichever is asked for: the same bits
+    const int rp = pad16(r), slices = gp.sp.C * gp.sp.ncl;
     GradParams p;
+    std::memset(&p, 0, sizeof(p));
     CUtensorMap tmAct[2], tmSmall[2];
     int nj = 0;
     if (dA) {
       AB_TRY(make_map(&tmAct[nj], dY, (uint64_t)N, m, m, 64, 64));
       AB_TRY(make_map(&tmSmall[nj], T, (uint64_t)N, r, r, 64, 64));
-      p.job[nj].P = m; p.job[nj].chunks = (m + 255) / 256; p.job[nj].partial = w.pA;
+      p.job[nj].chunks = tiles256(m); p.job[nj].out = grad_out(gp.sp, w.pA, dA, m, r, false);
       ++nj;
     }
     if (dB) {
       AB_TRY(make_map(&tmAct[nj], x, (uint64_t)N, n, n, 64, 64));
       AB_TRY(make_map(&tmSmall[nj], w.dT, (uint64_t)N, r, r, 64, 64));
-      p.job[nj].P = n; p.job[nj].chunks = (n + 255) / 256; p.job[nj].partial = w.pB;
+      p.job[nj].chunks = tiles256(n); p.job[nj].out = grad_out(gp.sp, w.pB, dB, n, r, true);
       ++nj;
     }
     if (nj == 1) { tmAct[1] = tmAct[0]; tmSmall[1] = tmSmall[0]; p.job[1] = p.job[0]; p.job[1].chunks = 0; }
-    p.njobs = nj; p.r = rp; p.natoms = gp.natoms; p.ns = gp.ns; p.slot_bytes = gp.slot_bytes;
-    p.slices = gp.slices; p.rows_per_slice = gp.rows_per_slice; p.N = (int)N; p.clear_status = first ? 1 : 0; p.status = w.status;
+    p.r = rp; p.natoms = gp.natoms; p.ns = gp.ns; p.slot_bytes = gp.slot_bytes;
+    p.slices = slices; p.rows_per_slice = gp.sp.per * 64; p.N = (int)N; p.clear_status = first ? 1 : 0; p.status = w.status;
     p.job0_independent = (after_chain && dA) ? 1 : 0;   // job 0 is the dA job whenever dA is asked for
     AB_CUDA_OK(cudaFuncSetAttribute(grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gp.smem));
-    const unsigned grid = (unsigned)((p.job[0].chunks + p.job[1].chunks) * gp.slices);
-    AB_LAUNCH_DEP(grad_kernel, dim3(grid), dim3(192), gp.smem, st, tmAct[0], tmSmall[0], tmAct[1], tmSmall[1], p);
+    const unsigned grid = (unsigned)((p.job[0].chunks + p.job[1].chunks) * slices);
+    AB_LAUNCH_CLUSTER(gp.sp.C, grad_kernel, dim3(grid), dim3(192), gp.smem, st, tmAct[0], tmSmall[0], tmAct[1], tmSmall[1], p);
     AB_LAUNCH_OK();
-    {
+    if (gp.sp.ncl > 1) {
       const int nA = dA ? (int)(((int64_t)m * r / 4 + 255) / 256) : 0;
       const int nB = dB ? ((n + 31) / 32) * ((r + 31) / 32) : 0;
       AB_LAUNCH_DEP(reduce_partials_kernel, dim3(nA + nB), dim3(256), 0, st, static_cast<const float*>(w.pA), dA, m, nA,
-                 static_cast<const float*>(w.pB), dB, n, gp.slices, r, rp);
+                 static_cast<const float*>(w.pB), dB, n, gp.sp.ncl, r, rp);
       AB_LAUNCH_OK();
     }
     first = false;
@@ -1293,7 +1366,7 @@ ConvGeom conv_geom(int B, int H, int W, int in_ch, int sign, int tap_stride, int
   return g;
 }
 
-struct ConvGradPlan { int natoms, ns, slot_bytes, spi, kb, bhk, box_rows, cpt, slices, slabs_per_slice, nslabs; size_t smem; bool ok; };
+struct ConvGradPlan { int natoms, ns, slot_bytes, spi, kb, bhk, box_rows, cpt, nslabs; GradSplit sp; size_t smem; bool ok; };
 ConvGradPlan conv_grad_plan(int B, int H, int W, int C, int rp) {
   ConvGradPlan pl;
   pl.natoms = (rp + 63) / 64;
@@ -1307,14 +1380,7 @@ ConvGradPlan conv_grad_plan(int B, int H, int W, int C, int rp) {
   else { pl.kb = 1; pl.bhk = W <= 64 ? 64 / W : 1; pl.spi = (H + pl.bhk - 1) / pl.bhk; pl.nslabs = B * pl.spi; }
   pl.box_rows = W * pl.bhk * pl.kb;
   pl.cpt = (C + 255) / 256;
-  const int chunks = 9 * pl.cpt;
-  int sms = sm_count();
-  if (sms <= 0) sms = 1;
-  int slices = sms / chunks;
-  if (slices < 1) slices = 1;
-  if (slices > pl.nslabs) slices = pl.nslabs;
-  pl.slabs_per_slice = (pl.nslabs + slices - 1) / slices;
-  pl.slices = (pl.nslabs + pl.slabs_per_slice - 1) / pl.slabs_per_slice;
+  pl.sp = grad_split(pl.nslabs, 9 * pl.cpt, rp);
   return pl;
 }
 
@@ -1322,15 +1388,14 @@ struct ConvWs { int* status; bf16 *T, *dT; float *pA, *pB; size_t bytes; };
 ConvWs conv_ws(void* ws, int B, int H, int W, int C, int m, int r) {
   const int64_t N = (int64_t)B * H * W;
   const int rp = pad16(r);
-  GradPlan ga = grad_plan(N, m, 0, r);
-  ConvGradPlan gb = conv_grad_plan(B, H, W, C, rp);
+  const GradSplit ga = grad_plan(N, m, 0, r).sp, gb = conv_grad_plan(B, H, W, C, rp).sp;
   Arena ar(ws, 0);
   ConvWs w;
   w.status = ar.take_n<int>(64);
   w.T = ar.take_n<bf16>((size_t)N * r);
   w.dT = ar.take_n<bf16>((size_t)N * r);
-  w.pA = ar.take_n<float>((size_t)ga.slices * m * rp);
-  w.pB = ar.take_n<float>((size_t)gb.slices * 9 * C * rp);
+  w.pA = ar.take_n<float>(grad_partial(ga, m, rp));
+  w.pB = ar.take_n<float>(grad_partial(gb, 9 * (int64_t)C, rp));
   w.bytes = align_up(ar.used, 256);
   return w;
 }
@@ -1410,20 +1475,23 @@ int conv_tc_backward(const void* x, const void* dY, const void* A, const void* B
     CUtensorMap tmAct, tmSmall;
     AB_TRY(make_map(&tmAct, dY, (uint64_t)N, m, m, 64, 64));
     AB_TRY(make_map(&tmSmall, T, (uint64_t)N, r, r, 64, 64));
-    p.job[0].P = m; p.job[0].chunks = (m + 255) / 256; p.job[0].partial = w.pA;
+    p.job[0].chunks = tiles256(m); p.job[0].out = grad_out(gp.sp, w.pA, dA, m, r, false);
     p.job[1] = p.job[0]; p.job[1].chunks = 0;
-    p.njobs = 1; p.r = rp; p.natoms = gp.natoms; p.ns = gp.ns; p.slot_bytes = gp.slot_bytes;
-    p.slices = gp.slices; p.rows_per_slice = gp.rows_per_slice; p.N = (int)N; p.clear_status = first ? 1 : 0;
+    const int slices = gp.sp.C * gp.sp.ncl;
+    p.r = rp; p.natoms = gp.natoms; p.ns = gp.ns; p.slot_bytes = gp.slot_bytes;
+    p.slices = slices; p.rows_per_slice = gp.sp.per * 64; p.N = (int)N; p.clear_status = first ? 1 : 0;
     p.status = w.status; p.job0_independent = 0;
     AB_CUDA_OK(cudaFuncSetAttribute(grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gp.smem));
-    AB_LAUNCH_DEP(grad_kernel, dim3((unsigned)(p.job[0].chunks * gp.slices)), dim3(192), gp.smem, st, tmAct, tmSmall, tmAct,
-                  tmSmall, p);
+    AB_LAUNCH_CLUSTER(gp.sp.C, grad_kernel, dim3((unsigned)(p.job[0].chunks * slices)), dim3(192), gp.smem, st, tmAct, tmSmall, tmAct,
+                      tmSmall, p);
     AB_LAUNCH_OK();
     first = false;
-    const int nA = (int)(((int64_t)m * r / 4 + 255) / 256);
-    AB_LAUNCH_DEP(reduce_partials_kernel, dim3(nA), dim3(256), 0, st, static_cast<const float*>(w.pA), dA, m, nA,
-                  static_cast<const float*>(w.pA), static_cast<float*>(nullptr), 0, gp.slices, r, rp);
-    AB_LAUNCH_OK();
+    if (gp.sp.ncl > 1) {
+      const int nA = (int)(((int64_t)m * r / 4 + 255) / 256);
+      AB_LAUNCH_DEP(reduce_partials_kernel, dim3(nA), dim3(256), 0, st, static_cast<const float*>(w.pA), dA, m, nA,
+                    static_cast<const float*>(w.pA), static_cast<float*>(nullptr), 0, gp.sp.ncl, r, rp);
+      AB_LAUNCH_OK();
+    }
   }
   if (dB) {
     ConvGradPlan gp = conv_grad_plan(B, H, W, C, rp);
@@ -1433,15 +1501,18 @@ int conv_tc_backward(const void* x, const void* dY, const void* A, const void* B
     AB_TRY(make_tensor_map_nhwc(&tmX4, x, B, H, W, C, W, gp.bhk, gp.kb));
     AB_TRY(make_tensor_map_nhwc(&tmT4, w.dT, B, H, W, r, W, gp.bhk, gp.kb));
     p.B = B; p.H = H; p.W = W; p.C = C; p.r = rp; p.natoms = gp.natoms; p.ns = gp.ns; p.slot_bytes = gp.slot_bytes;
-    p.spi = gp.spi; p.kb = gp.kb; p.bhk = gp.bhk; p.box_rows = gp.box_rows; p.cpt = gp.cpt; p.slices = gp.slices;
-    p.slabs_per_slice = gp.slabs_per_slice; p.nslabs = gp.nslabs; p.partial = w.pB; p.status = w.status;
+    const int slices = gp.sp.C * gp.sp.ncl;
+    p.spi = gp.spi; p.kb = gp.kb; p.bhk = gp.bhk; p.box_rows = gp.box_rows; p.cpt = gp.cpt; p.slices = slices;
+    p.slabs_per_slice = gp.sp.per; p.nslabs = gp.nslabs; p.out = grad_out(gp.sp, w.pB, dB, 9 * C, r, true); p.status = w.status;
     AB_CUDA_OK(cudaFuncSetAttribute(conv_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gp.smem));
-    AB_LAUNCH_DEP(conv_grad_kernel, dim3((unsigned)(9 * gp.cpt * gp.slices)), dim3(192), gp.smem, st, tmX4, tmT4, p);
+    AB_LAUNCH_CLUSTER(gp.sp.C, conv_grad_kernel, dim3((unsigned)(9 * gp.cpt * slices)), dim3(192), gp.smem, st, tmX4, tmT4, p);
     AB_LAUNCH_OK();
-    const int nB = ((9 * C + 31) / 32) * ((r + 31) / 32);
-    AB_LAUNCH_DEP(reduce_partials_kernel, dim3(nB), dim3(256), 0, st, static_cast<const float*>(w.pB), static_cast<float*>(nullptr),
-                  0, 0, static_cast<const float*>(w.pB), dB, 9 * C, gp.slices, r, rp);
-    AB_LAUNCH_OK();
+    if (gp.sp.ncl > 1) {
+      const int nB = ((9 * C + 31) / 32) * ((r + 31) / 32);
+      AB_LAUNCH_DEP(reduce_partials_kernel, dim3(nB), dim3(256), 0, st, static_cast<const float*>(w.pB), static_cast<float*>(nullptr),
+                    0, 0, static_cast<const float*>(w.pB), dB, 9 * C, gp.sp.ncl, r, rp);
+      AB_LAUNCH_OK();
+    }
   }
   if (first) AB_CUDA_OK(cudaMemsetAsync(w.status, 0, sizeof(int), st));
   return AB_OK;
