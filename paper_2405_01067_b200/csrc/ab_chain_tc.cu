@@ -7,8 +7,8 @@
 //   backward: In = dY, F1 = A^T (r x m), F2 = B^T (n x r), Out = dX, S = dT   (A and B read as they lie)
 // grad_kernel: dA = dY^T T and dB^T = x^T dT are reductions over the rows; a CTA owns 256 output rows (a
 // slice of m or of n) and one slice of the N rows and streams 64-row slabs of both operands (both "MN-major": the reduction
-// index is the slow one in memory).  The slices of a tile form clusters, whose CTAs add their accumulators through
-// distributed shared memory in ascending order; where a tile has more than one cluster, reduce_partials_kernel adds those sums.
+// index is the slow one in memory).  Where a tile has several slices each leaves its sums in memory and
+// reduce_partials_kernel adds them in a fixed order.
 //
 // All operand tiles are TMA boxes of 64 bf16 (128 bytes) x rows with 128-byte swizzle.  Every mbarrier
 // wait gives up after about a second, raises AB_ERR_TIMEOUT in the status word and unwinds to the common
@@ -608,7 +608,7 @@ __device__ __forceinline__ void grad_mma_loop(Bars* bars, uint8_t* ring, int nk,
 // ---------------------------------------------------------------------------------------------
 // grad kernel: partial[slice][p][j] = sum_{k in slice} act[k][p] * small[k][j]
 // Where a tile's sums go: element (row, col) to dst[row * ld + col], or, transposed, to dst[col * ld + row].  A tile with
-// several clusters leaves one set of sums per cluster, `stride` elements apart.
+// several slices leaves one set of sums per slice, `stride` elements apart.
 struct GradOut {
   float* dst;
   int64_t ld, stride;
@@ -622,70 +622,70 @@ struct GradJob {
 struct GradParams {
   GradJob job[2];
   int r, natoms, ns, slot_bytes;
-  int slices, rows_per_slice;   // slices: CTAs per tile; rows_per_slice is a multiple of 64
+  int slices, rows_per_slice;   // rows_per_slice is a multiple of 64
   int N;
   int clear_status;
   int job0_independent;   // 1: job 0 reads nothing the kernel before this one in the stream writes (see grad_kernel)
   int* status;
 };
 
-// The end of both gradient kernels: 2 x 128 accumulator rows of r columns -> this CTA's shared memory -> sums over the CTAs
-// of the cluster, in ascending order, each CTA for its share of the rows -> global memory.  Every thread of the
-// CTA comes here, also after a wait that gave up (the outputs are then undefined, the status says so).
-// A row takes r + 4 floats: with r a multiple of 16 eight lanes' 16-byte accesses then fall into different banks.
-__device__ __forceinline__ void grad_finish(uint8_t* ring, uint32_t tmem_base, bool have, int r, int row0, int cluster_index,
-                                            const GradOut& o) {
-  namespace cg = cooperative_groups;
-  cg::cluster_group cluster = cg::this_cluster();
-  const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+// The end of both gradient kernels: 2 x 128 accumulator rows of r columns -> this CTA's shared memory -> global memory, two
+// rows per warp instruction (from the registers a warp instruction would touch 32 rows).  Every thread of the CTA
+// comes here, also after a wait that gave up (the outputs are then undefined, the status says so).
+// A row takes r + 4 floats of shared memory: with r a multiple of 16 eight lanes' 16-byte accesses then fall into different
+// banks.  Slices were also added inside clusters: through distributed shared memory the sums come at 10 to 15
+// bytes a cycle and SM, and 8-CTA clusters leave 20 SMs empty (convolution of the ResNet layer: 57.5 us against 22 us,
+// and 6 to 9 us for the separate reduction).
+__device__ __forceinline__ void grad_finish(uint8_t* ring, int ring_bytes, uint32_t tmem_base, bool have, int r, int row0,
+                                            int slice, const GradOut& o) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   float* tile = reinterpret_cast<float*>(ring);
-  const int ldt = r + 4, share = 128 / C;
-  float* dst = o.dst + (int64_t)cluster_index * o.stride;
-  for (int mt = 0; mt < 2 && row0 + 128 * mt < o.rows; ++mt) {
+  const int ldt = r + 4;
+  const int halves = 256 * ldt * 4 <= ring_bytes ? 2 : 1;      // accumulators per pass
+  float* dst = o.dst + (int64_t)slice * o.stride;
+  for (int m0 = 0; m0 < 2 && row0 + 128 * m0 < o.rows; m0 += halves) {
+    const int grow0 = row0 + 128 * m0;
+    int rows = o.rows - grow0;
+    if (rows > 128 * halves) rows = 128 * halves;
     if (warp >= 2) {
-      const int q = warp & 3, row = q * 32 + lane;
-      const uint32_t t = tmem_base + 256 * mt + ((uint32_t)(q * 32) << 16);
-      for (int c0 = 0; c0 < r; c0 += 16) {
-        float v[16];
-        if (have) tmem_ld16(t + c0, v);
-        else {
+      for (int h = 0; 128 * h < rows; ++h) {
+        const int q = warp & 3, row = 128 * h + q * 32 + lane;
+        const uint32_t t = tmem_base + 256 * (m0 + h) + ((uint32_t)(q * 32) << 16);
+        for (int c0 = 0; c0 < r; c0 += 64) {
+          uint32_t v[4][16];
+          if (have) {
 #pragma unroll
-          for (int i = 0; i < 16; ++i) v[i] = 0.f;
-        }
-        float4* d = reinterpret_cast<float4*>(tile + row * ldt + c0);
+            for (int g = 0; g < 4; ++g) if (c0 + 16 * g < r) tmem_ld16_nowait(t + c0 + 16 * g, v[g]);
+            tmem_wait_ld();
+          } else {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) d[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
-      }
-    }
-    if (C > 1) cluster.sync(); else __syncthreads();
-    const int groups = r >> 2;
-    for (int e = tid; e < share * groups; e += blockDim.x) {
-      const int lr = rank * share + e % share, c = (e / share) * 4;       // neighbouring threads: neighbouring rows
-      float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (C == 8) {
-        float4 v[8];
+            for (int g = 0; g < 4; ++g)
 #pragma unroll
-        for (int k = 0; k < 8; ++k) v[k] = *reinterpret_cast<const float4*>(cluster.map_shared_rank(tile, k) + lr * ldt + c);
-        s = v[0];
+              for (int i = 0; i < 16; ++i) v[g][i] = 0u;
+          }
+          uint4* d = reinterpret_cast<uint4*>(tile + row * ldt + c0);
 #pragma unroll
-        for (int k = 1; k < 8; ++k) { s.x += v[k].x; s.y += v[k].y; s.z += v[k].z; s.w += v[k].w; }
-      } else {
-        for (int k = 0; k < C; ++k) {
-          const float4 v = *reinterpret_cast<const float4*>((C > 1 ? cluster.map_shared_rank(tile, k) : tile) + lr * ldt + c);
-          s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+          for (int g = 0; g < 4; ++g)
+            if (c0 + 16 * g < r) {
+#pragma unroll
+              for (int i = 0; i < 4; ++i) d[4 * g + i] = make_uint4(v[g][4 * i], v[g][4 * i + 1], v[g][4 * i + 2], v[g][4 * i + 3]);
+            }
         }
       }
-      const int row = row0 + 128 * mt + lr;
-      if (row >= o.rows || c >= o.cols) continue;
-      if (!o.transposed) {
-        *reinterpret_cast<float4*>(dst + (int64_t)row * o.ld + c) = s;       // cols is a multiple of 4
-      } else {
-        float* d = dst + (int64_t)c * o.ld + row;
-        d[0] = s.x; d[o.ld] = s.y; d[2 * o.ld] = s.z; d[3 * o.ld] = s.w;
+    }
+    __syncthreads();
+    if (o.transposed) {              // neighbouring lanes take neighbouring rows
+      for (int c = warp; c < o.cols; c += 6)
+        for (int row = lane; row < rows; row += 32) dst[(int64_t)c * o.ld + grow0 + row] = tile[row * ldt + c];
+    } else {
+      for (int c = 4 * (lane & 15); c < o.cols; c += 64) {         // cols and ld are multiples of 4
+        float* d = dst + (int64_t)grow0 * o.ld + c;
+#pragma unroll 4
+        for (int row = 2 * warp + (lane >> 4); row < rows; row += 12)
+          *reinterpret_cast<float4*>(d + (int64_t)row * o.ld) = *reinterpret_cast<const float4*>(tile + row * ldt + c);
       }
     }
-    if (C > 1) cluster.sync(); else __syncthreads();     // the tile is reused, or the CTA leaves
+    __syncthreads();
   }
 }
 
@@ -701,7 +701,6 @@ grad_kernel(const __grid_constant__ CUtensorMap tmAct0, const __grid_constant__ 
 
   // which job, which 128-row chunk of its output, which slice of the N rows
   int tile = blockIdx.x;
-  const int cluster_size = (int)cooperative_groups::this_cluster().num_blocks();
   const int slice = tile % p.slices;
   tile /= p.slices;
   int jb = 0;
@@ -766,7 +765,7 @@ grad_kernel(const __grid_constant__ CUtensorMap tmAct0, const __grid_constant__ 
     __syncthreads();
   }
   tc_fence_after();
-  grad_finish(ring, tmem_base, nk > 0 && !failed, p.r, chunk * 256, slice / cluster_size, p.job[jb].out);
+  grad_finish(ring, p.ns * p.slot_bytes, tmem_base, nk > 0 && !failed, p.r, chunk * 256, slice, p.job[jb].out);
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
@@ -802,7 +801,6 @@ conv_grad_kernel(const __grid_constant__ CUtensorMap tmX4, const __grid_constant
   Bars* bars = reinterpret_cast<Bars*>(ring + (size_t)p.ns * p.slot_bytes);
   const int warp = (int)uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
   int tile = blockIdx.x;
-  const int cluster_size = (int)cooperative_groups::this_cluster().num_blocks();
   const int slice = tile % p.slices;
   const int chunk = tile / p.slices;
   const int tap = chunk / p.cpt, cwin = (chunk - tap * p.cpt) * 256;
@@ -820,9 +818,12 @@ conv_grad_kernel(const __grid_constant__ CUtensorMap tmX4, const __grid_constant
     tma_prefetch_desc(&tmX4); tma_prefetch_desc(&tmT4);
   }
   {
-    uint4* z = reinterpret_cast<uint4*>(ring);
-    const int n16 = p.ns * p.slot_bytes / 16;
-    for (int i = threadIdx.x; i < n16; i += blockDim.x) z[i] = make_uint4(0u, 0u, 0u, 0u);
+    // a box has box_rows of a tile's 64 rows: the rest stay zero
+    const int per = (64 - p.box_rows) * 8, n16 = p.ns * (p.slot_bytes / 8192) * per;
+    for (int i = threadIdx.x; i < n16; i += blockDim.x) {
+      const int t = i / per;
+      reinterpret_cast<uint4*>(ring + (size_t)t * 8192 + p.box_rows * 128)[i - t * per] = make_uint4(0u, 0u, 0u, 0u);
+    }
     fence_proxy_async_smem();
   }
   if (warp == 1) tmem_alloc(&bars->tmem_base, kTmemCols);
@@ -869,7 +870,7 @@ conv_grad_kernel(const __grid_constant__ CUtensorMap tmX4, const __grid_constant
   GradOut o = p.out;
   o.dst += p.out.transposed ? (int64_t)tap * p.C : (int64_t)tap * p.C * p.out.ld;
   o.rows = p.C;
-  grad_finish(ring, tmem_base, nk > 0 && !failed, p.r, cwin, slice / cluster_size, o);
+  grad_finish(ring, p.ns * p.slot_bytes, tmem_base, nk > 0 && !failed, p.r, cwin, slice, o);
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
@@ -878,49 +879,81 @@ conv_grad_kernel(const __grid_constant__ CUtensorMap tmX4, const __grid_constant
   }
 }
 
-// Sums the clusters' partials in ascending order (fixed order: identical bits every run).
-//   blocks [0, nA):  dA[p][j]  = sum_s pA[s][p][j]            (float4 per thread)
-//   blocks [nA, ..): dB[j][q]  = sum_s pB[s][q][j]            (32 x 32 tiles transposed through shared memory)
-__global__ void __launch_bounds__(256)
+// Sums the slices' partials in a fixed order (identical bits every run).
+//   blocks [0, nA):  dA[p][j]  = sum_s pA[s][p][j]
+//   blocks [nA, ..): dB[j][q]  = sum_s pB[s][q][j]            (tiles transposed through shared memory)
+// The partials lie in L2 and the kernel waits for them: a thread that walks the slices alone makes slices / 4 trips of
+// about 800 cycles (104 slices of 256 x 128: 38 us).  So G threads share an element (4 columns), each sums every G-th
+// slice, and the first adds the G sums (6 us).
+constexpr int kReduceT = 256;
+__host__ __device__ inline int reduce_groups(int slices) { return slices >= 24 ? 8 : slices >= 12 ? 4 : slices >= 6 ? 2 : 1; }
+// rows x float4 columns of a transposed tile: 256 / G of them, rows as long as a 128-byte line as far as they go
+__host__ __device__ inline int reduce_rows(int G) { return G == 8 ? 16 : 32; }
+__device__ __forceinline__ float4 sum_slices(const float* src, int64_t stride, int first, int slices, int step) {
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  int k = first;
+  for (; k + 7 * step < slices; k += 8 * step) {
+    float4 v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = __ldcg(reinterpret_cast<const float4*>(src + (k + i * step) * stride));
+#pragma unroll
+    for (int i = 0; i < 8; ++i) { acc.x += v[i].x; acc.y += v[i].y; acc.z += v[i].z; acc.w += v[i].w; }
+  }
+#pragma unroll 4
+  for (; k < slices; k += step) {
+    const float4 v = __ldcg(reinterpret_cast<const float4*>(src + k * stride));
+    acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
+  }
+  return acc;
+}
+__global__ void __launch_bounds__(kReduceT)
 reduce_partials_kernel(const float* __restrict__ pA, float* __restrict__ dA, int PA, int nA,
                        const float* __restrict__ pB, float* __restrict__ dB, int PB, int slices, int r, int rp) {
-  // r: columns of the results; rp: row length of the partials (r rounded up to 16)
+  // r: columns of the results, a multiple of 4; rp: row length of the partials (r rounded up to 16)
+  __shared__ float4 part[kReduceT];
+  __shared__ float turned[32][33];
+  const int G = reduce_groups(slices), items = kReduceT / G;
+  const int g = threadIdx.x / items, e = threadIdx.x - g * items;
+  const bool first = (int)blockIdx.x < nA;
+  const int r4 = r >> 2, rows = reduce_rows(G), c4 = items / rows;
+  const int tiles_j = (r4 + c4 - 1) / c4, t = (int)blockIdx.x - nA;
+  int64_t row;
+  int col;
+  int64_t i4 = 0;
+  if (first) {
+    i4 = (int64_t)blockIdx.x * items + e;
+    row = i4 / r4;
+    col = 4 * (int)(i4 - row * r4);
+  } else {
+    row = (int64_t)(t / tiles_j) * rows + e / c4;
+    col = 4 * ((t % tiles_j) * c4 + e % c4);
+  }
+  const bool live = col < r && row < (first ? PA : PB);
   dep_wait();
   dep_launch();
-  if ((int)blockIdx.x < nA) {
-    const int64_t total4 = (int64_t)PA * r / 4;
-    const int64_t i4 = (int64_t)blockIdx.x * 256 + threadIdx.x;
-    if (i4 >= total4) return;
-    const int64_t prow = (i4 * 4) / r;
-    const int col = (int)((i4 * 4) % r);
-    const float* src = pA + prow * rp + col;
-    const int64_t slice_stride = (int64_t)PA * rp;
-    float4 acc = *reinterpret_cast<const float4*>(src);
-#pragma unroll 4
-    for (int s = 1; s < slices; ++s) {
-      const float4 v = *reinterpret_cast<const float4*>(src + s * slice_stride);
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (live) acc = sum_slices((first ? pA : pB) + row * rp + col, (int64_t)(first ? PA : PB) * rp, g, slices, G);
+  part[threadIdx.x] = acc;
+  __syncthreads();
+  if (g == 0) {
+    for (int i = 1; i < G; ++i) {
+      const float4 v = part[i * items + e];
       acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
     }
-    reinterpret_cast<float4*>(dA)[i4] = acc;
-    return;
+    if (first) {
+      if (live) reinterpret_cast<float4*>(dA)[i4] = acc;
+    } else {
+      float* d = &turned[e / c4][4 * (e % c4)];
+      d[0] = acc.x; d[1] = acc.y; d[2] = acc.z; d[3] = acc.w;
+    }
   }
-  __shared__ float tile[32][33];
-  const int t = blockIdx.x - nA;
-  const int tiles_j = (r + 31) / 32;
-  const int q0 = (t / tiles_j) * 32, j0 = (t % tiles_j) * 32;
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  for (int i = ty; i < 32; i += 8) {
-    const int q = q0 + i, j = j0 + tx;
-    float acc = 0.f;
-    if (q < PB && j < r)
-#pragma unroll 4
-      for (int s = 0; s < slices; ++s) acc += pB[((int64_t)s * PB + q) * rp + j];
-    tile[i][tx] = acc;
-  }
+  if (first) return;
   __syncthreads();
-  for (int i = ty; i < 32; i += 8) {
-    const int j = j0 + i, q = q0 + tx;
-    if (j < r && q < PB) dB[(int64_t)j * PB + q] = tile[tx][i];
+  const int64_t q0 = (int64_t)(t / tiles_j) * rows;
+  const int j0 = (t % tiles_j) * c4 * 4;
+  for (int i = threadIdx.x; i < rows * c4 * 4; i += kReduceT) {
+    const int j = i / rows, q = i - j * rows;
+    if (j0 + j < r && q0 + q < PB) dB[(int64_t)(j0 + j) * PB + q0 + q] = turned[q][j];
   }
 }
 
@@ -943,33 +976,19 @@ __global__ void bounded_wait_selftest_kernel(int* status, unsigned long long lim
 // Launch with programmatic stream serialisation (see dep_wait): only for kernels that call dep_wait()
 // before their first access to global memory.
 template <typename... KArgs, typename... Args>
-cudaError_t launch_dep_cluster(int cluster, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                               Args&&... args) {
+cudaError_t launch_dep(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute at[2];
+  cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
-  at[1].id = cudaLaunchAttributeClusterDimension;
-  at[1].val.clusterDim.x = cluster; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
   cfg.attrs = at;
-  cfg.numAttrs = cluster > 1 ? 2 : 1;
+  cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
-template <typename... KArgs, typename... Args>
-cudaError_t launch_dep(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
-  return launch_dep_cluster(1, kernel, grid, block, smem, st, std::forward<Args>(args)...);
-}
-#define AB_LAUNCH_CLUSTER(...)                             \
-  do {                                                     \
-    if (launch_dep_cluster(__VA_ARGS__) != cudaSuccess) {  \
-      cudaGetLastError();                                  \
-      return AB_ERR_CUDA;                                  \
-    }                                                      \
-  } while (0)
 #define AB_LAUNCH_DEP(...)                         \
   do {                                             \
     if (launch_dep(__VA_ARGS__) != cudaSuccess) {  \
@@ -1051,25 +1070,22 @@ ChainPlan chain_plan(int rp, int max_blocks, bool f1_mn) {
   return pl;
 }
 
-// How the slabs of a gradient reduction are dealt: clusters of C CTAs, ncl clusters per 256-row tile, per slabs per CTA.  The
-// split with the least time by what was measured: about 0.7 us a slab with the device full, 3 us to fill and empty a CTA, 4 us
-// for a reduction launch and its traffic at 4 TB/s; resident clusters of 8 / 4 / 2 / 1 CTAs: 16 / 36 / 74 / one per SM.
-struct GradSplit { int C, ncl, per; };
+// How the slabs of a gradient reduction are dealt: slices per 256-row tile, slabs per slice.  The split with the least time by
+// what was measured: 0.55 us a slab, 5 us to fill and empty a CTA and to write its sums; several slices
+// take a reduction launch of 3 us that reads them all at 3 TB/s.  Few slabs thus go to fewer CTAs than there are SMs.
+struct GradSplit { int slices, per; };
 GradSplit grad_split(int64_t slabs, int tiles, int rp) {
   const int sms = sm_count() > 0 ? sm_count() : 1;
-  GradSplit best = {1, 1, (int)slabs};
+  GradSplit best = {1, (int)slabs};
   double best_t = 1e30;
-  for (int C = 1; C <= 8; C *= 2) {
-    if (C > slabs) break;
-    int resident = C == 8 ? sms / 9 : C == 4 ? sms / 4 - 1 : sms / C;
-    if (resident < 1) resident = 1;
-    for (int ncl = 1; ncl <= 32 && (int64_t)C * ncl <= slabs; ++ncl) {
-      const int64_t per = (slabs + (int64_t)C * ncl - 1) / ((int64_t)C * ncl);
-      const int waves = (tiles * ncl + resident - 1) / resident;
-      double t = waves * (0.7 * (double)per + 3.0);
-      if (ncl > 1) t += 4.0 + 2.0 * ncl * tiles * 256.0 * rp * 4.0 / 4e6;
-      if (t < best_t) { best_t = t; best = {C, ncl, (int)per}; }
-    }
+  for (int want = 1; want <= sms && want <= slabs; ++want) {
+    const int64_t per = (slabs + want - 1) / want;
+    const int slices = (int)((slabs + per - 1) / per);
+    if (slices != want) continue;
+    const int waves = (tiles * slices + sms - 1) / sms;
+    double t = waves * (0.55 * (double)per + 5.0);
+    if (slices > 1) t += 3.0 + (double)slices * tiles * 256.0 * rp * 4.0 / 3e6;
+    if (t < best_t) { best_t = t; best = {slices, (int)per}; }
   }
   return best;
 }
@@ -1083,19 +1099,24 @@ GradPlan grad_plan(int64_t N, int m, int n, int r) {
   const int fixed = (int)sizeof(Bars) + 1024;
   pl.ns = (kSmemLimit - fixed) / pl.slot_bytes;
   if (pl.ns > kMaxStages) pl.ns = kMaxStages;
-  pl.smem = (size_t)fixed + (size_t)pl.ns * pl.slot_bytes;      // the ring also holds 128 x (r + 4) sums: at most 133 KB of it
+  pl.smem = (size_t)fixed + (size_t)pl.ns * pl.slot_bytes;      // the ring also takes 128 x (r + 4) sums: at most 133 KB of it
   pl.sp = grad_split((N + 63) / 64, tiles256(m) + tiles256(n), pad16(r));
   return pl;
 }
-// floats of the clusters' partial sums of an output of `rows` rows
-size_t grad_partial(const GradSplit& s, int64_t rows, int rp) { return s.ncl > 1 ? (size_t)s.ncl * rows * rp : 0; }
+// floats of the slices' sums of an output of `rows` rows, where there is more than one slice
+size_t grad_partial(const GradSplit& s, int64_t rows, int rp) { return s.slices > 1 ? (size_t)s.slices * rows * rp : 0; }
 GradOut grad_out(const GradSplit& sp, float* partial, float* dst, int rows, int r, bool transposed) {
   GradOut o;
   const int rp = pad16(r);
   o.rows = rows;
-  if (sp.ncl > 1) { o.dst = partial; o.ld = rp; o.stride = (int64_t)rows * rp; o.cols = rp; o.transposed = 0; }
+  if (sp.slices > 1) { o.dst = partial; o.ld = rp; o.stride = (int64_t)rows * rp; o.cols = rp; o.transposed = 0; }
   else { o.dst = dst; o.ld = transposed ? rows : r; o.stride = 0; o.cols = r; o.transposed = transposed ? 1 : 0; }
   return o;
+}
+struct ReduceGrid { int a, b; };          // blocks of reduce_partials_kernel
+ReduceGrid reduce_grid(const GradSplit& sp, int64_t rowsA, int64_t rowsB, int r) {
+  const int G = reduce_groups(sp.slices), items = kReduceT / G, rows = reduce_rows(G), c4 = items / rows, r4 = r / 4;
+  return {(int)((rowsA * r4 + items - 1) / items), (int)((rowsB + rows - 1) / rows) * ((r4 + c4 - 1) / c4)};
 }
 
 struct BwdWs { int* status; bf16 *T, *dT; float *pA, *pB; size_t bytes; };
@@ -1311,7 +1332,7 @@ int chain_tc_backward(const void* x, const void* dY, const void* A, const void* 
   }
   if (dA || dB) {
     const GradPlan gp = grad_plan(N, m, n, r);     // the same split whichever is asked for: the same bits
-    const int rp = pad16(r), slices = gp.sp.C * gp.sp.ncl;
+    const int rp = pad16(r), slices = gp.sp.slices;
     GradParams p;
     std::memset(&p, 0, sizeof(p));
     CUtensorMap tmAct[2], tmSmall[2];
@@ -1334,13 +1355,13 @@ int chain_tc_backward(const void* x, const void* dY, const void* A, const void* 
     p.job0_independent = (after_chain && dA) ? 1 : 0;   // job 0 is the dA job whenever dA is asked for
     AB_CUDA_OK(cudaFuncSetAttribute(grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gp.smem));
     const unsigned grid = (unsigned)((p.job[0].chunks + p.job[1].chunks) * slices);
-    AB_LAUNCH_CLUSTER(gp.sp.C, grad_kernel, dim3(grid), dim3(192), gp.smem, st, tmAct[0], tmSmall[0], tmAct[1], tmSmall[1], p);
+    AB_LAUNCH_DEP(grad_kernel, dim3(grid), dim3(192), gp.smem, st, tmAct[0], tmSmall[0], tmAct[1], tmSmall[1], p);
     AB_LAUNCH_OK();
-    if (gp.sp.ncl > 1) {
-      const int nA = dA ? (int)(((int64_t)m * r / 4 + 255) / 256) : 0;
-      const int nB = dB ? ((n + 31) / 32) * ((r + 31) / 32) : 0;
-      AB_LAUNCH_DEP(reduce_partials_kernel, dim3(nA + nB), dim3(256), 0, st, static_cast<const float*>(w.pA), dA, m, nA,
-                 static_cast<const float*>(w.pB), dB, n, gp.sp.ncl, r, rp);
+    if (slices > 1) {
+      const ReduceGrid rg = reduce_grid(gp.sp, dA ? m : 0, dB ? n : 0, r);
+      const int nA = rg.a, nB = rg.b;
+      AB_LAUNCH_DEP(reduce_partials_kernel, dim3(nA + nB), dim3(kReduceT), 0, st, static_cast<const float*>(w.pA), dA, m, nA,
+                 static_cast<const float*>(w.pB), dB, n, slices, r, rp);
       AB_LAUNCH_OK();
     }
     first = false;
@@ -1477,19 +1498,19 @@ int conv_tc_backward(const void* x, const void* dY, const void* A, const void* B
     AB_TRY(make_map(&tmSmall, T, (uint64_t)N, r, r, 64, 64));
     p.job[0].chunks = tiles256(m); p.job[0].out = grad_out(gp.sp, w.pA, dA, m, r, false);
     p.job[1] = p.job[0]; p.job[1].chunks = 0;
-    const int slices = gp.sp.C * gp.sp.ncl;
+    const int slices = gp.sp.slices;
     p.r = rp; p.natoms = gp.natoms; p.ns = gp.ns; p.slot_bytes = gp.slot_bytes;
     p.slices = slices; p.rows_per_slice = gp.sp.per * 64; p.N = (int)N; p.clear_status = first ? 1 : 0;
     p.status = w.status; p.job0_independent = 0;
     AB_CUDA_OK(cudaFuncSetAttribute(grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gp.smem));
-    AB_LAUNCH_CLUSTER(gp.sp.C, grad_kernel, dim3((unsigned)(p.job[0].chunks * slices)), dim3(192), gp.smem, st, tmAct, tmSmall, tmAct,
+    AB_LAUNCH_DEP(grad_kernel, dim3((unsigned)(p.job[0].chunks * slices)), dim3(192), gp.smem, st, tmAct, tmSmall, tmAct,
                       tmSmall, p);
     AB_LAUNCH_OK();
     first = false;
-    if (gp.sp.ncl > 1) {
-      const int nA = (int)(((int64_t)m * r / 4 + 255) / 256);
-      AB_LAUNCH_DEP(reduce_partials_kernel, dim3(nA), dim3(256), 0, st, static_cast<const float*>(w.pA), dA, m, nA,
-                    static_cast<const float*>(w.pA), static_cast<float*>(nullptr), 0, gp.sp.ncl, r, rp);
+    if (slices > 1) {
+      const int nA = reduce_grid(gp.sp, m, 0, r).a;
+      AB_LAUNCH_DEP(reduce_partials_kernel, dim3(nA), dim3(kReduceT), 0, st, static_cast<const float*>(w.pA), dA, m, nA,
+                    static_cast<const float*>(w.pA), static_cast<float*>(nullptr), 0, slices, r, rp);
       AB_LAUNCH_OK();
     }
   }
@@ -1501,16 +1522,16 @@ int conv_tc_backward(const void* x, const void* dY, const void* A, const void* B
     AB_TRY(make_tensor_map_nhwc(&tmX4, x, B, H, W, C, W, gp.bhk, gp.kb));
     AB_TRY(make_tensor_map_nhwc(&tmT4, w.dT, B, H, W, r, W, gp.bhk, gp.kb));
     p.B = B; p.H = H; p.W = W; p.C = C; p.r = rp; p.natoms = gp.natoms; p.ns = gp.ns; p.slot_bytes = gp.slot_bytes;
-    const int slices = gp.sp.C * gp.sp.ncl;
+    const int slices = gp.sp.slices;
     p.spi = gp.spi; p.kb = gp.kb; p.bhk = gp.bhk; p.box_rows = gp.box_rows; p.cpt = gp.cpt; p.slices = slices;
     p.slabs_per_slice = gp.sp.per; p.nslabs = gp.nslabs; p.out = grad_out(gp.sp, w.pB, dB, 9 * C, r, true); p.status = w.status;
     AB_CUDA_OK(cudaFuncSetAttribute(conv_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gp.smem));
-    AB_LAUNCH_CLUSTER(gp.sp.C, conv_grad_kernel, dim3((unsigned)(9 * gp.cpt * slices)), dim3(192), gp.smem, st, tmX4, tmT4, p);
+    AB_LAUNCH_DEP(conv_grad_kernel, dim3((unsigned)(9 * gp.cpt * slices)), dim3(192), gp.smem, st, tmX4, tmT4, p);
     AB_LAUNCH_OK();
-    if (gp.sp.ncl > 1) {
-      const int nB = ((9 * C + 31) / 32) * ((r + 31) / 32);
-      AB_LAUNCH_DEP(reduce_partials_kernel, dim3(nB), dim3(256), 0, st, static_cast<const float*>(w.pB), static_cast<float*>(nullptr),
-                    0, 0, static_cast<const float*>(w.pB), dB, 9 * C, gp.sp.ncl, r, rp);
+    if (slices > 1) {
+      const int nB = reduce_grid(gp.sp, 0, 9 * (int64_t)C, r).b;
+      AB_LAUNCH_DEP(reduce_partials_kernel, dim3(nB), dim3(kReduceT), 0, st, static_cast<const float*>(w.pB), static_cast<float*>(nullptr),
+                    0, 0, static_cast<const float*>(w.pB), dB, 9 * C, slices, r, rp);
       AB_LAUNCH_OK();
     }
   }
