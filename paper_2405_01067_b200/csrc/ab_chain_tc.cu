@@ -1210,13 +1210,36 @@ int launch_chain_ex(const ChainLaunch& L, cudaStream_t st) {
   return AB_OK;
 }
 
+// Whether the chain runs as two products by tiles.  The fused kernel takes every row through whole factors on one SM: with
+// few rows that is a long walk on few SMs, and S in memory costs next to nothing.  Measured (us, fused / by tiles,
+// 768 -> 192 -> 3072): 64 rows 21.8 / 8.5, 6173 26.2 / 17.4, 8800 26.5 / 23.1, 10500 28.7 / 32.5; 776 -> 120 -> 1000: 64 rows
+// 14.2 / 8.3, 8800 20.0 / 14.5, 25088 30.7 / 34.4: hence up to one 128-row block for every two SMs.  Factors of a few tiles
+// are no long walk (256 -> 32 -> 256: 5.9 / 6.9).  The first product alone (us, chain kernel / tiles): K 3072 12608 rows
+// 24.1 / 17.0, 25088 33.2 / 44.7; K 256 25088 rows 6.3 / 4.7, 50432 9.2 / 6.1.
+bool by_tiles(int64_t N, int K1, int r, int P) {
+  const int64_t blocks = (N + 127) / 128;
+  const int sms = sm_count();
+  if (P == 0) return K1 <= 512 || 3 * blocks <= 2 * sms;
+  const int walk = (K1 + 63) / 64 + (P + kChunk - 1) / kChunk * ((r + 63) / 64);
+  return 2 * blocks <= sms && walk > 6;
+}
+
 // S = In F1^T (saved to Sg if not null), Out = S F2^T (skipped if Out is null).
 // f_mn = false: F1 is given as r x K1 (row stride ldF1) and F2 as P x r (row stride ldF2);
 // f_mn = true : F1 is given transposed, K1 x r, and F2 transposed, r x P (the factors A and B as they lie in
 //               memory when the chain runs backwards).
+// P is given even where Out is not wanted: which kernels run, and with that the bits of S, depends on the shape alone.
+// scratch: N x r for S where Sg is null; without it the fused kernel runs.
 int launch_chain(const void* In, int64_t N, int K1, const void* F1, int ldF1, const void* F2, int ldF2, int P,
-                 bool f_mn, void* Out, void* Sg, int r, int* status, bool clear_status, cudaStream_t st,
+                 bool f_mn, void* Out, void* Sg, void* scratch, int r, int* status, bool clear_status, cudaStream_t st,
                  bool stall_selftest = false, unsigned long long wait_ns = kWaitLimitNs) {
+  void* S = Sg ? Sg : scratch;
+  if (!stall_selftest && S && by_tiles(N, K1, r, P)) {
+    const TileProduct first = {In, N, K1, F1, ldF1, f_mn, S, r}, second = {S, N, r, F2, ldF2, f_mn, Out, P};
+    AB_TRY(tile_product(first, clear_status, status, st));
+    if (Out && P > 0) AB_TRY(tile_product(second, false, status, st));
+    return AB_OK;
+  }
   ChainLaunch L;
   L.In = In; L.N = N; L.K1 = K1; L.F1 = F1; L.ldF1 = ldF1; L.f1_rows = 0; L.f1_cols = 0; L.F2 = F2; L.ldF2 = ldF2; L.P = P;
   L.f_mn = f_mn; L.Out = Out; L.Sg = Sg; L.s_ld = r; L.s_cols = r; L.r = r; L.cv = nullptr; L.status = status;
@@ -1246,7 +1269,7 @@ int chain_stall_selftest(void* ws, size_t ws_bytes, unsigned limit_us, cudaStrea
   void* F1 = base + 256 + 65536;         // 16 x 64
   void* F2 = base + 256 + 2 * 65536;     // 64 x 16
   void* Out = base + 256 + 3 * 65536;    // 256 x 64
-  return launch_chain(In, 256, 64, F1, 64, F2, 16, 64, false, Out, nullptr, 16, status, true, st, true,
+  return launch_chain(In, 256, 64, F1, 64, F2, 16, 64, false, Out, nullptr, nullptr, 16, status, true, st, true,
                       (unsigned long long)limit_us * 1000ull);
 }
 
@@ -1291,7 +1314,7 @@ bool chain_tc_supported(int64_t N, int m, int n, int r, int ldA, int ldB, int dt
   return chain_plan(pad16(r), 1, false).ok && chain_plan(pad16(r), 1, true).ok;
 }
 
-size_t chain_tc_forward_ws(int64_t, int, int, int) { return 256; }
+size_t chain_tc_forward_ws(int64_t N, int, int, int r) { return 256 + align_up((size_t)N * r * sizeof(bf16), 256); }
 size_t chain_tc_backward_ws(int64_t N, int m, int n, int r) {
   if (r % 8 != 0 || r < 8 || r > 256) return 0;
   return bwd_ws(nullptr, N, m, n, r).bytes;
@@ -1303,7 +1326,9 @@ int chain_tc_forward(const void* x, const void* A, const void* B, void* y, void*
   if (!ws || ws_bytes < 256) return AB_ERR_WORKSPACE;
   if (T_save && !aligned(T_save, 16)) return AB_ERR_INVALID_ARG;
   int* status = static_cast<int*>(ws);
-  return launch_chain(x, N, n, B, ldB, A, ldA, m, false, y, T_save, r, status, true, st);
+  // S has room behind the status word in a workspace of the size that was asked for
+  void* scratch = ws_bytes >= chain_tc_forward_ws(N, m, n, r) ? static_cast<char*>(ws) + 256 : nullptr;
+  return launch_chain(x, N, n, B, ldB, A, ldA, m, false, y, T_save, scratch, r, status, true, st);
 }
 
 int chain_tc_backward(const void* x, const void* dY, const void* A, const void* B,
@@ -1320,13 +1345,13 @@ int chain_tc_backward(const void* x, const void* dY, const void* A, const void* 
   bool after_chain = false;   // the dT/dX chain kernel is the launch right before the gradient kernel
   const bf16* T = static_cast<const bf16*>(T_saved);
   if (dA && !T) {   // recompute T = x B^T (first product only)
-    AB_TRY(launch_chain(x, N, n, B, ldB, nullptr, 0, 0, false, nullptr, w.T, r, w.status, first, st));
+    AB_TRY(launch_chain(x, N, n, B, ldB, A, ldA, m, false, nullptr, w.T, nullptr, r, w.status, first, st));
     first = false;
     T = w.T;
   }
   if (dX || dB) {
     // dT = dY A (kept for dB), dX = dT B: the chain with F1 = A^T and F2 = B^T, i.e. A and B as they lie
-    AB_TRY(launch_chain(dY, N, m, A, ldA, B, ldB, n, true, dX, dB ? w.dT : nullptr, r, w.status, first, st));
+    AB_TRY(launch_chain(dY, N, m, A, ldA, B, ldB, n, true, dX, dB ? w.dT : nullptr, w.dT, r, w.status, first, st));
     first = false;
     after_chain = true;
   }
@@ -1475,7 +1500,7 @@ int conv_tc_backward(const void* x, const void* dY, const void* A, const void* B
     T = w.T;
   }
   if (dX || dB) {
-    AB_TRY(launch_chain(dY, N, m, A, ldA, nullptr, 0, 0, true, nullptr, w.dT, r, w.status, first, st));   // dT = dY A
+    AB_TRY(launch_chain(dY, N, m, A, ldA, nullptr, 0, 0, true, nullptr, w.dT, nullptr, r, w.status, first, st));   // dT = dY A
     first = false;
   }
   if (dX) {

@@ -161,6 +161,11 @@ int chain_tc_backward(const void* x, const void* dY, const void* A, const void* 
                       int64_t N, int m, int n, int r, int ldA, int ldB,
                       void* ws, size_t ws_bytes, cudaStream_t st);
 
+// ---- bf16 products by tiles (ab_tile_tc.cu) ------------------------------------------------------
+// D = X F^T: X is N x K, D is N x P (both without gaps), F is P x K, or, f_mn, K x P; row stride ldF.  K, P, ldF multiples of 8.
+struct TileProduct { const void* X; int64_t N; int K; const void* F; int ldF; bool f_mn; void* D; int P; };
+int tile_product(const TileProduct& t, bool clear_status, int* status, cudaStream_t st);
+
 // ---- small fp32 products and layers (ab_layer_small.cu) -----------------------------------------
 // C[p][q] = sum over k of U[p * u_p + k * u_k] V[q * v_q + k * v_k], row stride ldc; sums of 16 products in fp32, those
 // in fp64.  One or two products with the same reduction length in one launch; status: cleared if not null.
