@@ -66,16 +66,30 @@ __device__ __forceinline__ bool split_warp_wait(SplitBars* b, uint64_t* bar, uin
   return __all_sync(0xffffffffu, ok);
 }
 
-// A consumer warp's place in the ring of tile records.
-struct RecordReader {
+// A consumer warp's walk over its CTA's tiles.  Several problems: records handed round by the finder warp.  One problem: it lies
+// in the kernel's parameters and a tile follows from its number, so no warp waits for another (through records 3300 cycles
+// passed from the start to the first load, as many as two slabs take; 768 x 768 x 192 11.4 -> 7.9 us, of it also
+// the epilogue without scaling code, 4300 -> 2200 cycles).
+struct TileAt { const SplitGemm* P; int m0, n0; };
+template <bool kOne, int BN>
+struct TileReader {
   int slot = 0, ph = 0;
-  // the next record, or null after the last one (or when a wait gave up)
-  __device__ __forceinline__ const TileRecord* next(SplitBars* b, int* status) {
-    if (!split_warp_wait(b, &b->rec_full[slot], ph, status)) return nullptr;
-    const TileRecord* r = &b->rec[slot];
-    return __any_sync(0xffffffffu, r->last) ? nullptr : r;
+  // the next tile; P is null after the last one (or when a wait gave up)
+  __device__ __forceinline__ TileAt next(SplitBars* b, const SplitGemm* probs, int ntiles, int* status) {
+    if constexpr (kOne) {
+      const int tile = (int)blockIdx.x + slot++ * (int)gridDim.x;
+      if (tile >= ntiles) return {nullptr, 0, 0};
+      const int tn = (probs->N + BN - 1) / BN, tm = tile / tn;
+      return {probs, tm * kM, (tile - tm * tn) * BN};
+    } else {
+      if (!split_warp_wait(b, &b->rec_full[slot], ph, status)) return {nullptr, 0, 0};
+      const TileRecord* r = &b->rec[slot];
+      if (__any_sync(0xffffffffu, r->last)) return {nullptr, 0, 0};
+      return {&r->P, r->m0, r->n0};
+    }
   }
   __device__ __forceinline__ void done(SplitBars* b) {     // the record has been read
+    if constexpr (kOne) return;
     __syncwarp();
     if ((threadIdx.x & 31) == 0) mbar_arrive(&b->rec_empty[slot]);
     if (++slot == kRing) { slot = 0; ph ^= 1; }
@@ -198,8 +212,8 @@ __device__ __forceinline__ void store_slab(const OperandSlab<kRows, kBf16>& s, u
   }
 }
 
-template <int BN, bool kBf16>
-__device__ __forceinline__ void gemm_split_body(const SplitGemm* probs, int nprobs, int ntiles, int* status, bool clear_status) {
+template <int BN, bool kBf16, bool kOne>
+__device__ __forceinline__ void gemm_split_body(const SplitGemm* probs, int nprobs, int ntiles, int* status) {
   using C = Cfg<BN, kBf16>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -219,10 +233,10 @@ __device__ __forceinline__ void gemm_split_body(const SplitGemm* probs, int npro
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *reinterpret_cast<volatile uint32_t*>(&bars->tmem_base);
-  dep_wait();
-  dep_launch();
-  // a wait gives up only after about a second: this cannot wipe a raised error
-  if (clear_status && blockIdx.x == 0 && tid == 0) atomicExch(status, 0);
+  if constexpr (!kOne) {       // one problem: each role finds its first tile before it waits
+    dep_wait();
+    dep_launch();
+  }
 
   if (warp < kConvWarps) {
     // ------------------------------------------------------------ converters
@@ -231,24 +245,26 @@ __device__ __forceinline__ void gemm_split_body(const SplitGemm* probs, int npro
     using SB = OperandSlab<BN, kBf16>;
     OperandCursor<kM, kBf16> ca;
     OperandCursor<BN, kBf16> cb;
-    SA a;
-    SB b;
-    RecordReader rd;
+    TileReader<kOne, BN> rd;
     int K = 0, k0 = 0, slot = 0, ph = 1;
     auto open = [&]() -> bool {
-      const TileRecord* r = rd.next(bars, status);
-      if (!r) return false;
-      ca.start(r->P.A, r->P.lda, r->P.a_mn, r->m0, r->P.M, tid);
-      cb.start(r->P.B, r->P.ldb, r->P.b_mn, r->n0, r->P.N, tid);
-      K = r->P.K;
+      const TileAt t = rd.next(bars, probs, ntiles, status);
+      if (!t.P) return false;
+      ca.start(t.P->A, t.P->lda, t.P->a_mn, t.m0, t.P->M, tid);
+      cb.start(t.P->B, t.P->ldb, t.P->b_mn, t.n0, t.P->N, tid);
+      K = t.P->K;
       k0 = 0;
       rd.done(bars);
       return true;
     };
-    bool more = open();
-    if (more) { ca.load(a, min(64, K)); cb.load(b, min(64, K)); k0 = 64; }
-    while (more) {
-      if (!split_warp_wait(bars, &bars->empty[slot], ph, status)) break;
+    auto load = [&](SA& a, SB& b) { ca.load(a, min(64, K - k0)); cb.load(b, min(64, K - k0)); k0 += 64; };
+    auto fetch = [&](SA& a, SB& b) -> bool {
+      if (k0 >= K && !open()) return false;
+      load(a, b);
+      return true;
+    };
+    auto put = [&](const SA& a, const SB& b) -> bool {
+      if (!split_warp_wait(bars, &bars->empty[slot], ph, status)) return false;
       uint8_t* dst = smem + (size_t)slot * C::kStage;
       store_slab<kM, kBf16>(a, dst + ca.soff, (ca.mn ? SA::kStepMn : SA::kStepK) * 128);
       store_slab<BN, kBf16>(b, dst + C::kPieces * C::kABytes + cb.soff, (cb.mn ? SB::kStepMn : SB::kStepK) * 128);
@@ -256,22 +272,36 @@ __device__ __forceinline__ void gemm_split_body(const SplitGemm* probs, int npro
       __syncwarp();
       if (lane == 0) mbar_arrive(&bars->full[slot]);
       if (++slot == C::kStages) { slot = 0; ph ^= 1; }
-      if (k0 >= K) more = open();
-      if (more) { ca.load(a, min(64, K - k0)); cb.load(b, min(64, K - k0)); k0 += 64; }
+      return true;
+    };
+    bool h0 = open();
+    if constexpr (kOne) {
+      dep_wait();
+      dep_launch();
+      // a wait gives up only after about a second: this cannot wipe a raised error
+      if (blockIdx.x == 0 && tid == 0) atomicExch(status, 0);
+    }
+    SA a0;
+    SB b0;
+    if (h0) load(a0, b0);
+    while (h0) {
+      if (!put(a0, b0)) break;
+      h0 = fetch(a0, b0);
     }
   } else if (warp >= kMmaWarp) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsMma));
     if (warp == kMmaWarp) {
       // ---------------------------------------------------------- MMA issuer (see elect_one for the uniform loop)
-      RecordReader rd;
+      if constexpr (kOne) dep_launch();
+      TileReader<kOne, BN> rd;
       int slot = 0, ph = 0;
       bool ok = true;
       const uint32_t sbase = uniform(smem_u32(smem)), tbase = uniform(tmem_base);
       for (int it = 0; ok; ++it) {
-        const TileRecord* r = rd.next(bars, status);
-        if (!r) break;
-        const int amn = (int)uniform(r->P.a_mn), bmn = (int)uniform(r->P.b_mn), K = (int)uniform(r->P.K),
-                  ncols = (int)uniform(min(BN, r->P.N - r->n0));
+        const TileAt t = rd.next(bars, probs, ntiles, status);
+        if (!t.P) break;
+        const int amn = (int)uniform(t.P->a_mn), bmn = (int)uniform(t.P->b_mn), K = (int)uniform(t.P->K),
+                  ncols = (int)uniform(min(BN, t.P->N - t.n0));
         rd.done(bars);
         const uint32_t idesc = instr_desc_bf16(kM, (ncols + 15) & ~15, amn, bmn);
         const int buf = it & 1;
@@ -311,7 +341,7 @@ __device__ __forceinline__ void gemm_split_body(const SplitGemm* probs, int npro
         if (ok && elect_one()) tc_commit(&bars->acc_full[buf]);
         __syncwarp();
       }
-    } else if (warp == kFindWarp) {
+    } else if (!kOne) {
       // ---------------------------------------------------------- tile finder
       int idx = 0, slot = 0, ph = 1;
       for (int tile = blockIdx.x;; tile += gridDim.x) {
@@ -348,16 +378,20 @@ __device__ __forceinline__ void gemm_split_body(const SplitGemm* probs, int npro
     const int qw = warp & 3;                             // the quarter of the TMEM lanes this warp may read
     uint8_t* mystg = stg + qw * 4096;
     const uint32_t lane_base = (uint32_t)(qw * 32) << 16;
-    RecordReader rd;
+    if constexpr (kOne) {
+      dep_wait();
+      dep_launch();
+    }
+    TileReader<kOne, BN> rd;
     for (int it = 0;; ++it) {
-      const TileRecord* r = rd.next(bars, status);
-      if (!r) break;
-      const int M = r->P.M, N = r->P.N, c_bf16 = r->P.c_bf16, m0 = r->m0, n0 = r->n0;
-      const int64_t ldc = r->P.ldc;
-      void* Cp = r->P.C;
-      const float *row_vec = r->P.row_vec, *col_vec = r->P.col_vec, thr = r->P.thr;
-      const int row_mode = r->P.row_mode, col_mode = r->P.col_mode;
-      const int *lr = r->P.live_rows, *lc = r->P.live_cols;
+      const TileAt t = rd.next(bars, probs, ntiles, status);
+      if (!t.P) break;
+      const int M = t.P->M, N = t.P->N, c_bf16 = t.P->c_bf16, m0 = t.m0, n0 = t.n0;
+      const int64_t ldc = t.P->ldc;
+      void* Cp = t.P->C;
+      const float *row_vec = t.P->row_vec, *col_vec = t.P->col_vec, thr = t.P->thr;
+      const int row_mode = t.P->row_mode, col_mode = t.P->col_mode;
+      const int *lr = t.P->live_rows, *lc = t.P->live_cols;
       rd.done(bars);
       const int live_r = lr ? min(*lr, M) : M, live_c = lc ? min(*lc, N) : N;
       const int row = m0 + qw * 32 + lane;
@@ -463,12 +497,12 @@ __device__ __forceinline__ void gemm_split_body(const SplitGemm* probs, int npro
 template <int BN>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_split_batched_kernel(const SplitGemm* __restrict__ probs, int nprobs, int ntiles, int* status) {
-  gemm_split_body<BN, false>(probs, nprobs, ntiles, status, false);
+  gemm_split_body<BN, false, false>(probs, nprobs, ntiles, status);
 }
 template <int BN, bool kBf16>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_split_one_kernel(const __grid_constant__ SplitGemm p, int ntiles, int* status) {
-  gemm_split_body<BN, kBf16>(&p, 1, ntiles, status, true);
+  gemm_split_body<BN, kBf16, true>(&p, 1, ntiles, status);
 }
 
 template <typename... KArgs, typename... Args>
@@ -493,17 +527,22 @@ int launch(void (*kernel)(KArgs...), size_t smem, int tiles, cudaStream_t st, Ar
 
 int tiles_of(const SplitGemm& p, int bn) { return ((p.M + kM - 1) / kM) * ((p.N + bn - 1) / bn); }
 
-// Tiles 128 columns wide where they give every SM one, else 64 (a 768 x 768 result: 72 CTAs instead of 36).
-int tile_width(int tiles128) { return tiles128 >= sm_count() ? 128 : 64; }
+// Tiles 128 or 64 columns wide, whichever takes less time: a wide one about one and a half times a narrow one (its A is converted
+// once instead of twice).  768 x 768: 36 or 72 tiles, one round of either: 64.  3072 x 768: 144 wide ones in one round, 288
+// narrow ones in two: 128 (10.4 us against 12.4 us).
+int tile_width(int tiles64, int tiles128) {
+  const int sms = sm_count() > 0 ? sm_count() : 1;
+  return 2 * ((tiles64 + sms - 1) / sms) >= 3 * ((tiles128 + sms - 1) / sms) ? 128 : 64;
+}
 
 }  // namespace
 
 SplitBatch gemm_split_plan(SplitGemm* probs, int count) {
   SplitBatch b;
-  int t128 = 0;
-  for (int i = 0; i < count; ++i) t128 += tiles_of(probs[i], 128);
+  int t64 = 0, t128 = 0;
+  for (int i = 0; i < count; ++i) { t64 += tiles_of(probs[i], 64); t128 += tiles_of(probs[i], 128); }
   b.count = count;
-  b.bn = tile_width(t128);
+  b.bn = tile_width(t64, t128);
   b.tiles = 0;
   for (int i = 0; i < count; ++i) { probs[i].first_tile = b.tiles; b.tiles += tiles_of(probs[i], b.bn); }
   return b;
