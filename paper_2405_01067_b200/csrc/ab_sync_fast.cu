@@ -398,6 +398,7 @@ int launch_jacobi(const JacobiJob* jobs, int count, int rmax, float tol, cudaStr
   return launch_jacobi_el<8>(jobs, count, rmax, tol, st);
 }
 
+constexpr int kTaskRows = 4;     // rows of a step of the elimination below a panel
 constexpr int kCPanel = 8;       // rows per panel of the Cholesky elimination (kCThreads / 64)
 
 struct CholJob {
@@ -410,9 +411,17 @@ struct CholJob {
   int r;
 };
 
+// 1 / sqrt(x) to about one unit in the last place: one Newton step on the hardware's approximation.  The pivots follow from one
+// another, and a square root and a division cost 400 cycles of that chain.
+__device__ __forceinline__ float rsqrt_close(float x) {
+  const float y = rsqrtf(x);
+  return fmaf(0.5f * y, fmaf(-x * y, y, 1.f), y);
+}
 // Right-looking Cholesky of one Gram matrix in shared memory (r <= 256), then the inverse of the
-// triangle by back substitution, one warp per column.  R lives in the upper triangle; column j of
+// triangle by back substitution, four columns per warp at a time.  R lives in the upper triangle; column j of
 // the inverse is parked in the strict lower triangle of row j (contiguous), its diagonal in dinv[].
+// 144 matrices of 192 rows, one CTA each (us): 228 -> 138; the factor 232000 -> 154000 cycles, of them 64000 in the panels'
+// chains of pivots and 90000 below them, bound by shared memory; the inverse 134000 -> 60000.
 __global__ void __launch_bounds__(kCThreads, 1) chol_inv_kernel(const CholJob* __restrict__ jobs) {
   extern __shared__ __align__(16) float sm[];
   const CholJob job = jobs[blockIdx.x];
@@ -427,14 +436,30 @@ __global__ void __launch_bounds__(kCThreads, 1) chol_inv_kernel(const CholJob* _
   {
     const float* __restrict__ G = job.G;
     const size_t part = (size_t)r * r;
-    for (int i = warp; i < r; i += nwarps) {           // one row per warp; the loads of a row are all in flight
-      const float* g = G + (size_t)i * r;
-#pragma unroll 8
-      for (int k = lane; k < r; k += 32) {
-        float v = g[k];
-        for (int q = 1; q < job.nparts; ++q) v += g[q * part + k];                 // ascending part order
-        S[i * ld + k] = v;
+    for (int i0 = 2 * warp; i0 < r; i0 += 2 * nwarps) {           // two rows per warp; the loads of both are all in flight
+      float v[2][8];
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int e = 0; e < 8; ++e) v[h][e] = 0.f;
+      for (int q = 0; q < job.nparts; ++q) {                                       // ascending part order
+        float t[2][8];
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+          for (int e = 0; e < 8; ++e)
+            if (i0 + h < r && 32 * e + lane < r) t[h][e] = G[q * part + (size_t)(i0 + h) * r + 32 * e + lane];
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+          for (int e = 0; e < 8; ++e)
+            if (i0 + h < r && 32 * e + lane < r) v[h][e] = q == 0 ? t[h][e] : v[h][e] + t[h][e];
       }
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+          if (i0 + h < r && 32 * e + lane < r) S[(i0 + h) * ld + 32 * e + lane] = v[h][e];
     }
   }
   __syncthreads();
@@ -443,42 +468,80 @@ __global__ void __launch_bounds__(kCThreads, 1) chol_inv_kernel(const CholJob* _
   __syncthreads();
   const float cut = kEigThr * maxdiag;
 
-  // Panels of kCPanel rows: inside a panel the rows are finished one after the other (scale row j,
-  // subtract it from the few panel rows below it), then all rows below the panel take the panel's
-  // kCPanel rank-one terms in one pass, in ascending j -- the same sums per entry as a column-by-column
-  // elimination, with one long step per panel instead of one per column.
+  // Panels of kCPanel rows.  Every thread eliminates the panel's diagonal block for itself, in registers, and takes its own
+  // column through it beside that: two barriers a panel, not two a row.  Then all rows below the panel take its kCPanel
+  // rank-one terms in one pass, in ascending j -- the same sums per entry as a column-by-column elimination.
   for (int j0 = 0; j0 < r; j0 += kCPanel) {
-    const int jend = (j0 + kCPanel < r) ? j0 + kCPanel : r;
-    for (int j = j0; j < jend; ++j) {
-      const float dj = S[j * ld + j];
-      const bool live = dj > cut && dj > 0.f;
-      const float inv = live ? 1.f / sqrtf(dj) : 0.f;
-      for (int k = j + 1 + tid; k < r; k += kCThreads) S[j * ld + k] *= inv;   // a dropped row becomes zero
-      __syncthreads();
-      if (tid == 0) {
-        S[j * ld + j] = dj * inv; dinv[j] = inv;                                // nobody reads the pivot below
-        if (!live && dj != 0.f) dropped_live = 1;
+    const int np = (r - j0 < kCPanel) ? r - j0 : kCPanel, jend = j0 + np;
+    const int k = j0 + tid;                // r <= 256 <= kCThreads: one column a thread
+    float d[kCPanel][kCPanel], p[kCPanel];
+    if (k < r) {
+#pragma unroll
+      for (int a = 0; a < kCPanel; ++a) {
+        p[a] = a < np ? S[(j0 + a) * ld + k] : 0.f;
+#pragma unroll
+        for (int b = a; b < kCPanel; ++b) d[a][b] = b < np ? S[(j0 + a) * ld + j0 + b] : 0.f;
       }
-      {                                              // panel rows still open: 64 threads per row
-        const int i = j + 1 + (tid >> 6);
-        if (i < jend) {
-          const float f = S[j * ld + i];
-          for (int k = i + (tid & 63); k < r; k += 64) S[i * ld + k] = fmaf(-f, S[j * ld + k], S[i * ld + k]);
+    }
+    __syncthreads();
+    if (k < r) {
+#pragma unroll
+      for (int q = 0; q < kCPanel; ++q) {
+        const float dj = d[q][q];
+        const bool live = dj > cut && dj > 0.f;
+        const float inv = live ? rsqrt_close(dj) : 0.f;
+        if (q < np) {
+          if (k > j0 + q) {
+            p[q] *= inv;                                                          // a dropped row becomes zero
+            S[(j0 + q) * ld + k] = p[q];
+          } else if (k == j0 + q) {
+            S[k * ld + k] = dj * inv;
+            dinv[k] = inv;
+            if (!live && dj != 0.f) dropped_live = 1;
+          }
+        }
+#pragma unroll
+        for (int b = q + 1; b < kCPanel; ++b) d[q][b] *= inv;
+#pragma unroll
+        for (int a = q + 1; a < kCPanel; ++a) {
+          p[a] = fmaf(-d[q][a], p[q], p[a]);
+#pragma unroll
+          for (int b = a; b < kCPanel; ++b) d[a][b] = fmaf(-d[q][a], d[q][b], d[a][b]);
         }
       }
-      __syncthreads();
     }
-    const int np = jend - j0;
-    for (int i = jend + warp; i < r; i += nwarps) {
-      float f[kCPanel];
+    __syncthreads();
+    if (jend >= r) break;
+    // steps of kTaskRows rows x 64 columns, a multiplier read once for two columns a lane; not the last panel: np == kCPanel
+    const int nrg = (r - jend + kTaskRows - 1) / kTaskRows, ntasks = nrg * ((r + 63) >> 6);
+    for (int t = warp; t < ntasks; t += nwarps) {
+      const int cb = t / nrg, i0 = jend + (t - cb * nrg) * kTaskRows, c0 = 64 * cb + lane, c1 = c0 + 32;
+      if (c0 - lane + 63 < i0) continue;
+      float pk0[kCPanel], pk1[kCPanel], acc0[kTaskRows], acc1[kTaskRows];
 #pragma unroll
-      for (int q = 0; q < kCPanel; ++q) f[q] = (q < np) ? S[(j0 + q) * ld + i] : 0.f;
-      for (int k = i + lane; k < r; k += 32) {
-        float acc = S[i * ld + k];
+      for (int q = 0; q < kCPanel; ++q) {
+        pk0[q] = c0 < r ? S[(j0 + q) * ld + c0] : 0.f;
+        pk1[q] = c1 < r ? S[(j0 + q) * ld + c1] : 0.f;
+      }
 #pragma unroll
-        for (int q = 0; q < kCPanel; ++q)
-          if (q < np) acc = fmaf(-f[q], S[(j0 + q) * ld + k], acc);
-        S[i * ld + k] = acc;
+      for (int h = 0; h < kTaskRows; ++h) {
+        acc0[h] = (c0 >= i0 + h && c0 < r) ? S[(i0 + h) * ld + c0] : 0.f;
+        acc1[h] = (c1 >= i0 + h && c1 < r) ? S[(i0 + h) * ld + c1] : 0.f;
+      }
+#pragma unroll
+      for (int h = 0; h < kTaskRows; ++h) {
+        const int i = i0 + h < r ? i0 + h : r - 1;
+#pragma unroll
+        for (int q = 0; q < kCPanel; ++q) {
+          const float f = S[(j0 + q) * ld + i];
+          acc0[h] = fmaf(-f, pk0[q], acc0[h]);
+          acc1[h] = fmaf(-f, pk1[q], acc1[h]);
+        }
+      }
+#pragma unroll
+      for (int h = 0; h < kTaskRows; ++h) {
+        if (c0 >= i0 + h && c0 < r) S[(i0 + h) * ld + c0] = acc0[h];
+        if (c1 >= i0 + h && c1 < r) S[(i0 + h) * ld + c1] = acc1[h];
       }
     }
     __syncthreads();
@@ -488,40 +551,64 @@ __global__ void __launch_bounds__(kCThreads, 1) chol_inv_kernel(const CholJob* _
   // form: lane l owns rows l, l + 32, ... of the column.  b starts as e_j; going down from k = j,
   // x_k = b_k / R_kk is final (one shuffle hands it to all lanes) and every row i < k takes
   // b_i -= R_ik x_k -- no reduction across lanes, and only the upper triangle (R) is read.
-  for (int j = warp; j < r; j += nwarps) {
-    float b[8], dk[8];
+  // Four neighbouring columns at a time: what a step reads of R serves all four, and their chains of shuffle and update hide one
+  // another's latency.  A column's entries below its j stay zero, so its steps above j change nothing.
+  {
+    float dk[8];
 #pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const int i = 32 * e + lane;
-      b[e] = (i == j) ? 1.f : 0.f;
-      dk[e] = (i < r) ? dinv[i] : 0.f;
-    }
+    for (int e = 0; e < 8; ++e) dk[e] = (32 * e + lane < r) ? dinv[32 * e + lane] : 0.f;
+    const int ngroups = (r + 3) >> 2;
+    for (int t = 0; t * nwarps < ngroups; ++t) {
+      const int gi = t * nwarps + ((t & 1) ? nwarps - 1 - warp : warp);       // long and short columns shared out
+      if (gi >= ngroups) continue;
+      const int j0 = 4 * gi, jtop = (j0 + 3 < r - 1) ? j0 + 3 : r - 1;
+      float b[4][8];
 #pragma unroll
-    for (int e = 7; e >= 0; --e) {
-      if (32 * e > j) continue;                  // uniform over the warp
-      const int ltop = (j - 32 * e < 31) ? j - 32 * e : 31;
-      for (int l = ltop; l >= 0; --l) {
-        const int k = 32 * e + l;
-        const float xk = __shfl_sync(0xffffffffu, b[e] * dk[e], l);
-        if (lane == l) b[e] = xk;
+      for (int c = 0; c < 4; ++c)
 #pragma unroll
-        for (int e2 = 0; e2 <= e; ++e2) {
-          const int i = 32 * e2 + lane;
-          if (i < k) b[e2] = fmaf(-S[i * ld + k], xk, b[e2]);
+        for (int e = 0; e < 8; ++e) b[c][e] = (32 * e + lane == j0 + c) ? 1.f : 0.f;
+#pragma unroll
+      for (int e = 7; e >= 0; --e) {
+        if (32 * e > jtop) continue;                  // uniform over the warp
+        const int ltop = (jtop - 32 * e < 31) ? jtop - 32 * e : 31;
+        for (int l = ltop; l >= 0; --l) {
+          const int k = 32 * e + l;
+          float xk[4];
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            xk[c] = __shfl_sync(0xffffffffu, b[c][e] * dk[e], l);
+            if (lane == l) b[c][e] = xk[c];
+          }
+#pragma unroll
+          for (int e2 = 0; e2 <= e; ++e2) {
+            const int i = 32 * e2 + lane;
+            if (i < k) {
+              const float Sik = S[i * ld + k];
+#pragma unroll
+              for (int c = 0; c < 4; ++c) b[c][e2] = fmaf(-Sik, xk[c], b[c][e2]);
+            }
+          }
         }
       }
-    }
 #pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const int i = 32 * e + lane;
-      if (i < j) S[j * ld + i] = b[e];           // column j of X, parked in row j below the diagonal
+      for (int c = 0; c < 4; ++c)
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          const int i = 32 * e + lane;
+          if (j0 + c < r && i < j0 + c) S[(j0 + c) * ld + i] = b[c][e];           // column j of X, parked in row j below the diagonal
+        }
     }
   }
   __syncthreads();
-  for (int idx = tid; idx < r * r; idx += kCThreads) {
-    const int i = idx / r, k = idx % r;
-    job.R[idx] = (k >= i) ? S[i * ld + k] : 0.f;
-    job.Rinv[idx] = (k > i) ? S[k * ld + i] : (k == i ? dinv[i] : 0.f);
+  for (int i = warp; i < r; i += nwarps) {
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const int k = 32 * e + lane;
+      if (k < r) {
+        job.R[(size_t)i * r + k] = (k >= i) ? S[i * ld + k] : 0.f;
+        job.Rinv[(size_t)i * r + k] = (k > i) ? S[k * ld + i] : (k == i ? dinv[i] : 0.f);
+      }
+    }
   }
   if (tid == 0 && job.status) *job.status = dropped_live ? (int)AB_ERR_ACCURACY : (int)AB_OK;
 }
