@@ -93,10 +93,9 @@ int recombine_mean_simt(const float* A_copies, int64_t strideA, const float* B_c
                         float* W, float* Abar, float* Bbar, int m, int n, int r, cudaStream_t st);
 
 // ---- general tensor-core GEMM (ab_gemm_tc.cu) --------------------------------------------------
-// C[M x N] = sum over terms of A_t B_t^T on the tensor cores; see the head of ab_gemm_tc.cu.
+// C[M x N] = A B^T on the tensor cores; see the head of ab_gemm_tc.cu.
 struct TcOperand {
-  const void* p[3];   // bf16 pieces: one (plain product) or three (hi, mid, lo of an fp32 matrix)
-  int pieces;
+  const void* p;      // bf16
   int64_t ld;         // row stride in elements, a multiple of 8
   bool mn;            // false: stored M x K (resp. N x K); true: stored K x M (resp. K x N)
 };
@@ -107,15 +106,12 @@ struct TcProblem {
   int M, N, K;
   bool c_f32;
   int ksplit;
-  const int* live_rows;   // optional device ints: rows / columns at or beyond them are written as zero
-  const int* live_cols;
 };
 bool gemm_tc_available();
 bool gemm_tc_problem_ok(const TcProblem& q);
-size_t gemm_tc_table_bytes(int count);
-// table_dev: device memory of gemm_tc_table_bytes(count); status: device int that receives AB_ERR_TIMEOUT
-// if a bounded wait ran out (never cleared here).
-int gemm_tc_batched(const TcProblem* probs, int count, void* table_dev, int* status, cudaStream_t st);
+// One or two problems; status: device int, cleared first, that receives AB_ERR_TIMEOUT if a bounded wait ran out.
+int gemm_tc_batched(const TcProblem* probs, int count, int* status, cudaStream_t st);
+// count and slice_stride multiples of 4, 16-byte aligned
 int sum_slices(const float* part, float* out, int64_t count, int64_t slice_stride, int slices, cudaStream_t st);
 
 // ---- batched fp32-accurate products with the split in the loader (ab_gemm_split.cu) --------------------------

@@ -1,23 +1,19 @@
 // General tensor-core GEMM on sm_100a: the products of the path that are plain contractions.
 //
-//   C[M x N] = sum over terms t of  A_t[M x K] * B_t[N x K]^T        (bf16 operands, fp32 accumulation in TMEM)
+//   C[M x N] = A[M x K] * B[N x K]^T        (bf16 operands, fp32 accumulation in TMEM)
 //
-// One term is the ordinary bf16 product (the dense layer of the full-rank phases: y = x W^T, dX = dY W,
-// dW = dY^T x).  Six terms are the fp32-accurate product of two fp32 matrices that were cut into three bf16
-// pieces each (hi + mid + lo carries 24 bits): hi*hi, hi*mid, mid*hi, hi*lo, lo*hi, mid*mid, the small terms
-// first.  bf16 products are exact in fp32, so what is lost is the three products of order 2^-24 and the
-// rounding of the fp32 sums.  This carries W = Abar Bbar, the Gram matrices and the long products of the
-// group synchronisation, which need the 1e-6 / 1e-4 bounds of the fp32 path.
+// the dense layer of the full-rank phases: y = x W^T, dX = dY W, dW = dY^T x.
 //
 // Either operand may lie K-major (M x K resp. N x K, row-major) or MN-major (stored K x M resp. K x N,
 // row-major); the shared-memory descriptors of the MMAs express the difference, nothing is transposed.
-// Many problems run in one launch: a table of problem records (tensor maps included) sits in device memory
-// and a CTA finds its problem and its 128 x 256 tile from its block index.  K may be cut into slices, each
-// writing its own partial result (summed afterwards in ascending order: fixed bits).
+// Up to two problems run in one launch; their records (tensor maps included) are kernel parameters and a CTA finds its problem
+// and its 128 x 256 tile from its block index.  (In a table in device memory they cost a copy in front of every launch, which
+// also kept the launch from overlapping the kernel before it.)  K may be cut into slices, each writing its own partial
+// result (summed afterwards in ascending order: fixed bits).  A slab of 64 is bound by the arrival of its 48 KB at 64 bytes a
+// cycle and SM, 768 cycles; its MMAs take 520.
 //
 // Warps (192 threads): 0 = TMA producer, 1 = MMA issuer and TMEM owner, 2..5 = epilogue (TMEM -> registers
 // -> a staging tile of the warp's own -> TMA store of 32 rows).  Every wait is bounded (see ab_tc_ptx.cuh).
-#include <vector>
 #include <cstring>
 
 #include "ab_common.cuh"
@@ -35,7 +31,7 @@ constexpr int kStage = kAStage + kBStage;
 constexpr int kStages = 4;
 constexpr int kStgBytes = 4096;           // 32 rows x 128 bytes
 constexpr int kTcThreads = 192;
-constexpr int kMaxTerms = 6;
+constexpr int kMaxProbs = 2;
 
 struct TcBars {
   uint64_t full[kStages], empty[kStages];
@@ -44,13 +40,10 @@ struct TcBars {
   int abort_any;
 };
 
-// One problem of a batch, as the kernel reads it from device memory.
 struct alignas(64) TcProblemDev {
-  CUtensorMap a[3], b[3];   // the pieces of A and of B (one piece for a plain bf16 product)
+  CUtensorMap a, b;
   CUtensorMap c;            // output, boxes of 32 rows x 128 bytes
   int M, N, K;
-  int nterms;
-  int term_a[kMaxTerms], term_b[kMaxTerms];
   int a_mn, b_mn;           // 1: stored K x M / K x N
   int c_f32;                // 1: fp32 output (32 columns per box), 0: bf16 (64 columns per box)
   int tiles_n;              // column tiles
@@ -58,8 +51,11 @@ struct alignas(64) TcProblemDev {
   int kslice;               // K per slice, a multiple of 64
   int c_rows;               // rows of one partial result in the output map (M when ksplit == 1)
   int first_tile;           // index of this problem's first tile among all tiles of the batch
-  const int* live_rows;     // optional device ints: rows / columns at or beyond them are written as zero
-  const int* live_cols;
+};
+struct TcBatch {
+  TcProblemDev prob[kMaxProbs];
+  int nprobs, ntiles;
+  int* status;
 };
 
 __device__ __forceinline__ void tc_raise(TcBars* b, int* status) {
@@ -72,14 +68,9 @@ struct TileInfo {
   const TcProblemDev* P;
   int m0, n0, slice, k_begin, k_end, nslab, ncols, nmma;
 };
-__device__ __forceinline__ TileInfo decode_tile(const TcProblemDev* __restrict__ probs, int nprobs, int tile) {
-  int lo = 0, hi = nprobs - 1;
-  while (lo < hi) {                       // the last problem whose first tile is <= tile
-    const int mid = (lo + hi + 1) >> 1;
-    if (probs[mid].first_tile <= tile) lo = mid; else hi = mid - 1;
-  }
+__device__ __forceinline__ TileInfo decode_tile(const TcBatch& p, int tile) {
   TileInfo ti;
-  ti.P = probs + lo;
+  ti.P = p.prob + (p.nprobs > 1 && tile >= p.prob[1].first_tile ? 1 : 0);
   int t = tile - ti.P->first_tile;
   ti.slice = t % ti.P->ksplit;
   t /= ti.P->ksplit;
@@ -99,7 +90,9 @@ __device__ __forceinline__ TileInfo decode_tile(const TcProblemDev* __restrict__
 // TMEM alternate between a CTA's tiles, so the epilogue of one tile (TMEM -> staging -> TMA stores) runs
 // beside the loads and MMAs of the next.
 __global__ void __launch_bounds__(kTcThreads, 1)
-gemm_tc_kernel(const TcProblemDev* __restrict__ probs, int nprobs, int ntiles, int* status) {
+gemm_tc_kernel(const __grid_constant__ TcBatch p) {
+  int* const status = p.status;
+  const int ntiles = p.ntiles;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   uint8_t* ring = smem;
@@ -118,6 +111,10 @@ gemm_tc_kernel(const TcProblemDev* __restrict__ probs, int nprobs, int ntiles, i
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *reinterpret_cast<volatile uint32_t*>(&bars->tmem_base);
+  dep_wait();            // nothing above touches global memory
+  dep_launch();
+  // a wait gives up only after about a second: this cannot wipe a raised error
+  if (blockIdx.x == 0 && threadIdx.x == 0) atomicExch(status, 0);
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
@@ -125,28 +122,25 @@ gemm_tc_kernel(const TcProblemDev* __restrict__ probs, int nprobs, int ntiles, i
       int slot = 0, ph = 1;
       bool ok = true;
       for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
-        const TileInfo ti = decode_tile(probs, nprobs, tile);
+        const TileInfo ti = decode_tile(p, tile);
         const TcProblemDev* P = ti.P;
-        const int a_mn = (int)uniform(P->a_mn), b_mn = (int)uniform(P->b_mn), nterms = (int)uniform(P->nterms), nslab = (int)uniform(ti.nslab);
-        for (int tix = 0; tix < nterms && ok; ++tix) {
-          const CUtensorMap* ma = &P->a[P->term_a[tix]];
-          const CUtensorMap* mb = &P->b[P->term_b[tix]];
-          for (int ks = 0; ks < nslab; ++ks) {
-            if (!mbar_wait_warp(&bars->empty[slot], ph)) { tc_raise(bars, status); ok = false; break; }
-            if (elect_one()) {
-              uint8_t* da = ring + (size_t)slot * kStage;
-              uint8_t* db = da + kAStage;
-              uint64_t* bar = &bars->full[slot];
-              const int k0 = ti.k_begin + ks * kBK;
-              mbar_arrive_expect_tx(bar, kStage);
-              if (a_mn) { for (int h = 0; h < 2; ++h) tma_load_2d(da + h * 8192, ma, bar, ti.m0 + 64 * h, k0); }
-              else tma_load_2d(da, ma, bar, k0, ti.m0);
-              if (b_mn) { for (int h = 0; h < 4; ++h) tma_load_2d(db + h * 8192, mb, bar, ti.n0 + 64 * h, k0); }
-              else tma_load_2d(db, mb, bar, k0, ti.n0);
-            }
-            __syncwarp();
-            if (++slot == kStages) { slot = 0; ph ^= 1; }
+        const int a_mn = (int)uniform(P->a_mn), b_mn = (int)uniform(P->b_mn), nslab = (int)uniform(ti.nslab);
+        const CUtensorMap *ma = &P->a, *mb = &P->b;
+        for (int ks = 0; ks < nslab; ++ks) {
+          if (!mbar_wait_warp(&bars->empty[slot], ph)) { tc_raise(bars, status); ok = false; break; }
+          if (elect_one()) {
+            uint8_t* da = ring + (size_t)slot * kStage;
+            uint8_t* db = da + kAStage;
+            uint64_t* bar = &bars->full[slot];
+            const int k0 = ti.k_begin + ks * kBK;
+            mbar_arrive_expect_tx(bar, kStage);
+            if (a_mn) { for (int h = 0; h < 2; ++h) tma_load_2d(da + h * 8192, ma, bar, ti.m0 + 64 * h, k0); }
+            else tma_load_2d(da, ma, bar, k0, ti.m0);
+            if (b_mn) { for (int h = 0; h < 4; ++h) tma_load_2d(db + h * 8192, mb, bar, ti.n0 + 64 * h, k0); }
+            else tma_load_2d(db, mb, bar, k0, ti.n0);
           }
+          __syncwarp();
+          if (++slot == kStages) { slot = 0; ph ^= 1; }
         }
       }
     }
@@ -157,8 +151,8 @@ gemm_tc_kernel(const TcProblemDev* __restrict__ probs, int nprobs, int ntiles, i
       bool ok = true;
       const uint32_t sbase = uniform(smem_u32(ring)), tmem = uniform(tmem_base);
       for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, ++it) {
-        const TileInfo ti = decode_tile(probs, nprobs, tile);
-        const int nterms = (int)uniform(ti.P->nterms), nslab = (int)uniform(ti.nslab), klen = (int)uniform(ti.k_end - ti.k_begin);
+        const TileInfo ti = decode_tile(p, tile);
+        const int nslab = (int)uniform(ti.nslab), klen = (int)uniform(ti.k_end - ti.k_begin);
         const int a_mn = (int)uniform(ti.P->a_mn), b_mn = (int)uniform(ti.P->b_mn);
         const uint32_t idesc = instr_desc_bf16(kBM, (int)uniform(ti.nmma), a_mn, b_mn);
         const uint64_t da0 = smem_desc_sw128(sbase, a_mn ? 8192 : 16), db0 = smem_desc_sw128(sbase + kAStage, b_mn ? 8192 : 16);
@@ -167,21 +161,19 @@ gemm_tc_kernel(const TcProblemDev* __restrict__ probs, int nprobs, int ntiles, i
         if (!mbar_wait_warp(&bars->acc_empty[b], ((it >> 1) & 1) ^ 1)) { tc_raise(bars, status); ok = false; break; }
         tc_fence_after();
         const uint32_t tacc = tmem + 256 * b;
-        for (int tix = 0; tix < nterms && ok; ++tix) {
-          for (int ks = 0; ks < nslab; ++ks) {
-            if (!mbar_wait_warp(&bars->full[slot], ph)) { tc_raise(bars, status); ok = false; break; }
-            tc_fence_after();
-            const uint64_t da = da0 + (uint64_t)(slot * (kStage >> 4)), db = db0 + (uint64_t)(slot * (kStage >> 4));
-            const int ksteps = (klen - ks * kBK + 15) >> 4;
-            if (elect_one()) {
+        for (int ks = 0; ks < nslab; ++ks) {
+          if (!mbar_wait_warp(&bars->full[slot], ph)) { tc_raise(bars, status); ok = false; break; }
+          tc_fence_after();
+          const uint64_t da = da0 + (uint64_t)(slot * (kStage >> 4)), db = db0 + (uint64_t)(slot * (kStage >> 4));
+          const int ksteps = (klen - ks * kBK + 15) >> 4;
+          if (elect_one()) {
 #pragma unroll
-              for (int kk = 0; kk < 4; ++kk)
-                if (kk < ksteps) tc_mma_bf16(tacc, da + as * kk, db + bs * kk, idesc, (tix | ks | kk) ? 1u : 0u);
-              tc_commit(&bars->empty[slot]);
-            }
-            __syncwarp();
-            if (++slot == kStages) { slot = 0; ph ^= 1; }
+            for (int kk = 0; kk < 4; ++kk)
+              if (kk < ksteps) tc_mma_bf16(tacc, da + as * kk, db + bs * kk, idesc, (ks | kk) ? 1u : 0u);
+            tc_commit(&bars->empty[slot]);
           }
+          __syncwarp();
+          if (++slot == kStages) { slot = 0; ph ^= 1; }
         }
         if (ok && elect_one()) tc_commit(&bars->acc_full[b]);
         __syncwarp();
@@ -195,10 +187,10 @@ gemm_tc_kernel(const TcProblemDev* __restrict__ probs, int nprobs, int ntiles, i
     int nst = 0, it = 0;
     bool ok = true;
     for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, ++it) {
-      const TileInfo ti = decode_tile(probs, nprobs, tile);
+      const TileInfo ti = decode_tile(p, tile);
       const TcProblemDev* P = ti.P;
       const int b = it & 1;
-      const bool have_acc = ti.nslab > 0 && P->nterms > 0;      // an empty reduction leaves zeros
+      const bool have_acc = ti.nslab > 0;      // an empty reduction leaves zeros
       {
         int w = 1;
         if (lane == 0) { w = mbar_wait(&bars->acc_full[b], (it >> 1) & 1) ? 1 : 0; if (!w) tc_raise(bars, status); }
@@ -206,9 +198,6 @@ gemm_tc_kernel(const TcProblemDev* __restrict__ probs, int nprobs, int ntiles, i
       }
       if (!ok) break;
       tc_fence_after();
-      const int grow = ti.m0 + qw * 32 + lane;           // row of C this thread holds
-      const int live_r = P->live_rows ? *P->live_rows : P->M;
-      const int live_c = P->live_cols ? *P->live_cols : P->N;
       const bool rows_in = ti.m0 + qw * 32 < P->M;
       const int c_f32 = P->c_f32;
       const int pcols = c_f32 ? 32 : 64;                 // columns of one 128-byte piece
@@ -233,12 +222,6 @@ gemm_tc_kernel(const TcProblemDev* __restrict__ probs, int nprobs, int ntiles, i
           if (lane == 0) mbar_arrive(&bars->acc_empty[b]);
         }
         if (!rows_in) continue;
-        const bool row_dead = grow >= live_r;
-#pragma unroll
-        for (int gq = 0; gq < 4; ++gq)
-#pragma unroll
-          for (int e = 0; e < 16; ++e)
-            if (row_dead || ti.n0 + c0 + gq * 16 + e >= live_c) v[gq][e] = 0u;
         uint8_t* buf = mystg + (nst & 1) * kStgBytes;
         ++nst;
         if (lane == 0) tma_store_wait_read<1>();
@@ -288,84 +271,96 @@ gemm_tc_kernel(const TcProblemDev* __restrict__ probs, int nprobs, int ntiles, i
   }
 }
 
-// out[i] = sum over slices of part[s][i], ascending s (fixed order); partials are rows_pad x ld, out is rows x ld
+// out[i] = sum over slices of part[s][i], ascending s (fixed order); four values a thread (count and stride are multiples of 4), up
+// to eight slices' loads in flight
 __global__ void __launch_bounds__(256)
-sum_slices_kernel(const float* __restrict__ part, float* __restrict__ out, int64_t count, int64_t slice_stride, int slices) {
+sum_slices_kernel(const float4* __restrict__ part, float4* __restrict__ out, int64_t count4, int64_t stride4, int slices) {
   const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
-  if (i >= count) return;
-  float acc = part[i];
-  for (int s = 1; s < slices; ++s) acc += part[i + s * slice_stride];
+  dep_wait();
+  dep_launch();
+  if (i >= count4) return;
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int s0 = 0; s0 < slices; s0 += 8) {
+    float4 v[8];
+#pragma unroll
+    for (int s = 0; s < 8; ++s)
+      if (s0 + s < slices) v[s] = __ldcg(part + i + (s0 + s) * stride4);
+#pragma unroll
+    for (int s = 0; s < 8; ++s)
+      if (s0 + s < slices) { acc.x += v[s].x; acc.y += v[s].y; acc.z += v[s].z; acc.w += v[s].w; }
+  }
   out[i] = acc;
+}
+
+template <typename... KArgs, typename... Args>
+int launch_after(void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  if (cudaLaunchKernelEx(&cfg, kernel, args...) != cudaSuccess) { (void)cudaGetLastError(); return AB_ERR_CUDA; }
+  AB_LAUNCH_OK();
+  return AB_OK;
 }
 
 }  // namespace
 
 int sum_slices(const float* part, float* out, int64_t count, int64_t slice_stride, int slices, cudaStream_t st) {
   if (count <= 0) return AB_OK;
-  sum_slices_kernel<<<(unsigned)((count + 255) / 256), 256, 0, st>>>(part, out, count, slice_stride, slices);
-  AB_LAUNCH_OK();
-  return AB_OK;
+  if (count % 4 != 0 || slice_stride % 4 != 0 || !aligned(part, 16) || !aligned(out, 16)) return AB_ERR_INVALID_ARG;
+  return launch_after(sum_slices_kernel, (unsigned)((count / 4 + 255) / 256), 256u, 0, st, reinterpret_cast<const float4*>(part),
+                      reinterpret_cast<float4*>(out), count / 4, slice_stride / 4, slices);
 }
 
 bool gemm_tc_available() { return tc_device_ok(); }
 
-size_t gemm_tc_table_bytes(int count) { return align_up((size_t)count * sizeof(TcProblemDev), 256); }
-
 bool gemm_tc_problem_ok(const TcProblem& q) {
   if (q.M <= 0 || q.N <= 0 || q.K <= 0) return false;
-  if (q.A.pieces != q.B.pieces || (q.A.pieces != 1 && q.A.pieces != 3)) return false;
-  if (q.A.ld % 8 != 0 || q.B.ld % 8 != 0) return false;
-  for (int i = 0; i < q.A.pieces; ++i)
-    if (!aligned(q.A.p[i], 16) || !aligned(q.B.p[i], 16)) return false;
+  if (q.A.ld % 8 != 0 || q.B.ld % 8 != 0 || !aligned(q.A.p, 16) || !aligned(q.B.p, 16)) return false;
   if (!aligned(q.C, 16) || (q.ldc * (q.c_f32 ? 4 : 2)) % 16 != 0) return false;
   if (q.ksplit < 1 || (q.ksplit > 1 && !q.c_f32)) return false;
   return true;
 }
 
-int gemm_tc_batched(const TcProblem* probs, int count, void* table_dev, int* status, cudaStream_t st) {
+int gemm_tc_batched(const TcProblem* probs, int count, int* status, cudaStream_t st) {
   if (count <= 0) return AB_OK;
-  if (!tc_device_ok()) return AB_ERR_UNSUPPORTED;
-  std::vector<TcProblemDev> tab((size_t)count);
+  if (count > kMaxProbs || !tc_device_ok()) return AB_ERR_UNSUPPORTED;
+  TcBatch batch;
+  std::memset(&batch, 0, sizeof(batch));
   int tiles = 0;
   for (int i = 0; i < count; ++i) {
     const TcProblem& q = probs[i];
     if (!gemm_tc_problem_ok(q)) return AB_ERR_UNSUPPORTED;
-    TcProblemDev& d = tab[i];
-    std::memset(&d, 0, sizeof(d));
-    for (int pc = 0; pc < q.A.pieces; ++pc) {
-      if (q.A.mn) AB_TRY(make_tensor_map_2d(&d.a[pc], q.A.p[pc], false, q.K, q.M, q.A.ld, 64, 64));
-      else AB_TRY(make_tensor_map_2d(&d.a[pc], q.A.p[pc], false, q.M, q.K, q.A.ld, 64, kBM));
-      if (q.B.mn) AB_TRY(make_tensor_map_2d(&d.b[pc], q.B.p[pc], false, q.K, q.N, q.B.ld, 64, 64));
-      else AB_TRY(make_tensor_map_2d(&d.b[pc], q.B.p[pc], false, q.N, q.K, q.B.ld, 64, kBN));
-    }
+    TcProblemDev& d = batch.prob[i];
+    if (q.A.mn) AB_TRY(make_tensor_map_2d(&d.a, q.A.p, false, q.K, q.M, q.A.ld, 64, 64));
+    else AB_TRY(make_tensor_map_2d(&d.a, q.A.p, false, q.M, q.K, q.A.ld, 64, kBM));
+    if (q.B.mn) AB_TRY(make_tensor_map_2d(&d.b, q.B.p, false, q.K, q.N, q.B.ld, 64, 64));
+    else AB_TRY(make_tensor_map_2d(&d.b, q.B.p, false, q.N, q.K, q.B.ld, 64, kBN));
     d.M = q.M; d.N = q.N; d.K = q.K;
-    if (q.A.pieces == 1) { d.nterms = 1; d.term_a[0] = 0; d.term_b[0] = 0; }
-    else {   // small terms first: mid*mid, lo*hi, hi*lo, mid*hi, hi*mid, hi*hi
-      const int ta[6] = {1, 2, 0, 1, 0, 0}, tb[6] = {1, 0, 2, 0, 1, 0};
-      d.nterms = 6;
-      for (int k = 0; k < 6; ++k) { d.term_a[k] = ta[k]; d.term_b[k] = tb[k]; }
-    }
     d.a_mn = q.A.mn ? 1 : 0; d.b_mn = q.B.mn ? 1 : 0; d.c_f32 = q.c_f32 ? 1 : 0;
     d.tiles_n = (q.N + kBN - 1) / kBN;
     d.ksplit = q.ksplit;
     const int slabs = (q.K + kBK - 1) / kBK;
     d.kslice = ((slabs + q.ksplit - 1) / q.ksplit) * kBK;
     d.c_rows = q.ksplit > 1 ? (q.M + kBM - 1) / kBM * kBM : q.M;
-    AB_TRY(make_tensor_map_2d(&d.c, q.C, q.c_f32, (uint64_t)d.c_rows * q.ksplit - (q.ksplit > 1 ? 0 : 0), q.N, q.ldc,
+    AB_TRY(make_tensor_map_2d(&d.c, q.C, q.c_f32, (uint64_t)d.c_rows * q.ksplit, q.N, q.ldc,
                               q.c_f32 ? 32 : 64, 32));
     d.first_tile = tiles;
-    d.live_rows = q.live_rows; d.live_cols = q.live_cols;
     tiles += ((q.M + kBM - 1) / kBM) * d.tiles_n * q.ksplit;
   }
-  AB_CUDA_OK(cudaMemcpyAsync(table_dev, tab.data(), tab.size() * sizeof(TcProblemDev), cudaMemcpyHostToDevice, st));
   const size_t smem = (size_t)kStages * kStage + 4 * 2 * kStgBytes + sizeof(TcBars) + 1024;
   AB_CUDA_OK(cudaFuncSetAttribute(gemm_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int sms = sm_count();
   if (sms <= 0) return AB_ERR_CUDA;
   const int grid = tiles < sms ? tiles : sms;
-  gemm_tc_kernel<<<(unsigned)grid, kTcThreads, smem, st>>>(static_cast<const TcProblemDev*>(table_dev), count, tiles, status);
-  AB_LAUNCH_OK();
-  return AB_OK;
+  batch.nprobs = count; batch.ntiles = tiles; batch.status = status;
+  return launch_after(gemm_tc_kernel, (unsigned)grid, (unsigned)kTcThreads, smem, st, batch);
 }
 
 }  // namespace ab
