@@ -772,6 +772,9 @@ grad_kernel(const __grid_constant__ CUtensorMap tmAct0, const __grid_constant__ 
     tc_fence_after();
     tmem_dealloc(tmem_base, kTmemCols);
   }
+  // Whatever is launched behind this kernel waits for this kernel alone.  Without a dB job (whose CTAs have waited above) it could
+  // be through while the chain kernel still writes dX and reads the workspace: no CTA leaves before that kernel is done.
+  dep_wait();
 }
 
 // ---------------------------------------------------------------------------------------------
