@@ -80,7 +80,7 @@ int general_forward(const void* x, const void* A, const void* B, void* y, void* 
   if (dt == AB_F32) {
     const float *x32 = static_cast<const float*>(x), *A32 = static_cast<const float*>(A), *B32 = static_cast<const float*>(B);
     float* T32 = T_save ? static_cast<float*>(T_save) : T;
-    if (layer_small_ok(N, m, n, r))
+    if (layer_small_ok(N, n, m, r, false))
       return layer_small_chain(x32, N, n, B32, ldB, 1, A32, ldA, 1, static_cast<float*>(y), m, static_cast<float*>(T_save), r, status, st);
     AB_CUDA_OK(cudaMemsetAsync(status, 0, sizeof(int), st));
     AB_TRY(gemm_simt(x, dt, n, 1, B, dt, 1, ldB, T32, AB_F32, r, N, r, n, st));       // T = x B^T
@@ -104,35 +104,49 @@ int general_backward(const void* x, const void* dY, const void* A, const void* B
   if (dt == AB_F32) {
     const float *x32 = static_cast<const float*>(x), *y32 = static_cast<const float*>(dY), *A32 = static_cast<const float*>(A),
                 *B32 = static_cast<const float*>(B);
-    const bool fused = layer_small_ok(N, m, n, r);
-    int* clear = status;              // the first kernel of the call clears the status word
-    if (!fused) { AB_CUDA_OK(cudaMemsetAsync(status, 0, sizeof(int), st)); clear = nullptr; }
+    const bool fused = layer_small_ok(N, m, n, r, true), fused_T = layer_small_ok(N, n, m, r, false);
+    // dA and dB in one launch where their tiles together leave room for a cut reduction (see gemm_small_pays)
+    const int64_t tiles = (int64_t)((m + 63) / 64 + (n + 63) / 64) * ((r + 63) / 64);
+    const bool pair = 2 * tiles < sm_count();
+    int* clear = status;              // the first kernel of the call clears the status word; the general ones do not
+    auto cleared = [&]() -> int {
+      if (clear) AB_CUDA_OK(cudaMemsetAsync(status, 0, sizeof(int), st));
+      clear = nullptr;
+      return AB_OK;
+    };
     if (dX || dB) {                   // dT = dY A, dX = dT B
       if (fused) {
         AB_TRY(layer_small_chain(y32, N, m, A32, 1, ldA, B32, 1, ldB, static_cast<float*>(dX), n, dB ? dT : nullptr, r, clear, st));
         clear = nullptr;
       } else {
+        AB_TRY(cleared());
         AB_TRY(gemm_simt(dY, dt, m, 1, A, dt, ldA, 1, dT, AB_F32, r, N, r, m, st));
         if (dX) AB_TRY(gemm_simt(dT, AB_F32, r, 1, B, dt, ldB, 1, dX, dt, n, N, n, r, st));
       }
     }
     const float* Ts = static_cast<const float*>(T_saved);
     if (dA && !Ts) {
-      if (fused) {
+      if (fused_T) {
         AB_TRY(layer_small_chain(x32, N, n, B32, ldB, 1, nullptr, 0, 0, nullptr, 0, T, r, clear, st));
         clear = nullptr;
       } else {
+        AB_TRY(cleared());
         AB_TRY(gemm_simt(x, dt, n, 1, B, dt, 1, ldB, T, AB_F32, r, N, r, n, st));
       }
       Ts = T;
     }
-    SmallProduct g[2];                // dA = dY^T T, dB = dT^T x: one launch
+    if (!pair) {                      // dA = dY^T T, dB = dT^T x
+      AB_TRY(cleared());
+      if (dA) AB_TRY(gemm_simt(dY, dt, 1, m, Ts, dt, r, 1, dA, AB_F32, r, m, r, N, st));
+      if (dB) AB_TRY(gemm_simt(dT, AB_F32, 1, r, x, dt, n, 1, dB, AB_F32, n, r, n, N, st));
+      return AB_OK;
+    }
+    SmallProduct g[2];
     int ng = 0;
     if (dA) g[ng++] = SmallProduct{y32, 1, m, Ts, 1, r, dA, r, m, r};
     if (dB) g[ng++] = SmallProduct{dT, 1, r, x32, 1, n, dB, n, r, n};
     if (ng > 0) { AB_TRY(gemm_small(g, ng, N, clear, st)); clear = nullptr; }
-    if (clear) AB_CUDA_OK(cudaMemsetAsync(status, 0, sizeof(int), st));
-    return AB_OK;
+    return cleared();
   }
   AB_CUDA_OK(cudaMemsetAsync(status, 0, sizeof(int), st));
   AB_TRY(gemm_simt(dY, dt, m, 1, A, dt, ldA, 1, dT, AB_F32, r, N, r, m, st));      // dT = dY A

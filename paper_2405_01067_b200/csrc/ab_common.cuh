@@ -167,9 +167,10 @@ int tile_product(const TileProduct& t, bool clear_status, int* status, cudaStrea
 // in fp64.  One or two products with the same reduction length in one launch; status: cleared if not null.
 struct SmallProduct { const float* U; int64_t u_p, u_k; const float* V; int64_t v_q, v_k; float* C; int64_t ldc; int P, Q; };
 int gemm_small(const SmallProduct* jobs, int njobs, int64_t K, int* status, cudaStream_t st);
+bool gemm_small_pays(int64_t M, int64_t N, int64_t K);
 // S = In F1^T, Out = S F2^T (Out null: only S; S null: not stored) for a layer small enough to be latency-bound;
 // F1(j, k) at F1[j * f1_j + k * f1_k], F2(p, j) at F2[p * f2_p + j * f2_j]
-bool layer_small_ok(int64_t N, int m, int n, int r);
+bool layer_small_ok(int64_t N, int K1, int P, int r, bool backward);
 int layer_small_chain(const float* In, int64_t N, int K1, const float* F1, int64_t f1_j, int64_t f1_k, const float* F2, int64_t f2_p,
                       int64_t f2_j, float* Out, int P, float* S, int r, int* status, cudaStream_t st);
 

@@ -1,7 +1,7 @@
 // Strided GEMMs on the fp32 pipes: the path for fp32 storage (where a reduced-precision
 // tensor-core pass would miss the 1e-4 bound) and for shapes the fused tensor-core chain does
 // not take.  Two kernels:
-//  - gemm_simt_kernel: any mix of fp32 / bf16 operands with at least one bf16.  64x64 output tile per CTA, 16-deep k
+//  - gemm_simt_kernel: any mix of fp32 / bf16 operands.  64x64 output tile per CTA, 16-deep k
 //    slabs staged in shared memory, 4x4 accumulators per thread.  Each 16-term partial dot
 //    product is formed in fp32 and added to a running fp64 sum, so long reductions keep ~1e-7
 //    relative accuracy; the order of additions is fixed by the shape alone.
@@ -331,7 +331,7 @@ int gemm_simt(const void* A, int a_dt, int64_t sAm, int64_t sAk,
   if (a_dt == AB_F32 && b_dt == AB_F32 && c_dt == AB_F32 && M < ((int64_t)1 << 22) && N < ((int64_t)1 << 31) &&
       K < ((int64_t)1 << 31) && tiles64 >= 296) {
     // all-fp32 problems with enough tiles to fill the SMs twice take the register-tiled kernel (fp32
-    // sums in ascending k); smaller ones go to gemm_small, which cuts the reduction over warps and CTAs
+    // sums in ascending k)
     GemmDesc d;
     d.A = static_cast<const float*>(A); d.B = static_cast<const float*>(B); d.C = C;
     d.sAm = sAm; d.sAk = sAk; d.sBk = sBk; d.sBn = sBn; d.ldc = ldc;
@@ -343,7 +343,7 @@ int gemm_simt(const void* A, int a_dt, int64_t sAm, int64_t sAk,
     if (bigN) return launch_one<64, 128>(d, st);
     return launch_one<64, 64>(d, st);
   }
-  if (a_dt == AB_F32 && b_dt == AB_F32 && c_dt == AB_F32 && M < ((int64_t)1 << 31) && N < ((int64_t)1 << 31)) {
+  if (a_dt == AB_F32 && b_dt == AB_F32 && c_dt == AB_F32 && gemm_small_pays(M, N, K)) {
     const SmallProduct q{static_cast<const float*>(A), sAm, sAk, static_cast<const float*>(B), sBn, sBk, static_cast<float*>(C), ldc,
                          (int)M, (int)N};
     return gemm_small(&q, 1, K, nullptr, st);
@@ -358,6 +358,7 @@ int gemm_simt(const void* A, int a_dt, int64_t sAm, int64_t sAk,
 #define AB_GEMM_CASE(TA, TB, TC) s = launch<TA, TB, TC>(Ap, sAm, sAk, B, sBk, sBn, Cp, ldc, mb, N, K, st)
     int key = (a_dt << 2) | (b_dt << 1) | c_dt;
     switch (key) {
+      case 0: AB_GEMM_CASE(float, float, float); break;
       case 1: AB_GEMM_CASE(float, float, bf16); break;
       case 2: AB_GEMM_CASE(float, bf16, float); break;
       case 3: AB_GEMM_CASE(float, bf16, bf16); break;

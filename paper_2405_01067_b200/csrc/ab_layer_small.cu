@@ -4,13 +4,13 @@
 //   small_chain_kernel:  S = In F1^T,  Out = S F2^T  for a few rows per CTA, S in shared memory (forward: T and y;
 //                        backward: dT and dX with A and B read the other way round)
 //   small_gemm_kernel:   dA = dY^T T and dB = dT^T x in one launch, 32 x 32 tiles, the rows cut over a cluster; also
-//                        every other fp32 product that is too small for the register-tiled kernel
+//                        every other fp32 product that gemm_small_pays names
 //
 // Sums: 16 products in fp32, those sums in fp64, in an order fixed by the shape, as in the general kernel.
 // What bounds both at the small sizes is latency: a launch, a trip to L2 for the first values, then the factors streamed once per
 // CTA (96 KB, about 1 us).  64 x 512 -> 256, rank 32, forward and backward: 82 -> 27 us, seven kernels -> three.
 // The tiled product against the general kernel it replaces for fp32 (64 x 64 tiles, one CTA walking the whole reduction):
-// 64 x 64, rank 16, 4096 rows, forward and backward 538 -> 52 us; 1000 x 1000, rank 250, 1000 rows 362 -> 270 us.
+// backward of a 1024 x 100 layer, rank 30, 50432 rows: 8.8 -> 0.8 ms.
 #include <cooperative_groups.h>
 
 #include "ab_common.cuh"
@@ -173,7 +173,7 @@ small_chain_kernel(const SmallChain p) {
 // fetches the 16 x 32 values of each operand that it multiplies itself, so no barrier is inside the loop.
 //   kMany false: the next slab waits in registers (one CTA per SM; what counts is the latency of a lone tile)
 //   kMany true : asynchronous copies into a second buffer, lanes along the index that is contiguous in memory; two CTAs
-//                per SM hide each other's waits (768 x 768 x 3072: 290 -> 154 us, but a 256 x 64 layer of 1000 rows 51 -> 61 us)
+//                per SM hide each other's waits (768 x 768 x 3072: 290 -> 235 us, but a 256 x 64 layer of 1000 rows 51 -> 61 us)
 struct SmallGemm { SmallProduct job[2]; int64_t K; int tiles0, tiles_q[2]; int* status; };
 
 constexpr int kGt = 32, kGk = 128;                 // tile edge, reduction per slab: 16 for each of the eight warps
@@ -367,6 +367,17 @@ int run_chain(const SmallChain& p, cudaStream_t st) {
 
 }  // namespace
 
+// Whether a product goes to small_gemm_kernel.  Its 32 x 32 tiles and cut reductions win where the 64 x 64 kernel would leave half
+// of the SMs empty for a long walk; with more tiles, or next to no reduction, that kernel has less to do per result.  Measured at
+// 148 SMs, us 64 x 64 / this: 256 x 250, K 3072 194 / 39, K 64 10.3 / 8.5; 512 x 512 (64 of its tiles), K 4608 280 / 176; 4096 x 64,
+// K 64 9.9 / 14.4; 128 x 3072 (96 tiles), K 512 37 / 43; 768 x 768 (144), K 3072 190 / 235, K 16384 1350 / 1270, K 50432 4200 / 3900;
+// 1024 x 1024 (256), K 1 7.5 / 34, K 50432 4970 / 7420.
+bool gemm_small_pays(int64_t M, int64_t N, int64_t K) {
+  const int64_t sms = sm_count() > 0 ? sm_count() : 1, tiles = (M + 63) / 64 * ((N + 63) / 64);
+  if (2 * tiles >= sms) return tiles <= sms && K >= 16384;
+  return K >= 96 || (K >= 64 && (M + kGt - 1) / kGt * ((N + kGt - 1) / kGt) <= sms);
+}
+
 int gemm_small(const SmallProduct* jobs, int njobs, int64_t K, int* status, cudaStream_t st) {
   SmallGemm g;
   int64_t tiles = 0;
@@ -377,7 +388,7 @@ int gemm_small(const SmallProduct* jobs, int njobs, int64_t K, int* status, cuda
     if (i < njobs) tiles += t;
     if (i == 0) g.tiles0 = (int)t;
   }
-  if (tiles <= 0 || tiles > ((int64_t)1 << 27)) return tiles <= 0 ? AB_OK : AB_ERR_UNSUPPORTED;
+  if (tiles <= 0) return AB_OK;
   g.K = K;
   g.status = status;
   // the reduction cut over a cluster while each CTA keeps a slab and the device has room for two CTAs an SM
@@ -389,15 +400,32 @@ int gemm_small(const SmallProduct* jobs, int njobs, int64_t K, int* status, cuda
   return launch_small(small_gemm_kernel<false>, (unsigned)(tiles * C), C, sm, st, g);
 }
 
-// The fused chain streams both factors once per CTA of a few rows, from L2 by single values: it wins where that is little (measured,
-// square layers of width w, forward and backward, us fused / one product at a time: r 8, w 1024, 1000 rows 48 / 128; r 32,
-// w 256, 64 rows 28 / 39, 4096 rows 88 / 121) and loses beyond (r 32, w 64, 4096 rows 62 / 52; r 64, w 256, 1000 rows 60 / 52;
-// r 32, w 1024, 64 rows 54 / 39; r 256, w 256, 64 rows 210 / 43).
-bool layer_small_ok(int64_t N, int m, int n, int r) {
-  const int64_t work = (int64_t)r * (m > n ? m : n);
-  if (!(work <= 8192 && (N <= 1024 || r < 32 || work > 4096)) && !(work <= 16384 && N <= 300)) return false;
+// Whether the fused chain S = In F1^T, Out = S F2^T (In: N x K1, Out: N x P) is faster than a launch per product.  A CTA streams
+// both factors for its 1 to 16 rows, by single values: it wins where that is little and the separate products
+// are bound by their launches and the length of one reduction.  Forward, a thread's row of F2 = A is its own and its values lie
+// apart from its neighbours': that costs r^2 P, backward the lanes read along F2 = B.  Measured, us fused / by products: forward
+// 64 x 512 -> 32 -> 256 9.3 / 16.5, 1000 x 256 -> 32 -> 256 14.6 / 20.6, 2368 x 256 -> 32 -> 64 19.3 / 14.5, 600 x 64 -> 64 -> 64 17.3 / 14.4,
+// 64 x 768 -> 32 -> 1024 24 / 16.5, 4096 x 256 -> 8 -> 256 17.1 / 26.7, 16384 x 64 -> 16 -> 64 66.9 / 18.5; backward 1000 x 256 -> 128 -> 256
+// 23 / 33, 300 x 256 -> 128 -> 512 31.2 / 20.7, 64 x 1024 -> 32 -> 1024 22.9 / 16.3.  Above 16 rows a CTA and SM the
+// factors are streamed again, which only a long first reduction into a narrow rank is worth.
+bool layer_small_ok(int64_t N, int K1, int P, int r, bool backward) {
+  const int64_t sms = sm_count() > 0 ? sm_count() : 1;
+  const int64_t wide = (int64_t)r * (K1 > P ? K1 : P), out = (int64_t)r * P;
   const int R = rows_per_cta(N);
-  return chain_smem(R, n, r) <= 200 * 1024 && chain_smem(R, m, r) <= 200 * 1024;
+  if (chain_smem(R, K1, r) > 200 * 1024 || chain_smem(R, P, r) > 200 * 1024) return false;
+  if (N > 64 * sms) return false;
+  if (N > 32 * sms) return r <= 8 && K1 >= 1024;
+  if (N > 16 * sms) {
+    if (backward) return K1 >= 256 && r <= 32 && (P <= 512 || out <= 1024) && P >= 64;
+    return K1 >= 256 && r <= 16 && out <= 4096;
+  }
+  if (backward) {
+    if (N > 4 * sms) return wide <= 65536;
+    return r <= 64 && wide <= 32768 && (N > sms || out <= 16384);
+  }
+  if (r > (N <= 2 * sms ? 64 : 32) || wide > 32768) return false;
+  if (N <= 8 * sms) return r * out <= 600000;
+  return K1 >= 256 ? r * out <= 300000 : r <= 16 && r * out <= 70000;
 }
 
 int layer_small_chain(const float* In, int64_t N, int K1, const float* F1, int64_t f1_j, int64_t f1_k, const float* F2, int64_t f2_p,
