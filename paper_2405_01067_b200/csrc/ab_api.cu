@@ -345,6 +345,15 @@ int ab_recombine(const void* Abar, const void* Bbar, float* W, int m, int n, int
   // The tensor-core kernel reports its waits to the workspace's first int; without one the product runs on the fp32 pipes.
   if (!ws || !aligned(ws, 256) || ws_bytes < 256 || !gemm_tc_available())
     return gemm_simt(Abar, dt, ldA, 1, Bbar, dt, ldB, 1, W, AB_F32, n, m, n, r, st);
+  // bf16 factors: the split kernel's converters move every operand tile through registers, which a product of several rounds
+  // pays for; the GEMM that loads its tiles by TMA has wider tiles and a later start.  Measured, us split / TMA: 3072 x 768, rank 256
+  // 6.6 / 7.3, rank 384 7.6 / 7.5, rank 768 10.9 / 9.3; 3072 x 1536, rank 128 7.7 / 7.3, rank 768 18.6 / 9.6; 3072 x 3072, rank 192
+  // 14.4 / 9.9, rank 768 34.3 / 15.6 (128 x 256 tiles times slabs of 64: 288, 432, 864; 288, 1728; 864, 3456).
+  if (dt == AB_BF16 && (int64_t)((m + 127) / 128) * ((n + 255) / 256) * ((r + 63) / 64) >= 2 * (int64_t)sm_count()) {
+    TcProblem q;
+    q.A = {Abar, ldA, false}; q.B = {Bbar, ldB, true}; q.C = W; q.ldc = n; q.M = m; q.N = n; q.K = r; q.c_f32 = true; q.ksplit = 1;
+    if (gemm_tc_problem_ok(q)) return gemm_tc_batched(&q, 1, static_cast<int*>(ws), st);
+  }
   SplitGemm p;
   memset(&p, 0, sizeof(p));
   p.A = Abar; p.lda = ldA; p.B = Bbar; p.ldb = ldB; p.b_mn = 1; p.C = W; p.ldc = n; p.M = m; p.N = n; p.K = r;

@@ -66,3 +66,20 @@ def test_lone_layer_gram_slices(ab, m, n, r):
     ref = np.linalg.svd(a.astype(np.float64) @ b.astype(np.float64), compute_uv=False)[:r]
     assert int(status[0].item()) == 0 and int(r_out[0].item()) == r
     assert np.max(np.abs(sigma[0].cpu().numpy() - ref) / ref) <= 1e-5      # well conditioned: a few 2^-24 sqrt(n)
+
+
+@pytest.mark.parametrize("m,n,r", [(1920, 2440, 296), (1921, 2440, 312), (3000, 1992, 200), (300, 20000, 128), (2560, 1024, 2000)])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_large_bf16_recombine(m, n, r, shift, ab):
+    """bf16 factors of many tiles: loaded by TMA where rows and bases allow it, else (shift) through the converters."""
+    g = torch.Generator(device="cuda").manual_seed(m + r)
+    big_a, big_b = (torch.randn(s, generator=g, device="cuda").bfloat16() for s in ((m * r + 8,), (r * n + 8,)))
+    A, B = big_a[shift:shift + m * r].view(m, r), big_b[shift:shift + r * n].view(r, n)
+    W = torch.full((m, n), float("nan"), device="cuda")
+    ws = ab.workspace(256, "cuda")
+    ws[:4] = 255
+    ab.ab_recombine(A, B, W=W, ws=ws)
+    want = A.double() @ B.double()
+    assert ab.workspace_status(ws) == 0
+    # products are exact, fp32 sums of up to 2000: sqrt(2000) 2^-24 = 2.7e-6 at worst
+    assert float((W.double() - want).norm() / want.norm()) <= 2.7e-6
