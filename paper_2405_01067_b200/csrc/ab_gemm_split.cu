@@ -292,7 +292,10 @@ __device__ __forceinline__ void gemm_split_body(const SplitGemm* probs, int npro
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsMma));
     if (warp == kMmaWarp) {
       // ---------------------------------------------------------- MMA issuer (see elect_one for the uniform loop)
-      if constexpr (kOne) dep_launch();
+      if constexpr (kOne) {      // no bounded wait starts before the kernel in front is done: it may take longer than a wait may
+        dep_wait();
+        dep_launch();
+      }
       TileReader<kOne, BN> rd;
       int slot = 0, ph = 0;
       bool ok = true;

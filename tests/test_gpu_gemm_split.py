@@ -83,3 +83,20 @@ def test_large_bf16_recombine(m, n, r, shift, ab):
     assert ab.workspace_status(ws) == 0
     # products are exact, fp32 sums of up to 2000: sqrt(2000) 2^-24 = 2.7e-6 at worst
     assert float((W.double() - want).norm() / want.norm()) <= 2.7e-6
+
+
+def test_a_kernel_in_front_may_take_longer_than_a_wait(ab):
+    """The waits inside the product are bounded by a second; a kernel in front of it that takes a second (the self-test of
+    the chain's waits) and lets it start early is not its own time."""
+    rng = np.random.default_rng(9)
+    a, b = rng.standard_normal((300, 64)).astype(np.float32), rng.standard_normal((64, 200)).astype(np.float32)
+    A, B, W = torch.from_numpy(a).cuda(), torch.from_numpy(b).cuda(), torch.empty((300, 200), device="cuda")
+    stall = ab.workspace(int(ab.lib().ab_selftest_chain_stall_workspace_bytes()), "cuda")
+    ws = ab.workspace(256, "cuda")
+    stream = torch.cuda.current_stream().cuda_stream
+    torch.cuda.synchronize()
+    assert ab.lib().ab_selftest_chain_stall(stall.data_ptr(), stall.numel(), 1_000_000, stream) == 0
+    ab.ab_recombine(A, B, W=W, ws=ws)
+    torch.cuda.synchronize()
+    assert ab.workspace_status(stall) == ab.AB_ERR_TIMEOUT and ab.workspace_status(ws) == 0
+    assert orc.rel_frob(W.cpu().numpy().astype(np.float64), orc.recombine(a, b)) <= 1e-6
