@@ -87,6 +87,18 @@ int ab_selftest_chain_stall(void* ws, size_t ws_bytes, unsigned limit_us, void* 
 size_t ab_selftest_chain_stall_workspace_bytes(void);
 
 /*
+ * Self-test of what a split does when its direct eigensolver cannot vouch for its vectors (no counterpart in the paper): count
+ * (1 .. 64) fp32 matrices [m,n] of W, one behind the other, are split as by ab_svd_split with sigma_cutoff 0, but matrix i
+ * goes through the Jacobi fallback if bit i of flagged is set, and a solver_status other than AB_OK takes the place of what the solver's
+ * first call reported about its waits.  A [count][m,r_max], B [count][r_max,n], sigma [count][min(r_max,m,n)]; r_out and
+ * dev_status: device int[count].  Short sides above 1184 do not take the direct solver and ignore both.
+ */
+int ab_selftest_split_fallback(const float* W, int m, int n, int r_max, int count, unsigned long long flagged, int solver_status,
+                               float* A, float* B, float* sigma, int* r_out, int* dev_status, void* ws, size_t ws_bytes,
+                               void* cuda_stream);
+size_t ab_selftest_split_fallback_workspace_bytes(int m, int n, int r_max, int count);
+
+/*
  * Scratch bytes a call needs (0 if none).  Arguments a given op does not use are ignored
  * (pass 0).  For AB_OP_SVD_SPLIT, r is r_max.  Returns 0 for unknown ops or bad sizes.
  */
@@ -250,7 +262,8 @@ int ab_recombine_mean(const void* A_copies, int64_t strideA, const void* B_copie
  *   W [m,n] dense of type w_dt.  A [m,r_max] (row stride r_max) and B [r_max,n] of type
  *   out_dt; columns of A and rows of B with index >= r' are zero.  sigma [r_cap] fp32,
  *   descending up to rounding; r_out: device int that receives r'; dev_status: device
- *   int that receives AB_OK, AB_ERR_NOT_CONVERGED or AB_ERR_ACCURACY.  sigma_cutoff = 0 keeps r_cap.
+ *   int that receives AB_OK, AB_ERR_NOT_CONVERGED, AB_ERR_ACCURACY or AB_ERR_TIMEOUT (a bounded wait between
+ *   the CTAs of the eigensolver ran out; the outputs are then undefined).  sigma_cutoff = 0 keeps r_cap.
  *   Accuracy domain: the decomposition works on the Gram matrix of the shorter side in fp32, so
  *   singular values below 2% of the largest lose relative accuracy (they keep absolute accuracy
  *   1e-6 * s_0).  If a value between 1e-5 and 2e-2 of the largest is among the kept ones,

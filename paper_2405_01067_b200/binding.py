@@ -26,6 +26,7 @@ EXPORTS = ["ab_status_string", "ab_version", "ab_launch_count", "ab_workspace_by
            "ab_group_average", "ab_recombine", "ab_svd_split", "ab_group_sync", "ab_sync_workspace_bytes",
            "ab_layer_forward_static", "ab_static_scratch_elems", "ab_adamw_step", "ab_lr_rebound_factor", "ab_selftest_bounded_wait",
            "ab_selftest_chain_stall", "ab_selftest_chain_stall_workspace_bytes",
+           "ab_selftest_split_fallback", "ab_selftest_split_fallback_workspace_bytes",
            "ab_dense_forward", "ab_dense_backward", "ab_conv3x3_forward", "ab_conv3x3_backward",
            "ab_conv3x3_workspace_bytes", "ab_recombine_mean"]
 
@@ -88,6 +89,10 @@ def lib() -> ctypes.CDLL:
     L.ab_selftest_chain_stall.restype = c_int
     L.ab_selftest_chain_stall.argtypes = [c_void_p, c_size_t, ctypes.c_uint, c_void_p]
     L.ab_selftest_chain_stall_workspace_bytes.restype = c_size_t
+    L.ab_selftest_split_fallback.restype = c_int
+    L.ab_selftest_split_fallback.argtypes = [c_void_p] + [c_int] * 4 + [ctypes.c_ulonglong, c_int] + [c_void_p] * 6 + [c_size_t, c_void_p]
+    L.ab_selftest_split_fallback_workspace_bytes.restype = c_size_t
+    L.ab_selftest_split_fallback_workspace_bytes.argtypes = [c_int] * 4
     L.ab_dense_forward.restype = c_int
     L.ab_dense_forward.argtypes = [c_void_p] * 3 + [c_int64, c_int, c_int, c_int, c_void_p, c_size_t, c_void_p]
     L.ab_dense_backward.restype = c_int
@@ -119,6 +124,22 @@ def ab_selftest_chain_stall(limit_us: int = 1000, stream=None) -> int:
     ws = workspace(int(lib().ab_selftest_chain_stall_workspace_bytes()), "cuda")
     _check(lib().ab_selftest_chain_stall(_ptr(ws), ws.numel(), int(limit_us), _stream(stream)), "ab_selftest_chain_stall")
     return workspace_status(ws)
+
+
+def ab_selftest_split_fallback(W, r_max: int, flagged: int, solver_status: int = AB_OK, stream=None):
+    """Splits W (count, m, n) with the matrices of `flagged` (a bit each) sent through the Jacobi fallback.  Returns (A, B,
+    sigma, r_out, status), a matrix per row."""
+    _dev_ok(W)
+    count, m, n = W.shape
+    dev = W.device
+    A, B = torch.empty((count, m, r_max), device=dev), torch.empty((count, r_max, n), device=dev)
+    sigma = torch.empty((count, min(r_max, m, n)), device=dev)
+    r_out, status = (torch.zeros((count,), dtype=torch.int32, device=dev) for _ in range(2))
+    ws = workspace(int(lib().ab_selftest_split_fallback_workspace_bytes(m, n, r_max, count)), dev)
+    _check(lib().ab_selftest_split_fallback(_ptr(W), m, n, r_max, count, int(flagged), int(solver_status), _ptr(A), _ptr(B), _ptr(sigma),
+                                            _ptr(r_out), _ptr(status), _ptr(ws), ws.numel(), _stream(stream)),
+           "ab_selftest_split_fallback")
+    return A, B, sigma, r_out, status
 
 
 def ab_launch_count() -> int:

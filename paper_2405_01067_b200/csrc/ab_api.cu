@@ -386,6 +386,38 @@ int ab_svd_split(const void* W, int m, int n, int r_max, float sigma_cutoff,
   return svd_batch(&it, 1, sigma_cutoff, ws, ws_bytes, static_cast<cudaStream_t>(cuda_stream));
 }
 
+static std::vector<SvdItem> selftest_split_items(const float* W, int m, int n, int r_max, int count, float* A, float* B, float* sigma,
+                                                 int* r_out, int* dev_status) {
+  std::vector<SvdItem> items((size_t)count);
+  const int r_cap = r_max < m ? (r_max < n ? r_max : n) : (m < n ? m : n);
+  for (int i = 0; i < count; ++i) {
+    SvdItem& it = items[i];
+    it.w_dt = it.out_dt = AB_F32; it.m = m; it.n = n; it.r_max = r_max;
+    it.W = W + (size_t)i * m * n; it.A = A + (size_t)i * m * r_max; it.B = B + (size_t)i * r_max * n;
+    it.sigma = sigma + (size_t)i * r_cap; it.r_out = r_out + i; it.dev_status = dev_status + i;
+  }
+  return items;
+}
+
+size_t ab_selftest_split_fallback_workspace_bytes(int m, int n, int r_max, int count) {
+  if (m <= 0 || n <= 0 || r_max <= 0 || count < 1 || count > 64) return 0;
+  const std::vector<SvdItem> items = selftest_split_items(nullptr, m, n, r_max, count, nullptr, nullptr, nullptr, nullptr, nullptr);
+  return svd_batch_ws(items.data(), count) + 256;
+}
+
+int ab_selftest_split_fallback(const float* W, int m, int n, int r_max, int count, unsigned long long flagged, int solver_status,
+                               float* A, float* B, float* sigma, int* r_out, int* dev_status, void* ws, size_t ws_bytes,
+                               void* cuda_stream) {
+  if (m <= 0 || n <= 0 || r_max <= 0 || count < 1 || count > 64 || !W || !A || !B || !sigma || !r_out || !dev_status)
+    return AB_ERR_INVALID_ARG;
+  if ((m < n ? m : n) > 3072) return AB_ERR_UNSUPPORTED;
+  if (!ws || !aligned(ws, 256)) return AB_ERR_WORKSPACE;
+  if (!have_device()) return AB_ERR_CUDA;
+  const std::vector<SvdItem> items = selftest_split_items(W, m, n, r_max, count, A, B, sigma, r_out, dev_status);
+  const SvdSelftest st{flagged, solver_status};
+  return svd_batch(items.data(), count, 0.f, ws, ws_bytes, static_cast<cudaStream_t>(cuda_stream), &st);
+}
+
 // Workspace of ab_group_sync: per matrix Abar, Bbar (fp32) and W (fp32), then the SVD batch.
 static size_t sync_layout(const ab_sync_desc* d, int L, int dt, void* ws, std::vector<float*>* Ab,
                           std::vector<float*>* Bb, std::vector<float*>* Wd, std::vector<SvdItem>* items, void** svd_ws) {

@@ -201,7 +201,11 @@ struct SvdItem {
   int* dev_status;
 };
 size_t svd_batch_ws(const SvdItem* items, int L);
-int svd_batch(const SvdItem* items, int L, float sigma_cutoff, void* ws, size_t ws_bytes, cudaStream_t st);
+// Self-test of what follows the direct solver: the first 64 matrices whose bit is set are flagged as if it had left their vectors
+// less than orthogonal; a status other than AB_OK stands for a wait that ran out in the solver's first call.
+struct SvdSelftest { unsigned long long flagged; int solver_status; };
+int svd_batch(const SvdItem* items, int L, float sigma_cutoff, void* ws, size_t ws_bytes, cudaStream_t st,
+              const SvdSelftest* selftest = nullptr);
 
 // ---- direct symmetric eigensolver (ab_eig.cu) ---------------------------------------------------
 // Leading eigenvectors of `count` symmetric matrices, fp64 inside: any orders up to kEigSmallMax in one call, or

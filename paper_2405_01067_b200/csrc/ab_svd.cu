@@ -555,8 +555,9 @@ long_norms_kernel(const float* __restrict__ Y, int64_t st_, int64_t sk, int L, i
   }
 }
 
+// solver: null, or what the direct solver's waits reported for the call this matrix was part of
 __global__ void rank_rule_kernel(const float* __restrict__ sigma, int r_cap, float cutoff, int* __restrict__ r_out,
-                                 const JState* __restrict__ st, int* __restrict__ dev_status) {
+                                 const JState* __restrict__ st, const int* __restrict__ solver, int* __restrict__ dev_status) {
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   float top = 0.f;
   for (int k = 0; k < r_cap; ++k) top = fmaxf(top, sigma[k]);
@@ -566,12 +567,19 @@ __global__ void rank_rule_kernel(const float* __restrict__ sigma, int r_cap, flo
   if (keep < 1) keep = 1;
   *r_out = keep;
   if (dev_status) {
-    int code = st->status;
+    int code = solver && *solver != AB_OK ? *solver : st->status;
     if (code == AB_OK)
       for (int k = 0; k < keep; ++k)
         if (sigma[k] < kDomainRel * top && sigma[k] > kZeroRel * top) code = AB_ERR_ACCURACY;
     *dev_status = code;
   }
+}
+
+// What the self-test of the fallback makes of the direct solver's verdicts (see SvdSelftest).
+__global__ void force_fallback_kernel(int* __restrict__ flags, int count, int* __restrict__ solver, unsigned long long flagged, int status) {
+  const int i = threadIdx.x;
+  if (i < count && (flagged >> i & 1ull)) flags[i] = 1;
+  if (i == 0 && status != AB_OK) *solver = status;
 }
 
 // long factor: F(t,k) = Ylong(k,t) / sqrt(sigma_k); short factor: F(k,u) = sqrt(sigma_k) Vr[k][u].
@@ -634,8 +642,8 @@ struct Layout {
   std::map<int, float*> X, Vt;
   std::map<int, JState*> st;
   std::map<int, void*> jobs;                  // short side up to kEigSmallMax: the in-shared-memory Jacobi's scratch
-  std::map<int, double*> eig;                 // direct solver: its scratch, EigJobs, fallback flags (and behind the flags of
-  std::map<int, int*> flags;                  //   a group two words on which the blocks of the fallback meet)
+  std::map<int, double*> eig;                 // direct solver: its scratch, EigJobs, fallback flags (and behind the flags of a
+  std::map<int, int*> flags;                  //   group two words on which the blocks of the fallback meet and the solver's status)
   std::map<int, EigJob*> ejobs;
   std::vector<ItemWs> item;
   size_t bytes;
@@ -644,6 +652,8 @@ struct Layout {
 // Matrices of one order that are solved (and hold scratch) at the same time: two or three of the large ones fill the
 // device in the reduction, a dozen in the steps behind it.
 int eig_chunk(int s) { return s <= kEigSmallMax ? 1 << 20 : 12; }
+// one status word per call of the direct solver: a wait that runs out leaves every matrix of that call undone
+int eig_calls(int s, int count) { return (count + eig_chunk(s) - 1) / eig_chunk(s); }
 
 Layout make_layout(const SvdItem* items, int L, void* ws) {
   Layout lo;
@@ -657,7 +667,7 @@ Layout make_layout(const SvdItem* items, int L, void* ws) {
     if (g.first <= kEigSmallMax) lo.jobs[g.first] = ar.take_n<char>(rows_jacobi_scratch_bytes((int)cnt));
     if (g.first <= eig_max()) {
       lo.ejobs[g.first] = ar.take_n<EigJob>(cnt);
-      lo.flags[g.first] = ar.take_n<int>(cnt + 2);
+      lo.flags[g.first] = ar.take_n<int>(cnt + 2 + eig_calls(g.first, (int)cnt));
       lo.eig[g.first] = ar.take_n<double>(std::min(cnt, (size_t)eig_chunk(g.first)) * eig_ws_doubles(g.first));
     }
   }
@@ -752,7 +762,8 @@ size_t svd_batch_ws(const SvdItem* items, int L) {
   return make_layout(items, L, nullptr).bytes;
 }
 
-int svd_batch(const SvdItem* items, int L, float sigma_cutoff, void* ws, size_t ws_bytes, cudaStream_t stream) {
+int svd_batch(const SvdItem* items, int L, float sigma_cutoff, void* ws, size_t ws_bytes, cudaStream_t stream,
+              const SvdSelftest* selftest) {
   Layout lo = make_layout(items, L, ws);
   if (lo.bytes > ws_bytes) return AB_ERR_WORKSPACE;
   // 1. Gram matrices into X
@@ -788,10 +799,14 @@ int svd_batch(const SvdItem* items, int L, float sigma_cutoff, void* ws, size_t 
         eig_bind(q, lo.eig[s] + (size_t)(j % chunk) * eig_ws_doubles(s));
       }
       AB_CUDA_OK(cudaMemsetAsync(lo.st[s], 0, sizeof(JState) * count, stream));
-      AB_CUDA_OK(cudaMemsetAsync(lo.flags[s], 0, sizeof(int) * (count + 2), stream));
+      AB_CUDA_OK(cudaMemsetAsync(lo.flags[s], 0, sizeof(int) * (count + 2 + eig_calls(s, count)), stream));
       AB_TRY(upload_async(lo.ejobs[s], ej.data(), ej.size() * sizeof(EigJob), stream));
       for (int j = 0; j < count; j += chunk)
-        AB_TRY(eig_direct(ej.data() + j, lo.ejobs[s] + j, std::min(chunk, count - j), s, &lo.st[s][j].status, stream));
+        AB_TRY(eig_direct(ej.data() + j, lo.ejobs[s] + j, std::min(chunk, count - j), s, lo.flags[s] + count + 2 + j / chunk, stream));
+      if (selftest) {
+        force_fallback_kernel<<<1, 64, 0, stream>>>(lo.flags[s], count, lo.flags[s] + count + 2, selftest->flagged, selftest->solver_status);
+        AB_LAUNCH_OK();
+      }
       if (small) {
         AB_TRY(rows_jacobi(lo.X[s], lo.Vt[s], lam, &lo.st[s]->status, sizeof(JState), lo.flags[s], count, s, lo.jobs[s], stream));
         int r_need = 0;
@@ -844,7 +859,9 @@ int svd_batch(const SvdItem* items, int L, float sigma_cutoff, void* ws, size_t 
       }
       long_norms_kernel<<<(p.r_cap + 31) / 32, 256, 0, stream>>>(w.Y, yt, yk, p.L, p.r_cap, it.sigma);
       AB_LAUNCH_OK();
-      rank_rule_kernel<<<1, 32, 0, stream>>>(it.sigma, p.r_cap, sigma_cutoff, it.r_out, lo.st[s] + j, it.dev_status);
+      const int count = (int)g.second.size();
+      const int* solver = solved ? lo.flags[s] + count + 2 + j / eig_chunk(s) : nullptr;
+      rank_rule_kernel<<<1, 32, 0, stream>>>(it.sigma, p.r_cap, sigma_cutoff, it.r_out, lo.st[s] + j, solver, it.dev_status);
       AB_LAUNCH_OK();
       // tall: A is the long factor (A[t][k], strides r_max, 1), B the short one (B[k][u], strides n, 1)
       // wide: B is the long factor (B[k][t], strides 1, n),     A the short one (A[u][k]: k stride 1, u stride r_max)
