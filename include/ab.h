@@ -15,6 +15,7 @@
  *    low-priority helper stream per device that ab_group_sync creates on first use (see there).
  *  - Calls are asynchronous on `cuda_stream` (a cudaStream_t passed as void*; NULL = the
  *    default stream).  Buffers must stay valid until the stream has run the call.
+ *  - Calls may be captured into a CUDA graph: what a call builds on the host becomes part of the graph.
  *  - Arguments that can be checked on the host (NULL, non-positive sizes, r > min(m,n),
  *    a short workspace, a misaligned pointer) are rejected with a negative status and
  *    nothing is launched.  Conditions only the device can see (an iteration that did not

@@ -24,7 +24,29 @@ int sm_count() {
   return sms;
 }
 
+// A piece of a host table as a kernel argument.
+struct TablePiece { uint4 v[240]; };
+__global__ void __launch_bounds__(256)
+put_table_kernel(const __grid_constant__ TablePiece p, unsigned char* __restrict__ dst, int bytes) {
+  const unsigned char* src = reinterpret_cast<const unsigned char*>(p.v);
+  for (int i = threadIdx.x; i < bytes; i += 256) dst[i] = src[i];
+}
+
 int upload_async(void* dst, const void* src, size_t bytes, cudaStream_t st) {
+  // Under stream capture a copy node would read the host table when the graph is launched, long after the table is gone; a kernel's
+  // arguments are part of the graph.
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  AB_CUDA_OK(cudaStreamIsCapturing(st, &cap));
+  if (cap != cudaStreamCaptureStatusNone) {
+    for (size_t o = 0; o < bytes; o += sizeof(TablePiece)) {
+      TablePiece p;
+      const int n = (int)(bytes - o < sizeof(TablePiece) ? bytes - o : sizeof(TablePiece));
+      memcpy(p.v, static_cast<const char*>(src) + o, (size_t)n);
+      put_table_kernel<<<1, 256, 0, st>>>(p, static_cast<unsigned char*>(dst) + o, n);
+      AB_LAUNCH_OK();
+    }
+    return AB_OK;
+  }
   constexpr size_t kPiece = 48 * 1024;
   for (size_t o = 0; o < bytes; o += kPiece)
     AB_CUDA_OK(cudaMemcpyAsync(static_cast<char*>(dst) + o, static_cast<const char*>(src) + o, bytes - o < kPiece ? bytes - o : kPiece,

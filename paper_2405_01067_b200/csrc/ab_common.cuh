@@ -137,7 +137,8 @@ int gemm_split_batched(const SplitGemm* d_probs, const SplitBatch& b, int* statu
 int gemm_split_one(SplitGemm p, bool src_bf16, int* status, cudaStream_t st);    // one problem; clears *status first
 
 // Copies a host table to the device in pieces the runtime stages without waiting for the stream (a pageable copy of
-// more than 64 KB waits until the stream has drained).
+// more than 64 KB waits until the stream has drained), under stream capture as arguments of kernels: either way the table may go
+// when the call returns.
 int upload_async(void* dst, const void* src, size_t bytes, cudaStream_t st);
 
 // ---- dense layer of the full-rank phases (ab_dense.cu) ------------------------------------------
