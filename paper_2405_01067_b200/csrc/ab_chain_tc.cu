@@ -31,7 +31,7 @@ constexpr int kMaxStages = 10;
 constexpr int kMaxStages2 = 6;         // 32 KB slots of the second product, carved from the same ring memory
 constexpr int kChunk = 256;            // output columns per accumulator of the second product
 constexpr int kAtom2Bytes = kChunk * 128;   // one 256 x 64 tile of F2
-constexpr int kSmemLimit = 227 * 1024;
+constexpr int kSmemLimit = kMaxSmem;
 constexpr int kTmemCols = 512;
 constexpr int kEpiThreads = 128;
 
@@ -1206,7 +1206,7 @@ int launch_chain_ex(const ChainLaunch& L, cudaStream_t st) {
   q.wait_ns = L.wait_ns; q.status = L.status;
   if (conv) q.cv = *L.cv;
   q.out_ptr = static_cast<bf16*>(L.Out); q.s_ptr = static_cast<bf16*>(L.Sg); q.s_ld = L.s_ld; q.s_cols = L.s_cols;
-  AB_CUDA_OK(cudaFuncSetAttribute(chain_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem));
+  AB_CUDA_OK(allow_smem(chain_kernel));
   AB_LAUNCH_DEP(chain_kernel, dim3((unsigned)grid), dim3(kChainThreads), pl.smem, st, tmIn, tmIn4, tmF1, tmF2, tmOut,
                 tmS, q);
   AB_LAUNCH_OK();
@@ -1381,7 +1381,7 @@ int chain_tc_backward(const void* x, const void* dY, const void* A, const void* 
     p.r = rp; p.natoms = gp.natoms; p.ns = gp.ns; p.slot_bytes = gp.slot_bytes;
     p.slices = slices; p.rows_per_slice = gp.sp.per * 64; p.N = (int)N; p.clear_status = first ? 1 : 0; p.status = w.status;
     p.job0_independent = (after_chain && dA) ? 1 : 0;   // job 0 is the dA job whenever dA is asked for
-    AB_CUDA_OK(cudaFuncSetAttribute(grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gp.smem));
+    AB_CUDA_OK(allow_smem(grad_kernel));
     const unsigned grid = (unsigned)((p.job[0].chunks + p.job[1].chunks) * slices);
     AB_LAUNCH_DEP(grad_kernel, dim3(grid), dim3(192), gp.smem, st, tmAct[0], tmSmall[0], tmAct[1], tmSmall[1], p);
     AB_LAUNCH_OK();
@@ -1530,7 +1530,7 @@ int conv_tc_backward(const void* x, const void* dY, const void* A, const void* B
     p.r = rp; p.natoms = gp.natoms; p.ns = gp.ns; p.slot_bytes = gp.slot_bytes;
     p.slices = slices; p.rows_per_slice = gp.sp.per * 64; p.N = (int)N; p.clear_status = first ? 1 : 0;
     p.status = w.status; p.job0_independent = 0;
-    AB_CUDA_OK(cudaFuncSetAttribute(grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gp.smem));
+    AB_CUDA_OK(allow_smem(grad_kernel));
     AB_LAUNCH_DEP(grad_kernel, dim3((unsigned)(p.job[0].chunks * slices)), dim3(192), gp.smem, st, tmAct, tmSmall, tmAct,
                       tmSmall, p);
     AB_LAUNCH_OK();
@@ -1553,7 +1553,7 @@ int conv_tc_backward(const void* x, const void* dY, const void* A, const void* B
     const int slices = gp.sp.slices;
     p.spi = gp.spi; p.kb = gp.kb; p.bhk = gp.bhk; p.box_rows = gp.box_rows; p.cpt = gp.cpt; p.slices = slices;
     p.slabs_per_slice = gp.sp.per; p.nslabs = gp.nslabs; p.out = grad_out(gp.sp, w.pB, dB, 9 * C, r, true); p.status = w.status;
-    AB_CUDA_OK(cudaFuncSetAttribute(conv_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gp.smem));
+    AB_CUDA_OK(allow_smem(conv_grad_kernel));
     AB_LAUNCH_DEP(conv_grad_kernel, dim3((unsigned)(9 * gp.cpt * slices)), dim3(192), gp.smem, st, tmX4, tmT4, p);
     AB_LAUNCH_OK();
     if (slices > 1) {

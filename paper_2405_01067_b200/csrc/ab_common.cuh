@@ -36,6 +36,14 @@ void count_launches(long long n);
     if (_s != AB_OK) return _s;                            \
   } while (0)
 
+// Lets a kernel take all the shared memory there is beside its static words.  The limit belongs to the kernel, not to a launch: a
+// thread that set its own call's figure could lower it between another thread's setting and launch, and that launch would fail.
+constexpr int kMaxSmem = 227 * 1024;
+template <typename K>
+inline cudaError_t allow_smem(K* kernel, int static_bytes = 0) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem - static_bytes);
+}
+
 // Multiprocessors of the current device (cached per device; 0 if the query fails).  Grid sizes that are
 // meant to fill the GPU are derived from it.
 int sm_count();

@@ -324,7 +324,7 @@ small_gemm_kernel(const __grid_constant__ SmallGemm p) {
 
 template <typename K, typename P>
 int launch_small(K* kernel, unsigned grid, int cluster, size_t smem, cudaStream_t st, const P& p) {
-  if (smem > 48 * 1024) AB_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  if (smem > 48 * 1024) AB_CUDA_OK(allow_smem(kernel));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(kThreads);

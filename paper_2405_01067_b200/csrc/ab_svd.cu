@@ -405,6 +405,7 @@ jacobi_sweeps_kernel(float* Xall, float* Vall, int s, int nb, int count, float t
     for (int m = threadIdx.x; m < count; m += blockDim.x) if (flags[m]) states[m].status = AB_ERR_TIMEOUT;
 }
 
+constexpr int kJacobiStatics = 2048;      // static shared memory of the kernels above, rounded up
 template <int PB, int kCl>
 size_t jacobi_smem_bytes(int s) {
   const int s4 = (s + 3) >> 2;
@@ -696,8 +697,8 @@ Layout make_layout(const SvdItem* items, int L, void* ws) {
 template <int PB, int CL>
 int run_jacobi_cl(float* X, float* Vt, JState* st, int s, int nb, int count, cudaStream_t stream) {
   const size_t smem = jacobi_smem_bytes<PB, CL>(s);
-  if (smem > 227 * 1024) return AB_ERR_UNSUPPORTED;
-  AB_CUDA_OK(cudaFuncSetAttribute(jacobi_pair_kernel<PB, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  if (smem > kMaxSmem - kJacobiStatics) return AB_ERR_UNSUPPORTED;
+  AB_CUDA_OK(allow_smem(jacobi_pair_kernel<PB, CL>, kJacobiStatics));
   const int nbe = nb + (nb & 1);
   const int rounds = nbe > 2 ? nbe - 1 : 1;
   const float tol = jacobi_tol(s);
@@ -736,8 +737,8 @@ int run_jacobi(float* X, float* Vt, JState* st, int s, int nb, int count, cudaSt
 template <int PB>
 int run_jacobi_fallback(float* X, float* Vt, JState* st, int* flags, int s, int nb, int count, cudaStream_t stream) {
   const size_t smem = jacobi_smem_bytes<PB, 1>(s);
-  if (smem > 227 * 1024) return AB_ERR_UNSUPPORTED;
-  AB_CUDA_OK(cudaFuncSetAttribute(jacobi_sweeps_kernel<PB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  if (smem > kMaxSmem - kJacobiStatics) return AB_ERR_UNSUPPORTED;
+  AB_CUDA_OK(allow_smem(jacobi_sweeps_kernel<PB>, kJacobiStatics));
   int per_sm = 0;
   AB_CUDA_OK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, jacobi_sweeps_kernel<PB>, 256, smem));
   const int sms = sm_count();

@@ -43,6 +43,7 @@ constexpr float kEigThr = 1e-6f;     // relative pivot cut of G_A, G_B (and of s
 // zero, is reported through the status word.
 constexpr float kFDomainRel = 1e-2f, kFZeroRel = 1e-6f;
 constexpr int kCThreads = 512;
+constexpr int kStatics = 256;          // the few static words of the kernels here, rounded up
 
 struct JacobiJob {
   const float* X;   // k x r input (row stride r)
@@ -358,9 +359,8 @@ template <int EL, int C>
 int try_launch_jacobi(const JacobiJob* jobs, int count, int rmax, float tol, cudaStream_t st) {
   cudaLaunchAttribute attr[1];
   cudaLaunchConfig_t cfg = jacobi_config<EL, C>(count, rmax, st, attr);
-  if (cfg.dynamicSmemBytes > 227u * 1024u) return C == 1 ? AB_ERR_UNSUPPORTED : 1;
-  AB_CUDA_OK(cudaFuncSetAttribute(jacobi_rows_cluster_kernel<EL, C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)cfg.dynamicSmemBytes));
+  if (cfg.dynamicSmemBytes > (size_t)(kMaxSmem - kStatics)) return C == 1 ? AB_ERR_UNSUPPORTED : 1;
+  AB_CUDA_OK(allow_smem(jacobi_rows_cluster_kernel<EL, C>, kStatics));
   if (C > 1) {
     // one CTA per SM: CTAs that share an SM would only take turns on its issue slots
     int resident = 0;
@@ -764,7 +764,7 @@ float rows_jacobi_tol(int s) { return 5e-7f * sqrtf((float)s) < 4e-6f ? 4e-6f : 
 
 bool rows_jacobi_fits(int count, int s) {
   if (s < 1 || s > 256 || count < 1) return false;
-  if (jacobi_smem_bytes(s, s, 1) <= 227 * 1024 - 256) return true;
+  if (jacobi_smem_bytes(s, s, 1) <= kMaxSmem - kStatics) return true;
   const int sms = sm_count();
   return sms > 0 && (long long)count * 2 <= sms && s >= 32;
 }
@@ -784,7 +784,7 @@ int rows_jacobi(const float* X, float* rows, float* norms, int* status, size_t s
 
 bool sync_factored_supported(const ab_sync_desc* d, int L) {
   // dynamic shared memory of the two single-CTA kernels, with room for their few static words
-  const size_t cap = 227 * 1024 - 256;
+  const size_t cap = kMaxSmem - kStatics;
   for (int i = 0; i < L; ++i)
     if (chol_smem_bytes(d[i].r) > cap || jacobi_smem_bytes(d[i].r, d[i].r, 1) > cap) return false;
   return true;
@@ -917,7 +917,7 @@ int sync_factored(const ab_sync_desc* d, int L, int K, float sigma_cutoff, int d
   if (any_w && !side) AB_TRY(run(kW, w.tc_status + 2, st));
   AB_TRY(run(kGram, w.tc_status, st));
   const size_t csm = chol_smem_bytes(rmax);
-  AB_CUDA_OK(cudaFuncSetAttribute(chol_inv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csm));
+  AB_CUDA_OK(allow_smem(chol_inv_kernel, kStatics));
   chol_inv_kernel<<<2 * L, kCThreads, csm, st>>>(w.cjobs);                                  // R_A, R_B and inverses
   AB_LAUNCH_OK();
   AB_TRY(run(kM, w.tc_status, st));

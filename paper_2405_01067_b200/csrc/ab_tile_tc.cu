@@ -227,7 +227,7 @@ int launch_tiles(const TileProduct& t, const TilePlan& pl, bool clear_status, in
   else AB_TRY(make_tensor_map_2d(&tmF, t.F, false, t.P, t.K, t.ldF, 64, cols));
   AB_TRY(make_tensor_map_2d(&tmD, t.D, false, (uint64_t)t.N, t.P, t.P, 64, 32));
   const size_t smem = 1024 + (size_t)ns * p.slot_bytes + sizeof(TileBars);
-  AB_CUDA_OK(cudaFuncSetAttribute(tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  AB_CUDA_OK(allow_smem(tile_kernel));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)((t.N + rows - 1) / rows * p.ncol));
   cfg.blockDim = dim3(kTileThreads);
