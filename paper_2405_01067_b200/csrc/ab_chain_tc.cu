@@ -1217,12 +1217,15 @@ int launch_chain_ex(const ChainLaunch& L, cudaStream_t st) {
 // few rows that is a long walk on few SMs, and S in memory costs next to nothing.  Measured (us, fused / by tiles,
 // 768 -> 192 -> 3072): 64 rows 21.8 / 8.5, 6173 26.2 / 17.4, 8800 26.5 / 23.1, 10500 28.7 / 32.5; 776 -> 120 -> 1000: 64 rows
 // 14.2 / 8.3, 8800 20.0 / 14.5, 25088 30.7 / 34.4: hence up to one 128-row block for every two SMs.  Factors of a few tiles
-// are no long walk (256 -> 32 -> 256: 5.9 / 6.9).  The first product alone (us, chain kernel / tiles): K 3072 12608 rows
-// 24.1 / 17.0, 25088 33.2 / 44.7; K 256 25088 rows 6.3 / 4.7, 50432 9.2 / 6.1.
+// are no long walk (256 -> 32 -> 256: 5.9 / 6.9); between (512 -> 64 -> 512) a lone forward is bound by the host's second launch, 8.6 / 11.4,
+// and the backward of 6173 rows, where the launches overlap, gains, 19.6 / 18.1.
+// The first product alone (us, chain kernel / tiles): K 3072 12608 rows 24.1 / 17.0, 25088 33.2 / 44.7; K 256, rank 128 25088 rows
+// 6.3 / 4.7, 50432 9.2 / 6.1; with the gradient behind it K 64 to 512, rank 32, 200704 rows 82 to 111 / 76 to 102, but rank 24, K 512
+// 118 / 138 and rank 8, K 256 102 / 120: many rows of a rank below 32 stay with the chain kernel.
 bool by_tiles(int64_t N, int K1, int r, int P) {
   const int64_t blocks = (N + 127) / 128;
   const int sms = sm_count();
-  if (P == 0) return K1 <= 512 || 3 * blocks <= 2 * sms;
+  if (P == 0) return 3 * blocks <= 2 * sms || (K1 <= 512 && r >= 32);
   const int walk = (K1 + 63) / 64 + (P + kChunk - 1) / kChunk * ((r + 63) / 64);
   return 2 * blocks <= sms && walk > 6;
 }
@@ -1231,8 +1234,8 @@ bool by_tiles(int64_t N, int K1, int r, int P) {
 // f_mn = false: F1 is given as r x K1 (row stride ldF1) and F2 as P x r (row stride ldF2);
 // f_mn = true : F1 is given transposed, K1 x r, and F2 transposed, r x P (the factors A and B as they lie in
 //               memory when the chain runs backwards).
-// P is given even where Out is not wanted: which kernels run, and with that the bits of S, depends on the shape alone.
-// scratch: N x r for S where Sg is null; without it the fused kernel runs.
+// P is given even where Out is not wanted: which kernels run, and with that the bits of S, depends on the shape and on whether
+// there is room for S, not on what is wanted.  scratch: N x r for S where Sg is null; without it the fused kernel runs.
 int launch_chain(const void* In, int64_t N, int K1, const void* F1, int ldF1, const void* F2, int ldF2, int P,
                  bool f_mn, void* Out, void* Sg, void* scratch, int r, int* status, bool clear_status, cudaStream_t st,
                  bool stall_selftest = false, unsigned long long wait_ns = kWaitLimitNs) {

@@ -102,3 +102,9 @@ def test_conv3x3_full_size_resnet_and_vgg(ab):
     (batch 1024, r = 32) at full size."""
     for (B, H, W, C, m, r) in [(128, 14, 14, 256, 256, 128), (1024, 4, 4, 512, 512, 32)]:
         check(ab, conv_case(970 + H, B, H, W, C, m, r))
+
+
+@pytest.mark.parametrize("r", [24, 32])
+def test_many_pixels_of_a_low_rank(ab, r):
+    """dT = dY A of more than two thirds of a 128-row block per SM: fused below rank 32, by tiles from there on."""
+    check(ab, conv_case(50 + r, 70, 14, 14, 64, 72, r))

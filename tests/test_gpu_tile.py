@@ -22,7 +22,7 @@ def _close(got, want, terms):
 
 @pytest.mark.parametrize("rows,m,n,r", [(1, 64, 768, 8), (63, 520, 72, 24), (65, 3072, 768, 192), (197, 768, 3072, 192),
                                         (129, 1000, 776, 120), (2049, 328, 2304, 256), (9472, 264, 392, 64), (9473, 264, 392, 64),
-                                        (12672, 64, 3072, 16)])
+                                        (12672, 64, 3072, 16), (63, 1032, 1000, 24)])
 @pytest.mark.parametrize("save", [True, False])
 def test_few_rows_layer(rows, m, n, r, save):
     x, A, B, dY = _bf16(rows, n, seed=1), _bf16(m, r, seed=2), _bf16(r, n, seed=3), _bf16(rows, m, seed=4)
