@@ -431,14 +431,16 @@ norms_sort_kernel(const float* __restrict__ Xall, int s, float* __restrict__ lam
   }
   __syncthreads();
   for (int i = threadIdx.x; i < s; i += 256) {
-    float li = lam_s[i];
+    // Compared by their bits, which for values that are not negative is the order of the values: NaN has a place as well, and perm
+    // is a permutation whatever the matrix holds (a rank that nothing took would leave an index of old workspace contents).
+    const unsigned li = __float_as_uint(lam_s[i]);
     int rank = 0;
     for (int j = 0; j < s; ++j) {
-      float lj = lam_s[j];
+      const unsigned lj = __float_as_uint(lam_s[j]);
       rank += (lj > li) || (lj == li && j < i);
     }
     perm_all[(size_t)mat * s + rank] = i;
-    lam_all[(size_t)mat * s + i] = li;
+    lam_all[(size_t)mat * s + i] = lam_s[i];
   }
 }
 
