@@ -9,7 +9,8 @@
  * Conventions for every call
  *  - Pointers are DEVICE pointers owned by the caller unless a parameter says "host".
  *    The library allocates no device memory; scratch space is passed in as `ws` (size from
- *    ab_workspace_bytes, 256-byte aligned).  No result depends on an earlier call.  What the
+ *    ab_workspace_bytes, 256-byte aligned) and belongs to the call until the stream has run it: calls that
+ *    may overlap on the GPU need a workspace each.  No result depends on an earlier call.  What the
  *    library does keep per process: a count of its kernel launches (ab_launch_count), cached
  *    device properties, the address of the built-in array of ab_layer_forward_static, and one
  *    low-priority helper stream per device that ab_group_sync creates on first use (see there).
@@ -109,9 +110,12 @@ size_t ab_workspace_bytes(int op, int64_t N, int m, int n, int r, int K, int dt)
  * Forward of the factorised layer (Eq. 3 used as a linear map): y = (x B^T) A^T.
  *   x [N,n], A [m,r] (row stride ldA >= r), B [r,n] (row stride ldB >= n), y [N,m], all of
  *   storage type dt.  T_save: NULL, or [N,r] of type dt that receives T = x B^T for the
- *   backward call.  The rank-r intermediate stays on chip when dt = AB_BF16, r is a
- *   multiple of 8 with 8 <= r <= 256 and m, n are multiples of 8; other shapes take a
- *   slower general kernel (same results to rounding).  N = 0 is a no-op.
+ *   backward call.  When dt = AB_BF16, r is a multiple of 8 with 8 <= r <= 256 and m, n are
+ *   multiples of 8 it runs on the tensor cores: many rows in one kernel that keeps the rank-r
+ *   intermediate on chip, few rows as two products with the intermediate in T_save or ws (a ws
+ *   that holds the status word alone, 256 bytes, is accepted and keeps it on chip there too;
+ *   sums are then added in another order).  Other shapes and fp32 take slower general kernels
+ *   (same results to rounding).  N = 0 is a no-op.
  *   Device status: the first int of ws receives AB_OK, or AB_ERR_TIMEOUT if a bounded
  *   on-chip wait of the fused kernel expired (outputs are then undefined).  The same holds
  *   for ab_layer_backward.
@@ -236,10 +240,10 @@ int ab_group_average(const void* base, int64_t stride_elems, int K, int64_t coun
 /*
  * Recombination (Algorithm 1: W <- A B): W [m,n] fp32 (dense) = Abar [m,r] Bbar [r,n],
  * factors of type dt, product accurate to fp32 rounding.  With a workspace of
- * ab_workspace_bytes(AB_OP_RECOMBINE, 0, m, n, r, 0, dt) bytes and n a multiple of 4 it runs on the tensor
- * cores: bf16 factors multiply exactly in fp32; fp32 factors are cut into three bf16 pieces each (24 bits)
- * and multiplied as six bf16 products accumulated in fp32.  With ws = NULL (or too small) the same product
- * runs on the fp32 pipes.
+ * ab_workspace_bytes(AB_OP_RECOMBINE, 0, m, n, r, 0, dt) bytes it runs on the tensor cores: bf16 factors
+ * multiply exactly in fp32; fp32 factors are cut into three bf16 pieces each (24 bits) and multiplied as six
+ * bf16 products accumulated in fp32 (an infinity, or a value that rounds to one in bf16, makes its row or
+ * column NaN).  With ws = NULL (or too small) the same product runs on the fp32 pipes.
  */
 int ab_recombine(const void* Abar, const void* Bbar, float* W, int m, int n, int r,
                  int ldA, int ldB, int dt, void* ws, size_t ws_bytes, void* cuda_stream);
