@@ -292,9 +292,9 @@ __device__ __forceinline__ void gemm_split_body(const SplitGemm* probs, int npro
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsMma));
     if (warp == kMmaWarp) {
       // ---------------------------------------------------------- MMA issuer (see elect_one for the uniform loop)
-      if constexpr (kOne) {      // no bounded wait starts before the kernel in front is done: it may take longer than a wait may
-        dep_wait();
-        dep_launch();
+      if constexpr (kOne) {
+        dep_launch();            // the kernel behind may set itself up already: it waits for this one as a whole
+        dep_wait();              // no bounded wait starts before the kernel in front is done: it may take longer than a wait may
       }
       TileReader<kOne, BN> rd;
       int slot = 0, ph = 0;
