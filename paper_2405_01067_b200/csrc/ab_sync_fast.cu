@@ -660,13 +660,21 @@ __global__ void fold_tc_status_kernel(const int* __restrict__ tc_status, int* __
 }
 
 // The long index of a Gram product is cut into slices, whose partial sums the Cholesky kernel adds in ascending order.  Short ones
-// give a lone matrix more CTAs for the product (2 us a slab of 64 with its start and end), long ones leave the one CTA that adds
-// them less to load (22 us a part of rank 192, 2.4 of rank 64): 8 r, from 128 (two slabs) to 768, at most kGramMaxParts slices.
-// Group sync, us, slices of 128 / 256 / 512 / 768: 3072 x 768, rank 192 776 / 727 / 662 / 643; 3072 x 3072, rank 128 494 / 473 / 454 /
-// 453; 512 x 4608, rank 64 231 / 230 / 226 / 230; 3072 x 3072, rank 32 158 / 159 / 162 / 163; 3072 x 64, rank 16 129 / 132 / 133 / 139;
-// all of ViT-B/16 1935 / 1755 / 1581 / 1548.
+// give a few matrices more CTAs for the product (2 us a slab of 64 with its start and end), long ones leave the one CTA that adds
+// them less to load (22 us a part of rank 192, 2.4 of rank 64): 8 r, and no shorter than gives every SM a tile, from 128 (two slabs)
+// to 768, at most kGramMaxParts slices.  Group sync, us, slices of 128 / 256 / 512 / 768: 3072 x 768, rank 192 776 / 727 / 662 / 643;
+// 3072 x 3072, rank 128 494 / 473 / 454 / 453; 512 x 4608, rank 64 231 / 230 / 226 / 230; 3072 x 3072, rank 32 158 / 159 / 162 / 163; 3072 x 64,
+// rank 16 129 / 132 / 133 / 139; all of ViT-B/16 1935 / 1755 / 1581 / 1548; 100 of 3072 x 3072, rank 32 at 256 / 768: 565 / 539.
 constexpr int kGramMaxParts = 16;
-int gram_slice(const ab_sync_desc& d) { return std::max(128, std::min(768, 8 * d.r)); }
+int gram_fill(const ab_sync_desc* d, int L) {       // the slice length with which every SM has a tile
+  int64_t work = 0;                     // tiles x length
+  for (int i = 0; i < L; ++i) {
+    const int64_t t = (d[i].r + 127) / 128;
+    work += t * (t + 1) / 2 * ((int64_t)d[i].m + d[i].n);
+  }
+  return (int)std::min<int64_t>(768, (work / std::max(sm_count(), 1) + 63) / 64 * 64);
+}
+int gram_slice(int r, int fill) { return std::max(128, std::min(768, std::max(8 * r, fill))); }
 int gram_per(int len, int slice) {      // length of a part, a multiple of 64
   const int parts = std::max(1, std::min(kGramMaxParts, (len + slice - 1) / slice));
   return ((len + parts - 1) / parts + 63) / 64 * 64;
@@ -692,6 +700,7 @@ struct FastWs {
 FastWs fast_layout(const ab_sync_desc* d, int L, void* ws) {
   FastWs w;
   Arena ar(ws, 0);
+  const int fill = gram_fill(d, L);
   auto each = [&](std::vector<float*>& v, auto count) {
     v.resize(L);
     for (int i = 0; i < L; ++i) v[i] = ar.take_n<float>(count(d[i]));
@@ -699,12 +708,12 @@ FastWs fast_layout(const ab_sync_desc* d, int L, void* ws) {
   each(w.Abar, [](const ab_sync_desc& x) { return (size_t)x.m * x.r; });
   each(w.Bbar, [](const ab_sync_desc& x) { return (size_t)x.r * x.n; });
   auto rr = [](const ab_sync_desc& x) { return (size_t)x.r * x.r; };
-  each(w.GA, [](const ab_sync_desc& x) { return (size_t)gram_parts(x.m, gram_slice(x)) * x.r * x.r; });
-  each(w.GB, [](const ab_sync_desc& x) { return (size_t)gram_parts(x.n, gram_slice(x)) * x.r * x.r; });
+  each(w.GA, [=](const ab_sync_desc& x) { return (size_t)gram_parts(x.m, gram_slice(x.r, fill)) * x.r * x.r; });
+  each(w.GB, [=](const ab_sync_desc& x) { return (size_t)gram_parts(x.n, gram_slice(x.r, fill)) * x.r * x.r; });
   each(w.RA, rr); each(w.RB, rr); each(w.IA, rr); each(w.IB, rr);
   each(w.M, rr); each(w.Vs, rr); each(w.Y1, rr); each(w.ZA, rr); each(w.ZB, rr);
   size_t ngemm = (size_t)7 * L;
-  for (int i = 0; i < L; ++i) ngemm += gram_parts(d[i].m, gram_slice(d[i])) + gram_parts(d[i].n, gram_slice(d[i]));
+  for (int i = 0; i < L; ++i) ngemm += gram_parts(d[i].m, gram_slice(d[i].r, fill)) + gram_parts(d[i].n, gram_slice(d[i].r, fill));
   w.gemms = ar.take_n<SplitGemm>(ngemm);
   w.cjobs = ar.take_n<CholJob>((size_t)2 * L);
   w.ajobs = ar.take_n<AvgJob>((size_t)2 * L);
@@ -792,6 +801,7 @@ int sync_factored(const ab_sync_desc* d, int L, int K, float sigma_cutoff, int d
   if (w.bytes > ws_bytes) return AB_ERR_WORKSPACE;
   if (!gemm_tc_available()) return AB_ERR_UNSUPPORTED;
   const int out_bf16 = (dt == AB_BF16) ? 1 : 0;
+  const int fill = gram_fill(d, L);
   int rmax = 0;
   bool any_w = false;
   for (int i = 0; i < L; ++i) { rmax = std::max(rmax, d[i].r); any_w = any_w || d[i].W_out != nullptr; }
@@ -808,7 +818,7 @@ int sync_factored(const ab_sync_desc* d, int L, int K, float sigma_cutoff, int d
     const int m = d[i].m, n = d[i].n, r = d[i].r;
     float *Ab = w.Abar[i], *Bb = w.Bbar[i];
     // G_A = Abar^T Abar, G_B = Bbar Bbar^T, upper tiles only, in slices of the long index
-    const int slice = gram_slice(d[i]), pa = gram_parts(m, slice), pb = gram_parts(n, slice);
+    const int slice = gram_slice(d[i].r, fill), pa = gram_parts(m, slice), pb = gram_parts(n, slice);
     for (int q = 0; q < pa; ++q) {
       const int per = gram_per(m, slice), k0 = q * per, k1 = std::min(m, k0 + per);
       const float* src = Ab + (size_t)k0 * r;
