@@ -13,7 +13,8 @@
 // At convergence the rows of V^T are eigenvectors of G (singular vectors of the short side)
 // and |x_i| = sigma_i^2.  The long-side factor is W V_r (or V_r^T W) by a GEMM; sigma_i is
 // re-measured as the norm of that product, which makes A^T A = B B^T = diag(sigma) hold by
-// construction.  No wait in these kernels can spin: every loop has a fixed trip count.
+// construction.  The Jacobi kernels launched round by round wait for nothing: every loop has a fixed trip count.  The fallback in
+// one cooperative launch (grid_meet) and the direct solver wait for other CTAs; those waits are bounded and reach the status word.
 //
 // Short sides up to eig_max() (1184) take the direct solver of ab_eig.cu; the Jacobi in shared memory (up to
 // kEigSmallMax) or the block Jacobi in one cooperative launch is its fallback.  Larger ones take the block Jacobi.

@@ -22,7 +22,7 @@ constexpr int kMaxTileStages = 6;
 
 struct TileParams {
   int K, nk;                // reduction length, slabs of 64
-  int rows, cols;           // rows loaded and stored per tile (32, 64 or 128), columns (a multiple of 16)
+  int rows, cols;           // rows loaded and stored per tile (64 or 128), columns (a multiple of 16)
   int ncol;                 // tiles across D
   int N, P;                 // rows and width of D
   int ns, slot_bytes;
@@ -172,7 +172,7 @@ tile_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUt
   }
 }
 
-// What one launch costs in SM cycles, by what was measured on tiles of 32 to 128 rows and 64 to 256 columns:
+// What one launch costs in SM cycles, by what was measured on tiles of 32 to 128 rows (32 never pays) and 64 to 256 columns:
 // a 128-byte row arrives every 2 cycles, an MMA step of 16 takes 51 / 65 / 98 / 130 cycles at 64 / 128 / 192 / 256 columns, a slab
 // 200 besides; a load takes 1100 cycles (2200 from many megabytes) and the stages of the CTAs on an SM hide it; a CTA starts, fills
 // and stores in about 4500, which those on the SM beside it hide.
