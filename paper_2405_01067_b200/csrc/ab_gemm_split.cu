@@ -344,7 +344,7 @@ __device__ __forceinline__ void gemm_split_body(const SplitGemm* probs, int npro
         if (ok && elect_one()) tc_commit(&bars->acc_full[buf]);
         __syncwarp();
       }
-    } else if (!kOne) {
+    } else if (!kOne && warp == kFindWarp) {
       // ---------------------------------------------------------- tile finder
       int idx = 0, slot = 0, ph = 1;
       for (int tile = blockIdx.x;; tile += gridDim.x) {

@@ -100,3 +100,25 @@ def test_a_kernel_in_front_may_take_longer_than_a_wait(ab):
     torch.cuda.synchronize()
     assert ab.workspace_status(stall) == ab.AB_ERR_TIMEOUT and ab.workspace_status(ws) == 0
     assert orc.rel_frob(W.cpu().numpy().astype(np.float64), orc.recombine(a, b)) <= 1e-6
+
+
+def test_records_of_many_tiles(ab):
+    """A batch whose CTAs take dozens of tiles each: the tile records go round their ring many times.  Every copy of a
+    matrix gives the bits of its first one, in every run."""
+    shapes = [(40, 24, 8), (130, 60, 12), (64, 200, 16), (24, 24, 4), (150, 150, 20)]
+    rng = np.random.default_rng(2)
+    kinds = [synth.planted_factors(rng, m, n, np.linspace(1.0, 0.3, r)) for m, n, r in shapes]
+    kinds = [(torch.from_numpy(a[None].copy()).cuda(), torch.from_numpy(b[None].copy()).cuda()) for a, b in kinds]
+    order = rng.integers(0, len(kinds), 2500)
+    plan = ab.SyncPlan([kinds[k][0] for k in order], [kinds[k][1] for k in order], 0.1, want_W=True)
+    for _ in range(3):
+        ab.ab_group_sync(plan, path=ab.AB_SYNC_FACTORED)
+    torch.cuda.synchronize()
+    assert torch.count_nonzero(plan.status) == 0
+    for k in range(len(kinds)):
+        mine = np.flatnonzero(order == k)
+        for out in (plan.A_out, plan.B_out, plan.sigma, plan.W_out):
+            assert bool((torch.stack([out[i] for i in mine]) == out[mine[0]]).all())
+        W = kinds[k][0][0].double() @ kinds[k][1][0].double()
+        got = plan.A_out[mine[0]].double() @ plan.B_out[mine[0]].double()
+        assert float((got - W).norm() / W.norm()) <= 1e-5
