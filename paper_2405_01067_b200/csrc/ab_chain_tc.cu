@@ -697,7 +697,7 @@ grad_kernel(const __grid_constant__ CUtensorMap tmAct0, const __grid_constant__ 
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   uint8_t* ring = smem;
   Bars* bars = reinterpret_cast<Bars*>(ring + (size_t)p.ns * p.slot_bytes);
-  const int warp = (int)uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
+  const int warp = (int)uniform(threadIdx.x >> 5);
 
   // which job, which 128-row chunk of its output, which slice of the N rows
   int tile = blockIdx.x;
@@ -802,7 +802,7 @@ conv_grad_kernel(const __grid_constant__ CUtensorMap tmX4, const __grid_constant
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   uint8_t* ring = smem;
   Bars* bars = reinterpret_cast<Bars*>(ring + (size_t)p.ns * p.slot_bytes);
-  const int warp = (int)uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
+  const int warp = (int)uniform(threadIdx.x >> 5);
   int tile = blockIdx.x;
   const int slice = tile % p.slices;
   const int chunk = tile / p.slices;
@@ -976,30 +976,6 @@ __global__ void bounded_wait_selftest_kernel(int* status, unsigned long long lim
 
 // ---------------------------------------------------------------------------------------------
 // host side
-// Launch with programmatic stream serialisation (see dep_wait): only for kernels that call dep_wait()
-// before their first access to global memory.
-template <typename... KArgs, typename... Args>
-cudaError_t launch_dep(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
-}
-#define AB_LAUNCH_DEP(...)                         \
-  do {                                             \
-    if (launch_dep(__VA_ARGS__) != cudaSuccess) {  \
-      cudaGetLastError();                          \
-      return AB_ERR_CUDA;                          \
-    }                                              \
-  } while (0)
-
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -1030,21 +1006,6 @@ bool device_is_sm100() {
     cache[dev] = (major == 10) ? 1 : 0;
   }
   return cache[dev] == 1;
-}
-
-// bf16 matrix [rows x cols], row stride ld elements, box of box_cols x box_rows, 128-byte swizzle
-int make_map(CUtensorMap* m, const void* ptr, uint64_t rows, uint64_t cols, uint64_t ld, uint32_t box_cols,
-             uint32_t box_rows) {
-  EncodeTiledFn fn = encode_fn();
-  if (!fn) return AB_ERR_CUDA;
-  cuuint64_t dims[2] = {cols, rows};
-  cuuint64_t strides[1] = {ld * 2};
-  cuuint32_t box[2] = {box_cols, box_rows};
-  cuuint32_t estr[2] = {1, 1};
-  CUresult rc = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), dims, strides, box, estr,
-                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return rc == CUDA_SUCCESS ? AB_OK : AB_ERR_CUDA;
 }
 
 // Ranks that are multiples of 8 but not of 16 run as the next multiple of 16: the tensor maps keep the
@@ -1174,24 +1135,24 @@ int launch_chain_ex(const ChainLaunch& L, cudaStream_t st) {
   CUtensorMap tmIn, tmIn4, tmF1, tmF2, tmOut, tmS;
   if (conv) {
     AB_TRY(make_tensor_map_nhwc(&tmIn4, L.In, L.cv->B, L.cv->H, L.cv->W, L.cv->in_ch, L.cv->W, L.cv->bh, L.cv->bb));
-    AB_TRY(make_map(&tmF1, L.F1, L.f1_rows, L.f1_cols, L.ldF1, 64, L.f_mn ? 64 : rp));
+    AB_TRY(make_tensor_map_2d(&tmF1, L.F1, false, L.f1_rows, L.f1_cols, L.ldF1, 64, L.f_mn ? 64 : rp));
     tmIn = tmF1;
   } else {
-    AB_TRY(make_map(&tmIn, L.In, (uint64_t)L.N, L.K1, L.K1, 64, 128));
+    AB_TRY(make_tensor_map_2d(&tmIn, L.In, false, (uint64_t)L.N, L.K1, L.K1, 64, 128));
     tmIn4 = tmIn;
-    if (L.f_mn) AB_TRY(make_map(&tmF1, L.F1, L.K1, L.r, L.ldF1, 64, 64));
-    else AB_TRY(make_map(&tmF1, L.F1, L.r, L.K1, L.ldF1, 64, rp));
+    if (L.f_mn) AB_TRY(make_tensor_map_2d(&tmF1, L.F1, false, L.K1, L.r, L.ldF1, 64, 64));
+    else AB_TRY(make_tensor_map_2d(&tmF1, L.F1, false, L.r, L.K1, L.ldF1, 64, rp));
   }
   // unused maps still have to be valid objects: alias them to another operand
   if (second) {
-    if (L.f_mn) AB_TRY(make_map(&tmF2, L.F2, L.r, L.P, L.ldF2, 64, 64));
-    else AB_TRY(make_map(&tmF2, L.F2, L.P, L.r, L.ldF2, 64, kChunk));
-    AB_TRY(make_map(&tmOut, L.Out, (uint64_t)L.N, L.P, L.P, 64, kGroupRows));
+    if (L.f_mn) AB_TRY(make_tensor_map_2d(&tmF2, L.F2, false, L.r, L.P, L.ldF2, 64, 64));
+    else AB_TRY(make_tensor_map_2d(&tmF2, L.F2, false, L.P, L.r, L.ldF2, 64, kChunk));
+    AB_TRY(make_tensor_map_2d(&tmOut, L.Out, false, (uint64_t)L.N, L.P, L.P, 64, kGroupRows));
   } else {
     tmF2 = tmF1;
     tmOut = tmF1;
   }
-  if (L.Sg) AB_TRY(make_map(&tmS, L.Sg, (uint64_t)L.N, conv ? L.cv->s_col_off + L.s_cols : L.s_cols, L.s_ld, 64, kGroupRows));
+  if (L.Sg) AB_TRY(make_tensor_map_2d(&tmS, L.Sg, false, (uint64_t)L.N, conv ? L.cv->s_col_off + L.s_cols : L.s_cols, L.s_ld, 64, kGroupRows));
   else tmS = tmF1;
   ChainParams q;
   std::memset(&q, 0, sizeof(q));
@@ -1207,9 +1168,7 @@ int launch_chain_ex(const ChainLaunch& L, cudaStream_t st) {
   if (conv) q.cv = *L.cv;
   q.out_ptr = static_cast<bf16*>(L.Out); q.s_ptr = static_cast<bf16*>(L.Sg); q.s_ld = L.s_ld; q.s_cols = L.s_cols;
   AB_CUDA_OK(allow_smem(chain_kernel));
-  AB_LAUNCH_DEP(chain_kernel, dim3((unsigned)grid), dim3(kChainThreads), pl.smem, st, tmIn, tmIn4, tmF1, tmF2, tmOut,
-                tmS, q);
-  AB_LAUNCH_OK();
+  AB_TRY(launch_after(chain_kernel, (unsigned)grid, kChainThreads, pl.smem, 1, st, tmIn, tmIn4, tmF1, tmF2, tmOut, tmS, q));
   return AB_OK;
 }
 
@@ -1369,14 +1328,14 @@ int chain_tc_backward(const void* x, const void* dY, const void* A, const void* 
     CUtensorMap tmAct[2], tmSmall[2];
     int nj = 0;
     if (dA) {
-      AB_TRY(make_map(&tmAct[nj], dY, (uint64_t)N, m, m, 64, 64));
-      AB_TRY(make_map(&tmSmall[nj], T, (uint64_t)N, r, r, 64, 64));
+      AB_TRY(make_tensor_map_2d(&tmAct[nj], dY, false, (uint64_t)N, m, m, 64, 64));
+      AB_TRY(make_tensor_map_2d(&tmSmall[nj], T, false, (uint64_t)N, r, r, 64, 64));
       p.job[nj].chunks = tiles256(m); p.job[nj].out = grad_out(gp.sp, w.pA, dA, m, r, false);
       ++nj;
     }
     if (dB) {
-      AB_TRY(make_map(&tmAct[nj], x, (uint64_t)N, n, n, 64, 64));
-      AB_TRY(make_map(&tmSmall[nj], w.dT, (uint64_t)N, r, r, 64, 64));
+      AB_TRY(make_tensor_map_2d(&tmAct[nj], x, false, (uint64_t)N, n, n, 64, 64));
+      AB_TRY(make_tensor_map_2d(&tmSmall[nj], w.dT, false, (uint64_t)N, r, r, 64, 64));
       p.job[nj].chunks = tiles256(n); p.job[nj].out = grad_out(gp.sp, w.pB, dB, n, r, true);
       ++nj;
     }
@@ -1386,14 +1345,12 @@ int chain_tc_backward(const void* x, const void* dY, const void* A, const void* 
     p.job0_independent = (after_chain && dA) ? 1 : 0;   // job 0 is the dA job whenever dA is asked for
     AB_CUDA_OK(allow_smem(grad_kernel));
     const unsigned grid = (unsigned)((p.job[0].chunks + p.job[1].chunks) * slices);
-    AB_LAUNCH_DEP(grad_kernel, dim3(grid), dim3(192), gp.smem, st, tmAct[0], tmSmall[0], tmAct[1], tmSmall[1], p);
-    AB_LAUNCH_OK();
+    AB_TRY(launch_after(grad_kernel, grid, 192, gp.smem, 1, st, tmAct[0], tmSmall[0], tmAct[1], tmSmall[1], p));
     if (slices > 1) {
       const ReduceGrid rg = reduce_grid(gp.sp, dA ? m : 0, dB ? n : 0, r);
       const int nA = rg.a, nB = rg.b;
-      AB_LAUNCH_DEP(reduce_partials_kernel, dim3(nA + nB), dim3(kReduceT), 0, st, static_cast<const float*>(w.pA), dA, m, nA,
-                 static_cast<const float*>(w.pB), dB, n, slices, r, rp);
-      AB_LAUNCH_OK();
+      AB_TRY(launch_after(reduce_partials_kernel, (unsigned)(nA + nB), kReduceT, 0, 1, st, static_cast<const float*>(w.pA), dA,
+                          m, nA, static_cast<const float*>(w.pB), dB, n, slices, r, rp));
     }
     first = false;
   }
@@ -1525,8 +1482,8 @@ int conv_tc_backward(const void* x, const void* dY, const void* A, const void* B
     GradParams p;
     std::memset(&p, 0, sizeof(p));
     CUtensorMap tmAct, tmSmall;
-    AB_TRY(make_map(&tmAct, dY, (uint64_t)N, m, m, 64, 64));
-    AB_TRY(make_map(&tmSmall, T, (uint64_t)N, r, r, 64, 64));
+    AB_TRY(make_tensor_map_2d(&tmAct, dY, false, (uint64_t)N, m, m, 64, 64));
+    AB_TRY(make_tensor_map_2d(&tmSmall, T, false, (uint64_t)N, r, r, 64, 64));
     p.job[0].chunks = tiles256(m); p.job[0].out = grad_out(gp.sp, w.pA, dA, m, r, false);
     p.job[1] = p.job[0]; p.job[1].chunks = 0;
     const int slices = gp.sp.slices;
@@ -1534,15 +1491,12 @@ int conv_tc_backward(const void* x, const void* dY, const void* A, const void* B
     p.slices = slices; p.rows_per_slice = gp.sp.per * 64; p.N = (int)N; p.clear_status = first ? 1 : 0;
     p.status = w.status; p.job0_independent = 0;
     AB_CUDA_OK(allow_smem(grad_kernel));
-    AB_LAUNCH_DEP(grad_kernel, dim3((unsigned)(p.job[0].chunks * slices)), dim3(192), gp.smem, st, tmAct, tmSmall, tmAct,
-                      tmSmall, p);
-    AB_LAUNCH_OK();
+    AB_TRY(launch_after(grad_kernel, (unsigned)(p.job[0].chunks * slices), 192, gp.smem, 1, st, tmAct, tmSmall, tmAct, tmSmall, p));
     first = false;
     if (slices > 1) {
       const int nA = reduce_grid(gp.sp, m, 0, r).a;
-      AB_LAUNCH_DEP(reduce_partials_kernel, dim3(nA), dim3(kReduceT), 0, st, static_cast<const float*>(w.pA), dA, m, nA,
-                    static_cast<const float*>(w.pA), static_cast<float*>(nullptr), 0, slices, r, rp);
-      AB_LAUNCH_OK();
+      AB_TRY(launch_after(reduce_partials_kernel, (unsigned)(nA), kReduceT, 0, 1, st, static_cast<const float*>(w.pA), dA, m, nA,
+                          static_cast<const float*>(w.pA), static_cast<float*>(nullptr), 0, slices, r, rp));
     }
   }
   if (dB) {
@@ -1557,13 +1511,11 @@ int conv_tc_backward(const void* x, const void* dY, const void* A, const void* B
     p.spi = gp.spi; p.kb = gp.kb; p.bhk = gp.bhk; p.box_rows = gp.box_rows; p.cpt = gp.cpt; p.slices = slices;
     p.slabs_per_slice = gp.sp.per; p.nslabs = gp.nslabs; p.out = grad_out(gp.sp, w.pB, dB, 9 * C, r, true); p.status = w.status;
     AB_CUDA_OK(allow_smem(conv_grad_kernel));
-    AB_LAUNCH_DEP(conv_grad_kernel, dim3((unsigned)(9 * gp.cpt * slices)), dim3(192), gp.smem, st, tmX4, tmT4, p);
-    AB_LAUNCH_OK();
+    AB_TRY(launch_after(conv_grad_kernel, (unsigned)(9 * gp.cpt * slices), 192, gp.smem, 1, st, tmX4, tmT4, p));
     if (slices > 1) {
       const int nB = reduce_grid(gp.sp, 0, 9 * (int64_t)C, r).b;
-      AB_LAUNCH_DEP(reduce_partials_kernel, dim3(nB), dim3(kReduceT), 0, st, static_cast<const float*>(w.pB), static_cast<float*>(nullptr),
-                    0, 0, static_cast<const float*>(w.pB), dB, 9 * C, slices, r, rp);
-      AB_LAUNCH_OK();
+      AB_TRY(launch_after(reduce_partials_kernel, (unsigned)(nB), kReduceT, 0, 1, st, static_cast<const float*>(w.pB),
+                          static_cast<float*>(nullptr), 0, 0, static_cast<const float*>(w.pB), dB, 9 * C, slices, r, rp));
     }
   }
   if (first) AB_CUDA_OK(cudaMemsetAsync(w.status, 0, sizeof(int), st));

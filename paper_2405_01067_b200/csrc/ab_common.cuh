@@ -6,6 +6,8 @@
 #include <stdint.h>
 #include <stddef.h>
 
+#include <utility>
+
 #include "ab.h"
 
 namespace ab {
@@ -42,6 +44,27 @@ constexpr int kMaxSmem = 227 * 1024;
 template <typename K>
 inline cudaError_t allow_smem(K* kernel, int static_bytes = 0) {
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem - static_bytes);
+}
+
+// Launch with programmatic stream serialisation, in clusters of `cluster` CTAs: the kernel may become resident while the one before it
+// in the stream still runs.  Only for kernels that wait for that one (tc::dep_wait) before they touch global memory.
+template <typename... KArgs, typename... Args>
+inline int launch_after(void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem, int cluster, cudaStream_t st, Args&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = cluster; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
+  if (cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...) != cudaSuccess) { (void)cudaGetLastError(); return AB_ERR_CUDA; }
+  AB_LAUNCH_OK();
+  return AB_OK;
 }
 
 // Multiprocessors of the current device (cached per device; 0 if the query fails).  Grid sizes that are

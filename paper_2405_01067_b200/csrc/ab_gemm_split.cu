@@ -513,19 +513,7 @@ int launch(void (*kernel)(KArgs...), size_t smem, int tiles, cudaStream_t st, Ar
   const int sms = sm_count();
   if (sms <= 0) return AB_ERR_CUDA;
   AB_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(tiles < sms ? tiles : sms));
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  if (cudaLaunchKernelEx(&cfg, kernel, args...) != cudaSuccess) { (void)cudaGetLastError(); return AB_ERR_CUDA; }
-  AB_LAUNCH_OK();
-  return AB_OK;
+  return launch_after(kernel, (unsigned)(tiles < sms ? tiles : sms), (unsigned)kThreads, smem, 1, st, args...);
 }
 
 int tiles_of(const SplitGemm& p, int bn) { return ((p.M + kM - 1) / kM) * ((p.N + bn - 1) / bn); }

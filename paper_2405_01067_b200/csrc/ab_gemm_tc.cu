@@ -292,29 +292,12 @@ sum_slices_kernel(const float4* __restrict__ part, float4* __restrict__ out, int
   out[i] = acc;
 }
 
-template <typename... KArgs, typename... Args>
-int launch_after(void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, Args... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(block);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  if (cudaLaunchKernelEx(&cfg, kernel, args...) != cudaSuccess) { (void)cudaGetLastError(); return AB_ERR_CUDA; }
-  AB_LAUNCH_OK();
-  return AB_OK;
-}
-
 }  // namespace
 
 int sum_slices(const float* part, float* out, int64_t count, int64_t slice_stride, int slices, cudaStream_t st) {
   if (count <= 0) return AB_OK;
   if (count % 4 != 0 || slice_stride % 4 != 0 || !aligned(part, 16) || !aligned(out, 16)) return AB_ERR_INVALID_ARG;
-  return launch_after(sum_slices_kernel, (unsigned)((count / 4 + 255) / 256), 256u, 0, st, reinterpret_cast<const float4*>(part),
+  return launch_after(sum_slices_kernel, (unsigned)((count / 4 + 255) / 256), 256u, 0, 1, st, reinterpret_cast<const float4*>(part),
                       reinterpret_cast<float4*>(out), count / 4, slice_stride / 4, slices);
 }
 
@@ -360,7 +343,7 @@ int gemm_tc_batched(const TcProblem* probs, int count, int* status, cudaStream_t
   if (sms <= 0) return AB_ERR_CUDA;
   const int grid = tiles < sms ? tiles : sms;
   batch.nprobs = count; batch.ntiles = tiles; batch.status = status;
-  return launch_after(gemm_tc_kernel, (unsigned)grid, (unsigned)kTcThreads, smem, st, batch);
+  return launch_after(gemm_tc_kernel, (unsigned)grid, (unsigned)kTcThreads, smem, 1, st, batch);
 }
 
 }  // namespace ab

@@ -322,24 +322,10 @@ small_gemm_kernel(const __grid_constant__ SmallGemm p) {
   if (C > 1) cluster.sync();                          // nobody leaves while a peer reads its sums
 }
 
-template <typename K, typename P>
-int launch_small(K* kernel, unsigned grid, int cluster, size_t smem, cudaStream_t st, const P& p) {
+template <typename P>
+int launch_small(void (*kernel)(const P), unsigned grid, int cluster, size_t smem, cudaStream_t st, const P& p) {
   if (smem > 48 * 1024) AB_CUDA_OK(allow_smem(kernel));
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute at[2];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  at[1].id = cudaLaunchAttributeClusterDimension;
-  at[1].val.clusterDim.x = cluster; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = cluster > 1 ? 2 : 1;
-  if (cudaLaunchKernelEx(&cfg, kernel, p) != cudaSuccess) { (void)cudaGetLastError(); return AB_ERR_CUDA; }
-  AB_LAUNCH_OK();
-  return AB_OK;
+  return launch_after(kernel, grid, (unsigned)kThreads, smem, cluster, st, p);
 }
 
 size_t chain_smem(int R, int K1, int r) { return sizeof(float) * (size_t)R * (((K1 + 3) & ~3) + ((r + 3) & ~3)) + sizeof(double) * kThreads * R; }

@@ -228,19 +228,7 @@ int launch_tiles(const TileProduct& t, const TilePlan& pl, bool clear_status, in
   AB_TRY(make_tensor_map_2d(&tmD, t.D, false, (uint64_t)t.N, t.P, t.P, 64, 32));
   const size_t smem = 1024 + (size_t)ns * p.slot_bytes + sizeof(TileBars);
   AB_CUDA_OK(allow_smem(tile_kernel));
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)((t.N + rows - 1) / rows * p.ncol));
-  cfg.blockDim = dim3(kTileThreads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  AB_CUDA_OK(cudaLaunchKernelEx(&cfg, tile_kernel, tmX, tmF, tmD, p));
-  AB_LAUNCH_OK();
-  return AB_OK;
+  return launch_after(tile_kernel, (unsigned)((t.N + rows - 1) / rows * p.ncol), (unsigned)kTileThreads, smem, 1, st, tmX, tmF, tmD, p);
 }
 
 }  // namespace
