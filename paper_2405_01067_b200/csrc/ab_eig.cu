@@ -209,6 +209,7 @@ struct Tridiag {
 #pragma unroll
             for (int q = 0; q < 4; ++q) col[4 * g + q] = (next && E0 + 1 < E) ? x.A[4 * g + q][E0 + 1 < E ? E0 + 1 : E0] : x.A[4 * g + q][E0];
           }
+          __syncwarp();                              // other lanes send what this one wrote
           // four row sums across the warp, each exchange halving what a lane still carries: lanes 8 q .. hold sum q
           const bool h2 = (lane & 16) != 0, h1 = (lane & 8) != 0;
           double t0 = (h2 ? ps[2] : ps[0]) + __shfl_xor_sync(0xffffffffu, h2 ? ps[0] : ps[2], 16);
