@@ -538,27 +538,32 @@ struct TriShared {
   unsigned* mask;            // bit k set: T splits between k and k + 1
   double norm;
 };
+// sm: s entries; one pass over global memory with the loads of four rounds in flight
 __device__ __forceinline__ void tri_load(const EigJob& job, TriShared& t, double2* sm, unsigned* mask, double* red) {
   const int s = job.s;
   t.de = sm; t.mask = mask;
+#pragma unroll 4
+  for (int k = threadIdx.x; k < s; k += blockDim.x) sm[k] = make_double2(job.d[k], k + 1 < s ? job.e[k] : 0.0);
+  for (int k = threadIdx.x; k < (s + 31) / 32; k += blockDim.x) mask[k] = 0u;
+  __syncthreads();
   double big = 0.0;
   for (int k = threadIdx.x; k < s; k += blockDim.x) {
-    const double l = k > 0 ? fabs(job.e[k - 1]) : 0.0, r = k + 1 < s ? fabs(job.e[k]) : 0.0;
-    big = fmax(big, fabs(job.d[k]) + l + r);
+    const double2 q = sm[k];
+    big = fmax(big, fabs(q.x) + (k > 0 ? fabs(sm[k - 1].y) : 0.0) + fabs(q.y));
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) big = fmax(big, __shfl_xor_sync(0xffffffffu, big, o));
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = big;
-  for (int k = threadIdx.x; k < (s + 31) / 32; k += blockDim.x) mask[k] = 0u;
   __syncthreads();
   big = 0.0;
   for (int k = 0; k < (int)(blockDim.x >> 5); ++k) big = fmax(big, red[k]);
   t.norm = big;
   const double inv = big > 0.0 ? 1.0 / big : 0.0;
   for (int k = threadIdx.x; k < s; k += blockDim.x) {
-    const double e = k + 1 < s ? job.e[k] * inv : 0.0;
+    const double2 q = sm[k];
+    const double e = q.y * inv;
     const bool cut = fabs(e) <= kSplitRel;
-    t.de[k] = make_double2(job.d[k] * inv, cut ? 0.0 : e);
+    sm[k] = make_double2(q.x * inv, cut ? 0.0 : e);
     if (cut) atomicOr(&mask[k >> 5], 1u << (k & 31));
   }
   __syncthreads();
@@ -579,101 +584,163 @@ __device__ __forceinline__ void tri_block(const TriShared& t, int s, int i, int&
   }
 }
 
-// Eigenvalues below x of the block [b0, b1): sign changes of the leading principal minors of T - x I.  The
-// three-term recurrence has one dependent multiply-add a step (8.6 cycles; a division form has a division, 63);
-// eight steps' coefficients are fetched ahead of their use, and every eight steps the pair is brought back to unit size.
-__device__ __forceinline__ int sturm_count(const double2* de, int b0, int b1, double x) {
-  double p0 = 0.0, p1 = 1.0, e2 = 0.0;
-  int cnt = 0;
-  for (int k = b0; k < b1; k += 8) {
-    double2 q[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) q[u] = de[k + u];        // (d, e^2); eight entries of padding behind the last
-    if (k + 8 > b1) {                                    // what is not in the block: a diagonal of 2, no sign change
-#pragma unroll
-      for (int u = 0; u < 8; ++u)
-        if (k + u >= b1) q[u] = make_double2(2.0, 0.0);
-    }
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const double p2 = fma(q[u].x - x, p1, -(e2 * p0));
-      cnt += (unsigned)(__double2hiint(p2) ^ __double2hiint(p1)) >> 31;
-      p0 = p1; p1 = p2;
-      e2 = q[u].y;
-    }
-    const int h = max(__double2hiint(p0) & 0x7ff00000, __double2hiint(p1) & 0x7ff00000);
-    if (h > 0 && h < 0x7fe00000) {
-      const double sc = __hiloint2double(0x7fe00000 - h, 0);
-      p0 *= sc; p1 *= sc;
-    }
+// T splits somewhere inside (the bit of the last row is always set)
+__device__ __forceinline__ bool tri_splits(const TriShared& t, int s) {
+  for (int w = 0; w < (s + 31) / 32; ++w)
+    if (t.mask[w] & (w == (s - 1) >> 5 ? ~(1u << ((s - 1) & 31)) : 0xffffffffu)) return true;
+  return false;
+}
+
+// the power of two that brings the larger of two numbers to unit size
+__device__ __forceinline__ double pair_scale(double p0, double p1) {
+  const int h = max(__double2hiint(p0) & 0x7ff00000, __double2hiint(p1) & 0x7ff00000);
+  return (h > 0 && h < 0x7fe00000) ? __hiloint2double(0x7fe00000 - h, 0) : 1.0;
+}
+
+// Eigenvalues below x of the block [b0, b1): sign changes of the leading principal minors p[k] of T - x I, scaled by
+// factors s[k] > 0 with s[k + 1] = s[k - 1] / e[k - 1]^2, which leaves
+//   p[k + 1] = beta[k] (d[k] - x) p[k] - p[k - 1],   beta[k] = s[k + 1] / s[k]:
+// two multiply-adds a step, one of them dependent (8.5 cycles), and the signs are collected by one shift.  ab: (beta d, beta).
+// Every eight steps the pair is brought back to unit size and beta starts at 1 again, for which the older of the two is scaled
+// by ratio: between splits e^2 >= 5e-32, so eight steps stay within 1e127.  The coefficients are fetched eight steps ahead.
+// Cycles a step, one warp and four warps a scheduler: 15 and 40 (unscaled, a difference, a product and a multiply-add a step: 23 and 49).
+__device__ __forceinline__ int sturm_count(const double2* ab, const double* ratio, int b0, int b1, double x) {
+  double p0 = 0.0, p1 = 1.0, sc = 1.0;
+  unsigned m = 0;
+  int cnt = 0, k0 = b0 & ~7;
+  auto step = [&](const double2 q) {
+    const double p2 = fma(fma(-x, q.y, q.x), p1, -p0);
+    m = __funnelshift_l((unsigned)__double2hiint(p2), m, 1);
+    p0 = p1; p1 = p2;
+  };
+  if (k0 < b0) {                                         // the rest of a group that the block starts inside of
+    for (int u = b0 - k0; u < 8; ++u) step(ab[k0 + u]);
+    unsigned keep = 0xffu >> (b0 - k0);
+    if (k0 + 8 > b1) keep &= 0xffu << (k0 + 8 - b1);
+    cnt = __popc((m ^ (m >> 1)) & keep);
+    k0 += 8;
+    if (k0 >= b1) return cnt;
+    sc = pair_scale(p0, p1);
+    p0 = p0 * ratio[k0 >> 3] * sc; p1 *= sc;
   }
-  return cnt;
+  double2 q[8];
+#pragma unroll
+  for (int u = 0; u < 8; ++u) q[u] = ab[k0 + u];         // padded to whole pairs of groups, and a group behind
+  for (;;) {
+#pragma unroll
+    for (int g = 0; g < 2; ++g) {
+      const double rn = ratio[(k0 >> 3) + g + 1];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        step(q[u]);
+        q[u] = ab[k0 + 8 * g + 8 + u];
+        if (u == 5) sc = pair_scale(p0, p1);             // two steps early, off the chain: they add 1e32 at most
+      }
+      p0 = p0 * rn * sc; p1 *= sc;
+    }
+    k0 += 16;
+    const unsigned chg = m ^ (m >> 1);
+    if (k0 >= b1) return cnt + __popc(chg & 0xffffu & (0xffffu << (k0 - b1)));
+    cnt += __popc(chg & 0xffffu);
+  }
 }
 
 // Position i of T carries the (i - b0)-th smallest eigenvalue of its block.  kLanes lanes share the position: each
 // pass cuts the interval into kLanes + 1 parts, so a lone matrix takes 32 lanes (11 passes) and a batch that fills the
-// device by itself 4 (23 passes, least work in all).
+// device by itself 4 (24 passes, least time in all: 2 take 35, and one warp a scheduler costs half of what four do).
+// Where T does not split, the positions below s - need carry values that nobody asks for: they get -2, below everything.
 template <int kLanes>
 __global__ void __launch_bounds__(128)
 tri_values_kernel(const EigJob* __restrict__ jobs) {
   extern __shared__ __align__(16) double2 eig_sm[];
   __shared__ unsigned mask[kMaxOrder / 32];
   __shared__ double red[4];
+  __shared__ double ratio[kMaxOrder / 8 + 4];
   const EigJob job = jobs[blockIdx.y];
   const int s = job.s;
-  const int per = 128 / kLanes;
+  constexpr int per = 128 / kLanes;
   if ((int)blockIdx.x * per >= s) return;
   TriShared t;
   tri_load(job, t, eig_sm, mask, red);
-  for (int k = threadIdx.x; k < s + 8; k += 128) {
-    const double e = k < s ? eig_sm[k].y : 0.0;
-    eig_sm[k] = make_double2(k < s ? eig_sm[k].x : 2.0, e * e);
+  const int i = blockIdx.x * per + threadIdx.x / kLanes, sub = threadIdx.x % kLanes;
+  const int unasked = tri_splits(t, s) ? 0 : s - job.need;
+  if ((int)(blockIdx.x + 1) * per <= unasked) {          // the same for the whole block
+    if (sub == 0) job.lam[i] = -2.0;
+    return;
+  }
+  int b0 = 0, b1 = 1;
+  const bool in = i < s && i >= unasked;
+  if (in) tri_block(t, s, i, b0, b1);
+  double lo = -1.0000001, hi = 1.0000001;
+  if (in && b1 - b0 == 1) { lo = hi = t.de[b0].x; }
+  __syncthreads();                                       // before the diagonal is scaled
+  for (int g = threadIdx.x; 8 * g < s; g += 128) {
+    double beta = 1.0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int k = 8 * g + u;
+      const double2 q = k < s ? eig_sm[k] : make_double2(2.0, 0.0);
+      eig_sm[k] = make_double2(q.x * beta, beta);
+      const double eb = q.y * q.y * beta;
+      if (u == 7) ratio[g + 1] = eb;
+      else beta = eb > 0.0 ? 1.0 / eb : 1.0;
+    }
   }
   __syncthreads();
-  const int i = blockIdx.x * per + threadIdx.x / kLanes, sub = threadIdx.x % kLanes;
-  const bool in = i < s;
-  int b0 = 0, b1 = 1;
-  if (in) tri_block(t, s, i, b0, b1);
   const int want = i - b0;
-  double lo = -1.0000001, hi = 1.0000001;
   const unsigned gmask = (0xffffffffu >> (32 - kLanes)) << ((threadIdx.x & 31) / kLanes * kLanes);
-  if (in && b1 - b0 == 1) { lo = hi = t.de[b0].x; }
   constexpr int kPasses = kLanes == 4 ? 24 : kLanes == 8 ? 18 : 11;
   for (int pass = 0; pass < kPasses; ++pass) {
     const double wdt = (hi - lo) * (1.0 / (kLanes + 1));
     const double x = lo + wdt * (sub + 1);
-    int below = 0;                                    // x is at or below the wanted eigenvalue
-    if (in && hi - lo > 2e-16 * fmax(fabs(lo), fabs(hi)) + 1e-18) below = sturm_count(t.de, b0, b1, x) <= want ? 1 : 0;
-    else below = 2;
-    const unsigned bal = __ballot_sync(0xffffffffu, below == 1) & gmask;
-    if (below != 2) {
+    const bool open = in && hi - lo > 2e-16 * fmax(fabs(lo), fabs(hi)) + 1e-18;
+    const bool below = open && sturm_count(t.de, ratio, b0, b1, x) <= want;        // x is at or below the wanted eigenvalue
+    const unsigned bal = __ballot_sync(0xffffffffu, below) & gmask;
+    if (open) {
       const int nb = __popc(bal);                     // counts rise with x: the first nb points are below
       const double l0 = lo;
       if (nb > 0) lo = l0 + wdt * nb;
       if (nb < kLanes) hi = l0 + wdt * (nb + 1);
     }
   }
-  if (in && sub == 0) { job.lam[i] = 0.5 * (lo + hi); if (i == 0) job.norm[0] = t.norm; }
+  if (i < s && sub == 0) { job.lam[i] = in ? 0.5 * (lo + hi) : -2.0; if (i == s - 1) job.norm[0] = t.norm; }
 }
 
-// Eigenvector of T at lam: L from the factorisation from the top, U from the one from the bottom, joined where the
-// joint pivot is smallest (twisted factorisation; Fernando, and Dhillon and Parlett).  Warp 0 of a block works
-// from the top, warp 1 from the bottom, a lane per eigenvalue.  z[k][i]: component k of vector i, not normalised;
-// outside its block a vector is zero.
+// Eigenvector z of T at lam (twisted factorisation; Fernando, and Dhillon and Parlett), without its divisions.  u
+// solves all rows of (T - lam) u = 0 but the last from the top, w all but the first from the bottom; z is u down to a row tw, w from
+// there on, joined at size 1.  The residual is the joint pivot in row tw, which is the constant e[k] (u[k] w[k+1] - u[k+1] w[k])
+// over u[tw] w[tw], so tw is where |u w| is largest.  A step is
+//   u[k+1] = ((lam - d[k]) u[k] - e[k-1] u[k-1]) / e[k],   the quotients of e worked out once for all lanes:
+// one dependent multiply-add, where the factorisation had a dependent division (145 cycles).  Every eight steps the pair is brought back to
+// unit size and the exponent noted.  A split (e = 0) starts the recurrence anew; outside its block a vector is zero.
+// A block works on 32 eigenvalues, a lane each: warp 0 from the top, warp 1 from the bottom, then all warps share the rows.
+// z[k][i]: component k of vector i, not normalised.
 // The blocks behind the vector blocks form the dot products inside each group of kGroup reflectors that the back
 // transform needs.
-__global__ void __launch_bounds__(64)
-tri_vectors_kernel(const EigJob* __restrict__ jobs, int vec_blocks) {
+constexpr int kVecWarps = 8;
+constexpr int kNoKey = -2147483647 - 1;
+
+// order of the size of |v| 2^e among values of any exponent: exponent and 13 bits
+__device__ __forceinline__ int size_key(double v, int e) {
+  const int hi = __double2hiint(v) & 0x7fffffff;
+  return hi < 0x00100000 ? kNoKey : ((hi >> 20) + e) * 8192 + ((hi >> 7) & 0x1fff);
+}
+inline size_t vectors_smem(int smax) {
+  return (size_t)smax * (sizeof(double2) * 3 + sizeof(double)) + (size_t)((smax + 7) / 8) * 64 * sizeof(int);
+}
+
+__global__ void __launch_bounds__(32 * kVecWarps)
+tri_vectors_kernel(const EigJob* __restrict__ jobs, int vec_blocks, int smax) {
   extern __shared__ __align__(16) double2 eig_sm[];
   __shared__ unsigned mask[kMaxOrder / 32];
-  __shared__ double red[2];
-  __shared__ double best_g[2][32];
-  __shared__ int best_k[2][32];
+  __shared__ double red[kVecWarps];
+  __shared__ double part[kVecWarps][32];
+  __shared__ int best_key[kVecWarps][32], best_row[kVecWarps][32];
   const EigJob job = jobs[blockIdx.y];
   const int s = job.s;
-  const int half = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if ((int)blockIdx.x >= vec_blocks) {
-    const int g = ((int)blockIdx.x - vec_blocks) * 2 + half, j0 = g * kGroup;
+    const int g = ((int)blockIdx.x - vec_blocks) * kVecWarps + warp, j0 = g * kGroup;
     if (j0 >= s) return;
     int idx = 0;
     for (int a = 0; a < kGroup; ++a)
@@ -689,90 +756,140 @@ tri_vectors_kernel(const EigJob* __restrict__ jobs, int vec_blocks) {
   if ((int)blockIdx.x * 32 >= s) return;
   TriShared t;
   tri_load(job, t, eig_sm, mask, red);
+  if (!tri_splits(t, s) && (int)blockIdx.x * 32 + 32 <= s - job.need) return;      // vectors that nobody asks for
+  double2* fwd = eig_sm + smax;               // (1 / e[k], e[k-1] / e[k])
+  double2* bwd = fwd + smax;                  // (1 / e[k-1], e[k] / e[k-1])
+  double* dd = reinterpret_cast<double*>(bwd + smax);
+  int* ex = reinterpret_cast<int*>(dd + smax);               // exponents of u, then of w: [group of eight rows][lane]
+  int* exw = ex + (smax + 7) / 8 * 32;
+  for (int k = threadIdx.x; k < s; k += 32 * kVecWarps) {
+    const double2 q = t.de[k];
+    const double el = k > 0 ? t.de[k - 1].y : 0.0;
+    const double ir = q.y != 0.0 ? 1.0 / q.y : 0.0, il = el != 0.0 ? 1.0 / el : 0.0;
+    fwd[k] = make_double2(ir, el * ir);
+    bwd[k] = make_double2(il, q.y * il);
+    dd[k] = q.x;
+  }
   const int i = blockIdx.x * 32 + lane;
   const bool in = i < s;
-  double* Lp = job.zp + i;
-  double* Up = job.zm + i;
-  int b0 = 0, b1 = 0;
+  double* up = job.zp + i;
+  double* wp = job.zm + i;
+  int b0 = s, b1 = 0;
   double lam = 0.0;
-  constexpr double tiny = 1e-290;
-  const double2* de = t.de;
-  if (in) {
-    tri_block(t, s, i, b0, b1);
-    lam = job.lam[i];
-    if (half == 0) {          // L[k] = e[k] / D+[k], k = b0 .. b1 - 2
-      double2 c = de[b0];
-      double D = c.x - lam;
-      for (int k = b0; k + 1 < b1; ++k) {
-        const double2 cn = de[k + 1];
-        if (fabs(D) < tiny) D = D < 0.0 ? -tiny : tiny;
-        const double L = c.y / D;
-        Lp[(size_t)k * s] = L;
-        D = fma(-L, c.y, cn.x - lam);
-        c = cn;
+  if (in) { tri_block(t, s, i, b0, b1); lam = job.lam[i]; }
+  // rows any lane of the block works on, in whole groups of eight
+  const int g0 = __reduce_min_sync(0xffffffffu, b0) >> 3, g1 = (__reduce_max_sync(0xffffffffu, b1) + 7) >> 3;
+  __syncthreads();
+  if (warp == 0) {
+    double u = 0.0, um = 0.0;
+    int E = 0;
+    for (int g = g0; g < g1; ++g) {
+      const int h = max(__double2hiint(u) & 0x7ff00000, __double2hiint(um) & 0x7ff00000);
+      if (h > 0 && h < 0x7fe00000) {
+        const double sc = __hiloint2double(0x7fe00000 - h, 0);
+        u *= sc; um *= sc; E += (h >> 20) - 1023;
       }
-    } else {                  // U[k] = e[k - 1] / D-[k], k = b1 - 1 .. b0 + 1
-      double D = de[b1 - 1].x - lam;
-      for (int k = b1 - 1; k > b0; --k) {
-        const double2 cn = de[k - 1];
-        if (fabs(D) < tiny) D = D < 0.0 ? -tiny : tiny;
-        const double U = cn.y / D;
-        Up[(size_t)k * s] = U;
-        D = fma(-U, cn.y, cn.x - lam);
+      ex[g * 32 + lane] = E;
+      const int k0 = 8 * g, n = min(8, s - k0);
+      const bool starts = __any_sync(0xffffffffu, (b0 >> 3) == g);
+      double2 q[8];
+      double d[8];
+#pragma unroll
+      for (int v = 0; v < 8; ++v)
+        if (v < n) { q[v] = fwd[k0 + v]; d[v] = dd[k0 + v]; }
+#pragma unroll
+      for (int v = 0; v < 8; ++v) {
+        if (v >= n) break;
+        if (starts && k0 + v == b0) { u = 1.0; um = 0.0; }
+        if (in) up[(size_t)(k0 + v) * s] = u;
+        const double un = fma((lam - d[v]) * q[v].x, u, -(q[v].y * um));
+        um = u; u = un;
+      }
+    }
+  } else if (warp == 1) {
+    double w = 0.0, wm = 0.0;
+    int E = 0;
+    for (int g = g1 - 1; g >= g0; --g) {
+      const int h = max(__double2hiint(w) & 0x7ff00000, __double2hiint(wm) & 0x7ff00000);
+      if (h > 0 && h < 0x7fe00000) {
+        const double sc = __hiloint2double(0x7fe00000 - h, 0);
+        w *= sc; wm *= sc; E += (h >> 20) - 1023;
+      }
+      exw[g * 32 + lane] = E;
+      const int k0 = 8 * g, n = min(8, s - k0);
+      const bool starts = __any_sync(0xffffffffu, (b1 - 1) >> 3 == g);
+      double2 q[8];
+      double d[8];
+#pragma unroll
+      for (int v = 0; v < 8; ++v)
+        if (v < n) { q[v] = bwd[k0 + v]; d[v] = dd[k0 + v]; }
+#pragma unroll
+      for (int v = 7; v >= 0; --v) {
+        if (v >= n) continue;
+        if (starts && k0 + v == b1 - 1) { w = 1.0; wm = 0.0; }
+        if (in) wp[(size_t)(k0 + v) * s] = w;
+        const double wn = fma((lam - d[v]) * q[v].x, w, -(q[v].y * wm));
+        wm = w; w = wn;
       }
     }
   }
   __syncthreads();
-  {                           // joint pivot at k: d - lam - e[k-1] L[k-1] - e[k] U[k+1]
-    double bg = 1e300;
-    int bk = b0;
-    if (in) {
-      const int mid = (b0 + b1) >> 1;
-      const int k0 = half ? mid : b0, k1 = half ? b1 : mid;
-#pragma unroll 8
-      for (int k = k0; k < k1; ++k) {
-        const double2 c = de[k];
-        double g = c.x - lam;
-        if (k > b0) g = fma(-de[k - 1].y, __ldcg(Lp + (size_t)(k - 1) * s), g);
-        if (k + 1 < b1) g = fma(-c.y, __ldcg(Up + (size_t)(k + 1) * s), g);
-        if (fabs(g) < bg) { bg = fabs(g); bk = k; }
+  {                           // where |u w| is largest
+    int key = kNoKey, row = min(b0, s - 1);
+    for (int g = g0 + warp; g < g1; g += kVecWarps) {
+      const int k0 = 8 * g, n = in ? min(8, s - k0) : 0;
+      double a[8], c[8], top = 0.0;
+      int at = k0;
+#pragma unroll
+      for (int v = 0; v < 8; ++v) {
+        a[v] = v < n ? up[(size_t)(k0 + v) * s] : 0.0;
+        c[v] = v < n ? wp[(size_t)(k0 + v) * s] : 0.0;
       }
+#pragma unroll
+      for (int v = 0; v < 8; ++v) {
+        const double p = fabs(a[v] * c[v]);
+        if (p > top) { top = p; at = k0 + v; }
+      }
+      const int ky = size_key(top, ex[g * 32 + lane] + exw[g * 32 + lane]);
+      if (ky > key) { key = ky; row = at; }
     }
-    best_g[half][lane] = bg;
-    best_k[half][lane] = bk;
+    best_key[warp][lane] = key;
+    best_row[warp][lane] = row;
   }
   __syncthreads();
+  int tw = best_row[0][lane], key = best_key[0][lane];
+#pragma unroll
+  for (int v = 1; v < kVecWarps; ++v)
+    if (best_key[v][lane] > key) { key = best_key[v][lane]; tw = best_row[v][lane]; }
+  const double ui = in ? 1.0 / up[(size_t)tw * s] : 0.0, wi = in ? 1.0 / wp[(size_t)tw * s] : 0.0;
+  const int eu = ex[(tw >> 3) * 32 + lane], ew = exw[(tw >> 3) * 32 + lane];
+  __syncthreads();            // before row tw is overwritten
   double n2 = 0.0;
-  const int tw = best_g[1][lane] < best_g[0][lane] ? best_k[1][lane] : best_k[0][lane];
-  if (in) {                   // eight factors fetched ahead of the chain that uses them
-    double z = 1.0;
-    if (half == 0) {
-      n2 = 1.0;
-      for (int k = tw - 1; k >= b0; k -= 8) {
-        double f[8];
+  for (int g = warp; 8 * g < s; g += kVecWarps) {
+    const int k0 = 8 * g, n = in ? min(8, s - k0) : 0;
+    const bool live = g >= g0 && g < g1;
+    double a[8], c[8];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) f[u] = k - u >= b0 ? Lp[(size_t)(k - u) * s] : 0.0;
+    for (int v = 0; v < 8; ++v) {
+      a[v] = live && v < n && k0 + v <= tw ? up[(size_t)(k0 + v) * s] : 0.0;
+      c[v] = live && v < n && k0 + v > tw ? wp[(size_t)(k0 + v) * s] : 0.0;
+    }
+    const double fu = live ? ldexp(ui, ex[g * 32 + lane] - eu) : 0.0, fw = live ? ldexp(wi, exw[g * 32 + lane] - ew) : 0.0;
 #pragma unroll
-        for (int u = 0; u < 8; ++u)
-          if (k - u >= b0) { z *= -f[u]; n2 = fma(z, z, n2); Lp[(size_t)(k - u) * s] = z; }
-      }
-      for (int k = 0; k < b0; ++k) Lp[(size_t)k * s] = 0.0;
-    } else {
-      for (int k = tw + 1; k < b1; k += 8) {
-        double f[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) f[u] = k + u < b1 ? Up[(size_t)(k + u) * s] : 0.0;
-#pragma unroll
-        for (int u = 0; u < 8; ++u)
-          if (k + u < b1) { z *= -f[u]; n2 = fma(z, z, n2); Lp[(size_t)(k + u) * s] = z; }
-      }
-      for (int k = b1; k < s; ++k) Lp[(size_t)k * s] = 0.0;
-      Lp[(size_t)tw * s] = 1.0;
+    for (int v = 0; v < 8; ++v) {
+      const double z = k0 + v <= tw ? a[v] * fu : c[v] * fw;
+      n2 = fma(z, z, n2);
+      if (v < n) up[(size_t)(k0 + v) * s] = z;
     }
   }
-  best_g[half][lane] = n2;
+  part[warp][lane] = n2;
   __syncthreads();
-  if (in && half == 0) job.inv[i] = 1.0 / sqrt(best_g[0][lane] + best_g[1][lane]);
+  if (in && warp == 0) {
+    n2 = 0.0;
+#pragma unroll
+    for (int v = 0; v < kVecWarps; ++v) n2 += part[v][lane];
+    job.inv[i] = 1.0 / sqrt(n2);
+  }
 }
 
 // ---- 4. back transform ----------------------------------------------------------------------------------
@@ -1124,7 +1241,7 @@ int launch_tridiag(const EigJob* jobs, int count, int CL, int* status, cudaStrea
 template <int L>
 int launch_values(const EigJob* jobs, int count, int smax, cudaStream_t st) {
   const int per = 128 / L;
-  tri_values_kernel<L><<<dim3((unsigned)((smax + per - 1) / per), (unsigned)count), 128, (smax + 8) * sizeof(double2), st>>>(jobs);
+  tri_values_kernel<L><<<dim3((unsigned)((smax + per - 1) / per), (unsigned)count), 128, (smax + 32) * sizeof(double2), st>>>(jobs);
   AB_LAUNCH_OK();
   return AB_OK;
 }
@@ -1199,13 +1316,15 @@ int eig_direct(const EigJob* h_jobs, const EigJob* d_jobs, int count, int smax, 
   else
     rc = 8 * count <= sms ? launch_tridiag<8, 4, 8, false>(d_jobs, count, 8, status, st) : launch_tridiag<8, 8, 8, false>(d_jobs, count, 4, status, st);
   AB_TRY(rc);
-  const long long values = (long long)count * smax;
+  long long values = 0;
+  for (int i = 0; i < count; ++i) values += h_jobs[i].need;
   if (values <= 16LL * sms) rc = launch_values<32>(d_jobs, count, smax, st);
   else if (values <= 64LL * sms) rc = launch_values<8>(d_jobs, count, smax, st);
   else rc = launch_values<4>(d_jobs, count, smax, st);
   AB_TRY(rc);
-  const int vb = (smax + 31) / 32, gb = ((smax + kGroup - 1) / kGroup + 1) / 2;
-  tri_vectors_kernel<<<dim3((unsigned)(vb + gb), (unsigned)count), 64, smax * sizeof(double2), st>>>(d_jobs, vb);
+  const int vb = (smax + 31) / 32, gb = ((smax + kGroup - 1) / kGroup + kVecWarps - 1) / kVecWarps;
+  AB_CUDA_OK(allow_smem(tri_vectors_kernel, 8192));
+  tri_vectors_kernel<<<dim3((unsigned)(vb + gb), (unsigned)count), 32 * kVecWarps, vectors_smem(smax), st>>>(d_jobs, vb, smax);
   AB_LAUNCH_OK();
   if (smax > 1024) return launch_back_big<10>(d_jobs, count, smax, st);
   if (smax > 768) return launch_back_big<8>(d_jobs, count, smax, st);
