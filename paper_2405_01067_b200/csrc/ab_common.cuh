@@ -252,7 +252,8 @@ struct EigJob {
   float* rows;        // need x s: unit rows, descending eigenvalue
   float* vals;        // need: the eigenvalue (gram 0) or its square root, 0 below 1e-6 of the largest (gram 1); may be null
   int* flag;          // set to 1 when close vectors came out less than orthogonal (the caller clears it)
-  double *xbuf, *refl, *zp, *zm, *d, *e, *gam, *lam, *inv, *cross, *norm;
+  double *xbuf, *refl, *tmat, *zp, *zm, *d, *e, *gam, *lam, *inv, *norm;
+  int* order;
 };
 size_t eig_ws_doubles(int s);
 void eig_bind(EigJob& j, double* ws);

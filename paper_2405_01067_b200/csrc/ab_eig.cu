@@ -36,7 +36,11 @@ constexpr double kCloseRel = 1e-7;      // eigenvalues closer than this fraction
 constexpr double kOrthTol = 4e-6;       // what the Jacobi route leaves at small orders
 constexpr int kMaxOrder = 1280;         // masks are sized for this order
 constexpr double kLive2 = 1e-290;       // a column whose squared norm is below this needs no reflector
-constexpr int kGroup = 4;               // reflectors applied together in the back transform
+constexpr int kGroup = 8;               // reflectors applied together in the back transform
+
+// Reflectors are rows of an even number of doubles (bulk copies of whole rows start and end on 16 bytes), zero before and
+// behind their elements.
+__host__ __device__ __forceinline__ int refl_ld(int s) { return (s + 1) & ~1; }
 
 // Eigenvalues (fractions of the norm) that carry nothing: a core's sigma below 1e-6 of the largest is zero to its
 // caller; a Gram matrix that was rounded to fp32 has noise of 2^-24 of its entries for eigenvalues down there.
@@ -226,10 +230,11 @@ struct Tridiag {
       if (warp == 0) {                               // off the chain: gamma, and what later kernels need
         x.gam = den > 0.0 ? 1.0 / den : 0.0;
         if (rank == j % CL) {
-          double* dst = job.refl + (size_t)j * s;
+          const int ld = refl_ld(s);
+          double* dst = job.refl + (size_t)j * ld;
 #pragma unroll
           for (int e = 0; e < E; ++e)
-            if (lane + 32 * e < s) dst[lane + 32 * e] = e < E0 ? 0.0 : vn[e];
+            if (lane + 32 * e < ld) dst[lane + 32 * e] = e < E0 ? 0.0 : vn[e];
           if (lane == 0) { job.d[j] = dj; job.e[j] = (j + 1 < s) ? beta : 0.0; job.gam[j] = x.gam; }
         }
       }
@@ -511,10 +516,11 @@ tridiag_grid_kernel(const EigJob* __restrict__ jobs, int count, int C, int* stat
       gam = live ? 1.0 / (nrm * (nrm + fabs(alpha))) : 0.0;
       // what later kernels need, from the owner of row j + 1 (it is still here)
       if ((j + 1) % C == cta) {
-        double* dst = job.refl + (size_t)j * s;
+        const int ld = refl_ld(s);
+        double* dst = job.refl + (size_t)j * ld;
 #pragma unroll
         for (int e = 0; e < E; ++e)
-          if (tid + kGridThreads * e < s) dst[tid + kGridThreads * e] = vn[e];
+          if (tid + kGridThreads * e < ld) dst[tid + kGridThreads * e] = vn[e];
         if (tid == 0) { job.d[j] = dj; job.e[j] = beta; job.gam[j] = gam; }
       }
 #pragma unroll
@@ -522,8 +528,8 @@ tridiag_grid_kernel(const EigJob* __restrict__ jobs, int count, int C, int* stat
     }
     if (*reinterpret_cast<volatile int*>(&dead)) break;
     if (last == s - 1) {                 // the last diagonal element is what its row would have sent
-      double* dst = job.refl + (size_t)(s - 1) * s;
-      for (int k = tid; k < s; k += kGridThreads) dst[k] = 0.0;
+      double* dst = job.refl + (size_t)(s - 1) * refl_ld(s);
+      for (int k = tid; k < refl_ld(s); k += kGridThreads) dst[k] = 0.0;
       if (tid == 0) { job.d[s - 1] = colbuf[(s - 1) / C]; job.e[s - 1] = 0.0; job.gam[s - 1] = 0.0; }
     }
     __syncthreads();                     // colbuf is read before the next matrix writes it
@@ -715,8 +721,8 @@ tri_values_kernel(const EigJob* __restrict__ jobs) {
 // unit size and the exponent noted.  A split (e = 0) starts the recurrence anew; outside its block a vector is zero.
 // A block works on 32 eigenvalues, a lane each: warp 0 from the top, warp 1 from the bottom, then all warps share the rows.
 // z[k][i]: component k of vector i, not normalised.
-// The blocks behind the vector blocks form the dot products inside each group of kGroup reflectors that the back
-// transform needs.
+// The block also sorts its vectors among all: order[rank] is the position of the vector with that rank (descending).
+// The blocks behind the vector blocks form the factors of the groups of reflectors (group_factor).
 constexpr int kVecWarps = 8;
 constexpr int kNoKey = -2147483647 - 1;
 
@@ -726,7 +732,41 @@ __device__ __forceinline__ int size_key(double v, int e) {
   return hi < 0x00100000 ? kNoKey : ((hi >> 20) + e) * 8192 + ((hi >> 7) & 0x1fff);
 }
 inline size_t vectors_smem(int smax) {
-  return (size_t)smax * (sizeof(double2) * 3 + sizeof(double)) + (size_t)((smax + 7) / 8) * 64 * sizeof(int);
+  const size_t n = (size_t)(smax + 7) / 8 * 8;
+  return n * (sizeof(double2) * 3 + 2 * sizeof(double) + 8 * sizeof(int));
+}
+
+// H[j0] ... H[j0 + 7] = I - V T V^T, T upper triangular (compact WY form; Schreiber and Van Loan), one warp a group.
+// A reflector of a small column has gamma up to 1e290 and v of 1e-145: the sums below pair a gamma with a dot product first.
+__device__ __forceinline__ void group_factor(const EigJob& job, int g, int j0, int lane) {
+  const int s = job.s, ld = refl_ld(s);
+  double dot[kGroup][kGroup];
+#pragma unroll
+  for (int a = 0; a < kGroup; ++a)
+#pragma unroll
+    for (int b = a + 1; b < kGroup; ++b) dot[a][b] = 0.0;
+  for (int k = (j0 & ~31) + lane; k < s; k += 32) {
+    double f[kGroup];
+#pragma unroll
+    for (int a = 0; a < kGroup; ++a) f[a] = j0 + a < s ? job.refl[(size_t)(j0 + a) * ld + k] : 0.0;
+#pragma unroll
+    for (int a = 0; a < kGroup; ++a)
+#pragma unroll
+      for (int b = a + 1; b < kGroup; ++b) dot[a][b] = fma(f[a], f[b], dot[a][b]);
+  }
+  double row[kGroup];                   // lane i: row i of T
+#pragma unroll
+  for (int b = 0; b < kGroup; ++b) {
+    const double gm = j0 + b < s ? job.gam[j0 + b] : 0.0;
+    double acc = 0.0;
+#pragma unroll
+    for (int a = 0; a < b; ++a) acc = fma(a >= lane ? row[a] : 0.0, warp_sum(dot[a][b]), acc);
+    row[b] = b == lane ? gm : b > lane ? -gm * acc : 0.0;
+  }
+  if (lane < kGroup) {
+#pragma unroll
+    for (int b = 0; b < kGroup; ++b) job.tmat[(size_t)g * kGroup * kGroup + lane * kGroup + b] = row[b];
+  }
 }
 
 __global__ void __launch_bounds__(32 * kVecWarps)
@@ -735,40 +775,34 @@ tri_vectors_kernel(const EigJob* __restrict__ jobs, int vec_blocks, int smax) {
   __shared__ unsigned mask[kMaxOrder / 32];
   __shared__ double red[kVecWarps];
   __shared__ double part[kVecWarps][32];
-  __shared__ int best_key[kVecWarps][32], best_row[kVecWarps][32];
+  __shared__ int best_key[kVecWarps][32], best_row[kVecWarps][32], rank_part[kVecWarps][32];
   const EigJob job = jobs[blockIdx.y];
   const int s = job.s;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if ((int)blockIdx.x >= vec_blocks) {
     const int g = ((int)blockIdx.x - vec_blocks) * kVecWarps + warp, j0 = g * kGroup;
-    if (j0 >= s) return;
-    int idx = 0;
-    for (int a = 0; a < kGroup; ++a)
-      for (int b = a + 1; b < kGroup; ++b, ++idx) {
-        double acc = 0.0;
-        if (j0 + b < s)
-          for (int k = j0 + b + lane; k < s; k += 32) acc = fma(job.refl[(size_t)(j0 + a) * s + k], job.refl[(size_t)(j0 + b) * s + k], acc);
-        acc = warp_sum(acc);
-        if (lane == 0) job.cross[g * 6 + idx] = acc;
-      }
+    if (j0 < s) group_factor(job, g, j0, lane);
     return;
   }
   if ((int)blockIdx.x * 32 >= s) return;
   TriShared t;
   tri_load(job, t, eig_sm, mask, red);
   if (!tri_splits(t, s) && (int)blockIdx.x * 32 + 32 <= s - job.need) return;      // vectors that nobody asks for
-  double2* fwd = eig_sm + smax;               // (1 / e[k], e[k-1] / e[k])
-  double2* bwd = fwd + smax;                  // (1 / e[k-1], e[k] / e[k-1])
-  double* dd = reinterpret_cast<double*>(bwd + smax);
-  int* ex = reinterpret_cast<int*>(dd + smax);               // exponents of u, then of w: [group of eight rows][lane]
-  int* exw = ex + (smax + 7) / 8 * 32;
-  for (int k = threadIdx.x; k < s; k += 32 * kVecWarps) {
-    const double2 q = t.de[k];
-    const double el = k > 0 ? t.de[k - 1].y : 0.0;
+  const int pad = (smax + 7) & ~7;            // whole groups of eight rows; those behind the last are zero
+  double2* fwd = eig_sm + pad;                // (1 / e[k], e[k-1] / e[k])
+  double2* bwd = fwd + pad;                   // (1 / e[k-1], e[k] / e[k-1])
+  double* dd = reinterpret_cast<double*>(bwd + pad);
+  double* lams = dd + pad;
+  int* ex = reinterpret_cast<int*>(lams + pad);                // exponents of u, then of w: [group of eight rows][lane]
+  int* exw = ex + pad * 4;
+  for (int k = threadIdx.x; k < pad; k += 32 * kVecWarps) {
+    const double2 q = k < s ? t.de[k] : make_double2(0.0, 0.0);
+    const double el = k > 0 && k < s ? t.de[k - 1].y : 0.0;
     const double ir = q.y != 0.0 ? 1.0 / q.y : 0.0, il = el != 0.0 ? 1.0 / el : 0.0;
     fwd[k] = make_double2(ir, el * ir);
     bwd[k] = make_double2(il, q.y * il);
     dd[k] = q.x;
+    if (k < s) lams[k] = job.lam[k];
   }
   const int i = blockIdx.x * 32 + lane;
   const bool in = i < s;
@@ -780,56 +814,36 @@ tri_vectors_kernel(const EigJob* __restrict__ jobs, int vec_blocks, int smax) {
   // rows any lane of the block works on, in whole groups of eight
   const int g0 = __reduce_min_sync(0xffffffffu, b0) >> 3, g1 = (__reduce_max_sync(0xffffffffu, b1) + 7) >> 3;
   __syncthreads();
-  if (warp == 0) {
+  if (warp < 2) {
+    const double2* cf = warp == 0 ? fwd : bwd;
+    double* out = warp == 0 ? up : wp;
+    int* exs = warp == 0 ? ex : exw;
+    const int first = warp == 0 ? b0 : b1 - 1;           // where this lane's block starts
     double u = 0.0, um = 0.0;
     int E = 0;
-    for (int g = g0; g < g1; ++g) {
+    double2 q[8];
+    double d[8];
+    const int dir = warp == 0 ? 1 : -1, flip = warp == 0 ? 0 : 7;
+    int g = warp == 0 ? g0 : g1 - 1;
+#pragma unroll
+    for (int v = 0; v < 8; ++v) { q[v] = cf[8 * g + (v ^ flip)]; d[v] = dd[8 * g + (v ^ flip)]; }
+    for (int n = g1 - g0; n > 0; --n, g += dir) {
       const int h = max(__double2hiint(u) & 0x7ff00000, __double2hiint(um) & 0x7ff00000);
       if (h > 0 && h < 0x7fe00000) {
         const double sc = __hiloint2double(0x7fe00000 - h, 0);
         u *= sc; um *= sc; E += (h >> 20) - 1023;
       }
-      ex[g * 32 + lane] = E;
-      const int k0 = 8 * g, n = min(8, s - k0);
-      const bool starts = __any_sync(0xffffffffu, (b0 >> 3) == g);
-      double2 q[8];
-      double d[8];
-#pragma unroll
-      for (int v = 0; v < 8; ++v)
-        if (v < n) { q[v] = fwd[k0 + v]; d[v] = dd[k0 + v]; }
+      exs[g * 32 + lane] = E;
+      const bool starts = __any_sync(0xffffffffu, first >> 3 == g);
+      const int gn = n > 1 ? g + dir : g;
 #pragma unroll
       for (int v = 0; v < 8; ++v) {
-        if (v >= n) break;
-        if (starts && k0 + v == b0) { u = 1.0; um = 0.0; }
-        if (in) up[(size_t)(k0 + v) * s] = u;
+        const int k = 8 * g + (v ^ flip);
+        if (starts && k == first) { u = 1.0; um = 0.0; }
+        if (in && k < s) out[(size_t)k * s] = u;
         const double un = fma((lam - d[v]) * q[v].x, u, -(q[v].y * um));
         um = u; u = un;
-      }
-    }
-  } else if (warp == 1) {
-    double w = 0.0, wm = 0.0;
-    int E = 0;
-    for (int g = g1 - 1; g >= g0; --g) {
-      const int h = max(__double2hiint(w) & 0x7ff00000, __double2hiint(wm) & 0x7ff00000);
-      if (h > 0 && h < 0x7fe00000) {
-        const double sc = __hiloint2double(0x7fe00000 - h, 0);
-        w *= sc; wm *= sc; E += (h >> 20) - 1023;
-      }
-      exw[g * 32 + lane] = E;
-      const int k0 = 8 * g, n = min(8, s - k0);
-      const bool starts = __any_sync(0xffffffffu, (b1 - 1) >> 3 == g);
-      double2 q[8];
-      double d[8];
-#pragma unroll
-      for (int v = 0; v < 8; ++v)
-        if (v < n) { q[v] = bwd[k0 + v]; d[v] = dd[k0 + v]; }
-#pragma unroll
-      for (int v = 7; v >= 0; --v) {
-        if (v >= n) continue;
-        if (starts && k0 + v == b1 - 1) { w = 1.0; wm = 0.0; }
-        if (in) wp[(size_t)(k0 + v) * s] = w;
-        const double wn = fma((lam - d[v]) * q[v].x, w, -(q[v].y * wm));
-        wm = w; w = wn;
+        q[v] = cf[8 * gn + (v ^ flip)]; d[v] = dd[8 * gn + (v ^ flip)];       // the next group's
       }
     }
   }
@@ -863,7 +877,22 @@ tri_vectors_kernel(const EigJob* __restrict__ jobs, int vec_blocks, int smax) {
     if (best_key[v][lane] > key) { key = best_key[v][lane]; tw = best_row[v][lane]; }
   const double ui = in ? 1.0 / up[(size_t)tw * s] : 0.0, wi = in ? 1.0 / wp[(size_t)tw * s] : 0.0;
   const int eu = ex[(tw >> 3) * 32 + lane], ew = exw[(tw >> 3) * 32 + lane];
+  {
+    int above = 0;
+#pragma unroll 8
+    for (int k = warp; k < s; k += kVecWarps) {
+      const double lk = lams[k];
+      above += (lk > lam || (lk == lam && k < i)) ? 1 : 0;
+    }
+    rank_part[warp][lane] = above;
+  }
   __syncthreads();            // before row tw is overwritten
+  if (in && warp == 0) {
+    int above = 0;
+#pragma unroll
+    for (int v = 0; v < kVecWarps; ++v) above += rank_part[v][lane];
+    job.order[above] = i;
+  }
   double n2 = 0.0;
   for (int g = warp; 8 * g < s; g += kVecWarps) {
     const int k0 = 8 * g, n = in ? min(8, s - k0) : 0;
@@ -893,331 +922,182 @@ tri_vectors_kernel(const EigJob* __restrict__ jobs, int vec_blocks, int smax) {
 }
 
 // ---- 4. back transform ----------------------------------------------------------------------------------
-// A warp carries NV vectors of E elements a lane through all reflectors, last one first.  kGroup reflectors are
-// applied together: their dot products with the vectors go through the warp reduction side by side, and the
-// products among themselves (cross) turn them into the coefficients one after the other would have had.  The eight
-// warps of a block share the reflectors through shared memory, the next group on its way while one is applied
-// (each warp fetching its own was bound by L2: 259 us for 72 matrices of order 192).
-constexpr int kBackWarps = 8;
-template <int E, int NV>
-struct BackGroups {
-  double (&z)[NV][E];
-  double (*fs)[kGroup][32 * E];
-  const double *gs, *xs;
-  double* red;               // this warp's NV x kGroup sums
-  int lane;
-  bool wanted;
-  // the reflectors whose first element lies in the 32-column group E0
-  template <int E0, typename F>
-  __device__ __forceinline__ void segment(int ngroups, F& fetch) {
-    constexpr int kPer = 32 / kGroup;
-    for (int g = min(ngroups, (E0 + 1) * kPer) - 1; g >= E0 * kPer; --g) {
-      asm volatile("cp.async.wait_group 0;" ::: "memory");
-      __syncthreads();                     // group g is here, and nobody reads the buffer of group g + 1 any more
-      if (g > 0) fetch(g - 1);
-      if (!wanted) continue;
-      double f[kGroup][E];
-#pragma unroll
-      for (int a = 0; a < kGroup; ++a)
-#pragma unroll
-        for (int e = E0; e < E; ++e) f[a][e] = fs[g & 1][a][lane + 32 * e];
-      double dt[NV * kGroup];
-#pragma unroll
-      for (int v = 0; v < NV; ++v)
-#pragma unroll
-        for (int a = 0; a < kGroup; ++a) {
-          double acc = 0.0;
-#pragma unroll
-          for (int e = E0; e < E; ++e) acc = fma(f[a][e], z[v][e], acc);
-          dt[v * kGroup + a] = acc;
-        }
-      // NV * kGroup sums across the warp, each exchange halving what a lane still carries; the sums then go round
-      // through shared memory
-      int width = 16;
-      double t;
-      if constexpr (NV == 4) {
-        const bool h = (lane & 16) != 0;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) dt[q] = (h ? dt[q + 8] : dt[q]) + __shfl_xor_sync(0xffffffffu, h ? dt[q] : dt[q + 8], 16);
-        width = 8;
-      }
-      {
-        const bool h = (lane & width) != 0;
-        if constexpr (NV >= 2) {
-#pragma unroll
-          for (int q = 0; q < 4; ++q) dt[q] = (h ? dt[q + 4] : dt[q]) + __shfl_xor_sync(0xffffffffu, h ? dt[q] : dt[q + 4], width);
-          width >>= 1;
-        }
-      }
-      {
-        const bool h = (lane & width) != 0;
-#pragma unroll
-        for (int q = 0; q < 2; ++q) dt[q] = (h ? dt[q + 2] : dt[q]) + __shfl_xor_sync(0xffffffffu, h ? dt[q] : dt[q + 2], width);
-        width >>= 1;
-        const bool h1 = (lane & width) != 0;
-        t = (h1 ? dt[1] : dt[0]) + __shfl_xor_sync(0xffffffffu, h1 ? dt[0] : dt[1], width);
-      }
-      constexpr int kRest = 32 / (NV * kGroup);        // lanes that still hold parts of the same sum
-#pragma unroll
-      for (int o = kRest / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-      __syncwarp();
-      if (lane % kRest == 0) red[lane / kRest] = t;
-      __syncwarp();
-      const double2 g01 = *reinterpret_cast<const double2*>(gs + g * kGroup), g23 = *reinterpret_cast<const double2*>(gs + g * kGroup + 2);
-      const double2 x01 = *reinterpret_cast<const double2*>(xs + g * 6), x23 = *reinterpret_cast<const double2*>(xs + g * 6 + 2),
-                    x45 = *reinterpret_cast<const double2*>(xs + g * 6 + 4);
-#pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        const double2 d01 = *reinterpret_cast<const double2*>(red + v * kGroup), d23 = *reinterpret_cast<const double2*>(red + v * kGroup + 2);
-        // cross: (0,1) (0,2) (0,3) (1,2) (1,3) (2,3); the last reflector acts first
-        const double c3 = g23.y * d23.y;
-        const double c2 = g23.x * fma(-c3, x45.y, d23.x);
-        const double c1 = g01.y * fma(-c3, x45.x, fma(-c2, x23.y, d01.y));
-        const double c0 = g01.x * fma(-c3, x23.x, fma(-c2, x01.y, fma(-c1, x01.x, d01.x)));
-#pragma unroll
-        for (int e = E0; e < E; ++e)
-          z[v][e] = fma(-c0, f[0][e], fma(-c1, f[1][e], fma(-c2, f[2][e], fma(-c3, f[3][e], z[v][e]))));
-      }
-    }
-    if constexpr (E0 > 0) segment<E0 - 1>(ngroups, fetch);
-  }
-};
-
-template <int E, int NV>
-__global__ void __launch_bounds__(32 * kBackWarps)
-back_transform_kernel(const EigJob* __restrict__ jobs) {
-  constexpr int S = 32 * E;
-  extern __shared__ __align__(16) double back_sm[];
-  double (*fs)[kGroup][S] = reinterpret_cast<double (*)[kGroup][S]>(back_sm);   // two groups of reflectors
-  double* gs = back_sm + 2 * kGroup * S;                                           // gamma, padded to a whole group
-  __shared__ __align__(16) double red[kBackWarps][NV * kGroup];
-  double* xs = gs + S + kGroup;                                                    // six products a group
-  const EigJob job = jobs[blockIdx.y];
-  const int s = job.s;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  if ((int)blockIdx.x * kBackWarps * NV >= s) return;
-  const int i0 = (blockIdx.x * kBackWarps + warp) * NV;
-  const int ngroups = (s + kGroup - 1) / kGroup;
-  for (int k = tid; k < ngroups * kGroup; k += 32 * kBackWarps) gs[k] = k < s ? job.gam[k] : 0.0;
-  for (int k = tid; k < ngroups * 6; k += 32 * kBackWarps) xs[k] = job.cross[k];
-  auto fetch = [&](int g) {              // reflector a of group g has its first element at j0 + a + 1
-    const int j0 = g * kGroup, k0 = j0 & ~31, w = S - k0;
-    for (int idx = tid; idx < kGroup * w; idx += 32 * kBackWarps) {
-      const int a = idx / w, k = k0 + idx - a * w;
-      double* d = &fs[g & 1][a][k];
-      if (k < s && j0 + a < s)
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(tc::smem_u32(d)), "l"(job.refl + (size_t)(j0 + a) * s + k) : "memory");
-      else
-        *d = 0.0;
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  };
-  // rank of each vector's eigenvalue among all (descending, ties by position)
-  int rank[NV];
-  double lam[NV];
-  bool wanted = false;
-#pragma unroll
-  for (int v = 0; v < NV; ++v) {
-    const int i = i0 + v;
-    lam[v] = i < s ? job.lam[i] : 0.0;
-    int c = 0;
-    for (int k = lane; k < s; k += 32) {
-      const double lk = job.lam[k];
-      c += (lk > lam[v] || (lk == lam[v] && k < i)) ? 1 : 0;
-    }
-    rank[v] = __reduce_add_sync(0xffffffffu, c);
-    if (i >= s) rank[v] = s;
-    wanted = wanted || rank[v] < job.need;
-  }
-  if (!__syncthreads_or(wanted)) return;
-  double z[NV][E];
-#pragma unroll
-  for (int v = 0; v < NV; ++v) {
-    const int i = i0 + v;
-    const double inv = i < s ? job.inv[i] : 0.0;
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-      const int k = lane + 32 * e;
-      z[v][e] = (wanted && i < s && k < s) ? job.zp[(size_t)k * s + i] * inv : 0.0;
-    }
-    // neighbours too close for the factorisation to keep apart: is this vector orthogonal to them?
-    if (i < s && rank[v] < job.need && lam[v] > null_rel(job)) {
-      for (int k0 = 0; k0 < s; k0 += 32) {
-        const int k = k0 + lane;
-        bool close = false;
-        if (k < s && k != i) {
-          const double lk = job.lam[k];
-          close = fabs(lk - lam[v]) < kCloseRel && (lk > lam[v] || (lk == lam[v] && k < i));
-        }
-        unsigned bal = __ballot_sync(0xffffffffu, close);
-        while (bal) {
-          const int kk = k0 + __ffs(bal) - 1;
-          bal &= bal - 1;
-          double acc = 0.0;
-#pragma unroll
-          for (int e = 0; e < E; ++e) {
-            const int q = lane + 32 * e;
-            if (q < s) acc = fma(z[v][e], job.zp[(size_t)q * s + kk], acc);
-          }
-          acc = warp_sum(acc) * job.inv[kk];
-          if (!(fabs(acc) <= kOrthTol) && lane == 0) *job.flag = 1;
-        }
-      }
-    }
-  }
-  fetch(ngroups - 1);
-  BackGroups<E, NV> bg{z, fs, gs, xs, red[warp], lane, wanted};
-  bg.template segment<E - 1>(ngroups, fetch);
-  const double norm = job.norm[0];
-#pragma unroll
-  for (int v = 0; v < NV; ++v) {
-    if (rank[v] >= job.need) continue;
-    float* dst = job.rows + (size_t)rank[v] * s;
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-      const int k = lane + 32 * e;
-      if (k < s) dst[k] = (float)z[v][e];
-    }
-    if (lane == 0 && job.vals) {
-      const double l = lam[v] * norm;
-      job.vals[rank[v]] = (float)(job.gram ? (l > 1e-12 * norm ? sqrt(l) : 0.0) : l);
-    }
-  }
+// Z <- (I - V T V^T) Z for groups of eight reflectors, last group first: y = V^T z, w = T y, z -= V w.  Each is a product of
+// 8 x 8 pieces on the fp64 tensor path (mma.sync m8n8k4; there is no tcgen05 form for fp64).  Its rate is that of plain
+// multiply-adds, but the sums across lanes and most of the instructions go: with a vector a warp, its dot products reduced by
+// shuffles, order 768 (192 vectors) took 407 us, now 121; 72 matrices of order 192 took 192, now 65.
+// A warp holds Z^T of eight vectors as accumulator pieces: piece t, lane l, element i is vector l / 4, component
+// 8 t + 2 (l % 4) + i.  That is at once the left operand of y^T = Z^T V, if step i of the reduction takes the components
+// 8 t + 2 (l % 4) + i; likewise y^T and w^T are passed on as they come out.  Column c of y and w stands for
+// reflector row_of(c) of the group, an order in which all reads of shared memory are free of bank conflicts.
+// RS warps share the components of the same eight vectors (pieces dealt in turn) and add their parts of y through shared memory: a
+// lone matrix, whose chain of groups is what counts; RS = 1: a batch.  The reflectors of a group and its T come by bulk copies, the next
+// groups' on their way while one is applied.  Columns that a group's reflectors do not reach are dropped kBlock pieces at a time.
+__device__ __forceinline__ void dmma(double (&c)[2], double a, double b) {
+  asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};" : "+d"(c[0]), "+d"(c[1]) : "d"(a), "d"(b));
 }
+__device__ __forceinline__ int row_of(int c) { return (c & 1) ? 4 + (((c >> 1) + 2) & 3) : c >> 1; }
 
-// The same for orders above kEigSmallMax: one vector a warp, reflectors read from shared memory where they are
-// used, finished columns dropped 128 at a time.
-constexpr int kBigWarps = 4;
-template <int EB>
-struct BackBig {
-  static constexpr int E = 4 * EB, S = 32 * E;
-  double (&z)[E];
-  double (*fs)[kGroup][S];
-  const double *gs, *xs;
-  double* red;
-  int lane;
-  bool wanted;
-  template <int B0, typename F>
-  __device__ __forceinline__ void segment(int ngroups, F& fetch) {
-    constexpr int kPer = 128 / kGroup, E0 = 4 * B0;
-    for (int g = min(ngroups, (B0 + 1) * kPer) - 1; g >= B0 * kPer; --g) {
-      asm volatile("cp.async.wait_group 0;" ::: "memory");
-      __syncthreads();                     // group g is here, and nobody reads the buffer of group g + 1 any more
-      if (g > 0) fetch(g - 1);
-      if (!wanted) continue;
-      const double (*f)[S] = fs[g & 1];
-      double d0 = 0.0, d1 = 0.0, d2 = 0.0, d3 = 0.0;
+template <int TW, int RS, int W>
+struct BackShape {
+  static constexpr int kCols = 8 * TW * RS;
+  static constexpr int kPitch = (kCols + 15) / 16 * 16 + 4;       // rows 32 bytes apart modulo the 128 of the banks
+  static constexpr int kBlock = RS > 1 ? (TW % 2 ? 1 : 2) : 4;     // pieces of a warp that are dropped together
+  static constexpr int kGroups = W / RS;                           // vector groups of a CTA
+  static constexpr int kY = RS > 1 ? 2 * kGroups * RS * 32 : 0;
+  static constexpr size_t kStageBytes = sizeof(double) * (kGroup * kPitch + kGroup * kGroup);
+  static constexpr int kStages = std::min(4, (int)((kMaxSmem - 1024 - sizeof(double2) * kY) / kStageBytes));      // groups in flight
+  static constexpr size_t kBytes = kStages * kStageBytes + sizeof(double2) * kY;
+  static_assert(TW % kBlock == 0 && W % RS == 0, "shape");
+};
+
+template <int TW, int RS, int W>
+struct BackState {
+  using B = BackShape<TW, RS, W>;
+  const double *fs, *ts;
+  double2* ys;
+  uint64_t* bars;
+  int* dead;
+  int stage, parity, g, sub, vg, lane;
+  // the groups whose first column lies in the pieces [Q0, Q0 + kBlock) of the warps, then the groups before them
+  template <int Q0, typename F>
+  __device__ __forceinline__ void segment(double (&z)[TW][2], F& fetch) {
+    constexpr int kPitch = B::kPitch, kStages = B::kStages;
+    const int lr = lane >> 2, lc = lane & 3, frow = row_of(lr), wrow0 = row_of(2 * lc), wrow1 = row_of(2 * lc + 1);
+    for (; g >= RS * Q0; --g) {
+      if (!tc::mbar_wait(&bars[stage], parity)) *reinterpret_cast<volatile int*>(dead) = 1;
+      __syncthreads();                     // group g is here, and nobody reads the stage of group g + 1 any more
+      if (*reinterpret_cast<volatile int*>(dead)) return;
+      if (threadIdx.x == 0 && g >= kStages - 1) fetch(g - (kStages - 1), stage == 0 ? kStages - 1 : stage - 1);
+      const double* f = fs + stage * kGroup * kPitch;
+      const double* t = ts + stage * kGroup * kGroup;
+      const double t0 = t[frow * kGroup + wrow0], t1 = t[frow * kGroup + wrow1];
+      double y[2] = {0.0, 0.0}, y1[2] = {0.0, 0.0}, w[2] = {0.0, 0.0};
 #pragma unroll
-      for (int e = E0; e < E; ++e) {
-        const int k = lane + 32 * e;
-        d0 = fma(f[0][k], z[e], d0); d1 = fma(f[1][k], z[e], d1); d2 = fma(f[2][k], z[e], d2); d3 = fma(f[3][k], z[e], d3);
+      for (int q = Q0; q < TW; ++q) {
+        const double2 v = *reinterpret_cast<const double2*>(f + frow * kPitch + 8 * (sub + RS * q) + 2 * lc);
+        dmma(y, z[q][0], v.x);
+        dmma(y1, z[q][1], v.y);
       }
-      const bool h2 = (lane & 16) != 0, h1 = (lane & 8) != 0;
-      const double t0 = (h2 ? d2 : d0) + __shfl_xor_sync(0xffffffffu, h2 ? d0 : d2, 16);
-      const double t1 = (h2 ? d3 : d1) + __shfl_xor_sync(0xffffffffu, h2 ? d1 : d3, 16);
-      double t = (h1 ? t1 : t0) + __shfl_xor_sync(0xffffffffu, h1 ? t0 : t1, 8);
-      t += __shfl_xor_sync(0xffffffffu, t, 4);
-      t += __shfl_xor_sync(0xffffffffu, t, 2);
-      t += __shfl_xor_sync(0xffffffffu, t, 1);
-      __syncwarp();
-      if ((lane & 7) == 0) red[lane >> 3] = t;
-      __syncwarp();
-      const double* x = xs + g * 6;
-      const double* gm = gs + g * kGroup;
-      const double c3 = gm[3] * red[3];
-      const double c2 = gm[2] * fma(-c3, x[5], red[2]);
-      const double c1 = gm[1] * fma(-c3, x[4], fma(-c2, x[3], red[1]));
-      const double c0 = gm[0] * fma(-c3, x[2], fma(-c2, x[1], fma(-c1, x[0], red[0])));
+      y[0] += y1[0]; y[1] += y1[1];
+      if constexpr (RS > 1) {
+        double2* yw = ys + ((g & 1) * B::kGroups + vg) * RS * 32;
+        yw[sub * 32 + lane] = make_double2(y[0], y[1]);
+        tc::named_bar_sync(1 + vg, 32 * RS);
+        double2 p[RS];
 #pragma unroll
-      for (int e = E0; e < E; ++e) {
-        const int k = lane + 32 * e;
-        z[e] = fma(-c0, f[0][k], fma(-c1, f[1][k], fma(-c2, f[2][k], fma(-c3, f[3][k], z[e]))));
+        for (int r = 0; r < RS; ++r) p[r] = yw[r * 32 + lane];
+#pragma unroll
+        for (int o = 1; o < RS; o *= 2)
+#pragma unroll
+          for (int r = 0; r < RS; r += 2 * o) { p[r].x += p[r + o].x; p[r].y += p[r + o].y; }
+        y[0] = p[0].x; y[1] = p[0].y;
       }
+      dmma(w, y[0], t0);
+      dmma(w, y[1], t1);
+      w[0] = -w[0]; w[1] = -w[1];
+#pragma unroll
+      for (int q = Q0; q < TW; ++q) {
+        const int c = 8 * (sub + RS * q) + lr;
+        dmma(z[q], w[0], f[wrow0 * kPitch + c]);
+        dmma(z[q], w[1], f[wrow1 * kPitch + c]);
+      }
+      if (++stage == kStages) { stage = 0; parity ^= 1; }
     }
-    if constexpr (B0 > 0) segment<B0 - 1>(ngroups, fetch);
+    if constexpr (Q0 > 0) {
+      if (*reinterpret_cast<volatile int*>(dead) == 0) segment<Q0 - B::kBlock>(z, fetch);
+    }
   }
 };
-template <int EB>
-__global__ void __launch_bounds__(32 * kBigWarps)
-back_transform_big_kernel(const EigJob* __restrict__ jobs) {
-  constexpr int E = 4 * EB, S = 32 * E;
-  extern __shared__ __align__(16) double back_sm[];
-  double (*fs)[kGroup][S] = reinterpret_cast<double (*)[kGroup][S]>(back_sm);
-  double* gs = back_sm + 2 * kGroup * S;
-  double* xs = gs + S + kGroup;
-  __shared__ __align__(16) double red[kBigWarps][kGroup];
+
+template <int TW, int RS, int W>
+__global__ void __launch_bounds__(32 * W)
+back_transform_kernel(const EigJob* __restrict__ jobs, int* status) {
+  using B = BackShape<TW, RS, W>;
+  constexpr int kPitch = B::kPitch, kBlock = B::kBlock;
+  extern __shared__ __align__(128) double back_sm[];
+  constexpr int kStages = B::kStages;
+  double* fs = back_sm;                                    // [kStages][kGroup][kPitch]
+  double* ts = fs + kStages * kGroup * kPitch;             // [kStages][kGroup][kGroup]
+  double2* ys = reinterpret_cast<double2*>(ts + kStages * kGroup * kGroup);
+  __shared__ uint64_t bars[kStages];
+  __shared__ int dead;
   const EigJob job = jobs[blockIdx.y];
-  const int s = job.s;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int i = blockIdx.x * kBigWarps + warp;
-  const int ngroups = (s + kGroup - 1) / kGroup;
-  const double lam = i < s ? job.lam[i] : 0.0;
-  int rank = s;
-  if (i < s) {
-    int c = 0;
-    for (int k = lane; k < s; k += 32) {
-      const double lk = job.lam[k];
-      c += (lk > lam || (lk == lam && k < i)) ? 1 : 0;
-    }
-    rank = __reduce_add_sync(0xffffffffu, c);
+  const int s = job.s, ld = refl_ld(s), ngroups = (s + kGroup - 1) / kGroup;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, lr = lane >> 2, lc = lane & 3;
+  const int sub = warp % RS, vg = warp / RS;
+  if ((int)blockIdx.x * 8 * B::kGroups >= job.need) return;
+  // what no copy fills: columns behind the rows, rows behind the last reflector (in the stage of the last group, the first one used)
+  for (int r = warp; r < kStages * kGroup; r += W) {
+    const bool none = r < kGroup && (ngroups - 1) * kGroup + r >= s;
+    for (int k = (none ? 0 : ld) + lane; k < kPitch; k += 32) fs[r * kPitch + k] = 0.0;
   }
-  const bool wanted = rank < job.need;
-  if (!__syncthreads_or(wanted)) return;
-  for (int k = tid; k < ngroups * kGroup; k += 32 * kBigWarps) gs[k] = k < s ? job.gam[k] : 0.0;
-  for (int k = tid; k < ngroups * 6; k += 32 * kBigWarps) xs[k] = job.cross[k];
-  auto fetch = [&](int g) {
-    const int j0 = g * kGroup, k0 = j0 & ~127, w = S - k0;
-    for (int idx = tid; idx < kGroup * w; idx += 32 * kBigWarps) {
-      const int a = idx / w, k = k0 + idx - a * w;
-      double* d = &fs[g & 1][a][k];
-      if (k < s && j0 + a < s)
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(tc::smem_u32(d)), "l"(job.refl + (size_t)(j0 + a) * s + k) : "memory");
-      else
-        *d = 0.0;
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
+  if (tid == 0) {
+    dead = 0;
+    for (int i = 0; i < kStages; ++i) tc::mbar_init(&bars[i], 1);
+    tc::fence_barrier_init();
+  }
+  tc::fence_proxy_async_smem();
+  __syncthreads();
+  auto fetch = [&](int g, int stage) {
+    const int j0 = g * kGroup, n = min(kGroup, s - j0), k0 = 8 * RS * kBlock * (g / (RS * kBlock));
+    const uint32_t bytes = (uint32_t)(ld - k0) * 8;
+    uint64_t* bar = &bars[stage];
+    tc::mbar_arrive_expect_tx(bar, n * bytes + kGroup * kGroup * 8);
+    for (int a = 0; a < n; ++a) tc::bulk_load(fs + (stage * kGroup + a) * kPitch + k0, job.refl + (size_t)(j0 + a) * ld + k0, bytes, bar);
+    tc::bulk_load(ts + stage * kGroup * kGroup, job.tmat + (size_t)g * kGroup * kGroup, kGroup * kGroup * 8, bar);
   };
-  fetch(ngroups - 1);
-  double z[E];
-  const double inv = i < s ? job.inv[i] : 0.0;
+  if (tid == 0)
+    for (int i = 0; i < kStages - 1 && i < ngroups; ++i) fetch(ngroups - 1 - i, i);
+  const int q0 = (blockIdx.x * B::kGroups + vg) * 8, mine = q0 + lr;
+  auto position = [&](int q) { const int i = job.order[q]; return (unsigned)i < (unsigned)s ? i : q; };   // NaN leaves holes in the order
+  double z[TW][2];
+  double lam = 0.0;
+  {
+    const int i = mine < job.need ? position(mine) : 0;
+    const double inv = mine < job.need ? job.inv[i] : 0.0;
+    lam = mine < job.need ? job.lam[i] : 0.0;
 #pragma unroll
-  for (int e = 0; e < E; ++e) {
-    const int k = lane + 32 * e;
-    z[e] = (wanted && k < s) ? job.zp[(size_t)k * s + i] * inv : 0.0;
+    for (int q = 0; q < TW; ++q)
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const int k = 8 * (sub + RS * q) + 2 * lc + e;
+        z[q][e] = (mine < job.need && k < s) ? job.zp[(size_t)k * s + i] * inv : 0.0;
+      }
   }
-  if (wanted && lam > null_rel(job)) {
-    for (int k0 = 0; k0 < s; k0 += 32) {
-      const int k = k0 + lane;
-      bool close = false;
-      if (k < s && k != i) {
-        const double lk = job.lam[k];
-        close = fabs(lk - lam) < kCloseRel && (lk > lam || (lk == lam && k < i));
-      }
-      unsigned bal = __ballot_sync(0xffffffffu, close);
-      while (bal) {
-        const int kk = k0 + __ffs(bal) - 1;
-        bal &= bal - 1;
-        double acc = 0.0;
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-          const int q = lane + 32 * e;
-          if (q < s) acc = fma(z[e], job.zp[(size_t)q * s + kk], acc);
-        }
-        acc = warp_sum(acc) * job.inv[kk];
-        if (!(fabs(acc) <= kOrthTol) && lane == 0) *job.flag = 1;
-      }
+  // neighbours too close for the factorisation to keep apart: is this vector orthogonal to those above it?
+  for (int q = q0 + sub; q < min(q0 + 8, job.need); q += RS) {
+    const int i = position(q);
+    const double li = job.lam[i];
+    if (!(li > null_rel(job))) continue;
+    for (int p = q - 1; p >= 0; --p) {
+      const int k = position(p);
+      if (!(fabs(job.lam[k] - li) < kCloseRel)) break;
+      double acc = 0.0;
+      for (int c = lane; c < s; c += 32) acc = fma(job.zp[(size_t)c * s + i], job.zp[(size_t)c * s + k], acc);
+      acc = warp_sum(acc) * job.inv[i] * job.inv[k];
+      if (!(fabs(acc) <= kOrthTol) && lane == 0) *job.flag = 1;
     }
   }
-  BackBig<EB> bb{z, fs, gs, xs, red[warp], lane, wanted};
-  bb.template segment<EB - 1>(ngroups, fetch);
-  if (!wanted) return;
-  float* dst = job.rows + (size_t)rank * s;
-#pragma unroll
-  for (int e = 0; e < E; ++e) {
-    const int k = lane + 32 * e;
-    if (k < s) dst[k] = (float)z[e];
+  BackState<TW, RS, W> x{fs, ts, ys, bars, &dead, 0, 0, ngroups - 1, sub, vg, lane};
+  x.template segment<TW - kBlock>(z, fetch);
+  if (*reinterpret_cast<volatile int*>(&dead)) {           // a copy never arrived
+    if (tid == 0) atomicExch(status, (int)AB_ERR_TIMEOUT);
+    return;
   }
-  if (lane == 0 && job.vals) job.vals[rank] = (float)(lam * job.norm[0]);
+  if (mine >= job.need) return;
+  float* dst = job.rows + (size_t)mine * s;
+#pragma unroll
+  for (int q = 0; q < TW; ++q)
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const int k = 8 * (sub + RS * q) + 2 * lc + e;
+      if (k < s) dst[k] = (float)z[q][e];
+    }
+  if (lc == 0 && sub == 0 && job.vals) {
+    const double norm = job.norm[0], l = lam * norm;
+    job.vals[mine] = (float)(job.gram ? (l > 1e-12 * norm ? sqrt(l) : 0.0) : l);
+  }
 }
 
 template <int E, int R, int W, bool kSingle>
@@ -1246,20 +1126,6 @@ int launch_values(const EigJob* jobs, int count, int smax, cudaStream_t st) {
   return AB_OK;
 }
 
-template <int E, int NV>
-int launch_back(const EigJob* jobs, int count, int smax, cudaStream_t st) {
-  const int per = kBackWarps * NV;
-  const size_t sm = sizeof(double) * (2 * kGroup * 32 * E + 32 * E + kGroup + (32 * E / kGroup + 1) * 6);
-  back_transform_kernel<E, NV><<<dim3((unsigned)((smax + per - 1) / per), (unsigned)count), 32 * kBackWarps, sm, st>>>(jobs);
-  AB_LAUNCH_OK();
-  return AB_OK;
-}
-// Four vectors a warp where the batch fills the device; one where it does not (the chain of a warp is then what counts).
-template <int E>
-int launch_back_e(const EigJob* jobs, int count, int smax, int sms, cudaStream_t st) {
-  return (long long)count * smax >= 32LL * sms ? launch_back<E, 4>(jobs, count, smax, st) : launch_back<E, 1>(jobs, count, smax, st);
-}
-
 template <int E>
 int launch_grid(const EigJob* jobs, int count, int smax, int sms, int* status, cudaStream_t st) {
   int per_sm = 0;
@@ -1273,28 +1139,32 @@ int launch_grid(const EigJob* jobs, int count, int smax, int sms, int* status, c
   return AB_OK;
 }
 
-template <int EB>
-int launch_back_big(const EigJob* jobs, int count, int smax, cudaStream_t st) {
-  constexpr int S = 128 * EB;
-  const size_t sm = sizeof(double) * (2 * kGroup * S + S + kGroup + (S / kGroup + 1) * 6);
-  AB_CUDA_OK(cudaFuncSetAttribute(back_transform_big_kernel<EB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-  back_transform_big_kernel<EB><<<dim3((unsigned)((smax + kBigWarps - 1) / kBigWarps), (unsigned)count), 32 * kBigWarps, sm, st>>>(jobs);
+template <int TW, int RS, int W>
+int launch_back(const EigJob* jobs, int count, int need, int* status, cudaStream_t st) {
+  using B = BackShape<TW, RS, W>;
+  constexpr int per = 8 * W / RS;
+  AB_CUDA_OK(allow_smem(back_transform_kernel<TW, RS, W>, 1024));
+  back_transform_kernel<TW, RS, W><<<dim3((unsigned)((need + per - 1) / per), (unsigned)count), 32 * W, B::kBytes, st>>>(jobs, status);
   AB_LAUNCH_OK();
   return AB_OK;
 }
 
 }  // namespace
 
-size_t eig_ws_doubles(int s) { return align_up((size_t)3 * s * s + (4 + 5 + 2) * (size_t)s + 64, 2); }
+size_t eig_ws_doubles(int s) {
+  const size_t n = (size_t)s, groups = (n + kGroup - 1) / kGroup;
+  return align_up(n * refl_ld(s) + 2 * n * n + groups * kGroup * kGroup + (4 + 5 + 1) * n + 8, 2);
+}
 
 // The largest order: the grid kernel needs all CTAs of a matrix resident together.
 int eig_max() { return std::min(1184, kGridRows * std::max(sm_count(), 1)); }
 
 void eig_bind(EigJob& j, double* ws) {
-  const size_t s = (size_t)j.s;
-  j.xbuf = ws; j.refl = j.xbuf + 4 * s; j.zp = j.refl + s * s; j.zm = j.zp + s * s;     // xbuf first: 16-byte aligned
-  j.d = j.zm + s * s; j.e = j.d + s; j.gam = j.e + s; j.lam = j.gam + s; j.inv = j.lam + s; j.cross = j.inv + s;
-  j.norm = j.cross + (s + 3) / 4 * 6;
+  const size_t s = (size_t)j.s, groups = (s + kGroup - 1) / kGroup;
+  j.xbuf = ws; j.refl = j.xbuf + 4 * s; j.tmat = j.refl + s * refl_ld(j.s);      // each of these 16-byte aligned
+  j.zp = j.tmat + groups * kGroup * kGroup; j.zm = j.zp + s * s;
+  j.d = j.zm + s * s; j.e = j.d + s; j.gam = j.e + s; j.lam = j.gam + s; j.inv = j.lam + s; j.norm = j.inv + s;
+  j.order = reinterpret_cast<int*>(j.norm + 1);
 }
 
 int eig_direct(const EigJob* h_jobs, const EigJob* d_jobs, int count, int smax, int* status, cudaStream_t st) {
@@ -1326,14 +1196,24 @@ int eig_direct(const EigJob* h_jobs, const EigJob* d_jobs, int count, int smax, 
   AB_CUDA_OK(allow_smem(tri_vectors_kernel, 8192));
   tri_vectors_kernel<<<dim3((unsigned)(vb + gb), (unsigned)count), 32 * kVecWarps, vectors_smem(smax), st>>>(d_jobs, vb, smax);
   AB_LAUNCH_OK();
-  if (smax > 1024) return launch_back_big<10>(d_jobs, count, smax, st);
-  if (smax > 768) return launch_back_big<8>(d_jobs, count, smax, st);
-  if (smax > 512) return launch_back_big<6>(d_jobs, count, smax, st);
-  if (smax > kEigSmallMax) return launch_back_big<4>(d_jobs, count, smax, st);
-  if (smax <= 64) return launch_back_e<2>(d_jobs, count, smax, sms, st);
-  if (smax <= 128) return launch_back_e<4>(d_jobs, count, smax, sms, st);
-  if (smax <= 192) return launch_back_e<6>(d_jobs, count, smax, sms, st);
-  return launch_back_e<8>(d_jobs, count, smax, sms, st);
+  // A warp to eight vectors where that gives a scheduler more than one warp, else eight warps to them (72 matrices of
+  // order 192, 23 warps of vectors an SM: 65 us against 137).
+  int need = 1;
+  for (int i = 0; i < count; ++i) need = std::max(need, h_jobs[i].need);
+  if (smax <= kEigSmallMax && values >= 48LL * sms) {
+    if (smax <= 64) return launch_back<8, 1, 4>(d_jobs, count, need, status, st);
+    if (smax <= 128) return launch_back<16, 1, 4>(d_jobs, count, need, status, st);
+    if (smax <= 192) return launch_back<24, 1, 4>(d_jobs, count, need, status, st);
+    return launch_back<32, 1, 4>(d_jobs, count, need, status, st);
+  }
+  if (smax <= 64) return launch_back<1, 8, 8>(d_jobs, count, need, status, st);
+  if (smax <= 128) return launch_back<2, 8, 8>(d_jobs, count, need, status, st);
+  if (smax <= 192) return launch_back<3, 8, 8>(d_jobs, count, need, status, st);
+  if (smax <= 256) return launch_back<4, 8, 8>(d_jobs, count, need, status, st);
+  if (smax <= 512) return launch_back<8, 8, 8>(d_jobs, count, need, status, st);
+  if (smax <= 768) return launch_back<12, 8, 8>(d_jobs, count, need, status, st);
+  if (smax <= 1024) return launch_back<16, 8, 8>(d_jobs, count, need, status, st);
+  return launch_back<20, 8, 8>(d_jobs, count, need, status, st);
 }
 
 }  // namespace ab
