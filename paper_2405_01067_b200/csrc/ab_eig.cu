@@ -36,6 +36,7 @@ constexpr double kCloseRel = 1e-7;      // eigenvalues closer than this fraction
 constexpr double kOrthTol = 4e-6;       // what the Jacobi route leaves at small orders
 constexpr int kMaxOrder = 1280;         // masks are sized for this order
 constexpr double kLive2 = 1e-290;       // a column whose squared norm is below this needs no reflector
+constexpr double kCancel = 0x1p-10;     // a squared norm below this fraction of its terms is summed again from the entries
 constexpr int kGroup = 8;               // reflectors applied together in the back transform
 
 // Reflectors are rows of an even number of doubles (bulk copies of whole rows start and end on 16 bytes), zero before and
@@ -343,17 +344,19 @@ tridiag_small_kernel(const EigJob* __restrict__ jobs, int* status) {
 }
 
 // ---- 1b. Householder reduction over the whole device ------------------------------------------------------
-// The same steps for orders a cluster cannot hold.  CTA c of the matrix's C = ceil(s / kGridRows) keeps rows c, c + C, ... in
-// registers; thread t owns columns t, t + 256, ... of all of them, so the vectors are spread over the CTA (every CTA works
-// out w and the next reflector for itself) and what crosses the device in a step is one (p_i, A[i][j+1]) pair per row.
+// The same steps for orders a cluster cannot hold.  CTA c of the matrix's C (s / kGridRows, whole clusters) keeps rows c, c + C,
+// ... in registers; thread t owns columns t, t + 256, ... of all of them, so the vectors are spread over the CTA (every
+// CTA works out w and the next reflector for itself) and what crosses the device in a step is one (p_i, A[i][j+1]) pair per row.
 // A pair is two 8-byte words, each carrying the step in its eight lowest mantissa bits (2^-44 of the value): a reader
-// polls the words of its own columns until the step matches, so data and signal are one trip through L2.
-// A CTA leaves when its last row is finished; every CTA that still reads the pairs of step j therefore sends a row
-// of step j + 1, and whoever has all of step j + 1 may overwrite the buffer of step j (two buffers, cleared before the launch).
-// All CTAs of a matrix have to be resident together: cooperative launch.  The polls are bounded.
-// Order 768: 2.21 ms, 2.9 us a step, nearly all of it latency (the poll, three barriers, three warp reductions, a
-// square root); the pass over 8 x 768 elements is 24 multiply-adds a thread.
-constexpr int kGridRows = 8, kGridThreads = 256;
+// polls the words until the step matches, so data and signal are one trip through L2.  Every CTA needs all pairs, but
+// each CTA of a cluster polls a share of them only and passes it on to the others (st.async onto a barrier of each receiver, two buffers
+// in turn): all CTAs polling everything was 1.2 MB a round at order 768, and the rounds held up the stores they waited for (3.1 us a step).
+// Who may overwrite what.  Buffers of a cluster: the barrier of step j + 1 counts a token of each CTA, sent once it
+// has read step j.  Pairs in memory: a cluster stays until its last row is finished, so whoever has all pairs of step j + 1
+// has one from every cluster that is still here, sent by a CTA that had all of step j, which its mates had read and passed on
+// by then; the buffer of step j may be written (two buffers, cleared before the launch).
+// All CTAs of a matrix have to be resident together: cooperative launch.  The waits are bounded.
+constexpr int kGridRows = 8;
 
 __device__ __forceinline__ double tag_word(double x, unsigned tag) {
   return __longlong_as_double((__double_as_longlong(x) & ~0xffll) | (long long)tag);
@@ -379,25 +382,59 @@ __device__ __forceinline__ bool poll_pair(const double2* p, unsigned tag, double
     if ((it & 1023u) == 1023u && tc::globaltimer_ns() - t0 > tc::kWaitLimitNs) return false;
   }
 }
-// sum over the CTA's eight warps of a value each warp has reduced into red[warp]
-__device__ __forceinline__ double sum8(const double* red) {
+// Four sums across a warp, each exchange halving what a lane still carries: lanes 8 q ... hold sum q.
+__device__ __forceinline__ double warp_sum4(double s0, double s1, double s2, double s3, int lane) {
+  const bool h2 = (lane & 16) != 0, h1 = (lane & 8) != 0;
+  const double t0 = (h2 ? s2 : s0) + __shfl_xor_sync(0xffffffffu, h2 ? s0 : s2, 16);
+  const double t1 = (h2 ? s3 : s1) + __shfl_xor_sync(0xffffffffu, h2 ? s1 : s3, 16);
+  double t = (h1 ? t1 : t0) + __shfl_xor_sync(0xffffffffu, h1 ? t0 : t1, 8);
+  t += __shfl_xor_sync(0xffffffffu, t, 4);
+  t += __shfl_xor_sync(0xffffffffu, t, 2);
+  t += __shfl_xor_sync(0xffffffffu, t, 1);
+  return t;
+}
+// sum over the CTA's W warps of a value each warp has left in red[warp]
+template <int W>
+__device__ __forceinline__ double sum_warps(const double* red) {
   const double2* r = reinterpret_cast<const double2*>(red);
-  const double2 a = r[0], b = r[1], c = r[2], d = r[3];
-  return ((a.x + a.y) + (b.x + b.y)) + ((c.x + c.y) + (d.x + d.y));
+  double2 a = r[0], b = r[1];
+  double t = (a.x + a.y) + (b.x + b.y);
+  if constexpr (W == 8) { a = r[2]; b = r[3]; t += (a.x + a.y) + (b.x + b.y); }
+  return t;
 }
 
-template <int E>
-__global__ void __launch_bounds__(kGridThreads, E <= 3 ? 2 : 1)
+// A step.  With x = v1 gamma and y = 2 c v1 - gamma p_j (c = gamma^2 p.v / 2) column j + 1 of the updated matrix is
+// (a - x p) + y v, where only y waits for a sum; its squared norm follows from the sums over b = a - x p:
+// b.b + 2 y b.v + y^2 v.v.  So one reduction over the CTA gives all that a step needs (there were two).  Where the terms
+// cancel to less than kCancel of their size (1 to 2 % of the steps of a decaying spectrum) the entries are summed themselves.
+// The square root stands beside the pass over the rows: its result is needed for element j + 1 of the reflector alone, whose products
+// are added as the row sums leave.
+// Order 768, cycles a step: 4300, of them 2100 outside the exchange; 5100 and 3500 with three barriers, two reductions and the
+// root in the chain; 6000 with all CTAs polling.  2.25 ms -> 1.55.
+template <int E, int W>
+__global__ void __launch_bounds__(32 * W, 1)
 tridiag_grid_kernel(const EigJob* __restrict__ jobs, int count, int C, int* status) {
-  constexpr int R = kGridRows;
-  __shared__ __align__(16) double red_pv[8], red_sq[8], red_row[R][8];
-  __shared__ double2 vw[R];              // (v_i, w_i) of this CTA's rows
-  __shared__ double colbuf[R];
-  __shared__ double sc[5];               // p_j, a_j, p_j+1, a_j+1, v_j+1
+  constexpr int R = kGridRows, T = 32 * W, S = T * E;
+  extern __shared__ __align__(16) double2 pairs[];                        // [2][S + kMaxCl]: the pairs of a step, behind them the mates' tokens
+  __shared__ __align__(16) double red[4][W], red_row[R][W], vrow[R];      // vrow: v of this CTA's rows
+  __shared__ double colbuf[R], vnext;                                     // column j + 1 of the rows; v_j+1
+  __shared__ uint64_t bar[2];
   __shared__ int dead;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int CL = (int)cg::this_cluster().num_blocks(), rank = (int)cg::this_cluster().block_rank();
   const int ngroups = gridDim.x / C, group = blockIdx.x / C, cta = blockIdx.x - group * C;
-  if (tid == 0) dead = 0;
+  const uint32_t pairs_at = tc::smem_u32(pairs), bar_off = tc::smem_u32(bar) - pairs_at;
+  uint32_t mate[kMaxCl];
+#pragma unroll
+  for (int c = 0; c < kMaxCl; ++c) mate[c] = map_rank(pairs_at, c < CL ? c : 0);
+  for (int k = tid; k < 2 * (S + kMaxCl); k += T) pairs[k] = make_double2(0.0, 0.0);       // columns behind the last stay zero
+  if (tid == 0) {
+    dead = 0;
+    tc::mbar_init(&bar[0], 1); tc::mbar_init(&bar[1], 1);
+    tc::fence_barrier_init();
+  }
+  cg::this_cluster().sync();             // barriers are ready before a mate sends
+  int uses = 0;                          // steps so far, over all matrices: buffer and parity
   for (int mat = group; mat < count; mat += ngroups) {
     const EigJob job = jobs[mat];
     const int s = job.s;
@@ -406,7 +443,7 @@ tridiag_grid_kernel(const EigJob* __restrict__ jobs, int count, int C, int* stat
     int slot[E];                         // which of this CTA's rows column k is, or -1
 #pragma unroll
     for (int e = 0; e < E; ++e) {
-      const int k = tid + kGridThreads * e;
+      const int k = tid + T * e;
       slot[e] = (k < s && k % C == cta) ? k / C : -1;
 #pragma unroll
       for (int r = 0; r < R; ++r) {
@@ -414,94 +451,139 @@ tridiag_grid_kernel(const EigJob* __restrict__ jobs, int count, int C, int* stat
         A[r][e] = (i < s && k < s) ? (double)job.X[(size_t)i * s + k] : 0.0;
       }
     }
-    int last = -1;                       // this CTA's last row
+    int last = -1;                       // the cluster's last row
 #pragma unroll
-    for (int r = 0; r < R; ++r)
-      if (cta + C * r < s) last = cta + C * r;
-    if (tid < R && cta + C * tid < s) {
+    for (int r = 0; r < R; ++r) {
+      const int i = cta - rank + C * r;
+      if (i < s) last = min(s, i + CL) - 1;
+    }
+    if (tid < R) {
       const int i = cta + C * tid;
-      st_relaxed(xb + i, tag_word(0.0, step_tag(0)), tag_word((double)job.X[(size_t)i * s], step_tag(0)));
+      if (i < s) st_relaxed(xb + i, tag_word(0.0, step_tag(0)), tag_word((double)job.X[(size_t)i * s], step_tag(0)));
+      vrow[tid] = 0.0;
+    }
+    if (tid == 0) vnext = 0.0;
+    __syncthreads();
+    const int share = (s + CL - 1) / CL, from = share * rank, upto = min(s, from + share);
+    if (tid < CL && last > 0) {          // tokens of the first step: this CTA has read the last step of the matrix before
+      const int buf = uses & 1;
+      const uint32_t m = map_rank(pairs_at, tid);
+      st_async(m + (uint32_t)(buf * (S + kMaxCl) + S + rank) * 16, 0.0, 0.0, m + bar_off + buf * 8);
     }
     double v[E];
 #pragma unroll
     for (int e = 0; e < E; ++e) v[e] = 0.0;
-    double gam = 0.0, v1 = 0.0;
-    for (int j = 0; j < last; ++j) {
-      const unsigned tag = step_tag(j);
-      const double2* rb = xb + (size_t)(j & 1) * s;
-      double w[E], vn[E], pv = 0.0;
+    double gam = 0.0, v1 = 0.0, x = 0.0;
+    unsigned tag = step_tag(0);
+    for (int j = 0; j < last; ++j, ++uses) {
+      const int buf = uses & 1;
+      const double2* pb = pairs + buf * (S + kMaxCl);
+      if (tid == 0) tc::mbar_arrive_expect_tx(&bar[buf], (uint32_t)(16 * (s - j + CL)));
       bool ok = true;
+      for (int k = max(from, j) + tid; k < upto; k += T) {
+        double2 q;
+        ok = poll_pair(xb + (size_t)(j & 1) * s + k, tag, q) && ok;
+        const uint32_t off = (uint32_t)(buf * (S + kMaxCl) + k) * 16;
+#pragma unroll
+        for (int c = 0; c < kMaxCl; ++c)
+          if (c < CL) st_async(mate[c] + off, q.x, q.y, mate[c] + bar_off + buf * 8);
+      }
+      const unsigned next_tag = tag == 255u ? 1u : tag + 1u;
+      // (v, p) of this CTA's rows, the two entries that everybody needs, and this thread's columns
+      double vr[R], pr[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r) vr[r] = vrow[r];
+      const double vj1 = vnext;
+      ok = tc::mbar_wait(&bar[buf], (uses >> 1) & 1) && ok;
+      if (!ok) *reinterpret_cast<volatile int*>(&dead) = 1;
+      double p[E], vn[E], pv = 0.0, bb = 0.0, bv = 0.0, vv = 0.0;
 #pragma unroll
       for (int e = 0; e < E; ++e) {
-        const int k = tid + kGridThreads * e;
-        w[e] = 0.0; vn[e] = 0.0;
-        if (k >= j && k < s) {
-          double2 q;
-          ok = poll_pair(rb + k, tag, q) && ok;
-          w[e] = q.x; vn[e] = q.y;
-          pv = fma(q.x, v[e], pv);
-          if (k == j) { sc[0] = q.x; sc[1] = q.y; }
-          if (k == j + 1) { sc[2] = q.x; sc[3] = q.y; sc[4] = v[e]; }
-        }
+        const int k = tid + T * e;
+        const double2 q = pb[k];
+        p[e] = k >= j ? q.x : 0.0;                       // what is before j is of an earlier step
+        vn[e] = k > j + 1 ? fma(-x, q.x, q.y) : 0.0;
+        const double vm = k > j + 1 ? v[e] : 0.0;
+        pv = fma(p[e], v[e], pv);
+        bb = fma(vn[e], vn[e], bb);
+        bv = fma(vn[e], vm, bv);
+        vv = fma(vm, vm, vv);
       }
-      if (!ok) *reinterpret_cast<volatile int*>(&dead) = 1;
-      pv = warp_sum(pv);
-      if (lane == 0) red_pv[warp] = pv;
+      const double2 qj = pb[j], qj1 = pb[j + 1];
+#pragma unroll
+      for (int r = 0; r < R; ++r) pr[r] = pb[min(cta + C * r, S - 1)].x;
+      const double t4 = warp_sum4(pv, bb, bv, vv, lane);
+      if ((lane & 7) == 0) red[lane >> 3][warp] = t4;
       __syncthreads();
       if (*reinterpret_cast<volatile int*>(&dead)) break;      // the same for all threads: a peer never answered
-      const double c = 0.5 * gam * (gam * sum8(red_pv));
-      const double wj = gam * sc[0] - c * v1;
-      double sq = 0.0;
+      if (tid < CL && j + 1 < last) {
+        const uint32_t m = map_rank(pairs_at, tid);
+        st_async(m + (uint32_t)((buf ^ 1) * (S + kMaxCl) + S + rank) * 16, 0.0, 0.0, m + bar_off + (buf ^ 1) * 8);
+      }
+      pv = sum_warps<W>(red[0]); bb = sum_warps<W>(red[1]); bv = sum_warps<W>(red[2]); vv = sum_warps<W>(red[3]);
+      const double c = 0.5 * gam * (gam * pv);           // gamma alone may be as large as 1e290
+      const double y = 2.0 * c * v1 - gam * qj.x, wj = gam * qj.x - c * v1;
+      double sq = bb + y * (2.0 * bv + y * vv);
+      double w[E];
 #pragma unroll
       for (int e = 0; e < E; ++e) {
-        const int k = tid + kGridThreads * e;
-        w[e] = gam * w[e] - c * v[e];
-        vn[e] = (k > j + 1) ? vn[e] - v1 * w[e] - wj * v[e] : 0.0;
-        sq = fma(vn[e], vn[e], sq);
-        if (slot[e] >= 0) vw[slot[e]] = make_double2(v[e], w[e]);
+        const int k = tid + T * e;
+        w[e] = fma(gam, p[e], -(c * v[e]));
+        vn[e] = k > j + 1 ? fma(y, v[e], vn[e]) : 0.0;
       }
-      sq = warp_sum(sq);
-      if (lane == 0) red_sq[warp] = sq;
-      const double dj = sc[1] - 2.0 * v1 * wj;
-      const double alpha = sc[3] - v1 * (gam * sc[2] - c * sc[4]) - wj * sc[4];
-      __syncthreads();
-      sq = sum8(red_sq);
+      if (!(sq >= kCancel * (bb + y * y * vv))) {        // the same in all CTAs: they work on the same bits
+        __syncthreads();                                 // red has been read
+        sq = 0.0;
+#pragma unroll
+        for (int e = 0; e < E; ++e) sq = fma(vn[e], vn[e], sq);
+        sq = warp_sum(sq);
+        if (lane == 0) red[0][warp] = sq;
+        __syncthreads();
+        sq = sum_warps<W>(red[0]);
+      }
+      const double dj = qj.y - 2.0 * v1 * wj, alpha = fma(y, vj1, fma(-x, qj1.x, qj1.y));
       const bool live = sq > kLive2;
+      double ps[R];
+#pragma unroll
+      for (int h = 0; h < R; h += 4) {
+#pragma unroll
+        for (int r = h; r < h + 4; ++r) ps[r] = 0.0;
+        if (cta + C * (h + 3) > j) {                     // of four rows that are not all finished
+#pragma unroll
+          for (int r = h; r < h + 4; ++r) {
+            const double wr = fma(gam, pr[r], -(c * vr[r]));      // the bits of w
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+              A[r][e] = fma(-vr[r], w[e], fma(-wr, v[e], A[r][e]));
+              ps[r] = fma(A[r][e], vn[e], ps[r]);
+            }
+          }
+        }
+      }
       const double nrm = sqrt(fma(alpha, alpha, sq));
       const double beta = live ? (alpha > 0.0 ? -nrm : nrm) : alpha;
       v1 = live ? alpha - beta : 0.0;
 #pragma unroll
       for (int e = 0; e < E; ++e) {
+        const int k = tid + T * e;
         if (!live) vn[e] = 0.0;
-        if (tid + kGridThreads * e == j + 1) vn[e] = v1;
-      }
-      double ps[R];
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        ps[r] = 0.0;
-        if (cta + C * r > j) {
-          const double2 q = vw[r];
-#pragma unroll
-          for (int e = 0; e < E; ++e) {
-            A[r][e] = fma(-q.x, w[e], fma(-q.y, v[e], A[r][e]));
-            ps[r] = fma(A[r][e], vn[e], ps[r]);
-          }
-        }
-      }
-#pragma unroll
-      for (int e = 0; e < E; ++e)
-        if (tid + kGridThreads * e == j + 1) {
+        if (k == j + 1) {
+          vn[e] = v1;
 #pragma unroll
           for (int r = 0; r < R; ++r) colbuf[r] = A[r][e];
         }
-      // eight row sums across the warp, each exchange halving what a lane still carries: lanes 4 r .. hold sum r
+        if (k == j + 2) vnext = vn[e];
+        if (slot[e] >= 0) vrow[slot[e]] = vn[e];
+        v[e] = vn[e];
+      }
       {
+        // eight row sums across the warp: lanes 4 r ... hold sum r
         const bool h3 = (lane & 16) != 0, h2 = (lane & 8) != 0, h1 = (lane & 4) != 0;
-        double t4[4], t2[2];
+        double t8[4], t2[2];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) t4[q] = (h3 ? ps[q + 4] : ps[q]) + __shfl_xor_sync(0xffffffffu, h3 ? ps[q] : ps[q + 4], 16);
+        for (int q = 0; q < 4; ++q) t8[q] = (h3 ? ps[q + 4] : ps[q]) + __shfl_xor_sync(0xffffffffu, h3 ? ps[q] : ps[q + 4], 16);
 #pragma unroll
-        for (int q = 0; q < 2; ++q) t2[q] = (h2 ? t4[q + 2] : t4[q]) + __shfl_xor_sync(0xffffffffu, h2 ? t4[q] : t4[q + 2], 8);
+        for (int q = 0; q < 2; ++q) t2[q] = (h2 ? t8[q + 2] : t8[q]) + __shfl_xor_sync(0xffffffffu, h2 ? t8[q] : t8[q + 2], 8);
         double t = (h1 ? t2[1] : t2[0]) + __shfl_xor_sync(0xffffffffu, h1 ? t2[0] : t2[1], 4);
         t += __shfl_xor_sync(0xffffffffu, t, 2);
         t += __shfl_xor_sync(0xffffffffu, t, 1);
@@ -510,31 +592,34 @@ tridiag_grid_kernel(const EigJob* __restrict__ jobs, int count, int C, int* stat
       __syncthreads();
       if (tid < R) {
         const int i = cta + C * tid;
-        if (i > j && i < s)
-          st_relaxed(xb + (size_t)((j + 1) & 1) * s + i, tag_word(sum8(red_row[tid]), step_tag(j + 1)), tag_word(colbuf[tid], step_tag(j + 1)));
+        if (i > j && i < s) {
+          const double a = colbuf[tid], sum = live ? fma(a, v1, sum_warps<W>(red_row[tid])) : 0.0;
+          st_relaxed(xb + (size_t)((j + 1) & 1) * s + i, tag_word(sum, next_tag), tag_word(a, next_tag));
+        }
       }
       gam = live ? 1.0 / (nrm * (nrm + fabs(alpha))) : 0.0;
-      // what later kernels need, from the owner of row j + 1 (it is still here)
+      x = v1 * gam;
+      tag = next_tag;
+      // what later kernels need, from the owner of row j + 1 (its cluster is still here)
       if ((j + 1) % C == cta) {
         const int ld = refl_ld(s);
         double* dst = job.refl + (size_t)j * ld;
 #pragma unroll
         for (int e = 0; e < E; ++e)
-          if (tid + kGridThreads * e < ld) dst[tid + kGridThreads * e] = vn[e];
+          if (tid + T * e < ld) dst[tid + T * e] = v[e];
         if (tid == 0) { job.d[j] = dj; job.e[j] = beta; job.gam[j] = gam; }
       }
-#pragma unroll
-      for (int e = 0; e < E; ++e) v[e] = vn[e];
     }
     if (*reinterpret_cast<volatile int*>(&dead)) break;
-    if (last == s - 1) {                 // the last diagonal element is what its row would have sent
+    if ((s - 1) % C == cta) {            // the last diagonal element is what its row would have sent
       double* dst = job.refl + (size_t)(s - 1) * refl_ld(s);
-      for (int k = tid; k < refl_ld(s); k += kGridThreads) dst[k] = 0.0;
+      for (int k = tid; k < refl_ld(s); k += T) dst[k] = 0.0;
       if (tid == 0) { job.d[s - 1] = colbuf[(s - 1) / C]; job.e[s - 1] = 0.0; job.gam[s - 1] = 0.0; }
     }
     __syncthreads();                     // colbuf is read before the next matrix writes it
   }
   if (tid == 0 && dead) atomicExch(status, (int)AB_ERR_TIMEOUT);
+  cg::this_cluster().sync();             // nobody leaves while a mate may still send to it
 }
 
 // ---- 2. and 3. the tridiagonal problem ------------------------------------------------------------------
@@ -1126,15 +1211,37 @@ int launch_values(const EigJob* jobs, int count, int smax, cudaStream_t st) {
   return AB_OK;
 }
 
-template <int E>
-int launch_grid(const EigJob* jobs, int count, int smax, int sms, int* status, cudaStream_t st) {
-  int per_sm = 0;
-  AB_CUDA_OK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tridiag_grid_kernel<E>, kGridThreads, 0));
-  int C = (smax + kGridRows - 1) / kGridRows;
-  if (per_sm * sms < C) return AB_ERR_UNSUPPORTED;
-  const int groups = std::min(count, per_sm * sms / C);
-  void* args[] = {(void*)&jobs, (void*)&count, (void*)&C, (void*)&status};
-  AB_CUDA_OK(cudaLaunchCooperativeKernel(tridiag_grid_kernel<E>, dim3((unsigned)(groups * C)), dim3(kGridThreads), args, 0, st));
+template <int E, int W>
+int launch_grid(const EigJob* jobs, int count, int smax, int* status, cudaStream_t st) {
+  const size_t sm = 2 * (size_t)(32 * W * E + kMaxCl) * sizeof(double2);
+  AB_CUDA_OK(allow_smem(tridiag_grid_kernel<E, W>, 2048));
+  cudaLaunchConfig_t cfg = {};
+  cfg.blockDim = dim3(32 * W);
+  cfg.dynamicSmemBytes = sm;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeCooperative;
+  attr[1].val.cooperative = 1;
+  cfg.attrs = attr;
+  // The size of clusters that leaves room for the most matrices at a time, the largest of those.
+  int best = 0, size = 0, groups = 0;
+  for (int CL = kMaxCl; CL >= 1; CL /= 2) {
+    const int C = ((smax + kGridRows - 1) / kGridRows + CL - 1) / CL * CL;
+    int clusters = 0;
+    attr[0].val.clusterDim.x = CL;
+    cfg.gridDim = dim3((unsigned)C);
+    cfg.numAttrs = 1;
+    AB_CUDA_OK(cudaOccupancyMaxActiveClusters(&clusters, tridiag_grid_kernel<E, W>, &cfg));
+    const int g = std::min(count, clusters * CL / C);
+    if (g > groups) { best = CL; size = C; groups = g; }
+  }
+  if (groups < 1) return AB_ERR_UNSUPPORTED;
+  attr[0].val.clusterDim.x = best;
+  cfg.gridDim = dim3((unsigned)(groups * size));
+  cfg.numAttrs = 2;
+  AB_CUDA_OK(cudaLaunchKernelEx(&cfg, tridiag_grid_kernel<E, W>, jobs, count, size, status));
   AB_LAUNCH_OK();
   return AB_OK;
 }
@@ -1151,9 +1258,11 @@ int launch_back(const EigJob* jobs, int count, int need, int* status, cudaStream
 
 }  // namespace
 
+static size_t xbuf_doubles(int s) { return s > kEigSmallMax ? (size_t)4 * s : 0; }
+
 size_t eig_ws_doubles(int s) {
   const size_t n = (size_t)s, groups = (n + kGroup - 1) / kGroup;
-  return align_up(n * refl_ld(s) + 2 * n * n + groups * kGroup * kGroup + (4 + 5 + 1) * n + 8, 2);
+  return align_up(xbuf_doubles(s) + n * refl_ld(s) + 2 * n * n + groups * kGroup * kGroup + (5 + 1) * n + 8, 2);
 }
 
 // The largest order: the grid kernel needs all CTAs of a matrix resident together.
@@ -1161,7 +1270,7 @@ int eig_max() { return std::min(1184, kGridRows * std::max(sm_count(), 1)); }
 
 void eig_bind(EigJob& j, double* ws) {
   const size_t s = (size_t)j.s, groups = (s + kGroup - 1) / kGroup;
-  j.xbuf = ws; j.refl = j.xbuf + 4 * s; j.tmat = j.refl + s * refl_ld(j.s);      // each of these 16-byte aligned
+  j.xbuf = ws; j.refl = j.xbuf + xbuf_doubles(j.s); j.tmat = j.refl + s * refl_ld(j.s);      // each of these 16-byte aligned
   j.zp = j.tmat + groups * kGroup * kGroup; j.zm = j.zp + s * s;
   j.d = j.zm + s * s; j.e = j.d + s; j.gam = j.e + s; j.lam = j.gam + s; j.inv = j.lam + s; j.norm = j.inv + s;
   j.order = reinterpret_cast<int*>(j.norm + 1);
@@ -1174,11 +1283,11 @@ int eig_direct(const EigJob* h_jobs, const EigJob* d_jobs, int count, int smax, 
   int rc;
   if (smax > kEigSmallMax) {
     for (int i = 0; i < count; ++i)       // no word of a step is there yet
-      AB_CUDA_OK(cudaMemsetAsync(h_jobs[i].xbuf, 0, (size_t)4 * h_jobs[i].s * sizeof(double), st));
-    if (smax <= 512) rc = launch_grid<2>(d_jobs, count, smax, sms, status, st);
-    else if (smax <= 768) rc = launch_grid<3>(d_jobs, count, smax, sms, status, st);
-    else if (smax <= 1024) rc = launch_grid<4>(d_jobs, count, smax, sms, status, st);
-    else rc = launch_grid<5>(d_jobs, count, smax, sms, status, st);
+      AB_CUDA_OK(cudaMemsetAsync(h_jobs[i].xbuf, 0, xbuf_doubles(h_jobs[i].s) * sizeof(double), st));
+    if (smax <= 512) rc = launch_grid<4, 4>(d_jobs, count, smax, status, st);
+    else if (smax <= 768) rc = launch_grid<6, 4>(d_jobs, count, smax, status, st);
+    else if (smax <= 1024) rc = launch_grid<4, 8>(d_jobs, count, smax, status, st);
+    else rc = launch_grid<5, 8>(d_jobs, count, smax, status, st);
   } else if (smax <= 64) rc = launch_tridiag<2, 8, 8, true>(d_jobs, count, 1, status, st);
   else if (smax <= 128) rc = launch_tridiag<4, 16, 8, true>(d_jobs, count, 1, status, st);
   else if (smax <= 192)
