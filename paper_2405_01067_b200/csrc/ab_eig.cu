@@ -53,6 +53,17 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
+// Four sums across a warp, each exchange halving what a lane still carries: lanes 8 q ... hold sum q.
+__device__ __forceinline__ double warp_sum4(double s0, double s1, double s2, double s3, int lane) {
+  const bool h2 = (lane & 16) != 0, h1 = (lane & 8) != 0;
+  const double t0 = (h2 ? s2 : s0) + __shfl_xor_sync(0xffffffffu, h2 ? s0 : s2, 16);
+  const double t1 = (h2 ? s3 : s1) + __shfl_xor_sync(0xffffffffu, h2 ? s1 : s3, 16);
+  double t = (h1 ? t1 : t0) + __shfl_xor_sync(0xffffffffu, h1 ? t0 : t1, 8);
+  t += __shfl_xor_sync(0xffffffffu, t, 4);
+  t += __shfl_xor_sync(0xffffffffu, t, 2);
+  t += __shfl_xor_sync(0xffffffffu, t, 1);
+  return t;
+}
 __device__ __forceinline__ uint32_t map_rank(uint32_t addr, uint32_t rank) {
   uint32_t r;
   asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
@@ -69,12 +80,16 @@ __device__ __forceinline__ void st_async(uint32_t addr, double x, double y, uint
 // The matrix lives in registers: element (i, k) in warp i mod (warps of the cluster), lane k mod 32, so a warp
 // holds R whole rows, E elements of each per lane.  Step j:
 //   - warp 0 of each CTA has received p = A v of the reflector before (v, gamma) and column j of
-//     the matrix as it was before that reflector's update;  w = gamma p - (gamma^2 p.v / 2) v;  it works out column j of the
-//     updated matrix and the next reflector v', and hands w and v' to the other warps;
-//   - all warps pass over their rows in registers: A -= v w^T + w v^T, p' = A v';  every row's p'_i and A[i][j+1] go
-//     to warp 0 of every CTA of the cluster.
-// So the rank-two update and the product with the next vector touch an element once, and a step is a chain of two
-// warp reductions, a square root, the pass and one exchange.  The vectors are worked out by one warp because fp64 issues
+//     the matrix as it was before that reflector's update, a;  w = gamma p - c v, c = gamma^2 p.v / 2;  column j of the updated
+//     matrix is (a - x p) + y v with x = v1 gamma, y = 2 c v1 - gamma p_j, where v1 is the first element of v.  Only y waits for a
+//     sum, and the squared norm of the column follows from sums over b = a - x p:  b.b + 2 y b.v + y^2 v.v.  So one reduction of four sums
+//     gives all that a step needs (it took two, one after the other).  Where the terms cancel to less than kCancel of their size
+//     (1 to 2 % of the steps of a decaying spectrum) the entries are summed themselves.  w and the next reflector v' go to the other warps;
+//   - all warps pass over their rows in registers: A -= v w^T + w v^T, p' = A v' without the first element of v', which the
+//     square root of warp 0 gives meanwhile;  every row's p'_i and A[i][j+1] go to warp 0 of every CTA of the cluster, which adds
+//     the first element's products A[i][j+1] v1' to p'.
+// So the rank-two update and the product with the next vector touch an element once, and a step is a chain of one
+// warp reduction, the pass and one exchange.  The vectors are worked out by one warp because fp64 issues
 // at half rate: with every warp doing it for itself (no hand-over) the copies took more issue slots than the pass (8100 cycles a step
 // at order 192).  Finished 32-column groups are dropped at compile time (segment<E0>).
 // The exchange is st.async onto an mbarrier of each receiver (two, used in turn): the data carry their own
@@ -98,6 +113,7 @@ struct Tridiag {
     double2 pa[2][S + kMaxCl];   // p and the next column; behind them the peers' tokens
     double2 stage_or_col[kChunk * S / 2];   // start: rows of X as fp64; afterwards each row warp's piece of column j + 1
     double v[2][S], w[S];
+    double first[2];                        // v1 of the reflectors
     uint64_t bar[2];
     int dead;
   };
@@ -109,49 +125,51 @@ struct Tridiag {
 
   struct Rows { double A[R][E]; double v[E]; double gam, v1; bool ok; uint32_t dst, dbar; };
 
-  // Warp 0, step j: from p and the column to w and the next reflector (left in shared memory).  Returns through vn,
-  // dj, beta what is to be stored, through nrm, alpha what gamma follows from.
+  // Warp 0, step j: from p and the column to w and the next reflector but its first element (left in shared memory).  Returns
+  // through vn, dj, alpha, sq what is to be stored and what the first element and gamma follow from.
   template <int E0>
-  __device__ __forceinline__ void vec_step(Rows& x, int j, double (&vn)[E], double& dj, double& beta, double& den) {
+  __device__ __forceinline__ void vec_step(Rows& x, int j, double (&vn)[E], double& dj, double& alpha, double& sq) {
     const int par = j & 1;
     if constexpr (kSingle) tc::named_bar_sync(2, kThreads);
     else x.ok = x.ok && tc::mbar_wait(&sh.bar[par], (j >> 1) & 1);
     const double2* pb = sh.pa[par];
-    double w[E], pv = 0.0;
+    const double xg = x.v1 * x.gam;
+    double p[E], pv = 0.0, bb = 0.0, bv = 0.0, vv = 0.0;
 #pragma unroll
     for (int e = E0; e < E; ++e) {
       const double2 q = pb[lane + 32 * e];
-      w[e] = q.x; vn[e] = q.y;
+      const bool ahead = e > E0 + 1 || lane + 32 * e > j + 1;
+      p[e] = fma(q.y, x.v1, q.x);
+      vn[e] = ahead ? fma(-xg, p[e], q.y) : 0.0;
+      const double vm = ahead ? x.v[e] : 0.0;
+      pv = fma(p[e], x.v[e], pv);
+      bb = fma(vn[e], vn[e], bb);
+      bv = fma(vn[e], vm, bv);
+      vv = fma(vm, vm, vv);
     }
     const int j1 = j + 1 < s ? j + 1 : j;
     const double2 qj = pb[j], qj1 = pb[j1];
-    const double vj1 = sh.v[par][j1];
-#pragma unroll
-    for (int e = E0; e < E; ++e) pv = fma(w[e], x.v[e], pv);
-    pv = warp_sum(pv);
+    const double vj1 = sh.v[par][j1], pj = fma(qj.y, x.v1, qj.x), pj1 = fma(qj1.y, x.v1, qj1.x);
+    const double t4 = warp_sum4(pv, bb, bv, vv, lane);
+    pv = __shfl_sync(0xffffffffu, t4, 0); bb = __shfl_sync(0xffffffffu, t4, 8);
+    bv = __shfl_sync(0xffffffffu, t4, 16); vv = __shfl_sync(0xffffffffu, t4, 24);
     const double c = 0.5 * x.gam * (x.gam * pv);    // gamma alone may be as large as 1e290
-    const double wj = x.gam * qj.x - c * x.v1;
-    double sq = 0.0;
+    const double y = 2.0 * c * x.v1 - x.gam * pj, wj = x.gam * pj - c * x.v1;
 #pragma unroll
     for (int e = E0; e < E; ++e) {
-      w[e] = x.gam * w[e] - c * x.v[e];
-      vn[e] = vn[e] - x.v1 * w[e] - wj * x.v[e];
-      if (e <= E0 + 1 && lane + 32 * e <= j + 1) vn[e] = 0.0;
-      sq = fma(vn[e], vn[e], sq);
-      sh.w[lane + 32 * e] = w[e];
-    }
-    sq = warp_sum(sq);
-    dj = qj.y - 2.0 * x.v1 * wj;
-    const double alpha = (j + 1 < s) ? qj1.y - x.v1 * (x.gam * qj1.x - c * vj1) - wj * vj1 : 0.0;
-    const bool live = sq > kLive2;
-    const double nrm = sqrt(fma(alpha, alpha, sq));
-    beta = live ? (alpha > 0.0 ? -nrm : nrm) : alpha;
-    x.v1 = live ? alpha - beta : 0.0;
-    den = live ? nrm * (nrm + fabs(alpha)) : 0.0;
-#pragma unroll
-    for (int e = E0; e < E; ++e) {
-      if (e <= E0 + 1 && lane + 32 * e == j + 1) vn[e] = x.v1;
+      const bool ahead = e > E0 + 1 || lane + 32 * e > j + 1;
+      sh.w[lane + 32 * e] = x.gam * p[e] - c * x.v[e];
+      vn[e] = ahead ? fma(y, x.v[e], vn[e]) : 0.0;
       sh.v[par ^ 1][lane + 32 * e] = vn[e];
+    }
+    sq = bb + y * (2.0 * bv + y * vv);
+    dj = qj.y - 2.0 * x.v1 * wj;
+    alpha = (j + 1 < s) ? fma(y, vj1, fma(-xg, pj1, qj1.y)) : 0.0;
+    if (!(sq >= kCancel * (bb + y * y * vv))) {
+      sq = 0.0;
+#pragma unroll
+      for (int e = E0; e < E; ++e) sq = fma(vn[e], vn[e], sq);
+      sq = warp_sum(sq);
     }
     if constexpr (!kSingle) {
       if (lane == 0 && !x.ok) sh.dead = 1;                 // a peer never answered: all warps leave
@@ -180,9 +198,19 @@ struct Tridiag {
     const int jend = min(32 * E0 + 32, s);
     for (int j = 32 * E0; j < jend; ++j) {
       const int par = j & 1;
-      double w[E], vn[E], dj = 0.0, beta = 0.0, den = 0.0;
-      if (warp == 0) vec_step<E0>(x, j, vn, dj, beta, den);
+      double w[E], vn[E], dj = 0.0, alpha = 0.0, sq = 0.0, beta = 0.0, den = 0.0;
+      if (warp == 0) vec_step<E0>(x, j, vn, dj, alpha, sq);
       tc::named_bar_sync(1, kThreads);               // w and v' are there
+      if (warp == 0) {
+        const bool live = sq > kLive2;
+        const double nrm = sqrt(fma(alpha, alpha, sq));
+        beta = live ? (alpha > 0.0 ? -nrm : nrm) : alpha;
+        x.v1 = live ? alpha - beta : 0.0;
+        den = live ? nrm * (nrm + fabs(alpha)) : 0.0;
+        if (lane == 0) sh.first[par ^ 1] = x.v1;     // for the other warps' next pass
+      } else if (lane == (j & 31)) {
+        x.v[E0] = sh.first[par];                     // v of the step before was without its first element, j
+      }
       if constexpr (!kSingle) {
         if (*reinterpret_cast<volatile int*>(&sh.dead)) return;
       }
@@ -230,6 +258,9 @@ struct Tridiag {
       if constexpr (kSingle) { if (warp != 0) bar_arrive(2, kThreads); }
       if (warp == 0) {                               // off the chain: gamma, and what later kernels need
         x.gam = den > 0.0 ? 1.0 / den : 0.0;
+#pragma unroll
+        for (int e = E0; e < E; ++e)
+          if (e <= E0 + 1 && lane + 32 * e == j + 1) vn[e] = x.v1;
         if (rank == j % CL) {
           const int ld = refl_ld(s);
           double* dst = job.refl + (size_t)j * ld;
@@ -296,6 +327,7 @@ struct Tridiag {
     for (int i = threadIdx.x; i < S; i += kThreads) sh.v[0][i] = sh.v[1][i] = sh.w[i] = 0.0;
     if (threadIdx.x == 0) {
       sh.dead = 0;
+      sh.first[0] = sh.first[1] = 0.0;
       if (!kSingle) { tc::mbar_init(&sh.bar[0], 1); tc::mbar_init(&sh.bar[1], 1); tc::fence_barrier_init(); }
     }
     if constexpr (kSingle) __syncthreads(); else cg::this_cluster().sync();   // buffers and barriers are ready before a peer writes
@@ -381,17 +413,6 @@ __device__ __forceinline__ bool poll_pair(const double2* p, unsigned tag, double
     if (word_tag(v.x) == tag && word_tag(v.y) == tag) return true;
     if ((it & 1023u) == 1023u && tc::globaltimer_ns() - t0 > tc::kWaitLimitNs) return false;
   }
-}
-// Four sums across a warp, each exchange halving what a lane still carries: lanes 8 q ... hold sum q.
-__device__ __forceinline__ double warp_sum4(double s0, double s1, double s2, double s3, int lane) {
-  const bool h2 = (lane & 16) != 0, h1 = (lane & 8) != 0;
-  const double t0 = (h2 ? s2 : s0) + __shfl_xor_sync(0xffffffffu, h2 ? s0 : s2, 16);
-  const double t1 = (h2 ? s3 : s1) + __shfl_xor_sync(0xffffffffu, h2 ? s1 : s3, 16);
-  double t = (h1 ? t1 : t0) + __shfl_xor_sync(0xffffffffu, h1 ? t0 : t1, 8);
-  t += __shfl_xor_sync(0xffffffffu, t, 4);
-  t += __shfl_xor_sync(0xffffffffu, t, 2);
-  t += __shfl_xor_sync(0xffffffffu, t, 1);
-  return t;
 }
 // sum over the CTA's W warps of a value each warp has left in red[warp]
 template <int W>
