@@ -528,55 +528,81 @@ gather_rows_kernel(const float* __restrict__ Vt, const int* __restrict__ perm, i
   for (int u = threadIdx.x; u < s; u += 256) Vr[(size_t)k * s + u] = src[u] * inv;
 }
 
-// sigma[k] = norm over t of Ylong(k,t), Ylong(k,t) = Y[t*st_ + k*sk].  32 values of k per CTA.
+// sigma[k] = norm over t of Ylong(k,t), Ylong(k,t) = Y[t*st_ + k*sk].
+// Neighbouring k adjacent in memory: a cluster of kNormCl CTAs takes 32 values of k, a lane each, the warps of all of them
+// sharing the t; the parts are added in the order of the warps.  One CTA to 32 values walked 3072 rows in
+// 384 dependent rounds: 57 us for 192 values, 4 of them now.  Neighbouring t adjacent: a CTA a k (70 us -> 5, 128 values of 2304).
+constexpr int kNormCl = 8;
 __global__ void __launch_bounds__(256)
-long_norms_kernel(const float* __restrict__ Y, int64_t st_, int64_t sk, int L, int r_cap, float* __restrict__ sigma) {
-  __shared__ double red[8][33];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (sk == 1) {                      // neighbouring k adjacent in memory: lane = k, warps stride over t
-    const int k = blockIdx.x * 32 + lane;
-    double acc = 0.0;
-    if (k < r_cap)
-      for (int t = warp; t < L; t += 8) { float v = Y[(int64_t)t * st_ + k]; acc += (double)v * v; }
-    red[warp][lane] = acc;
-    __syncthreads();
-    if (warp == 0 && k < r_cap) {
-      double t = 0.0;
+long_norms_kernel(const float* __restrict__ Y, int64_t st_, int L, int r_cap, float* __restrict__ sigma) {
+  __shared__ double red[8][32];
+  __shared__ double part[kNormCl][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, rank = blockIdx.x % kNormCl;
+  const int k = blockIdx.x / kNormCl * 32 + lane;
+  double acc = 0.0;
+  if (k < r_cap) {
+#pragma unroll 8
+    for (int t = rank * 8 + warp; t < L; t += 8 * kNormCl) { const float v = Y[(int64_t)t * st_ + k]; acc += (double)v * v; }
+  }
+  red[warp][lane] = acc;
+  __syncthreads();
+  auto cluster = cooperative_groups::this_cluster();
+  if (warp == 0) {
+    acc = 0.0;
 #pragma unroll
-      for (int i = 0; i < 8; ++i) t += red[i][lane];
-      sigma[k] = (float)sqrt(t);
-    }
-  } else {                            // neighbouring t adjacent: one warp walks one k
-    for (int kk = warp; kk < 32; kk += 8) {
-      const int k = blockIdx.x * 32 + kk;
-      if (k >= r_cap) continue;
-      double acc = 0.0;
-      for (int t = lane; t < L; t += 32) { float v = Y[(int64_t)t * st_ + (int64_t)k * sk]; acc += (double)v * v; }
+    for (int i = 0; i < 8; ++i) acc += red[i][lane];
+    *cluster.map_shared_rank(&part[rank][lane], 0) = acc;
+  }
+  cluster.sync();
+  if (rank == 0 && warp == 0 && k < r_cap) {
+    acc = 0.0;
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-      if (lane == 0) sigma[k] = (float)sqrt(acc);
-    }
+    for (int i = 0; i < kNormCl; ++i) acc += part[i][lane];
+    sigma[k] = (float)sqrt(acc);
+  }
+}
+__global__ void __launch_bounds__(256)
+long_norms_rows_kernel(const float* __restrict__ Y, int64_t sk, int L, float* __restrict__ sigma) {
+  __shared__ double red[8];
+  const float* y = Y + (int64_t)blockIdx.x * sk;
+  double acc = 0.0;
+#pragma unroll 4
+  for (int t = threadIdx.x; t < L; t += 256) { const float v = y[t]; acc += (double)v * v; }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    acc = 0.0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) acc += red[i];
+    sigma[blockIdx.x] = (float)sqrt(acc);
   }
 }
 
-// solver: null, or what the direct solver's waits reported for the call this matrix was part of
-__global__ void rank_rule_kernel(const float* __restrict__ sigma, int r_cap, float cutoff, int* __restrict__ r_out,
-                                 const JState* __restrict__ st, const int* __restrict__ solver, int* __restrict__ dev_status) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// The rank rule, by every block of 256 threads for itself: how many values reach cutoff times the largest (at least one);
+// outside: whether one of those that are kept lies outside the accuracy domain.
+__device__ __forceinline__ int rank_rule(const float* __restrict__ sigma, int r_cap, float cutoff, bool& outside) {
+  __shared__ float red[8];
   float top = 0.f;
-  for (int k = 0; k < r_cap; ++k) top = fmaxf(top, sigma[k]);
+  for (int k = threadIdx.x; k < r_cap; k += 256) top = fmaxf(top, sigma[k]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = top;
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < 8; ++i) top = fmaxf(top, red[i]);
   const float thr = cutoff * top;
   int keep = 0;
-  for (int k = 0; k < r_cap; ++k) keep += (sigma[k] >= thr) ? 1 : 0;
-  if (keep < 1) keep = 1;
-  *r_out = keep;
-  if (dev_status) {
-    int code = solver && *solver != AB_OK ? *solver : st->status;
-    if (code == AB_OK)
-      for (int k = 0; k < keep; ++k)
-        if (sigma[k] < kDomainRel * top && sigma[k] > kZeroRel * top) code = AB_ERR_ACCURACY;
-    *dev_status = code;
+  for (int k0 = 0; k0 < r_cap; k0 += 256) {
+    const int k = k0 + (int)threadIdx.x;
+    keep += __syncthreads_count(k < r_cap && sigma[k] >= thr);
   }
+  if (keep < 1) keep = 1;
+  bool out = false;
+  for (int k = threadIdx.x; k < keep; k += 256) out = out || (sigma[k] < kDomainRel * top && sigma[k] > kZeroRel * top);
+  outside = __syncthreads_or(out) != 0;
+  return keep;
 }
 
 // What the self-test of the fallback makes of the direct solver's verdicts (see SvdSelftest).
@@ -586,34 +612,48 @@ __global__ void force_fallback_kernel(int* __restrict__ flags, int count, int* _
   if (i == 0 && status != AB_OK) *solver = status;
 }
 
+// Applies the rank rule and writes the factors.
 // long factor: F(t,k) = Ylong(k,t) / sqrt(sigma_k); short factor: F(k,u) = sqrt(sigma_k) Vr[k][u].
-// Columns/rows k >= r' (and k >= r_cap) are written as zero.
+// Columns/rows k >= r' (and k >= r_cap) are written as zero.  tall: the long factor is A (L x r_max), the short one B (r_max x s);
+// else the long one is B (r_max x L), the short one A (s x r_max).  A warp a row of the results.
+// solver: null, or what the direct solver's waits reported for the call this matrix was part of
 template <typename TO>
-__global__ void write_factors_kernel(const float* __restrict__ Y, int64_t yt, int64_t yk,
-                                     const float* __restrict__ Vr, const float* __restrict__ sigma,
-                                     const int* __restrict__ r_out, int L, int s, int r_cap, int r_max,
-                                     TO* __restrict__ Flong, int64_t lt, int64_t lk,
-                                     TO* __restrict__ Fshort, int64_t sk_, int64_t su) {
-  const int rk = *r_out;
-  const int64_t nlong = (int64_t)L * r_max, nshort = (int64_t)s * r_max;
-  const int64_t step = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < nlong + nshort; idx += step) {
-    if (idx < nlong) {
-      // walk the long factor in its own memory order
-      int64_t t, k;
-      if (lk == 1) { t = idx / r_max; k = idx - t * r_max; } else { k = idx / L; t = idx - k * L; }
-      float v = 0.f;
-      if (k < rk && k < r_cap) {
-        float sg = sigma[k];
-        v = sg > 0.f ? Y[t * yt + k * yk] * rsqrtf(sg) : 0.f;
+__global__ void __launch_bounds__(256)
+write_factors_kernel(const float* __restrict__ Y, const float* __restrict__ Vr, const float* __restrict__ sigma, int tall, int L, int s,
+                     int r_cap, int r_max, float cutoff, TO* __restrict__ Flong, TO* __restrict__ Fshort, int* __restrict__ r_out,
+                     const JState* __restrict__ st, const int* __restrict__ solver, int* __restrict__ dev_status) {
+  bool outside;
+  const int rk = rank_rule(sigma, r_cap, cutoff, outside), keep = rk < r_cap ? rk : r_cap;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    *r_out = rk;
+    if (dev_status) {
+      const int code = solver && *solver != AB_OK ? *solver : st->status;
+      *dev_status = code == AB_OK && outside ? (int)AB_ERR_ACCURACY : code;
+    }
+  }
+  const int lane = threadIdx.x & 31, nlong = tall ? L : r_max, nshort = tall ? r_max : s;
+  for (int row = blockIdx.x * 8 + (threadIdx.x >> 5); row < nlong + nshort; row += gridDim.x * 8) {
+    const bool is_long = row < nlong;
+    const int i = is_long ? row : row - nlong;
+    if (is_long == (tall != 0)) {          // a row runs over k
+      TO* dst = (is_long ? Flong : Fshort) + (int64_t)i * r_max;
+      for (int k = lane; k < r_max; k += 32) {
+        float v = 0.f;
+        if (k < keep) {
+          const float sg = sigma[k];
+          if (is_long) v = sg > 0.f ? Y[(int64_t)i * r_cap + k] * rsqrtf(sg) : 0.f;
+          else v = sqrtf(sg) * Vr[(int64_t)k * s + i];
+        }
+        from_f32(dst[k], v);
       }
-      from_f32(Flong[t * lt + k * lk], v);
-    } else {
-      int64_t j = idx - nlong, k, u;
-      if (su == 1) { k = j / s; u = j - k * s; } else { u = j / r_max; k = j - u * r_max; }
-      float v = 0.f;
-      if (k < rk && k < r_cap) v = sqrtf(sigma[k]) * Vr[k * (int64_t)s + u];
-      from_f32(Fshort[k * sk_ + u * su], v);
+    } else {                               // a row is one k
+      const int n = is_long ? L : s;
+      TO* dst = (is_long ? Flong : Fshort) + (int64_t)i * n;
+      const float* src = is_long ? Y + (int64_t)i * L : Vr + (int64_t)i * s;
+      float f = 0.f;
+      if (i < keep) f = !is_long ? sqrtf(sigma[i]) : sigma[i] > 0.f ? rsqrtf(sigma[i]) : 0.f;
+      const bool zero = i >= keep || (is_long && !(sigma[i] > 0.f));
+      for (int t = lane; t < n; t += 32) from_f32(dst[t], zero ? 0.f : src[t] * f);
     }
   }
 }
@@ -861,26 +901,32 @@ int svd_batch(const SvdItem* items, int L, float sigma_cutoff, void* ws, size_t 
         AB_TRY(gemm_simt(w.Vr, AB_F32, s, 1, it.W, it.w_dt, it.n, 1, w.Y, AB_F32, it.n, p.r_cap, it.n, it.m, stream));
         yt = 1; yk = it.n;
       }
-      long_norms_kernel<<<(p.r_cap + 31) / 32, 256, 0, stream>>>(w.Y, yt, yk, p.L, p.r_cap, it.sigma);
+      if (p.tall) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)((p.r_cap + 31) / 32 * kNormCl));
+        cfg.blockDim = dim3(256);
+        cfg.stream = stream;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = kNormCl; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr; cfg.numAttrs = 1;
+        AB_CUDA_OK(cudaLaunchKernelEx(&cfg, long_norms_kernel, (const float*)w.Y, yt, p.L, p.r_cap, it.sigma));
+      } else {
+        long_norms_rows_kernel<<<p.r_cap, 256, 0, stream>>>(w.Y, yk, p.L, it.sigma);
+      }
       AB_LAUNCH_OK();
       const int count = (int)g.second.size();
       const int* solver = solved ? lo.flags[s] + count + 2 + j / eig_chunk(s) : nullptr;
-      rank_rule_kernel<<<1, 32, 0, stream>>>(it.sigma, p.r_cap, sigma_cutoff, it.r_out, lo.st[s] + j, solver, it.dev_status);
-      AB_LAUNCH_OK();
-      // tall: A is the long factor (A[t][k], strides r_max, 1), B the short one (B[k][u], strides n, 1)
-      // wide: B is the long factor (B[k][t], strides 1, n),     A the short one (A[u][k]: k stride 1, u stride r_max)
+      const int rows = p.tall ? p.L + it.r_max : it.r_max + p.s;
+      const unsigned grid = (unsigned)std::min((rows + 7) / 8, std::max(sm_count(), 1) * 4);
       void* Fl = p.tall ? it.A : it.B;
       void* Fs = p.tall ? it.B : it.A;
-      int64_t lt = p.tall ? it.r_max : 1, lk = p.tall ? 1 : it.n;
-      int64_t sk = p.tall ? it.n : 1, su = p.tall ? 1 : it.r_max;
-      int64_t total = (int64_t)(p.L + s) * it.r_max;
-      unsigned grid = (unsigned)std::min<int64_t>((total + 255) / 256, (int64_t)std::max(sm_count(), 1) * 8);
       if (it.out_dt == AB_F32)
-        write_factors_kernel<float><<<grid, 256, 0, stream>>>(w.Y, yt, yk, w.Vr, it.sigma, it.r_out, p.L, s, p.r_cap,
-                                                             it.r_max, (float*)Fl, lt, lk, (float*)Fs, sk, su);
+        write_factors_kernel<float><<<grid, 256, 0, stream>>>(w.Y, w.Vr, it.sigma, p.tall, p.L, p.s, p.r_cap, it.r_max, sigma_cutoff,
+                                                             (float*)Fl, (float*)Fs, it.r_out, lo.st[s] + j, solver, it.dev_status);
       else
-        write_factors_kernel<bf16><<<grid, 256, 0, stream>>>(w.Y, yt, yk, w.Vr, it.sigma, it.r_out, p.L, s, p.r_cap,
-                                                            it.r_max, (bf16*)Fl, lt, lk, (bf16*)Fs, sk, su);
+        write_factors_kernel<bf16><<<grid, 256, 0, stream>>>(w.Y, w.Vr, it.sigma, p.tall, p.L, p.s, p.r_cap, it.r_max, sigma_cutoff,
+                                                            (bf16*)Fl, (bf16*)Fs, it.r_out, lo.st[s] + j, solver, it.dev_status);
       AB_LAUNCH_OK();
     }
   }
