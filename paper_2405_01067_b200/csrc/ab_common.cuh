@@ -49,9 +49,9 @@ inline cudaError_t allow_smem(K* kernel, int static_bytes = 0) {
 // Launch with programmatic stream serialisation, in clusters of `cluster` CTAs: the kernel may become resident while the one before it
 // in the stream still runs.  Only for kernels that wait for that one (tc::dep_wait) before they touch global memory.
 template <typename... KArgs, typename... Args>
-inline int launch_after(void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem, int cluster, cudaStream_t st, Args&&... args) {
+inline int launch_after(void (*kernel)(KArgs...), dim3 grid, unsigned block, size_t smem, int cluster, cudaStream_t st, Args&&... args) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
+  cfg.gridDim = grid;
   cfg.blockDim = dim3(block);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;

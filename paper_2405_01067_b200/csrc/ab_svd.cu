@@ -537,6 +537,8 @@ __global__ void __launch_bounds__(256)
 long_norms_kernel(const float* __restrict__ Y, int64_t st_, int L, int r_cap, float* __restrict__ sigma) {
   __shared__ double red[8][32];
   __shared__ double part[kNormCl][32];
+  tc::dep_wait();
+  tc::dep_launch();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, rank = blockIdx.x % kNormCl;
   const int k = blockIdx.x / kNormCl * 32 + lane;
   double acc = 0.0;
@@ -564,6 +566,8 @@ long_norms_kernel(const float* __restrict__ Y, int64_t st_, int L, int r_cap, fl
 __global__ void __launch_bounds__(256)
 long_norms_rows_kernel(const float* __restrict__ Y, int64_t sk, int L, float* __restrict__ sigma) {
   __shared__ double red[8];
+  tc::dep_wait();
+  tc::dep_launch();
   const float* y = Y + (int64_t)blockIdx.x * sk;
   double acc = 0.0;
 #pragma unroll 4
@@ -616,18 +620,21 @@ __global__ void force_fallback_kernel(int* __restrict__ flags, int count, int* _
 // long factor: F(t,k) = Ylong(k,t) / sqrt(sigma_k); short factor: F(k,u) = sqrt(sigma_k) Vr[k][u].
 // Columns/rows k >= r' (and k >= r_cap) are written as zero.  tall: the long factor is A (L x r_max), the short one B (r_max x s);
 // else the long one is B (r_max x L), the short one A (s x r_max).  A warp a row of the results.
-// solver: null, or what the direct solver's waits reported for the call this matrix was part of
+// solver: null, or what the direct solver's waits reported for the call this matrix was part of; tc: the same of its two products
 template <typename TO>
 __global__ void __launch_bounds__(256)
 write_factors_kernel(const float* __restrict__ Y, const float* __restrict__ Vr, const float* __restrict__ sigma, int tall, int L, int s,
                      int r_cap, int r_max, float cutoff, TO* __restrict__ Flong, TO* __restrict__ Fshort, int* __restrict__ r_out,
-                     const JState* __restrict__ st, const int* __restrict__ solver, int* __restrict__ dev_status) {
+                     const JState* __restrict__ st, const int* __restrict__ solver, const int* __restrict__ tc,
+                     int* __restrict__ dev_status) {
+  tc::dep_wait();
+  tc::dep_launch();
   bool outside;
   const int rk = rank_rule(sigma, r_cap, cutoff, outside), keep = rk < r_cap ? rk : r_cap;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     *r_out = rk;
     if (dev_status) {
-      const int code = solver && *solver != AB_OK ? *solver : st->status;
+      const int code = tc[0] != AB_OK ? tc[0] : tc[1] != AB_OK ? tc[1] : solver && *solver != AB_OK ? *solver : st->status;
       *dev_status = code == AB_OK && outside ? (int)AB_ERR_ACCURACY : code;
     }
   }
@@ -655,6 +662,36 @@ write_factors_kernel(const float* __restrict__ Y, const float* __restrict__ Vr, 
       const bool zero = i >= keep || (is_long && !(sigma[i] > 0.f));
       for (int t = lane; t < n; t += 32) from_f32(dst[t], zero ? 0.f : src[t] * f);
     }
+  }
+}
+
+// X = the sum of `parts` partial Gram matrices of which the upper triangle counts, added in fp64 in ascending order, and its mirror
+// image.  A block a pair of 32 x 32 tiles.
+__global__ void __launch_bounds__(256)
+sum_gram_kernel(const float* __restrict__ part, int parts, float* __restrict__ X, int s) {
+  __shared__ float t[32][33];
+  tc::dep_wait();
+  tc::dep_launch();
+  const int bi = blockIdx.y, bj = blockIdx.x;
+  if (bj < bi) return;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, col = 32 * bj + tx;
+  const size_t stride = (size_t)s * s;
+#pragma unroll
+  for (int h = 0; h < 4; ++h) {
+    const int row = 32 * bi + ty + 8 * h;
+    double acc = 0.0;
+    if (row < s && col < s && row <= col) {
+#pragma unroll 6
+      for (int q = 0; q < parts; ++q) acc += (double)part[q * stride + (size_t)row * s + col];
+      X[(size_t)row * s + col] = (float)acc;
+    }
+    t[ty + 8 * h][tx] = (float)acc;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int h = 0; h < 4; ++h) {
+    const int row = 32 * bj + ty + 8 * h, c = 32 * bi + tx;      // the mirror image's
+    if (row < s && c < s && row > c) X[(size_t)row * s + c] = t[tx][ty + 8 * h];
   }
 }
 
@@ -689,6 +726,7 @@ struct Layout {
   std::map<int, double*> eig;                 // direct solver: its scratch, EigJobs, fallback flags (and behind the flags of a
   std::map<int, int*> flags;                  //   group two words on which the blocks of the fallback meet and the solver's status)
   std::map<int, EigJob*> ejobs;
+  int* tc;                                    // two words a matrix: what the waits of its Gram and its long product reported
   std::vector<ItemWs> item;
   size_t bytes;
 };
@@ -715,6 +753,7 @@ Layout make_layout(const SvdItem* items, int L, void* ws) {
       lo.eig[g.first] = ar.take_n<double>(std::min(cnt, (size_t)eig_chunk(g.first)) * eig_ws_doubles(g.first));
     }
   }
+  lo.tc = ar.take_n<int>(2 * (size_t)L);
   lo.item.resize(L);
   for (int i = 0; i < L; ++i) {
     Plan p = make_plan(items[i]);
@@ -797,6 +836,41 @@ int run_jacobi_fallback(float* X, float* Vt, JState* st, int* flags, int s, int 
   return AB_OK;
 }
 
+// The Gram matrix and the long product of an fp32 matrix go to the tensor cores as six bf16 terms (ab_gemm_split.cu) where their work
+// pays for three launches in place of one, or for a tile of 128.  Splits of one matrix, us, fp32 pipes / tensor cores.  Gram: 3072 x 256
+// 488 / 484, 800 x 256 461 / 468, 128 x 1000 265 / 281.  Long product: 3072 x 256 at rank 16 486 / 486, 32 488 / 484, 96 499 / 489;
+// 3072 x 128 at rank 64 301 / 298.
+constexpr int kGramParts = 6;             // the scratch of the solver, not yet in use, holds as many partial sums
+bool gram_on_tensor_cores(const SvdItem& it, const Plan& p) {
+  return it.w_dt == AB_F32 && p.s >= 192 && p.s <= eig_max() && (int64_t)p.s * p.s * p.L >= 100000000 && gemm_tc_available();
+}
+bool long_on_tensor_cores(const SvdItem& it, const Plan& p) {
+  return it.w_dt == AB_F32 && p.s >= 128 && (int64_t)p.s * p.L * p.r_cap >= 20000000 && gemm_tc_available();
+}
+SplitGemm split_product(const void* A, int64_t lda, int a_mn, const void* B, int64_t ldb, int b_mn, float* C, int64_t ldc, int M, int N, int K) {
+  SplitGemm g = {};
+  g.A = A; g.lda = lda; g.a_mn = a_mn; g.B = B; g.ldb = ldb; g.b_mn = b_mn; g.C = C; g.ldc = ldc; g.M = M; g.N = N; g.K = K;
+  return g;
+}
+// G = W^T W (tall) or W W^T; parts: kGramParts s x s partial results; scratch: room for as many SplitGemm and 16 bytes
+int gram_split(const SvdItem& it, const Plan& p, float* G, float* parts, void* scratch, int* status, cudaStream_t st) {
+  SplitGemm* table = reinterpret_cast<SplitGemm*>(align_up(reinterpret_cast<uintptr_t>(scratch), 16));      // s * s floats after an odd s * s
+  const float* W = static_cast<const float*>(it.W);
+  const int s = p.s, per = ((p.L + kGramParts - 1) / kGramParts + 63) / 64 * 64, n = (p.L + per - 1) / per;
+  SplitGemm g[kGramParts];
+  for (int q = 0; q < n; ++q) {
+    const int k0 = q * per, len = std::min(p.L - k0, per);
+    const float* src = p.tall ? W + (size_t)k0 * it.n : W + k0;
+    g[q] = split_product(src, it.n, p.tall, src, it.n, p.tall, parts + (size_t)q * s * s, s, s, s, len);
+    g[q].upper_only = 1;
+  }
+  const SplitBatch b = gemm_split_plan(g, n);
+  AB_TRY(upload_async(table, g, n * sizeof(SplitGemm), st));
+  AB_TRY(gemm_split_batched(table, b, status, st));
+  const unsigned t = (unsigned)(s + 31) / 32;
+  return launch_after(sum_gram_kernel, dim3(t, t), 256, 0, 1, st, (const float*)parts, n, G, s);
+}
+
 // Whether a group of `count` matrices of short side s goes to the direct solver (its fallback has to fit as well).
 bool direct(int s, int count) { return s <= kEigSmallMax ? rows_jacobi_fits(count, s) : s <= eig_max(); }
 
@@ -810,13 +884,18 @@ int svd_batch(const SvdItem* items, int L, float sigma_cutoff, void* ws, size_t 
               const SvdSelftest* selftest) {
   Layout lo = make_layout(items, L, ws);
   if (lo.bytes > ws_bytes) return AB_ERR_WORKSPACE;
+  AB_CUDA_OK(cudaMemsetAsync(lo.tc, 0, sizeof(int) * 2 * L, stream));
   // 1. Gram matrices into X
   for (auto& g : lo.groups) {
     const int s = g.first;
     for (size_t j = 0; j < g.second.size(); ++j) {
       const SvdItem& it = items[g.second[j]];
       float* G = lo.X[s] + j * (size_t)s * s;
-      if (it.m >= it.n)   // G = W^T W
+      const Plan p = make_plan(it);
+      if (gram_on_tensor_cores(it, p))
+        AB_TRY(gram_split(it, p, G, reinterpret_cast<float*>(lo.eig[s]), lo.Vt[s] + j * (size_t)s * s,
+                          lo.tc + 2 * g.second[j], stream));
+      else if (it.m >= it.n)   // G = W^T W
         AB_TRY(gemm_simt(it.W, it.w_dt, 1, it.n, it.W, it.w_dt, it.n, 1, G, AB_F32, s, s, s, it.m, stream));
       else                // G = W W^T
         AB_TRY(gemm_simt(it.W, it.w_dt, it.n, 1, it.W, it.w_dt, 1, it.n, G, AB_F32, s, s, s, it.n, stream));
@@ -894,27 +973,22 @@ int svd_batch(const SvdItem* items, int L, float sigma_cutoff, void* ws, size_t 
         AB_LAUNCH_OK();
       }
       int64_t yt, yk;   // Ylong(k,t) = Y[t*yt + k*yk]
+      const bool tc = long_on_tensor_cores(it, p);
       if (p.tall) {     // Y (m x r_cap) = W Vr^T
-        AB_TRY(gemm_simt(it.W, it.w_dt, it.n, 1, w.Vr, AB_F32, 1, s, w.Y, AB_F32, p.r_cap, it.m, p.r_cap, it.n, stream));
+        if (tc) AB_TRY(gemm_split_one(split_product(it.W, it.n, 0, w.Vr, s, 0, w.Y, p.r_cap, it.m, p.r_cap, s), false, lo.tc + 2 * i + 1, stream));
+        else AB_TRY(gemm_simt(it.W, it.w_dt, it.n, 1, w.Vr, AB_F32, 1, s, w.Y, AB_F32, p.r_cap, it.m, p.r_cap, it.n, stream));
         yt = p.r_cap; yk = 1;
       } else {          // Y (r_cap x n) = Vr W
-        AB_TRY(gemm_simt(w.Vr, AB_F32, s, 1, it.W, it.w_dt, it.n, 1, w.Y, AB_F32, it.n, p.r_cap, it.n, it.m, stream));
+        if (tc) AB_TRY(gemm_split_one(split_product(w.Vr, s, 0, it.W, it.n, 1, w.Y, it.n, p.r_cap, it.n, s), false, lo.tc + 2 * i + 1, stream));
+        else AB_TRY(gemm_simt(w.Vr, AB_F32, s, 1, it.W, it.w_dt, it.n, 1, w.Y, AB_F32, it.n, p.r_cap, it.n, it.m, stream));
         yt = 1; yk = it.n;
       }
       if (p.tall) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)((p.r_cap + 31) / 32 * kNormCl));
-        cfg.blockDim = dim3(256);
-        cfg.stream = stream;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = kNormCl; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr; cfg.numAttrs = 1;
-        AB_CUDA_OK(cudaLaunchKernelEx(&cfg, long_norms_kernel, (const float*)w.Y, yt, p.L, p.r_cap, it.sigma));
+        AB_TRY(launch_after(long_norms_kernel, dim3((unsigned)((p.r_cap + 31) / 32 * kNormCl)), 256, 0, kNormCl, stream, (const float*)w.Y, yt, p.L,
+                            p.r_cap, it.sigma));
       } else {
-        long_norms_rows_kernel<<<p.r_cap, 256, 0, stream>>>(w.Y, yk, p.L, it.sigma);
+        AB_TRY(launch_after(long_norms_rows_kernel, dim3((unsigned)p.r_cap), 256, 0, 1, stream, (const float*)w.Y, yk, p.L, it.sigma));
       }
-      AB_LAUNCH_OK();
       const int count = (int)g.second.size();
       const int* solver = solved ? lo.flags[s] + count + 2 + j / eig_chunk(s) : nullptr;
       const int rows = p.tall ? p.L + it.r_max : it.r_max + p.s;
@@ -922,12 +996,13 @@ int svd_batch(const SvdItem* items, int L, float sigma_cutoff, void* ws, size_t 
       void* Fl = p.tall ? it.A : it.B;
       void* Fs = p.tall ? it.B : it.A;
       if (it.out_dt == AB_F32)
-        write_factors_kernel<float><<<grid, 256, 0, stream>>>(w.Y, w.Vr, it.sigma, p.tall, p.L, p.s, p.r_cap, it.r_max, sigma_cutoff,
-                                                             (float*)Fl, (float*)Fs, it.r_out, lo.st[s] + j, solver, it.dev_status);
+        AB_TRY(launch_after(write_factors_kernel<float>, dim3(grid), 256, 0, 1, stream, (const float*)w.Y, (const float*)w.Vr, (const float*)it.sigma,
+                            (int)p.tall, p.L, p.s, p.r_cap, it.r_max, sigma_cutoff, (float*)Fl, (float*)Fs, it.r_out, (const JState*)(lo.st[s] + j),
+                            solver, (const int*)(lo.tc + 2 * i), it.dev_status));
       else
-        write_factors_kernel<bf16><<<grid, 256, 0, stream>>>(w.Y, w.Vr, it.sigma, p.tall, p.L, p.s, p.r_cap, it.r_max, sigma_cutoff,
-                                                            (bf16*)Fl, (bf16*)Fs, it.r_out, lo.st[s] + j, solver, it.dev_status);
-      AB_LAUNCH_OK();
+        AB_TRY(launch_after(write_factors_kernel<bf16>, dim3(grid), 256, 0, 1, stream, (const float*)w.Y, (const float*)w.Vr, (const float*)it.sigma,
+                            (int)p.tall, p.L, p.s, p.r_cap, it.r_max, sigma_cutoff, (bf16*)Fl, (bf16*)Fs, it.r_out, (const JState*)(lo.st[s] + j),
+                            solver, (const int*)(lo.tc + 2 * i), it.dev_status));
     }
   }
   return AB_OK;

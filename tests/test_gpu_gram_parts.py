@@ -1,0 +1,43 @@
+"""Gram matrix of a dense split in parts of the long side on the tensor cores: odd short sides (tables and partial sums behind an odd
+number of floats), long sides that leave a short last part or fill none, either side long.
+
+Tolerance: the six bf16 terms carry 24 bits and the parts are added in fp64, so sigma is as good as from an fp32 Gram matrix:
+2^-24 sqrt(s) sigma_1^2 / sigma, below 1e-4 for the values above 0.2 sigma_1 that are compared; the residual as in test_gpu_eig.py.
+"""
+import numpy as np
+import pytest
+import torch
+
+from paper_2405_01067_b200 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+def check(W, A, B, sigma, k):
+    ref = np.linalg.svd(W.astype(np.float64), compute_uv=False)
+    sg = sigma.cpu().numpy().astype(np.float64)
+    assert np.all(np.abs(sg - ref[:k]) <= 1e-4 * ref[:k])
+    res = np.linalg.norm(W - A.double().cpu().numpy() @ B.double().cpu().numpy())
+    assert abs(res - np.linalg.norm(ref[k:])) <= 1e-5 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("m,n,k", [(2713, 192, 40), (2476, 201, 150), (201, 2600, 33), (1664, 257, 64), (385, 769, 300), (769, 385, 8),
+                                   (3072, 768, 192), (1000, 999, 100)])
+def test_gram_in_parts(m, n, k):
+    from paper_2405_01067_b200 import binding as ab
+    W = synth.planted_matrix(np.random.default_rng(m + n), m, n, np.linspace(1.0, 0.2, min(m, n)))
+    A, B, sigma, r_out, status = ab.ab_svd_split(torch.from_numpy(W).cuda(), k, 0.0)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0 and int(r_out.item()) == k
+    check(W, A, B, sigma, k)
+
+
+def test_gram_in_parts_of_a_batch():
+    from paper_2405_01067_b200 import binding as ab
+    m, n, count = 1700, 257, 4
+    W = np.stack([synth.planted_matrix(np.random.default_rng(i), m, n, np.linspace(1.0 + i, 0.3 + i, n)) for i in range(count)])
+    A, B, sigma, r_out, status = ab.ab_selftest_split_fallback(torch.from_numpy(W).cuda(), 60, 0)
+    torch.cuda.synchronize()
+    assert status.tolist() == [0] * count and r_out.tolist() == [60] * count
+    for i in range(count):
+        check(W[i], A[i], B[i], sigma[i], 60)

@@ -19,7 +19,7 @@ def test_batches_of_large_orders(s, count):
         a, b = synth.planted_factors(rng, m, n, np.linspace(1.0 + i, 0.3, r))
         As.append(torch.from_numpy(a[None].copy()).cuda())
         Bs.append(torch.from_numpy(b[None].copy()).cuda())
-    plan = ab.SyncPlan(As, Bs, 0.1)
+    plan = ab.SyncPlan(As, Bs, 0.046)         # no value of these spectra lies within 2e-3 of it
     A_out, B_out, sigma, r_out, status = ab.ab_group_sync(plan, path=ab.AB_SYNC_DENSE)
     torch.cuda.synchronize()
     assert torch.count_nonzero(status) == 0
@@ -27,7 +27,7 @@ def test_batches_of_large_orders(s, count):
         W = As[i][0].double().cpu().numpy() @ Bs[i][0].double().cpu().numpy()
         ref = np.linalg.svd(W, compute_uv=False)
         keep = int(r_out[i].item())
-        assert keep == int(np.sum(ref[:r] >= 0.1 * ref[0]))
+        assert keep == int(np.sum(ref[:r] >= 0.046 * ref[0]))
         sg = sigma[i].cpu().numpy().astype(np.float64)
         assert np.all(np.abs(sg[:keep] - ref[:keep]) <= 1e-4 * ref[:keep])
         prod = A_out[i].double().cpu().numpy() @ B_out[i].double().cpu().numpy()
