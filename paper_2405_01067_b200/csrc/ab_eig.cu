@@ -368,6 +368,9 @@ __global__ void __launch_bounds__(32 * W, 1)
 tridiag_small_kernel(const EigJob* __restrict__ jobs, int* status) {
   using T = Tridiag<E, R, W, kSingle>;
   extern __shared__ __align__(16) unsigned char tri_sm[];
+  tc::dep_wait();
+  // A batch leaves a few SMs empty, and the blocks of the kernel behind would crowd there (72 matrices of order 192: + 120 us).
+  if (gridDim.x <= 32) tc::dep_launch();
   const int CL = kSingle ? 1 : (int)cg::this_cluster().num_blocks();
   const EigJob job = jobs[blockIdx.x / CL];
   T t{*reinterpret_cast<typename T::Shared*>(tri_sm), job, job.s, CL, kSingle ? 0 : (int)cg::this_cluster().block_rank(),
@@ -768,6 +771,8 @@ tri_values_kernel(const EigJob* __restrict__ jobs) {
   __shared__ unsigned mask[kMaxOrder / 32];
   __shared__ double red[4];
   __shared__ double ratio[kMaxOrder / 8 + 4];
+  tc::dep_wait();
+  tc::dep_launch();
   const EigJob job = jobs[blockIdx.y];
   const int s = job.s;
   constexpr int per = 128 / kLanes;
@@ -882,6 +887,8 @@ tri_vectors_kernel(const EigJob* __restrict__ jobs, int vec_blocks, int smax) {
   __shared__ double red[kVecWarps];
   __shared__ double part[kVecWarps][32];
   __shared__ int best_key[kVecWarps][32], best_row[kVecWarps][32], rank_part[kVecWarps][32];
+  tc::dep_wait();
+  tc::dep_launch();
   const EigJob job = jobs[blockIdx.y];
   const int s = job.s;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1128,6 +1135,8 @@ back_transform_kernel(const EigJob* __restrict__ jobs, int* status) {
   double2* ys = reinterpret_cast<double2*>(ts + kStages * kGroup * kGroup);
   __shared__ uint64_t bars[kStages];
   __shared__ int dead;
+  tc::dep_wait();
+  tc::dep_launch();
   const EigJob job = jobs[blockIdx.y];
   const int s = job.s, ld = refl_ld(s), ngroups = (s + kGroup - 1) / kGroup;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, lr = lane >> 2, lc = lane & 3;
@@ -1210,26 +1219,13 @@ template <int E, int R, int W, bool kSingle>
 int launch_tridiag(const EigJob* jobs, int count, int CL, int* status, cudaStream_t st) {
   const size_t sm = sizeof(typename Tridiag<E, R, W, kSingle>::Shared);
   AB_CUDA_OK(cudaFuncSetAttribute(tridiag_small_kernel<E, R, W, kSingle>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(count * CL));
-  cfg.blockDim = dim3(32 * W);
-  cfg.dynamicSmemBytes = sm;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = CL; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr; cfg.numAttrs = 1;
-  AB_CUDA_OK(cudaLaunchKernelEx(&cfg, tridiag_small_kernel<E, R, W, kSingle>, jobs, status));
-  AB_LAUNCH_OK();
-  return AB_OK;
+  return launch_after(tridiag_small_kernel<E, R, W, kSingle>, dim3((unsigned)(count * CL)), 32 * W, sm, CL, st, jobs, status);
 }
 
 template <int L>
 int launch_values(const EigJob* jobs, int count, int smax, cudaStream_t st) {
   const int per = 128 / L;
-  tri_values_kernel<L><<<dim3((unsigned)((smax + per - 1) / per), (unsigned)count), 128, (smax + 32) * sizeof(double2), st>>>(jobs);
-  AB_LAUNCH_OK();
-  return AB_OK;
+  return launch_after(tri_values_kernel<L>, dim3((unsigned)((smax + per - 1) / per), (unsigned)count), 128, (smax + 32) * sizeof(double2), 1, st, jobs);
 }
 
 template <int E, int W>
@@ -1272,9 +1268,8 @@ int launch_back(const EigJob* jobs, int count, int need, int* status, cudaStream
   using B = BackShape<TW, RS, W>;
   constexpr int per = 8 * W / RS;
   AB_CUDA_OK(allow_smem(back_transform_kernel<TW, RS, W>, 1024));
-  back_transform_kernel<TW, RS, W><<<dim3((unsigned)((need + per - 1) / per), (unsigned)count), 32 * W, B::kBytes, st>>>(jobs, status);
-  AB_LAUNCH_OK();
-  return AB_OK;
+  return launch_after(back_transform_kernel<TW, RS, W>, dim3((unsigned)((need + per - 1) / per), (unsigned)count), 32 * W, B::kBytes, 1, st, jobs,
+                      status);
 }
 
 }  // namespace
@@ -1324,8 +1319,7 @@ int eig_direct(const EigJob* h_jobs, const EigJob* d_jobs, int count, int smax, 
   AB_TRY(rc);
   const int vb = (smax + 31) / 32, gb = ((smax + kGroup - 1) / kGroup + kVecWarps - 1) / kVecWarps;
   AB_CUDA_OK(allow_smem(tri_vectors_kernel, 8192));
-  tri_vectors_kernel<<<dim3((unsigned)(vb + gb), (unsigned)count), 32 * kVecWarps, vectors_smem(smax), st>>>(d_jobs, vb, smax);
-  AB_LAUNCH_OK();
+  AB_TRY(launch_after(tri_vectors_kernel, dim3((unsigned)(vb + gb), (unsigned)count), 32 * kVecWarps, vectors_smem(smax), 1, st, d_jobs, vb, smax));
   // A warp to eight vectors where that gives a scheduler more than one warp, else eight warps to them (72 matrices of
   // order 192, 23 warps of vectors an SM: 65 us against 137).
   int need = 1;

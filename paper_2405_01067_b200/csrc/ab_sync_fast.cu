@@ -24,6 +24,7 @@
 #include <cooperative_groups.h>
 
 #include "ab_common.cuh"
+#include "ab_tc_ptx.cuh"
 
 namespace ab {
 namespace {
@@ -80,6 +81,8 @@ jacobi_rows_cluster_kernel(const JacobiJob* __restrict__ jobs, float tol) {
   cg::cluster_group cluster = cg::this_cluster();
   extern __shared__ __align__(16) float sm[];
   const int crank = (kC == 1) ? 0 : (int)cluster.block_rank();
+  tc::dep_wait();
+  tc::dep_launch();
   const JacobiJob job = jobs[blockIdx.x / kC];
   if (*job.flag == 0) return;                  // the same for every CTA of the cluster
   const int k = job.k, r = job.r, ld = r + 1;
@@ -357,7 +360,7 @@ cudaLaunchConfig_t jacobi_config(int count, int rmax, cudaStream_t st, cudaLaunc
 // Returns 1 when it declined, so that the caller tries a narrower cluster.
 template <int EL, int C>
 int try_launch_jacobi(const JacobiJob* jobs, int count, int rmax, float tol, cudaStream_t st) {
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   cudaLaunchConfig_t cfg = jacobi_config<EL, C>(count, rmax, st, attr);
   if (cfg.dynamicSmemBytes > (size_t)(kMaxSmem - kStatics)) return C == 1 ? AB_ERR_UNSUPPORTED : 1;
   AB_CUDA_OK(allow_smem(jacobi_rows_cluster_kernel<EL, C>, kStatics));
@@ -373,6 +376,9 @@ int try_launch_jacobi(const JacobiJob* jobs, int count, int rmax, float tol, cud
     }
     if (resident < count) return 1;
   }
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.numAttrs = 2;
   AB_CUDA_OK(cudaLaunchKernelEx(&cfg, jacobi_rows_cluster_kernel<EL, C>, jobs, tol));
   AB_LAUNCH_OK();
   return AB_OK;
@@ -424,6 +430,8 @@ __device__ __forceinline__ float rsqrt_close(float x) {
 // chains of pivots and 90000 below them, bound by shared memory; the inverse 134000 -> 60000.
 __global__ void __launch_bounds__(kCThreads, 1) chol_inv_kernel(const CholJob* __restrict__ jobs) {
   extern __shared__ __align__(16) float sm[];
+  tc::dep_wait();
+  tc::dep_launch();
   const CholJob job = jobs[blockIdx.x];
   const int r = job.r, ld = r + 1;
   float* S = sm;                       // r x ld
@@ -621,6 +629,8 @@ __global__ void __launch_bounds__(128)
 fast_rank_rule_kernel(const float* const* __restrict__ sigma, const int* __restrict__ rs,
                       float cutoff, int* const* __restrict__ r_out,
                       const int* __restrict__ jstatus, int* __restrict__ dev_status, int L) {
+  tc::dep_wait();
+  tc::dep_launch();
   const int i = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (i >= L) return;
   const float* sg = sigma[i];
@@ -653,6 +663,8 @@ fast_rank_rule_kernel(const float* const* __restrict__ sigma, const int* __restr
 
 // A bounded wait that ran out inside one of the tensor-core launches or the eigensolver of the call reaches every matrix's status.
 __global__ void fold_tc_status_kernel(const int* __restrict__ tc_status, int* __restrict__ dev_status, int L) {
+  tc::dep_wait();
+  tc::dep_launch();
   int bad = AB_OK;
   for (int k = 0; k < 4; ++k) if (tc_status[k] != AB_OK) bad = tc_status[k];
   if (bad == AB_OK) return;
@@ -921,8 +933,7 @@ int sync_factored(const ab_sync_desc* d, int L, int K, float sigma_cutoff, int d
   AB_TRY(run(kGram, w.tc_status, st));
   const size_t csm = chol_smem_bytes(rmax);
   AB_CUDA_OK(allow_smem(chol_inv_kernel, kStatics));
-  chol_inv_kernel<<<2 * L, kCThreads, csm, st>>>(w.cjobs);                                  // R_A, R_B and inverses
-  AB_LAUNCH_OK();
+  AB_TRY(launch_after(chol_inv_kernel, dim3((unsigned)(2 * L)), kCThreads, csm, 1, st, (const CholJob*)w.cjobs));       // R_A, R_B and inverses
   AB_TRY(run(kM, w.tc_status, st));
   int side_rc = AB_OK;
   if (side && cudaEventRecord(fork, st) != cudaSuccess) side_rc = AB_ERR_CUDA;
@@ -933,9 +944,8 @@ int sync_factored(const ab_sync_desc* d, int L, int K, float sigma_cutoff, int d
     if (side_rc == AB_OK) side_rc = run(kW, w.tc_status + 2, side);
     if (side_rc == AB_OK && cudaEventRecord(join, side) != cudaSuccess) side_rc = AB_ERR_CUDA;
   }
-  fast_rank_rule_kernel<<<(L + 3) / 4, 128, 0, st>>>(w.sig_ptrs, w.rs, sigma_cutoff, w.rout_ptrs, w.jstatus,
-                                                         dev_status, L);
-  AB_LAUNCH_OK();
+  AB_TRY(launch_after(fast_rank_rule_kernel, dim3((unsigned)((L + 3) / 4)), 128, 0, 1, st, (const float* const*)w.sig_ptrs, (const int*)w.rs, sigma_cutoff,
+                      (int* const*)w.rout_ptrs, (const int*)w.jstatus, dev_status, L));
   AB_TRY(run(kZ1, w.tc_status, st));
   AB_TRY(run(kZ2, w.tc_status, st));
   AB_TRY(run(kOut, w.tc_status + 1, st));
@@ -944,8 +954,7 @@ int sync_factored(const ab_sync_desc* d, int L, int K, float sigma_cutoff, int d
     if (side_rc != AB_OK) { (void)cudaGetLastError(); return side_rc; }
   }
   if (dev_status) {
-    fold_tc_status_kernel<<<1, 128, 0, st>>>(w.tc_status, dev_status, L);
-    AB_LAUNCH_OK();
+    AB_TRY(launch_after(fold_tc_status_kernel, dim3(1), 128, 0, 1, st, (const int*)w.tc_status, dev_status, L));
   }
   return AB_OK;
 }
