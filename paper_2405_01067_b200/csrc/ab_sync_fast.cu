@@ -444,6 +444,39 @@ __global__ void __launch_bounds__(kCThreads, 1) chol_inv_kernel(const CholJob* _
   {
     const float* __restrict__ G = job.G;
     const size_t part = (size_t)r * r;
+    if ((r & 3) == 0 && (reinterpret_cast<uintptr_t>(G) & 15u) == 0) {
+      // groups of four values of the upper triangle, four a thread and three parts at a time: up to twelve 16-byte loads in flight
+      const int rc = r >> 2, n = r * rc;
+      const size_t part4 = part >> 2;
+      const float4* G4 = reinterpret_cast<const float4*>(G);
+      for (int c0 = tid; c0 < n; c0 += 4 * kCThreads) {
+        float4 v[4];
+        int at[4];                                               // place in S, or -1
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int c = c0 + u * kCThreads, row = c / rc, col = 4 * (c - row * rc);
+          at[u] = c < n && col + 3 >= row ? row * ld + col : -1;
+          v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        for (int q0 = 0; q0 < job.nparts; q0 += 3) {             // ascending part order
+          float4 t[3][4];
+#pragma unroll
+          for (int q = 0; q < 3; ++q)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              t[q][u] = make_float4(0.f, 0.f, 0.f, 0.f);
+              if (at[u] >= 0 && q0 + q < job.nparts) t[q][u] = __ldcg(G4 + (q0 + q) * part4 + c0 + u * kCThreads);
+            }
+#pragma unroll
+          for (int q = 0; q < 3; ++q)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) { v[u].x += t[q][u].x; v[u].y += t[q][u].y; v[u].z += t[q][u].z; v[u].w += t[q][u].w; }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (at[u] >= 0) { S[at[u]] = v[u].x; S[at[u] + 1] = v[u].y; S[at[u] + 2] = v[u].z; S[at[u] + 3] = v[u].w; }
+      }
+    } else
     for (int i0 = 2 * warp; i0 < r; i0 += 2 * nwarps) {           // two rows per warp; the loads of both are all in flight
       float v[2][8];
 #pragma unroll
