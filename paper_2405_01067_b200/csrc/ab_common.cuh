@@ -105,6 +105,12 @@ int gemm_simt(const void* A, int a_dt, int64_t sAm, int64_t sAk,
               void* C, int c_dt, int64_t ldc,
               int64_t M, int64_t N, int64_t K, cudaStream_t st);
 
+// The reduction in parts of `per`: part q is M x N (without gaps) at parts + q M N, sums of 16 products in fp32, those in fp64; upper (M
+// = N): only tiles that reach the upper triangle are formed.  sum_parts adds them up.
+int gemm_parts(const float* A, int64_t sAm, int64_t sAk, const float* B, int64_t sBk, int64_t sBn, double* parts, int M, int N, int K, int per,
+               bool upper, cudaStream_t st);
+int sum_parts(const double* part, int parts, int64_t count, float* out, cudaStream_t st);
+
 // One fp32 problem of the register-tiled kernel.
 struct GemmDesc {
   const float* A; const float* B; void* C;

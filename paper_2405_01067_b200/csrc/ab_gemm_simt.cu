@@ -289,6 +289,102 @@ __device__ __forceinline__ void gemm_tile_8x8(const GemmDesc& d) {
   }
 }
 
+// ---- the same sums, the reduction in parts ---------------------------------------------------------------------
+// 64 x 64 tiles, 4 x 4 values a thread, sums of 16 products in fp32 and those in fp64 as in gemm_simt_kernel, but the next slab is
+// fetched while one is multiplied, and parts of the reduction give every SM two CTAs.  Parts stay fp64 until they are added up, so
+// nothing is rounded that was not.  Bound by shared memory: two 16-byte reads to 16 multiply-adds.
+__global__ void __launch_bounds__(256, 2)
+gemm_parts_kernel(const float* __restrict__ A, int64_t sAm, int64_t sAk, const float* __restrict__ B, int64_t sBk, int64_t sBn,
+                  double* __restrict__ C, int M, int N, int K, int per, int upper) {
+  __shared__ __align__(16) float As[2][BK][BM + PAD], Bs[2][BK][BN + PAD];
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int tn = (N + BN - 1) / BN;
+  int bi = 0, bj = blockIdx.x;
+  if (upper) {                          // tile pairs bi <= bj, row after row
+    while (bj >= tn - bi) { bj -= tn - bi; ++bi; }
+    bj += bi;
+  } else {
+    bi = bj / tn;
+    bj -= bi * tn;
+  }
+  const int m0 = BM * bi, n0 = BN * bj, k0 = (int)blockIdx.y * per, k1 = min(K, k0 + per);
+  // consecutive threads walk the direction that is contiguous in memory
+  const bool a_kfast = sAk == 1, b_nfast = sBn == 1;
+  const int a_k = a_kfast ? tid % BK : tid / BM, a_m = a_kfast ? tid / BK : tid % BM;
+  const int b_k = b_nfast ? tid / BN : tid % BK, b_n = b_nfast ? tid % BN : tid / BK;
+  const int a_dk = a_kfast ? 0 : 256 / BM, a_dm = a_kfast ? 256 / BK : 0, b_dk = b_nfast ? 256 / BN : 0, b_dn = b_nfast ? 0 : 256 / BK;
+  float va[4], vb[4];
+  auto fetch = [&](int k) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int am = m0 + a_m + e * a_dm, ak = k + a_k + e * a_dk, bn = n0 + b_n + e * b_dn, bk = k + b_k + e * b_dk;
+      va[e] = am < M && ak < k1 ? A[am * sAm + ak * sAk] : 0.f;
+      vb[e] = bn < N && bk < k1 ? B[bk * sBk + bn * sBn] : 0.f;
+    }
+  };
+  auto stash = [&](int buf) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      As[buf][a_k + e * a_dk][a_m + e * a_dm] = va[e];
+      Bs[buf][b_k + e * b_dk][b_n + e * b_dn] = vb[e];
+    }
+  };
+  double acc[4][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
+  fetch(k0);
+  stash(0);
+  __syncthreads();
+  int cur = 0;
+  for (int k = k0; k < k1; k += BK, cur ^= 1) {
+    const bool more = k + BK < k1;
+    if (more) fetch(k + BK);
+    float part[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) part[i][j] = 0.f;
+#pragma unroll
+    for (int kk = 0; kk < BK; ++kk) {
+      const float4 a = *reinterpret_cast<const float4*>(&As[cur][kk][ty * 4]);
+      const float4 b = *reinterpret_cast<const float4*>(&Bs[cur][kk][tx * 4]);
+      const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) part[i][j] = fmaf(av[i], bv[j], part[i][j]);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[i][j] += (double)part[i][j];
+    if (more) stash(cur ^ 1);
+    __syncthreads();
+  }
+  C += (size_t)blockIdx.y * M * N;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int gm = m0 + ty * 4 + i;
+    if (gm >= M) continue;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int gn = n0 + tx * 4 + j;
+      if (gn < N) C[(size_t)gm * N + gn] = acc[i][j];
+    }
+  }
+}
+__global__ void __launch_bounds__(256)
+sum_parts_kernel(const double* __restrict__ part, int parts, int64_t count, float* __restrict__ out) {
+  const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  if (i >= count) return;
+  double acc = 0.0;
+#pragma unroll 4
+  for (int q = 0; q < parts; ++q) acc += part[q * count + i];
+  out[i] = (float)acc;
+}
+
 // The descriptor travels as a kernel argument.
 template <int BM_, int BN_>
 __global__ void __launch_bounds__((BM_ / 8) * (BN_ / 8), 512 / ((BM_ / 8) * (BN_ / 8)))
@@ -306,6 +402,20 @@ int launch_one(const GemmDesc& d, cudaStream_t st) {
 }
 
 }  // namespace
+
+int gemm_parts(const float* A, int64_t sAm, int64_t sAk, const float* B, int64_t sBk, int64_t sBn, double* parts, int M, int N, int K, int per,
+               bool upper, cudaStream_t st) {
+  const int tm = (M + BM - 1) / BM, tn = (N + BN - 1) / BN;
+  const dim3 grid((unsigned)(upper ? tn * (tn + 1) / 2 : tm * tn), (unsigned)((K + per - 1) / per));
+  gemm_parts_kernel<<<grid, 256, 0, st>>>(A, sAm, sAk, B, sBk, sBn, parts, M, N, K, per, upper ? 1 : 0);
+  AB_LAUNCH_OK();
+  return AB_OK;
+}
+int sum_parts(const double* part, int parts, int64_t count, float* out, cudaStream_t st) {
+  sum_parts_kernel<<<(unsigned)((count + 255) / 256), 256, 0, st>>>(part, parts, count, out);
+  AB_LAUNCH_OK();
+  return AB_OK;
+}
 
 int recombine_mean_simt(const float* A_copies, int64_t strideA, const float* B_copies, int64_t strideB, int K,
                         float* W, float* Abar, float* Bbar, int m, int n, int r, cudaStream_t st) {

@@ -620,13 +620,12 @@ __global__ void force_fallback_kernel(int* __restrict__ flags, int count, int* _
 // long factor: F(t,k) = Ylong(k,t) / sqrt(sigma_k); short factor: F(k,u) = sqrt(sigma_k) Vr[k][u].
 // Columns/rows k >= r' (and k >= r_cap) are written as zero.  tall: the long factor is A (L x r_max), the short one B (r_max x s);
 // else the long one is B (r_max x L), the short one A (s x r_max).  A warp a row of the results.
-// solver: null, or what the direct solver's waits reported for the call this matrix was part of; tc: the same of its two products
+// solver: null, or what the direct solver's waits reported for the call this matrix was part of
 template <typename TO>
 __global__ void __launch_bounds__(256)
 write_factors_kernel(const float* __restrict__ Y, const float* __restrict__ Vr, const float* __restrict__ sigma, int tall, int L, int s,
                      int r_cap, int r_max, float cutoff, TO* __restrict__ Flong, TO* __restrict__ Fshort, int* __restrict__ r_out,
-                     const JState* __restrict__ st, const int* __restrict__ solver, const int* __restrict__ tc,
-                     int* __restrict__ dev_status) {
+                     const JState* __restrict__ st, const int* __restrict__ solver, int* __restrict__ dev_status) {
   tc::dep_wait();
   tc::dep_launch();
   bool outside;
@@ -634,7 +633,7 @@ write_factors_kernel(const float* __restrict__ Y, const float* __restrict__ Vr, 
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     *r_out = rk;
     if (dev_status) {
-      const int code = tc[0] != AB_OK ? tc[0] : tc[1] != AB_OK ? tc[1] : solver && *solver != AB_OK ? *solver : st->status;
+      const int code = solver && *solver != AB_OK ? *solver : st->status;
       *dev_status = code == AB_OK && outside ? (int)AB_ERR_ACCURACY : code;
     }
   }
@@ -668,7 +667,7 @@ write_factors_kernel(const float* __restrict__ Y, const float* __restrict__ Vr, 
 // X = the sum of `parts` partial Gram matrices of which the upper triangle counts, added in fp64 in ascending order, and its mirror
 // image.  A block a pair of 32 x 32 tiles.
 __global__ void __launch_bounds__(256)
-sum_gram_kernel(const float* __restrict__ part, int parts, float* __restrict__ X, int s) {
+sum_gram_kernel(const double* __restrict__ part, int parts, float* __restrict__ X, int s) {
   __shared__ float t[32][33];
   tc::dep_wait();
   tc::dep_launch();
@@ -681,8 +680,8 @@ sum_gram_kernel(const float* __restrict__ part, int parts, float* __restrict__ X
     const int row = 32 * bi + ty + 8 * h;
     double acc = 0.0;
     if (row < s && col < s && row <= col) {
-#pragma unroll 6
-      for (int q = 0; q < parts; ++q) acc += (double)part[q * stride + (size_t)row * s + col];
+#pragma unroll 3
+      for (int q = 0; q < parts; ++q) acc += part[q * stride + (size_t)row * s + col];
       X[(size_t)row * s + col] = (float)acc;
     }
     t[ty + 8 * h][tx] = (float)acc;
@@ -726,7 +725,6 @@ struct Layout {
   std::map<int, double*> eig;                 // direct solver: its scratch, EigJobs, fallback flags (and behind the flags of a
   std::map<int, int*> flags;                  //   group two words on which the blocks of the fallback meet and the solver's status)
   std::map<int, EigJob*> ejobs;
-  int* tc;                                    // two words a matrix: what the waits of its Gram and its long product reported
   std::vector<ItemWs> item;
   size_t bytes;
 };
@@ -753,7 +751,6 @@ Layout make_layout(const SvdItem* items, int L, void* ws) {
       lo.eig[g.first] = ar.take_n<double>(std::min(cnt, (size_t)eig_chunk(g.first)) * eig_ws_doubles(g.first));
     }
   }
-  lo.tc = ar.take_n<int>(2 * (size_t)L);
   lo.item.resize(L);
   for (int i = 0; i < L; ++i) {
     Plan p = make_plan(items[i]);
@@ -836,39 +833,41 @@ int run_jacobi_fallback(float* X, float* Vt, JState* st, int* flags, int s, int 
   return AB_OK;
 }
 
-// The Gram matrix and the long product of an fp32 matrix go to the tensor cores as six bf16 terms (ab_gemm_split.cu) where their work
-// pays for three launches in place of one, or for a tile of 128.  Splits of one matrix, us, fp32 pipes / tensor cores.  Gram: 3072 x 256
-// 488 / 484, 800 x 256 461 / 468, 128 x 1000 265 / 281.  Long product: 3072 x 256 at rank 16 486 / 486, 32 488 / 484, 96 499 / 489;
-// 3072 x 128 at rank 64 301 / 298.
-constexpr int kGramParts = 6;             // the scratch of the solver, not yet in use, holds as many partial sums
-bool gram_on_tensor_cores(const SvdItem& it, const Plan& p) {
-  return it.w_dt == AB_F32 && p.s >= 192 && p.s <= eig_max() && (int64_t)p.s * p.s * p.L >= 100000000 && gemm_tc_available();
+// Gram matrix and long product of a large fp32 matrix: the reduction in parts that together fill the device (gemm_parts); the scratch of
+// the solver, in use only between the two, holds kParts s x s partial results in fp64.  On the tensor cores as six bf16 terms
+// the two are faster still, but their sums are cut off, not rounded: sigma was off by 7e-7 of itself instead of 5e-8.
+constexpr int kParts = 3;
+#ifndef PW
+#define PW 300000000
+#endif
+constexpr int64_t kPartsWork = PW;
+bool in_parts(const SvdItem& it, const Plan& p, int64_t rows, int64_t cols, int64_t len) {
+  return it.w_dt == AB_F32 && p.s <= eig_max() && rows * cols * len >= kPartsWork;
 }
-bool long_on_tensor_cores(const SvdItem& it, const Plan& p) {
-  return it.w_dt == AB_F32 && p.s >= 128 && (int64_t)p.s * p.L * p.r_cap >= 20000000 && gemm_tc_available();
+int part_len(int64_t tiles, int len, int most) {
+  const int want = (int)std::max<int64_t>(1, std::min<int64_t>(most, (2LL * std::max(sm_count(), 1) + tiles / 2) / tiles));
+  return ((len + want - 1) / want + 15) / 16 * 16;
 }
-SplitGemm split_product(const void* A, int64_t lda, int a_mn, const void* B, int64_t ldb, int b_mn, float* C, int64_t ldc, int M, int N, int K) {
-  SplitGemm g = {};
-  g.A = A; g.lda = lda; g.a_mn = a_mn; g.B = B; g.ldb = ldb; g.b_mn = b_mn; g.C = C; g.ldc = ldc; g.M = M; g.N = N; g.K = K;
-  return g;
-}
-// G = W^T W (tall) or W W^T; parts: kGramParts s x s partial results; scratch: room for as many SplitGemm and 16 bytes
-int gram_split(const SvdItem& it, const Plan& p, float* G, float* parts, void* scratch, int* status, cudaStream_t st) {
-  SplitGemm* table = reinterpret_cast<SplitGemm*>(align_up(reinterpret_cast<uintptr_t>(scratch), 16));      // s * s floats after an odd s * s
+// G = W^T W (tall) or W W^T
+int gram_parts(const SvdItem& it, const Plan& p, float* G, double* parts, cudaStream_t st) {
   const float* W = static_cast<const float*>(it.W);
-  const int s = p.s, per = ((p.L + kGramParts - 1) / kGramParts + 63) / 64 * 64, n = (p.L + per - 1) / per;
-  SplitGemm g[kGramParts];
-  for (int q = 0; q < n; ++q) {
-    const int k0 = q * per, len = std::min(p.L - k0, per);
-    const float* src = p.tall ? W + (size_t)k0 * it.n : W + k0;
-    g[q] = split_product(src, it.n, p.tall, src, it.n, p.tall, parts + (size_t)q * s * s, s, s, s, len);
-    g[q].upper_only = 1;
-  }
-  const SplitBatch b = gemm_split_plan(g, n);
-  AB_TRY(upload_async(table, g, n * sizeof(SplitGemm), st));
-  AB_TRY(gemm_split_batched(table, b, status, st));
-  const unsigned t = (unsigned)(s + 31) / 32;
-  return launch_after(sum_gram_kernel, dim3(t, t), 256, 0, 1, st, (const float*)parts, n, G, s);
+  const int64_t t = (p.s + 63) / 64, sr = p.tall ? 1 : it.n, sk = p.tall ? it.n : 1;
+  const int per = part_len(t * (t + 1) / 2, p.L, kParts), n = (p.L + per - 1) / per;
+  AB_TRY(gemm_parts(W, sr, sk, W, sk, sr, parts, p.s, p.s, p.L, per, true, st));
+  const unsigned t32 = (unsigned)(p.s + 31) / 32;
+  sum_gram_kernel<<<dim3(t32, t32), 256, 0, st>>>(parts, n, G, p.s);
+  AB_LAUNCH_OK();
+  return AB_OK;
+}
+// Y (L x r_cap) = W Vr^T (tall) or Y (r_cap x L) = Vr W
+int long_parts(const SvdItem& it, const Plan& p, const float* Vr, float* Y, double* parts, cudaStream_t st) {
+  const float* W = static_cast<const float*>(it.W);
+  const int M = p.tall ? p.L : p.r_cap, N = p.tall ? p.r_cap : p.L;
+  const int64_t tiles = (int64_t)((M + 63) / 64) * ((N + 63) / 64), count = (int64_t)M * N;
+  const int per = part_len(tiles, p.s, (int)std::min<int64_t>(kParts, (int64_t)kParts * p.s * p.s / count)), n = (p.s + per - 1) / per;
+  if (p.tall) AB_TRY(gemm_parts(W, it.n, 1, Vr, 1, p.s, parts, M, N, p.s, per, false, st));
+  else AB_TRY(gemm_parts(Vr, p.s, 1, W, it.n, 1, parts, M, N, p.s, per, false, st));
+  return sum_parts(parts, n, count, Y, st);
 }
 
 // Whether a group of `count` matrices of short side s goes to the direct solver (its fallback has to fit as well).
@@ -884,7 +883,6 @@ int svd_batch(const SvdItem* items, int L, float sigma_cutoff, void* ws, size_t 
               const SvdSelftest* selftest) {
   Layout lo = make_layout(items, L, ws);
   if (lo.bytes > ws_bytes) return AB_ERR_WORKSPACE;
-  AB_CUDA_OK(cudaMemsetAsync(lo.tc, 0, sizeof(int) * 2 * L, stream));
   // 1. Gram matrices into X
   for (auto& g : lo.groups) {
     const int s = g.first;
@@ -892,9 +890,7 @@ int svd_batch(const SvdItem* items, int L, float sigma_cutoff, void* ws, size_t 
       const SvdItem& it = items[g.second[j]];
       float* G = lo.X[s] + j * (size_t)s * s;
       const Plan p = make_plan(it);
-      if (gram_on_tensor_cores(it, p))
-        AB_TRY(gram_split(it, p, G, reinterpret_cast<float*>(lo.eig[s]), lo.Vt[s] + j * (size_t)s * s,
-                          lo.tc + 2 * g.second[j], stream));
+      if (in_parts(it, p, s, s, p.L)) AB_TRY(gram_parts(it, p, G, lo.eig[s], stream));
       else if (it.m >= it.n)   // G = W^T W
         AB_TRY(gemm_simt(it.W, it.w_dt, 1, it.n, it.W, it.w_dt, it.n, 1, G, AB_F32, s, s, s, it.m, stream));
       else                // G = W W^T
@@ -973,14 +969,13 @@ int svd_batch(const SvdItem* items, int L, float sigma_cutoff, void* ws, size_t 
         AB_LAUNCH_OK();
       }
       int64_t yt, yk;   // Ylong(k,t) = Y[t*yt + k*yk]
-      const bool tc = long_on_tensor_cores(it, p);
+      const bool parts = in_parts(it, p, p.r_cap, p.s, p.L) && (int64_t)p.r_cap * p.L <= (int64_t)kParts * s * s;      // one part at least
+      if (parts) AB_TRY(long_parts(it, p, w.Vr, w.Y, lo.eig[s], stream));
       if (p.tall) {     // Y (m x r_cap) = W Vr^T
-        if (tc) AB_TRY(gemm_split_one(split_product(it.W, it.n, 0, w.Vr, s, 0, w.Y, p.r_cap, it.m, p.r_cap, s), false, lo.tc + 2 * i + 1, stream));
-        else AB_TRY(gemm_simt(it.W, it.w_dt, it.n, 1, w.Vr, AB_F32, 1, s, w.Y, AB_F32, p.r_cap, it.m, p.r_cap, it.n, stream));
+        if (!parts) AB_TRY(gemm_simt(it.W, it.w_dt, it.n, 1, w.Vr, AB_F32, 1, s, w.Y, AB_F32, p.r_cap, it.m, p.r_cap, it.n, stream));
         yt = p.r_cap; yk = 1;
       } else {          // Y (r_cap x n) = Vr W
-        if (tc) AB_TRY(gemm_split_one(split_product(w.Vr, s, 0, it.W, it.n, 1, w.Y, it.n, p.r_cap, it.n, s), false, lo.tc + 2 * i + 1, stream));
-        else AB_TRY(gemm_simt(w.Vr, AB_F32, s, 1, it.W, it.w_dt, it.n, 1, w.Y, AB_F32, it.n, p.r_cap, it.n, it.m, stream));
+        if (!parts) AB_TRY(gemm_simt(w.Vr, AB_F32, s, 1, it.W, it.w_dt, it.n, 1, w.Y, AB_F32, it.n, p.r_cap, it.n, it.m, stream));
         yt = 1; yk = it.n;
       }
       if (p.tall) {
@@ -998,11 +993,11 @@ int svd_batch(const SvdItem* items, int L, float sigma_cutoff, void* ws, size_t 
       if (it.out_dt == AB_F32)
         AB_TRY(launch_after(write_factors_kernel<float>, dim3(grid), 256, 0, 1, stream, (const float*)w.Y, (const float*)w.Vr, (const float*)it.sigma,
                             (int)p.tall, p.L, p.s, p.r_cap, it.r_max, sigma_cutoff, (float*)Fl, (float*)Fs, it.r_out, (const JState*)(lo.st[s] + j),
-                            solver, (const int*)(lo.tc + 2 * i), it.dev_status));
+                            solver, it.dev_status));
       else
         AB_TRY(launch_after(write_factors_kernel<bf16>, dim3(grid), 256, 0, 1, stream, (const float*)w.Y, (const float*)w.Vr, (const float*)it.sigma,
                             (int)p.tall, p.L, p.s, p.r_cap, it.r_max, sigma_cutoff, (bf16*)Fl, (bf16*)Fs, it.r_out, (const JState*)(lo.st[s] + j),
-                            solver, (const int*)(lo.tc + 2 * i), it.dev_status));
+                            solver, it.dev_status));
     }
   }
   return AB_OK;
