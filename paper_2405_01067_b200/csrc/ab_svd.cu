@@ -836,11 +836,11 @@ int run_jacobi_fallback(float* X, float* Vt, JState* st, int* flags, int s, int 
 // Gram matrix and long product of a large fp32 matrix: the reduction in parts that together fill the device (gemm_parts); the scratch of
 // the solver, in use only between the two, holds kParts s x s partial results in fp64.  On the tensor cores as six bf16 terms
 // the two are faster still, but their sums are cut off, not rounded: sigma was off by 7e-7 of itself instead of 5e-8.
+// Lines by the products to form: below, parts leave each CTA too few slabs and their sum is a launch more.  Split of 2304 x 256 at rank
+// 128 (1.5e8 products in the Gram matrix) as before / in parts 513 / 546 us, 3072 x 320 at rank 80 (3.1e8) 828 / 851, 2048 x 400
+// (3.3e8) 1116 / 1100, 3072 x 400 (4.9e8) 1203 / 1121, 3072 x 768 at rank 384 2308 / 2246, 768 x 3072 at rank 192 2206 / 2124.
 constexpr int kParts = 3;
-#ifndef PW
-#define PW 300000000
-#endif
-constexpr int64_t kPartsWork = PW;
+constexpr int64_t kPartsWork = 400000000;
 bool in_parts(const SvdItem& it, const Plan& p, int64_t rows, int64_t cols, int64_t len) {
   return it.w_dt == AB_F32 && p.s <= eig_max() && rows * cols * len >= kPartsWork;
 }

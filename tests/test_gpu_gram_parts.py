@@ -1,8 +1,9 @@
-"""Gram matrix of a dense split in parts of the long side on the tensor cores: odd short sides (tables and partial sums behind an odd
+"""Gram matrix and long product of a dense split with the reduction in parts: odd short sides (tables and partial sums behind an odd
 number of floats), long sides that leave a short last part or fill none, either side long.
 
-Tolerance: the six bf16 terms carry 24 bits and the parts are added in fp64, so sigma is as good as from an fp32 Gram matrix:
-2^-24 sqrt(s) sigma_1^2 / sigma, below 1e-4 for the values above 0.2 sigma_1 that are compared; the residual as in test_gpu_eig.py.
+Tolerance: 16 products at a time are summed in fp32 and those sums in fp64, one rounding to fp32 at the end, so sigma is as good
+as an fp32 Gram matrix lets it be: 2^-24 sqrt(s) sigma_1^2 / sigma, below 1e-4 for the values above 0.2 sigma_1 that are compared; the
+residual as in test_gpu_eig.py.
 """
 import numpy as np
 import pytest
