@@ -35,11 +35,14 @@ constexpr int kRegsConv = 152, kRegsEpi = 120, kRegsMma = 80;
 static_assert(2 * kRegsConv + kRegsEpi + kRegsMma <= 512, "");
 constexpr int kRing = 4;                 // tile records on their way to the other warps
 
+// Bytes of a piece of an operand tile: where the index of the rows is contiguous, its lines are 64 values long, also of 32 rows.
+constexpr int piece_bytes(int rows) { return (rows < 64 ? 64 : rows) * 128; }
+
 template <int BN, bool kBf16>
 struct Cfg {
   static constexpr int kPieces = kBf16 ? 1 : 3;
   static constexpr int kStages = kBf16 ? 4 : 2;
-  static constexpr int kABytes = kM * 128, kBBytes = BN * 128;
+  static constexpr int kABytes = piece_bytes(kM), kBBytes = piece_bytes(BN);
   static constexpr int kStage = kPieces * (kABytes + kBBytes);
   static constexpr size_t kSmem = (size_t)kStages * kStage + 4 * 4096 + 1024 + 2048;
 };
@@ -185,7 +188,7 @@ struct OperandCursor {
 // into the 128-byte-swizzled tile(s): lines of 128 bytes (64 values); piece p at dst + p * kPieceBytes
 template <int kRows, bool kBf16>
 __device__ __forceinline__ void store_slab(const OperandSlab<kRows, kBf16>& s, uint8_t* dst, uint32_t estep) {
-  constexpr int kPieceBytes = kRows * 128;
+  constexpr int kPieceBytes = piece_bytes(kRows);
 #pragma unroll
   for (int e = 0; e < OperandSlab<kRows, kBf16>::kF; ++e) {
     uint8_t* b = dst + e * estep;
@@ -518,12 +521,22 @@ int launch(void (*kernel)(KArgs...), size_t smem, int tiles, cudaStream_t st, Ar
 
 int tiles_of(const SplitGemm& p, int bn) { return ((p.M + kM - 1) / kM) * ((p.N + bn - 1) / bn); }
 
-// Tiles 128 or 64 columns wide, whichever takes less time: a wide one about one and a half times a narrow one (its A is converted
-// once instead of twice).  768 x 768: 36 or 72 tiles, one round of either: 64.  3072 x 768: 144 wide ones in one round, 288
+// Tiles of a batch, and of a problem too large for narrow_tiles: 128 or 64 columns wide, whichever takes less time: a wide one about one
+// and a half times a narrow one (its A is converted once instead of twice).  768 x 768: 36 or 72 tiles, one round of either: 64.  3072 x 768: 144 wide ones in one round, 288
 // narrow ones in two: 128 (10.4 us against 12.4 us).
 int tile_width(int tiles64, int tiles128) {
   const int sms = sm_count() > 0 ? sm_count() : 1;
   return 2 * ((tiles64 + sms - 1) / sms) >= 3 * ((tiles128 + sms - 1) / sms) ? 128 : 64;
+}
+
+// Up to how many tiles of 32 columns a lone problem takes them.  What a CTA converts and writes is a chain of latencies, so less of it
+// is faster as long as every tile has an SM, and the CTAs of the launch behind find room beside.  us a launch in a row of twelve, 64 wide
+// / 32 wide: 256 x 256, rank 64, fp32 4.9 / 4.4, bf16 3.4 / 3.2; 512 x 512, rank 192 7.5 / 6.8, 4.6 / 4.2; 1000 x 448 (112
+// tiles), rank 192 7.7 / 7.3, 4.8 / 4.6.  With nearly every SM taken the next launch waits outside, which a reduction of one slab
+// and the lighter bf16 conversion do not make up for: 768 x 768 (144 tiles), rank 64 5.4 / 5.6, 3.6 / 4.0, rank 192 7.7 / 7.6, 4.7 / 4.8.
+int narrow_tiles(bool src_bf16, int K) {
+  const int sms = sm_count();
+  return !src_bf16 && K > 64 ? sms : sms / 5 * 4;
 }
 
 }  // namespace
@@ -546,6 +559,11 @@ int gemm_split_batched(const SplitGemm* d_probs, const SplitBatch& b, int* statu
 }
 
 int gemm_split_one(SplitGemm p, bool src_bf16, int* status, cudaStream_t st) {
+  const int t32 = tiles_of(p, 32);
+  if (t32 <= narrow_tiles(src_bf16, p.K)) {
+    if (src_bf16) return launch(gemm_split_one_kernel<32, true>, Cfg<32, true>::kSmem, t32, st, p, t32, status);
+    return launch(gemm_split_one_kernel<32, false>, Cfg<32, false>::kSmem, t32, st, p, t32, status);
+  }
   const SplitBatch b = gemm_split_plan(&p, 1);
   if (src_bf16) {
     if (b.bn == 128) return launch(gemm_split_one_kernel<128, true>, Cfg<128, true>::kSmem, b.tiles, st, p, b.tiles, status);
