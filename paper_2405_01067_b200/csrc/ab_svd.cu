@@ -537,6 +537,8 @@ __global__ void __launch_bounds__(256)
 long_norms_kernel(const float* __restrict__ Y, int64_t st_, int L, int r_cap, float* __restrict__ sigma) {
   __shared__ double red[8][32];
   __shared__ double part[kNormCl][32];
+  auto cluster = cooperative_groups::this_cluster();
+  auto started = cluster.barrier_arrive();
   tc::dep_wait();
   tc::dep_launch();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, rank = blockIdx.x % kNormCl;
@@ -548,7 +550,7 @@ long_norms_kernel(const float* __restrict__ Y, int64_t st_, int L, int r_cap, fl
   }
   red[warp][lane] = acc;
   __syncthreads();
-  auto cluster = cooperative_groups::this_cluster();
+  cluster.barrier_wait(std::move(started));      // rank 0 runs: its shared memory may be written
   if (warp == 0) {
     acc = 0.0;
 #pragma unroll
