@@ -36,7 +36,6 @@ constexpr double kCloseRel = 1e-7;      // eigenvalues closer than this fraction
 constexpr double kOrthTol = 4e-6;       // what the Jacobi route leaves at small orders
 constexpr int kMaxOrder = 1280;         // masks are sized for this order
 constexpr double kLive2 = 1e-290;       // a column whose squared norm is below this needs no reflector
-constexpr double kCancel = 0x1p-10;     // a squared norm below this fraction of its terms is summed again from the entries
 constexpr int kGroup = 8;               // reflectors applied together in the back transform
 
 // Reflectors are rows of an even number of doubles (bulk copies of whole rows start and end on 16 bytes), zero before and
@@ -53,17 +52,6 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// Four sums across a warp, each exchange halving what a lane still carries: lanes 8 q ... hold sum q.
-__device__ __forceinline__ double warp_sum4(double s0, double s1, double s2, double s3, int lane) {
-  const bool h2 = (lane & 16) != 0, h1 = (lane & 8) != 0;
-  const double t0 = (h2 ? s2 : s0) + __shfl_xor_sync(0xffffffffu, h2 ? s0 : s2, 16);
-  const double t1 = (h2 ? s3 : s1) + __shfl_xor_sync(0xffffffffu, h2 ? s1 : s3, 16);
-  double t = (h1 ? t1 : t0) + __shfl_xor_sync(0xffffffffu, h1 ? t0 : t1, 8);
-  t += __shfl_xor_sync(0xffffffffu, t, 4);
-  t += __shfl_xor_sync(0xffffffffu, t, 2);
-  t += __shfl_xor_sync(0xffffffffu, t, 1);
-  return t;
-}
 __device__ __forceinline__ uint32_t map_rank(uint32_t addr, uint32_t rank) {
   uint32_t r;
   asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
@@ -81,13 +69,15 @@ __device__ __forceinline__ void st_async(uint32_t addr, double x, double y, uint
 // holds R whole rows, E elements of each per lane.  Step j:
 //   - warp 0 of each CTA has received p = A v of the reflector before (v, gamma) and column j of
 //     the matrix as it was before that reflector's update, a;  w = gamma p - c v, c = gamma^2 p.v / 2;  column j of the updated
-//     matrix is (a - x p) + y v with x = v1 gamma, y = 2 c v1 - gamma p_j, where v1 is the first element of v.  Only y waits for a
-//     sum, and the squared norm of the column follows from sums over b = a - x p:  b.b + 2 y b.v + y^2 v.v.  So one reduction of four sums
-//     gives all that a step needs (it took two, one after the other).  Where the terms cancel to less than kCancel of their size
-//     (1 to 2 % of the steps of a decaying spectrum) the entries are summed themselves.  w and the next reflector v' go to the other warps;
-//   - all warps pass over their rows in registers: A -= v w^T + w v^T, p' = A v' without the first element of v', which the
-//     square root of warp 0 gives meanwhile;  every row's p'_i and A[i][j+1] go to warp 0 of every CTA of the cluster, which adds
-//     the first element's products A[i][j+1] v1' to p'.
+//     matrix is (a - x p) + y v with x = v1 gamma, y = 2 c v1 - gamma p_j, where v1 is the first element of v, and only y waits for a
+//     sum.  w and the next reflector v' go to the other warps;
+//   - all warps pass over their rows in registers: A -= v w^T + w v^T, p' = A v' without the first element of v';  every row's p'_i
+//     and A[i][j+1] go to warp 0 of every CTA of the cluster;
+//   - while they travel, warp 0 sums the squares of the column and takes their root, which gives the first element of v';  it adds that
+//     element's products A[i][j+1] v1' to the p' that it receives.
+// The squares are those of the column's own entries.  Sums over b = a - x p, known a reduction earlier (b.b + 2 y b.v + y^2 v.v), cancel:
+// reflectors were then orthogonal to 1e-13 in place of 7e-16.  With the root in front of warp 0's pass a split of 256 x 2304 took 515 us
+// against 503.
 // So the rank-two update and the product with the next vector touch an element once, and a step is a chain of one
 // warp reduction, the pass and one exchange.  The vectors are worked out by one warp because fp64 issues
 // at half rate: with every warp doing it for itself (no hand-over) the copies took more issue slots than the pass (8100 cycles a step
@@ -126,33 +116,26 @@ struct Tridiag {
   struct Rows { double A[R][E]; double v[E]; double gam, v1; bool ok; uint32_t dst, dbar; };
 
   // Warp 0, step j: from p and the column to w and the next reflector but its first element (left in shared memory).  Returns
-  // through vn, dj, alpha, sq what is to be stored and what the first element and gamma follow from.
+  // through vn, dj, alpha what is to be stored and what the first element and gamma follow from.
   template <int E0>
-  __device__ __forceinline__ void vec_step(Rows& x, int j, double (&vn)[E], double& dj, double& alpha, double& sq) {
+  __device__ __forceinline__ void vec_step(Rows& x, int j, double (&vn)[E], double& dj, double& alpha) {
     const int par = j & 1;
     if constexpr (kSingle) tc::named_bar_sync(2, kThreads);
     else x.ok = x.ok && tc::mbar_wait(&sh.bar[par], (j >> 1) & 1);
     const double2* pb = sh.pa[par];
     const double xg = x.v1 * x.gam;
-    double p[E], pv = 0.0, bb = 0.0, bv = 0.0, vv = 0.0;
+    double p[E], pv = 0.0;
 #pragma unroll
     for (int e = E0; e < E; ++e) {
       const double2 q = pb[lane + 32 * e];
-      const bool ahead = e > E0 + 1 || lane + 32 * e > j + 1;
       p[e] = fma(q.y, x.v1, q.x);
-      vn[e] = ahead ? fma(-xg, p[e], q.y) : 0.0;
-      const double vm = ahead ? x.v[e] : 0.0;
+      vn[e] = fma(-xg, p[e], q.y);
       pv = fma(p[e], x.v[e], pv);
-      bb = fma(vn[e], vn[e], bb);
-      bv = fma(vn[e], vm, bv);
-      vv = fma(vm, vm, vv);
     }
     const int j1 = j + 1 < s ? j + 1 : j;
     const double2 qj = pb[j], qj1 = pb[j1];
     const double vj1 = sh.v[par][j1], pj = fma(qj.y, x.v1, qj.x), pj1 = fma(qj1.y, x.v1, qj1.x);
-    const double t4 = warp_sum4(pv, bb, bv, vv, lane);
-    pv = __shfl_sync(0xffffffffu, t4, 0); bb = __shfl_sync(0xffffffffu, t4, 8);
-    bv = __shfl_sync(0xffffffffu, t4, 16); vv = __shfl_sync(0xffffffffu, t4, 24);
+    pv = warp_sum(pv);
     const double c = 0.5 * x.gam * (x.gam * pv);    // gamma alone may be as large as 1e290
     const double y = 2.0 * c * x.v1 - x.gam * pj, wj = x.gam * pj - c * x.v1;
 #pragma unroll
@@ -162,15 +145,8 @@ struct Tridiag {
       vn[e] = ahead ? fma(y, x.v[e], vn[e]) : 0.0;
       sh.v[par ^ 1][lane + 32 * e] = vn[e];
     }
-    sq = bb + y * (2.0 * bv + y * vv);
     dj = qj.y - 2.0 * x.v1 * wj;
     alpha = (j + 1 < s) ? fma(y, vj1, fma(-xg, pj1, qj1.y)) : 0.0;
-    if (!(sq >= kCancel * (bb + y * y * vv))) {
-      sq = 0.0;
-#pragma unroll
-      for (int e = E0; e < E; ++e) sq = fma(vn[e], vn[e], sq);
-      sq = warp_sum(sq);
-    }
     if constexpr (!kSingle) {
       if (lane == 0 && !x.ok) sh.dead = 1;                 // a peer never answered: all warps leave
       if (x.ok && j + 1 < s) open_step(par ^ 1, s - 1 - j);
@@ -198,19 +174,10 @@ struct Tridiag {
     const int jend = min(32 * E0 + 32, s);
     for (int j = 32 * E0; j < jend; ++j) {
       const int par = j & 1;
-      double w[E], vn[E], dj = 0.0, alpha = 0.0, sq = 0.0, beta = 0.0, den = 0.0;
-      if (warp == 0) vec_step<E0>(x, j, vn, dj, alpha, sq);
+      double w[E], vn[E], dj = 0.0, alpha = 0.0, beta = 0.0, den = 0.0;
+      if (warp == 0) vec_step<E0>(x, j, vn, dj, alpha);
       tc::named_bar_sync(1, kThreads);               // w and v' are there
-      if (warp == 0) {
-        const bool live = sq > kLive2;
-        const double nrm = sqrt(fma(alpha, alpha, sq));
-        beta = live ? (alpha > 0.0 ? -nrm : nrm) : alpha;
-        x.v1 = live ? alpha - beta : 0.0;
-        den = live ? nrm * (nrm + fabs(alpha)) : 0.0;
-        if (lane == 0) sh.first[par ^ 1] = x.v1;     // for the other warps' next pass
-      } else if (lane == (j & 31)) {
-        x.v[E0] = sh.first[par];                     // v of the step before was without its first element, j
-      }
+      if (warp != 0 && lane == (j & 31)) x.v[E0] = sh.first[par];      // v of the step before was without its first element, j
       if constexpr (!kSingle) {
         if (*reinterpret_cast<volatile int*>(&sh.dead)) return;
       }
@@ -256,7 +223,17 @@ struct Tridiag {
         }
       }
       if constexpr (kSingle) { if (warp != 0) bar_arrive(2, kThreads); }
-      if (warp == 0) {                               // off the chain: gamma, and what later kernels need
+      if (warp == 0) {                               // beside the exchange: the first element, gamma, and what later kernels need
+        double sq = 0.0;
+#pragma unroll
+        for (int e = E0; e < E; ++e) sq = fma(vn[e], vn[e], sq);
+        sq = warp_sum(sq);
+        const bool live = sq > kLive2;
+        const double nrm = sqrt(fma(alpha, alpha, sq));
+        beta = live ? (alpha > 0.0 ? -nrm : nrm) : alpha;
+        x.v1 = live ? alpha - beta : 0.0;
+        den = live ? nrm * (nrm + fabs(alpha)) : 0.0;
+        if (lane == 0) sh.first[par ^ 1] = x.v1;     // for the other warps' next pass
         x.gam = den > 0.0 ? 1.0 / den : 0.0;
 #pragma unroll
         for (int e = E0; e < E; ++e)
@@ -428,19 +405,15 @@ __device__ __forceinline__ double sum_warps(const double* red) {
 }
 
 // A step.  With x = v1 gamma and y = 2 c v1 - gamma p_j (c = gamma^2 p.v / 2) column j + 1 of the updated matrix is
-// (a - x p) + y v, where only y waits for a sum; its squared norm follows from the sums over b = a - x p:
-// b.b + 2 y b.v + y^2 v.v.  So one reduction over the CTA gives all that a step needs (there were two).  Where the terms
-// cancel to less than kCancel of their size (1 to 2 % of the steps of a decaying spectrum) the entries are summed themselves.
-// The square root stands beside the pass over the rows: its result is needed for element j + 1 of the reflector alone, whose products
-// are added as the row sums leave.
-// Order 768, cycles a step: 4300, of them 2100 outside the exchange; 5100 and 3500 with three barriers, two reductions and the
-// root in the chain; 6000 with all CTAs polling.  2.25 ms -> 1.55.
+// (a - x p) + y v, where only y waits for a sum.  The sum of its squares and their root stand beside the pass over the rows (the
+// CTA's warps meet between its halves): what follows from them is needed for element j + 1 of the reflector alone, whose products are
+// added as the row sums leave.
 template <int E, int W>
 __global__ void __launch_bounds__(32 * W, 1)
 tridiag_grid_kernel(const EigJob* __restrict__ jobs, int count, int C, int* status) {
   constexpr int R = kGridRows, T = 32 * W, S = T * E;
   extern __shared__ __align__(16) double2 pairs[];                        // [2][S + kMaxCl]: the pairs of a step, behind them the mates' tokens
-  __shared__ __align__(16) double red[4][W], red_row[R][W], vrow[R];      // vrow: v of this CTA's rows
+  __shared__ __align__(16) double red_pv[W], red_sq[W], red_row[R][W], vrow[R];      // vrow: v of this CTA's rows
   __shared__ double colbuf[R], vnext;                                     // column j + 1 of the rows; v_j+1
   __shared__ uint64_t bar[2];
   __shared__ int dead;
@@ -520,53 +493,40 @@ tridiag_grid_kernel(const EigJob* __restrict__ jobs, int count, int C, int* stat
       const double vj1 = vnext;
       ok = tc::mbar_wait(&bar[buf], (uses >> 1) & 1) && ok;
       if (!ok) *reinterpret_cast<volatile int*>(&dead) = 1;
-      double p[E], vn[E], pv = 0.0, bb = 0.0, bv = 0.0, vv = 0.0;
+      double p[E], vn[E], pv = 0.0;
 #pragma unroll
       for (int e = 0; e < E; ++e) {
         const int k = tid + T * e;
         const double2 q = pb[k];
         p[e] = k >= j ? q.x : 0.0;                       // what is before j is of an earlier step
-        vn[e] = k > j + 1 ? fma(-x, q.x, q.y) : 0.0;
-        const double vm = k > j + 1 ? v[e] : 0.0;
+        vn[e] = fma(-x, q.x, q.y);
         pv = fma(p[e], v[e], pv);
-        bb = fma(vn[e], vn[e], bb);
-        bv = fma(vn[e], vm, bv);
-        vv = fma(vm, vm, vv);
       }
       const double2 qj = pb[j], qj1 = pb[j + 1];
 #pragma unroll
       for (int r = 0; r < R; ++r) pr[r] = pb[min(cta + C * r, S - 1)].x;
-      const double t4 = warp_sum4(pv, bb, bv, vv, lane);
-      if ((lane & 7) == 0) red[lane >> 3][warp] = t4;
+      pv = warp_sum(pv);
+      if (lane == 0) red_pv[warp] = pv;
       __syncthreads();
       if (*reinterpret_cast<volatile int*>(&dead)) break;      // the same for all threads: a peer never answered
       if (tid < CL && j + 1 < last) {
         const uint32_t m = map_rank(pairs_at, tid);
         st_async(m + (uint32_t)((buf ^ 1) * (S + kMaxCl) + S + rank) * 16, 0.0, 0.0, m + bar_off + (buf ^ 1) * 8);
       }
-      pv = sum_warps<W>(red[0]); bb = sum_warps<W>(red[1]); bv = sum_warps<W>(red[2]); vv = sum_warps<W>(red[3]);
+      pv = sum_warps<W>(red_pv);
       const double c = 0.5 * gam * (gam * pv);           // gamma alone may be as large as 1e290
       const double y = 2.0 * c * v1 - gam * qj.x, wj = gam * qj.x - c * v1;
-      double sq = bb + y * (2.0 * bv + y * vv);
-      double w[E];
+      double w[E], sq = 0.0;
 #pragma unroll
       for (int e = 0; e < E; ++e) {
         const int k = tid + T * e;
         w[e] = fma(gam, p[e], -(c * v[e]));
         vn[e] = k > j + 1 ? fma(y, v[e], vn[e]) : 0.0;
-      }
-      if (!(sq >= kCancel * (bb + y * y * vv))) {        // the same in all CTAs: they work on the same bits
-        __syncthreads();                                 // red has been read
-        sq = 0.0;
-#pragma unroll
-        for (int e = 0; e < E; ++e) sq = fma(vn[e], vn[e], sq);
-        sq = warp_sum(sq);
-        if (lane == 0) red[0][warp] = sq;
-        __syncthreads();
-        sq = sum_warps<W>(red[0]);
+        sq = fma(vn[e], vn[e], sq);
       }
       const double dj = qj.y - 2.0 * v1 * wj, alpha = fma(y, vj1, fma(-x, qj1.x, qj1.y));
-      const bool live = sq > kLive2;
+      sq = warp_sum(sq);
+      if (lane == 0) red_sq[warp] = sq;
       double ps[R];
 #pragma unroll
       for (int h = 0; h < R; h += 4) {
@@ -583,7 +543,10 @@ tridiag_grid_kernel(const EigJob* __restrict__ jobs, int count, int C, int* stat
             }
           }
         }
+        if (h == 0) __syncthreads();                     // the parts of the squares are there
       }
+      sq = sum_warps<W>(red_sq);                         // the same in all CTAs: they work on the same bits
+      const bool live = sq > kLive2;
       const double nrm = sqrt(fma(alpha, alpha, sq));
       const double beta = live ? (alpha > 0.0 ? -nrm : nrm) : alpha;
       v1 = live ? alpha - beta : 0.0;
