@@ -838,13 +838,27 @@ int run_jacobi_fallback(float* X, float* Vt, JState* st, int* flags, int s, int 
 // Gram matrix and long product of a large fp32 matrix: the reduction in parts that together fill the device (gemm_parts); the scratch of
 // the solver, in use only between the two, holds kParts s x s partial results in fp64.  On the tensor cores as six bf16 terms
 // the two are faster still, but their sums are cut off, not rounded: sigma was off by 7e-7 of itself instead of 5e-8.
-// Lines by the products to form: below, parts leave each CTA too few slabs and their sum is a launch more.  Split of 2304 x 256 at rank
-// 128 (1.5e8 products in the Gram matrix) as before / in parts 513 / 546 us, 3072 x 320 at rank 80 (3.1e8) 828 / 851, 2048 x 400
-// (3.3e8) 1116 / 1100, 3072 x 400 (4.9e8) 1203 / 1121, 3072 x 768 at rank 384 2308 / 2246, 768 x 3072 at rank 192 2206 / 2124.
+// Lower line, by the products to form: below, parts leave each CTA too few slabs and their sum is a launch more.  Split of 2304 x 256 at
+// rank 128 (1.5e8 products in the Gram matrix) by gemm_simt / in parts 513 / 546 us, 3072 x 320 at rank 80 (3.1e8) 828 / 851, 2048 x 400
+// (3.3e8) 1116 / 1100, 2600 x 400 (4.2e8) 1162 / 1139.
+// The Gram matrix also needs half as many CTAs as there are SMs: with three parts at most, fewer tiles leave the device idle however long
+// the reduction is, while gemm_simt's kernel for few tiles cuts it over clusters.  21 tiles (63 CTAs): 2800 x 384 962 / 992, 40000 x 384
+// 1811 / 2058; 10 tiles: 20000 x 256 750 / 1011; one: 100000 x 64 641 / 2648.  28 tiles (84 CTAs): 8000 x 448 1389 / 1277, 40000 x 448
+// 2697 / 2273; 55: 40000 x 640 4631 / 3464.
+// Long product, also against the 8 x 8 kernel that gemm_simt has from 296 tiles on: 3072 x 768 at rank 192 (144 tiles) 2292 / 2216, at 400
+// (336) 2425 / 2363, at 576 (432) 2399 / 2384; 4096 x 1024 at rank 320 3431 / 3285, at 512 3467 / 3435; 768 x 3072 at rank 480
+// 2404 / 2403.  There sigma is off by 3.3e-8 of the largest where that kernel's fp32 sums left 5.5e-8.
 constexpr int kParts = 3;
 constexpr int64_t kPartsWork = 400000000;
-bool in_parts(const SvdItem& it, const Plan& p, int64_t rows, int64_t cols, int64_t len) {
-  return it.w_dt == AB_F32 && p.s <= eig_max() && rows * cols * len >= kPartsWork;
+bool in_parts(const SvdItem& it, const Plan& p, int64_t rows, int64_t len) {
+  return it.w_dt == AB_F32 && p.s <= eig_max() && rows * p.s * len >= kPartsWork;
+}
+bool gram_in_parts(const SvdItem& it, const Plan& p) {
+  const int64_t t = (p.s + 63) / 64, ctas = kParts * (t * (t + 1) / 2);
+  return in_parts(it, p, p.s, p.L) && 2 * ctas >= sm_count();
+}
+bool long_in_parts(const SvdItem& it, const Plan& p) {      // room for one part at least
+  return in_parts(it, p, p.r_cap, p.L) && (int64_t)p.r_cap * p.L <= (int64_t)kParts * p.s * p.s;
 }
 int part_len(int64_t tiles, int len, int most) {
   const int want = (int)std::max<int64_t>(1, std::min<int64_t>(most, (2LL * std::max(sm_count(), 1) + tiles / 2) / tiles));
@@ -892,7 +906,7 @@ int svd_batch(const SvdItem* items, int L, float sigma_cutoff, void* ws, size_t 
       const SvdItem& it = items[g.second[j]];
       float* G = lo.X[s] + j * (size_t)s * s;
       const Plan p = make_plan(it);
-      if (in_parts(it, p, s, s, p.L)) AB_TRY(gram_parts(it, p, G, lo.eig[s], stream));
+      if (gram_in_parts(it, p)) AB_TRY(gram_parts(it, p, G, lo.eig[s], stream));
       else if (it.m >= it.n)   // G = W^T W
         AB_TRY(gemm_simt(it.W, it.w_dt, 1, it.n, it.W, it.w_dt, it.n, 1, G, AB_F32, s, s, s, it.m, stream));
       else                // G = W W^T
@@ -971,7 +985,7 @@ int svd_batch(const SvdItem* items, int L, float sigma_cutoff, void* ws, size_t 
         AB_LAUNCH_OK();
       }
       int64_t yt, yk;   // Ylong(k,t) = Y[t*yt + k*yk]
-      const bool parts = in_parts(it, p, p.r_cap, p.s, p.L) && (int64_t)p.r_cap * p.L <= (int64_t)kParts * s * s;      // one part at least
+      const bool parts = long_in_parts(it, p);
       if (parts) AB_TRY(long_parts(it, p, w.Vr, w.Y, lo.eig[s], stream));
       if (p.tall) {     // Y (m x r_cap) = W Vr^T
         if (!parts) AB_TRY(gemm_simt(it.W, it.w_dt, it.n, 1, w.Vr, AB_F32, 1, s, w.Y, AB_F32, p.r_cap, it.m, p.r_cap, it.n, stream));
