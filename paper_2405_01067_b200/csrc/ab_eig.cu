@@ -37,6 +37,7 @@ constexpr double kOrthTol = 4e-6;       // what the Jacobi route leaves at small
 constexpr int kMaxOrder = 1280;         // masks are sized for this order
 constexpr double kLive2 = 1e-290;       // a column whose squared norm is below this needs no reflector
 constexpr int kGroup = 8;               // reflectors applied together in the back transform
+constexpr int kFewClose = 12;           // up to this many close vectors above one are compared with it one by one
 
 // Reflectors are rows of an even number of doubles (bulk copies of whole rows start and end on 16 bytes), zero before and
 // behind their elements.
@@ -1143,18 +1144,35 @@ back_transform_kernel(const EigJob* __restrict__ jobs, int* status) {
         z[q][e] = (mine < job.need && k < s) ? job.zp[(size_t)k * s + i] * inv : 0.0;
       }
   }
-  // neighbours too close for the factorisation to keep apart: is this vector orthogonal to those above it?
+  // Neighbours too close for the factorisation to keep apart: is this vector orthogonal to those above it?  A few pairs are formed by
+  // the whole warp, one after the other, more of them side by side, a lane each: neighbours in the order are neighbours in memory.
   for (int q = q0 + sub; q < min(q0 + 8, job.need); q += RS) {
     const int i = position(q);
     const double li = job.lam[i];
     if (!(li > null_rel(job))) continue;
-    for (int p = q - 1; p >= 0; --p) {
-      const int k = position(p);
-      if (!(fabs(job.lam[k] - li) < kCloseRel)) break;
+    for (int top = q - 1; top >= 0; top -= 32) {           // a lane a neighbour
+      const int p = top - lane, k = p >= 0 ? position(p) : i;
+      const unsigned apart = __ballot_sync(0xffffffffu, !(p >= 0 && fabs(job.lam[k] - li) < kCloseRel));
+      const int n = apart ? __ffs(apart) - 1 : 32;
       double acc = 0.0;
-      for (int c = lane; c < s; c += 32) acc = fma(job.zp[(size_t)c * s + i], job.zp[(size_t)c * s + k], acc);
-      acc = warp_sum(acc) * job.inv[i] * job.inv[k];
-      if (!(fabs(acc) <= kOrthTol) && lane == 0) *job.flag = 1;
+      if (n > kFewClose) {
+        if (lane < n) {
+          const double *zi = job.zp + i, *zk = job.zp + k;
+#pragma unroll 16
+          for (int c = 0; c < s; ++c) acc = fma(zi[(size_t)c * s], zk[(size_t)c * s], acc);
+        }
+      } else {
+        for (int u = 0; u < n; ++u) {
+          const int ku = __shfl_sync(0xffffffffu, k, u);
+          double t = 0.0;
+#pragma unroll 4
+          for (int c = lane; c < s; c += 32) t = fma(job.zp[(size_t)c * s + i], job.zp[(size_t)c * s + ku], t);
+          t = warp_sum(t);
+          if (lane == u) acc = t;
+        }
+      }
+      if (lane < n && !(fabs(acc * job.inv[i] * job.inv[k]) <= kOrthTol)) *job.flag = 1;
+      if (n < 32) break;
     }
   }
   BackState<TW, RS, W> x{fs, ts, ys, bars, &dead, 0, 0, ngroups - 1, sub, vg, lane};
