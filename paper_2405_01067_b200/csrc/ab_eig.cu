@@ -8,8 +8,9 @@
 //   4. back_transform_kernel: u = H z, rows sorted by descending eigenvalue, rounded to fp32
 //
 // Everything up to the last rounding is fp64.  C = M^T M is formed in fp64 from the fp32 matrix M, so an
-// eigenvalue carries an absolute error of 1e-16 of the largest and squaring costs no accuracy: a singular value
-// of 1 % of the largest is good to 1e-12 before it is rounded to fp32.
+// eigenvalue carries an absolute error of up to 4e-15 of the largest (2e-14 above order 256, where the words that cross the device
+// keep 44 bits) and squaring costs no accuracy: a singular value of 1 % of the largest is good to 2e-11 before it is
+// rounded to fp32.
 //
 // Why not the one-sided Jacobi that this replaces (it stays as the fallback, see below): its sweeps are chains of
 // dependent steps -- s - 1 rounds a sweep, eight to thirteen sweeps, every step a dot product, a reduction across a warp, a
@@ -406,9 +407,9 @@ __device__ __forceinline__ double sum_warps(const double* red) {
 }
 
 // A step.  With x = v1 gamma and y = 2 c v1 - gamma p_j (c = gamma^2 p.v / 2) column j + 1 of the updated matrix is
-// (a - x p) + y v, where only y waits for a sum.  The sum of its squares and their root stand beside the pass over the rows (the
-// CTA's warps meet between its halves): what follows from them is needed for element j + 1 of the reflector alone, whose products are
-// added as the row sums leave.
+// (a - x p) + y v, where only y waits for a sum.  The sum of its squares goes through the CTA's reduction of the row sums: their root
+// is needed for element j + 1 of the reflector alone, whose products are added as the row sums leave.  Split of 3072 x 768
+// 2130 us, 2000 x 600 1700; with the squares reduced and their root taken between the halves of the pass (a barrier more) 2240 and 1811.
 template <int E, int W>
 __global__ void __launch_bounds__(32 * W, 1)
 tridiag_grid_kernel(const EigJob* __restrict__ jobs, int count, int C, int* status) {
@@ -526,8 +527,6 @@ tridiag_grid_kernel(const EigJob* __restrict__ jobs, int count, int C, int* stat
         sq = fma(vn[e], vn[e], sq);
       }
       const double dj = qj.y - 2.0 * v1 * wj, alpha = fma(y, vj1, fma(-x, qj1.x, qj1.y));
-      sq = warp_sum(sq);
-      if (lane == 0) red_sq[warp] = sq;
       double ps[R];
 #pragma unroll
       for (int h = 0; h < R; h += 4) {
@@ -544,25 +543,16 @@ tridiag_grid_kernel(const EigJob* __restrict__ jobs, int count, int C, int* stat
             }
           }
         }
-        if (h == 0) __syncthreads();                     // the parts of the squares are there
       }
-      sq = sum_warps<W>(red_sq);                         // the same in all CTAs: they work on the same bits
-      const bool live = sq > kLive2;
-      const double nrm = sqrt(fma(alpha, alpha, sq));
-      const double beta = live ? (alpha > 0.0 ? -nrm : nrm) : alpha;
-      v1 = live ? alpha - beta : 0.0;
 #pragma unroll
       for (int e = 0; e < E; ++e) {
         const int k = tid + T * e;
-        if (!live) vn[e] = 0.0;
         if (k == j + 1) {
-          vn[e] = v1;
 #pragma unroll
           for (int r = 0; r < R; ++r) colbuf[r] = A[r][e];
         }
         if (k == j + 2) vnext = vn[e];
         if (slot[e] >= 0) vrow[slot[e]] = vn[e];
-        v[e] = vn[e];
       }
       {
         // eight row sums across the warp: lanes 4 r ... hold sum r
@@ -576,8 +566,15 @@ tridiag_grid_kernel(const EigJob* __restrict__ jobs, int count, int C, int* stat
         t += __shfl_xor_sync(0xffffffffu, t, 2);
         t += __shfl_xor_sync(0xffffffffu, t, 1);
         if ((lane & 3) == 0) red_row[lane >> 2][warp] = t;
+        sq = warp_sum(sq);
+        if (lane == 0) red_sq[warp] = sq;
       }
       __syncthreads();
+      sq = sum_warps<W>(red_sq);                         // the same in all CTAs: they work on the same bits
+      const bool live = sq > kLive2;
+      const double nrm = sqrt(fma(alpha, alpha, sq));
+      const double beta = live ? (alpha > 0.0 ? -nrm : nrm) : alpha;
+      v1 = live ? alpha - beta : 0.0;
       if (tid < R) {
         const int i = cta + C * tid;
         if (i > j && i < s) {
@@ -588,6 +585,8 @@ tridiag_grid_kernel(const EigJob* __restrict__ jobs, int count, int C, int* stat
       gam = live ? 1.0 / (nrm * (nrm + fabs(alpha))) : 0.0;
       x = v1 * gam;
       tag = next_tag;
+#pragma unroll
+      for (int e = 0; e < E; ++e) v[e] = tid + T * e == j + 1 ? v1 : live ? vn[e] : 0.0;
       // what later kernels need, from the owner of row j + 1 (its cluster is still here)
       if ((j + 1) % C == cta) {
         const int ld = refl_ld(s);
