@@ -531,7 +531,7 @@ gather_rows_kernel(const float* __restrict__ Vt, const int* __restrict__ perm, i
 // sigma[k] = norm over t of Ylong(k,t), Ylong(k,t) = Y[t*st_ + k*sk].
 // Neighbouring k adjacent in memory: a cluster of kNormCl CTAs takes 32 values of k, a lane each, the warps of all of them
 // sharing the t; the parts are added in the order of the warps.  One CTA to 32 values walked 3072 rows in
-// 384 dependent rounds: 57 us for 192 values, 4 of them now.  Neighbouring t adjacent: a CTA a k (70 us -> 5, 128 values of 2304).
+// 384 dependent rounds: 57 us for 192 values, 10 now.  Neighbouring t adjacent: a CTA a k (70 us -> 5, 128 values of 2304).
 constexpr int kNormCl = 8;
 __global__ void __launch_bounds__(256)
 long_norms_kernel(const float* __restrict__ Y, int64_t st_, int L, int r_cap, float* __restrict__ sigma) {
